@@ -22,13 +22,13 @@
 //      operand.
 //
 // Roles (11 warps):
-//   warp 0 (one lane)  P producer: per k-block of 128 a 128 x 128 int8 TMA
+//   warp 0             P producer: per k-block of 128 a 128 x 128 int8 TMA
 //                      box of P (128-byte rows, 128-byte swizzle) into a
 //                      deep ring of its own.  Every row of a TMA box is a
 //                      request of its own; 128-byte rows move twice the
 //                      bytes per request of 64-byte ones (measured on
 //                      GB300: twice the bytes per second per SM).
-//   warp 10 (one lane) Q producer: Q's image with one bulk copy into a
+//   warp 10            Q producer: Q's image with one bulk copy into a
 //                      shallow ring (Q is read from L2).
 //   warps 6..9         converters: lane r of the warp with TMEM lane
 //                      quadrant q converts P row 32 q + r (128 int8, read
@@ -36,7 +36,7 @@
 //                      bf16 pairs and writes them to one of NA P slots in
 //                      TMEM (tcgen05.st, lane = row, the lower k of a pair
 //                      in the low half).
-//   warp 1 (one lane)  MMA issuer: tcgen05.mma kind::f16 with A in TMEM and
+//   warp 1             MMA issuer: tcgen05.mma kind::f16 with A in TMEM and
 //                      B in shared memory, into one of two TMEM accumulators
 //                      of QN fp32 columns.
 //   warps 2..5         epilogue: lane r of quadrant q owns P row 32 q + r.
@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(kThreadsS8tm, 1)
   auto acce_bar = [&](uint32_t b) { return bars + 8u * (2 * SP + 2 * SQ + 2 * NA + 2 + b); };
   const uint32_t drain_bar = bars + 8u * (2 * SP + 2 * SQ + 2 * NA + 4);
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);  // warp-uniform for the compiler
   const int lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
@@ -249,20 +249,20 @@ __global__ void __launch_bounds__(kThreadsS8tm, 1)
 
   if (warp == 0 || warp == kQWarp) {
     // -------------------------------------------- producers (P, then Q)
-    if (lane == 0) {
-      const bool is_p = warp == 0;
-      if (!is_p) griddep_wait();
-      const int ns = is_p ? SP : SQ;
-      uint32_t g = 0;
-      bool ok = true;
-      for (int u = blockIdx.x; ok && u < num_units; u += gridDim.x) {
-        const S8tmUnit w = decode_s8tm(p, u);
-        for (int kb = w.kb0; kb < w.kb1; ++kb) {
-          const uint32_t s = g % ns, ph = (g / ns) & 1u;
-          if (!mbar_wait(is_p ? pempty_bar(s) : qempty_bar(s), ph ^ 1u, abort_flag, p.err, p.wait_limit_ns)) {
-            ok = false;
-            break;
-          }
+    const bool is_p = warp == 0;
+    if (!is_p) griddep_wait();
+    const uint32_t ns = is_p ? SP : SQ;
+    uint32_t s = 0, ph = 0, g = 0;  // stage, its phase, copies issued
+    bool ok = true;
+    for (int u = blockIdx.x; ok && u < num_units; u += gridDim.x) {
+      const S8tmUnit w = decode_s8tm(p, u);
+      const uint8_t *q_src = static_cast<const uint8_t *>(p.q_img) + (int64_t)w.tq * p.num_kb * (int64_t)Cfg::kQBytes;
+      for (int kb = w.kb0; kb < w.kb1; ++kb) {
+        if (!mbar_wait_warp(is_p ? pempty_bar(s) : qempty_bar(s), ph ^ 1u, abort_flag, p.err, p.wait_limit_ns)) {
+          ok = false;
+          break;
+        }
+        if (elect_one()) {
           if (is_p) {
             mbar_arrive_expect_tx(pfull_bar(s), kPBytes);
             if constexpr (PK)
@@ -271,68 +271,78 @@ __global__ void __launch_bounds__(kThreadsS8tm, 1)
               tma_load_2d(sP + s * kPBytes, &tmP, w.tp * kBM, kb * kKB, pfull_bar(s));
           } else {
             mbar_arrive_expect_tx(qfull_bar(s), Cfg::kQBytes);
-            const uint8_t *q_src = static_cast<const uint8_t *>(p.q_img) +
-                                   ((int64_t)w.tq * p.num_kb + kb) * (int64_t)Cfg::kQBytes;
-            bulk_load(sQ + s * Cfg::kQBytes, q_src, Cfg::kQBytes, qfull_bar(s));
+            bulk_load(sQ + s * Cfg::kQBytes, q_src + (int64_t)kb * (int64_t)Cfg::kQBytes, Cfg::kQBytes, qfull_bar(s));
           }
-          ++g;
+        }
+        __syncwarp();
+        ++g;
+        if (++s == ns) {
+          s = 0;
+          ph ^= 1u;
         }
       }
-      // Every copy this thread issued has landed before the CTA may exit.
-      const uint32_t first = g > (uint32_t)ns ? g - ns : 0u;
-      for (uint32_t i = first; i < g; ++i)
-        mbar_wait_drain(is_p ? pfull_bar(i % ns) : qfull_bar(i % ns), (i / ns) & 1u, kDrainNs);
     }
+    // Every copy this warp issued has landed before the CTA may exit.
+    const uint32_t first = g > ns ? g - ns : 0u;
+    for (uint32_t i = first; i < g; ++i)
+      mbar_wait_drain(is_p ? pfull_bar(i % ns) : qfull_bar(i % ns), (i / ns) & 1u, kDrainNs);
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------- MMA issuer
-    if (lane == 0) {
-      constexpr uint32_t idesc = idesc_bf16_f32(kBM, QN, false);
-      uint32_t g = 0, acc_cnt = 0;
-      bool ok = true;
-      for (int u = blockIdx.x; ok && u < num_units; u += gridDim.x) {
-        const S8tmUnit w = decode_s8tm(p, u);
-        for (int kb_s = w.kb0; ok && kb_s < w.kb1; kb_s += p.slab_kb) {
-          const int kb_e = min(w.kb1, kb_s + p.slab_kb);
-          const uint32_t b = acc_cnt & 1u, aph = (acc_cnt >> 1) & 1u;
-          if (!mbar_wait(acce_bar(b), aph ^ 1u, abort_flag, p.err, p.wait_limit_ns)) {
+    constexpr uint32_t idesc = idesc_bf16_f32(kBM, QN, false);
+    // K-major, 128-byte swizzle, 8-row atoms 1024 bytes apart
+    const uint64_t dq = smem_desc_sw128(sQ, 16, 1024);
+    uint32_t s = 0, ph = 0, a = 0, tph = 0, acc_cnt = 0;
+    bool ok = true;
+    for (int u = blockIdx.x; ok && u < num_units; u += gridDim.x) {
+      const S8tmUnit w = decode_s8tm(p, u);
+      for (int kb_s = w.kb0; ok && kb_s < w.kb1; kb_s += p.slab_kb) {
+        const int kb_e = min(w.kb1, kb_s + p.slab_kb);
+        const uint32_t b = acc_cnt & 1u, aph = (acc_cnt >> 1) & 1u;
+        if (!mbar_wait_warp(acce_bar(b), aph ^ 1u, abort_flag, p.err, p.wait_limit_ns)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after_sync();
+        const uint32_t d_tmem = tmem_base + b * QN;
+        for (int kb = kb_s; kb < kb_e; ++kb) {
+          if (!mbar_wait_warp(qfull_bar(s), ph, abort_flag, p.err, p.wait_limit_ns) ||
+              !mbar_wait_warp(tfull_bar(a), tph, abort_flag, p.err, p.wait_limit_ns)) {
             ok = false;
             break;
           }
           tc_fence_after_sync();
-          const uint32_t d_tmem = tmem_base + b * QN;
-          for (int kb = kb_s; kb < kb_e; ++kb) {
-            const uint32_t s = g % SQ, ph = (g / SQ) & 1u;
-            const uint32_t a = g % NA, tph = (g / NA) & 1u;
-            if (!mbar_wait(qfull_bar(s), ph, abort_flag, p.err, p.wait_limit_ns) ||
-                !mbar_wait(tfull_bar(a), tph, abort_flag, p.err, p.wait_limit_ns)) {
-              ok = false;
-              break;
-            }
-            tc_fence_after_sync();
-            const uint32_t q0 = sQ + s * Cfg::kQBytes;
+          if (elect_one()) {
+            const uint64_t q0 = dq + s * (Cfg::kQBytes / 16);
             const uint32_t a_tmem = tmem_base + Cfg::kPCol0 + a * 64;
 #pragma unroll
-            for (int k = 0; k < kKB / 16; ++k) {
+            for (int k = 0; k < kKB / 16; ++k)
               // one K step of 16 is 8 packed columns of the P slot, and 32
-              // bytes along the rows of Q's half k / 4 (K-major, 128-byte
-              // swizzle, 8-row atoms 1024 bytes apart)
-              const uint32_t qh = q0 + (k >> 2) * Cfg::kQHalf, kk = k & 3;
-              const uint64_t bd = smem_desc_sw128(qh + kk * 32, 16, 1024);
-              tc_mma_bf16_tmem_a(d_tmem, a_tmem + k * 8, bd, idesc, (kb > kb_s || k > 0) ? 1u : 0u);
-            }
+              // bytes along the rows of Q's half k / 4
+              tc_mma_bf16_tmem_a(d_tmem, a_tmem + k * 8, q0 + (k >> 2) * (Cfg::kQHalf / 16) + (k & 3) * 2, idesc,
+                                 (kb > kb_s || k > 0) ? 1u : 0u);
             tc_commit(qempty_bar(s));  // the Q stage may be refilled once these MMAs finish
             tc_commit(tempty_bar(a));  // and the P slot reused
-            ++g;
           }
-          if (!ok) break;
-          tc_commit(accf_bar(b));
-          ++acc_cnt;
+          __syncwarp();
+          if (++s == SQ) {
+            s = 0;
+            ph ^= 1u;
+          }
+          if (++a == NA) {
+            a = 0;
+            tph ^= 1u;
+          }
         }
+        if (!ok) break;
+        if (elect_one()) tc_commit(accf_bar(b));
+        __syncwarp();
+        ++acc_cnt;
       }
-      tc_commit(drain_bar);
-      mbar_wait_drain(drain_bar, 0, kDrainNs);
     }
+    if (elect_one()) tc_commit(drain_bar);
+    __syncwarp();
+    mbar_wait_drain(drain_bar, 0, kDrainNs);
     __syncwarp();
   } else if (warp >= 2 + kEpiWarps) {
     // ------------------------------------------------------- converters

@@ -3,14 +3,14 @@
 // One CTA per SM loops over output tiles (the paper's output-stationary
 // mapping, Sec. 4.2.1: M and N are spread in space over independent workers,
 // K is reduced in time into a stationary accumulator).  Roles:
-//   warp 0 (one lane)  TMA producer: streams 128 x 64 A boxes and BN x 64 B
+//   warp 0             TMA producer: streams 128 x 64 A boxes and BN x 64 B
 //                      boxes into a STAGES-deep shared-memory ring (the
 //                      paper's double-buffered L1/L2 input tiles, Sec. 4.2.1,
 //                      deepened), each stage guarded by a full/empty mbarrier
 //                      pair.  The box shapes and the 128-byte swizzle play the
 //                      part of the paper's on-the-fly DMA layout transforms
 //                      (Sec. 4.3): matrices stay row-/column-major in memory.
-//   warp 1 (one lane)  MMA issuer: tcgen05.mma kind::f16 (bf16 x bf16 -> fp32)
+//   warp 1             MMA issuer: tcgen05.mma kind::f16 (bf16 x bf16 -> fp32)
 //                      into one of two TMEM accumulators; the first MMA of a
 //                      tile overwrites instead of accumulating, which takes
 //                      the place of the paper's zeroing kernel (Sec. 4.2.1).
@@ -490,7 +490,7 @@ __global__ void __launch_bounds__(TcCfg<BN, STAGES, B_KMAJOR, EPI, EPI_WARPS, TM
   auto acce_bar = [&](uint32_t b) { return bars + 8u * (2 * STAGES + 2 + b); };
   const uint32_t drain_bar = bars + 8u * (2 * STAGES + 4);
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);  // warp-uniform for the compiler
   const int lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
@@ -525,17 +525,16 @@ __global__ void __launch_bounds__(TcCfg<BN, STAGES, B_KMAJOR, EPI, EPI_WARPS, TM
 
   if (warp == 0) {
     // ------------------------------------------------------ TMA producer
-    if (lane == 0) {
-      uint32_t g = 0;
-      bool ok = true;
-      for (int u = blockIdx.x; ok && u < num_units; u += gridDim.x) {
-        const Unit w = decode_unit(p, u);
-        for (int kb = w.kb0; kb < w.kb1; ++kb) {
-          const uint32_t s = g % STAGES, ph = (g / STAGES) & 1u;
-          if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, p.err, p.wait_limit_ns)) {
-            ok = false;
-            break;
-          }
+    uint32_t s = 0, ph = 0, g = 0;  // stage, its phase, loads issued
+    bool ok = true;
+    for (int u = blockIdx.x; ok && u < num_units; u += gridDim.x) {
+      const Unit w = decode_unit(p, u);
+      for (int kb = w.kb0; kb < w.kb1; ++kb) {
+        if (!mbar_wait_warp(empty_bar(s), ph ^ 1u, abort_flag, p.err, p.wait_limit_ns)) {
+          ok = false;
+          break;
+        }
+        if (elect_one()) {
           mbar_arrive_expect_tx(full_bar(s), Cfg::kStageBytes);
           tma_load_2d(sA + s * kABytes, &tmA, kb * kBK, w.tm * kBM, full_bar(s));
           const uint32_t b_dst = sB + s * Cfg::kBBytes;
@@ -546,63 +545,66 @@ __global__ void __launch_bounds__(TcCfg<BN, STAGES, B_KMAJOR, EPI, EPI_WARPS, TM
             for (int j = 0; j < BN / 64; ++j)
               tma_load_2d(b_dst + j * (kBK * 128), &tmB, w.tn * BN + 64 * j, kb * kBK, full_bar(s));
           }
-          ++g;
+        }
+        __syncwarp();
+        ++g;
+        if (++s == STAGES) {
+          s = 0;
+          ph ^= 1u;
         }
       }
-      // Every load this thread issued has landed before the CTA may exit.
-      const uint32_t first = g > (uint32_t)STAGES ? g - STAGES : 0u;
-      for (uint32_t i = first; i < g; ++i) mbar_wait_drain(full_bar(i % STAGES), (i / STAGES) & 1u, kDrainNs);
     }
-    __syncwarp();  // lanes 1..31 wait here, so the warp reaches the CTA barrier converged
+    // Every load this warp issued has landed before the CTA may exit.
+    const uint32_t first = g > (uint32_t)STAGES ? g - STAGES : 0u;
+    for (uint32_t i = first; i < g; ++i) mbar_wait_drain(full_bar(i % STAGES), (i / STAGES) & 1u, kDrainNs);
+    __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------- MMA issuer
-    if (lane == 0) {
-      constexpr uint32_t idesc = idesc_bf16_f32(kBM, BN, !B_KMAJOR);
-      uint32_t g = 0, acc_cnt = 0;
-      bool ok = true;
-      for (int u = blockIdx.x; ok && u < num_units; u += gridDim.x) {
-        const Unit w = decode_unit(p, u);
-        for (int kb_s = w.kb0; ok && kb_s < w.kb1; kb_s += p.slab_kb) {
-          const int kb_e = min(w.kb1, kb_s + p.slab_kb);
-          const uint32_t b = acc_cnt & 1u, aph = (acc_cnt >> 1) & 1u;
-          if (!mbar_wait(acce_bar(b), aph ^ 1u, abort_flag, p.err, p.wait_limit_ns)) {
+    constexpr uint32_t idesc = idesc_bf16_f32(kBM, BN, !B_KMAJOR);
+    // K-major, 128-byte swizzle: rows 128 B apart, 8-row atoms 1024 B apart;
+    // one MMA step of K = 16 is 32 bytes along a row.  MN-major B: 64-wide N
+    // chunks kBK*128 B apart (LBO), 8-row K groups 1024 B apart (SBO); a K
+    // step of 16 rows is 2048 B.
+    const uint64_t da = smem_desc_sw128(sA, 16, 1024);
+    const uint64_t db = B_KMAJOR ? smem_desc_sw128(sB, 16, 1024) : smem_desc_sw128(sB, kBK * 128, 1024);
+    constexpr uint32_t kBStep = B_KMAJOR ? 32 / 16 : 2048 / 16;
+    uint32_t s = 0, ph = 0, acc_cnt = 0;
+    bool ok = true;
+    for (int u = blockIdx.x; ok && u < num_units; u += gridDim.x) {
+      const Unit w = decode_unit(p, u);
+      for (int kb_s = w.kb0; ok && kb_s < w.kb1; kb_s += p.slab_kb) {
+        const int kb_e = min(w.kb1, kb_s + p.slab_kb);
+        const uint32_t b = acc_cnt & 1u, aph = (acc_cnt >> 1) & 1u;
+        if (!mbar_wait_warp(acce_bar(b), aph ^ 1u, abort_flag, p.err, p.wait_limit_ns)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after_sync();
+        const uint32_t d_tmem = tmem_base + b * BN;
+        for (int kb = kb_s; kb < kb_e; ++kb) {
+          if (!mbar_wait_warp(full_bar(s), ph, abort_flag, p.err, p.wait_limit_ns)) {
             ok = false;
             break;
           }
           tc_fence_after_sync();
-          const uint32_t d_tmem = tmem_base + b * BN;
-          for (int kb = kb_s; kb < kb_e; ++kb) {
-            const uint32_t s = g % STAGES, ph = (g / STAGES) & 1u;
-            if (!mbar_wait(full_bar(s), ph, abort_flag, p.err, p.wait_limit_ns)) {
-              ok = false;
-              break;
-            }
-            tc_fence_after_sync();
-            const uint32_t a0 = sA + s * kABytes;
-            const uint32_t b0 = sB + s * Cfg::kBBytes;
-#pragma unroll
-            for (int k = 0; k < kBK / 16; ++k) {
-              // K-major, 128-byte swizzle: rows 128 B apart, 8-row atoms
-              // 1024 B apart; one MMA step of K = 16 is 32 bytes along a row.
-              const uint64_t ad = smem_desc_sw128(a0 + k * 32, 16, 1024);
-              // MN-major B: 64-wide N chunks kBK*128 B apart (LBO), 8-row
-              // K groups 1024 B apart (SBO); a K step of 16 rows is 2048 B.
-              const uint64_t bd = B_KMAJOR ? smem_desc_sw128(b0 + k * 32, 16, 1024)
-                                           : smem_desc_sw128(b0 + k * 2048, kBK * 128, 1024);
-              tc_mma_bf16(d_tmem, ad, bd, idesc, (kb > kb_s || k > 0) ? 1u : 0u);
-            }
-            tc_commit(empty_bar(s));  // stage s is free once these MMAs finish
-            ++g;
+          // stage s is free once these MMAs finish
+          tc_mma_kstep<kBStep>(d_tmem, da + s * (kABytes / 16), db + s * (Cfg::kBBytes / 16), idesc,
+                               kb > kb_s ? 1u : 0u, empty_bar(s));
+          if (++s == STAGES) {
+            s = 0;
+            ph ^= 1u;
           }
-          if (!ok) break;
-          tc_commit(accf_bar(b));  // accumulator b is ready for the epilogue
-          ++acc_cnt;
         }
+        if (!ok) break;
+        if (elect_one()) tc_commit(accf_bar(b));  // accumulator b is ready for the epilogue
+        __syncwarp();
+        ++acc_cnt;
       }
-      // All MMAs complete before TMEM is released.
-      tc_commit(drain_bar);
-      mbar_wait_drain(drain_bar, 0, kDrainNs);
     }
+    // All MMAs complete before TMEM is released.
+    if (elect_one()) tc_commit(drain_bar);
+    __syncwarp();
+    mbar_wait_drain(drain_bar, 0, kDrainNs);
     __syncwarp();
   } else {
     // --------------------------------------------------------- epilogue

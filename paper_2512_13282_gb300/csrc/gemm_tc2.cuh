@@ -2,7 +2,7 @@
 //
 // A cluster of two CTAs on neighbouring SMs owns a 256 x BN output tile.
 // Each CTA loads its own 128 rows of A and one half (BN/2 rows/columns) of
-// B into its shared memory; one thread of the leader CTA (rank 0) issues
+// B into its shared memory; one warp of the leader CTA (rank 0) issues
 // tcgen05.mma.cta_group::2 with M = 256, which reads the A and B halves of
 // both CTAs and leaves rows 0..127 of the tile in the leader's TMEM and rows
 // 128..255 in the peer's.  Per SM this halves the B bytes moved per flop,
@@ -70,13 +70,25 @@ __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr) {
   asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "n"(kCols) : "memory");
 }
 
-__device__ __forceinline__ void tc_mma_bf16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
-                                                 uint32_t idesc, uint32_t accumulate) {
+// tc_mma_kstep on a CTA pair: M = 256, the commit arrives on the mbarrier
+// at offset `bar` in both CTAs.
+template <uint32_t kBStep>
+__device__ __forceinline__ void tc_mma_kstep_pair(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
+                                                  uint32_t accumulate, uint32_t bar) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      "{\n\t.reg .pred e, p, t;\n\t.reg .b64 a1, a2, a3, b1, b2, b3;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 t, 0, 0;\n\t"
+      "add.s64 a1, %1, 2;\n\tadd.s64 a2, %1, 4;\n\tadd.s64 a3, %1, 6;\n\t"
+      "add.s64 b1, %2, %6;\n\tadd.s64 b2, %2, %7;\n\tadd.s64 b3, %2, %8;\n\t"
+      "@e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t"
+      "@e tcgen05.mma.cta_group::2.kind::f16 [%0], a1, b1, %3, t;\n\t"
+      "@e tcgen05.mma.cta_group::2.kind::f16 [%0], a2, b2, %3, t;\n\t"
+      "@e tcgen05.mma.cta_group::2.kind::f16 [%0], a3, b3, %3, t;\n\t"
+      "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%5], %9;\n\t}" ::
+          "r"(d_tmem),
+      "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(bar), "n"(kBStep), "n"(2 * kBStep), "n"(3 * kBStep),
+      "h"((uint16_t)0x3)
       : "memory");
 }
 
@@ -141,10 +153,11 @@ __global__ void __launch_bounds__(Tc2Cfg<BN, STAGES, B_KMAJOR, EPI, EPI_WARPS, T
   auto acce_bar = [&](uint32_t b) { return bars + 8u * (2 * STAGES + 2 + b); };
   const uint32_t drain_bar = bars + 8u * (2 * STAGES + 4);
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);  // warp-uniform for the compiler
   const int lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const bool leader = rank == 0;
+  const uint32_t full_leader = mapa_shared(full_bar(0), 0);  // the leader's full barriers (shared::cluster)
   const int cluster = blockIdx.x >> 1;
   const int num_clusters = gridDim.x >> 1;
 
@@ -181,22 +194,22 @@ __global__ void __launch_bounds__(Tc2Cfg<BN, STAGES, B_KMAJOR, EPI, EPI_WARPS, T
 
   if (warp == 0) {
     // ---------------------------------------------- TMA producer (both CTAs)
-    if (lane == 0) {
-      uint32_t g = 0;
-      bool ok = true;
-      for (int u = cluster; ok && u < num_units; u += num_clusters) {
-        const Unit w = decode_unit(p, u);
-        for (int kb = w.kb0; kb < w.kb1; ++kb) {
-          const uint32_t s = g % STAGES, ph = (g / STAGES) & 1u;
-          if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, p.err, p.wait_limit_ns)) {
-            ok = false;
-            break;
-          }
+    uint32_t s = 0, ph = 0, g = 0;  // stage, its phase, loads issued
+    bool ok = true;
+    for (int u = cluster; ok && u < num_units; u += num_clusters) {
+      const Unit w = decode_unit(p, u);
+      const int n0 = w.tn * BN + (int)rank * Cfg::kHalfN;
+      const int m0 = w.tm * kTileM + (int)rank * kBM;
+      for (int kb = w.kb0; kb < w.kb1; ++kb) {
+        if (!mbar_wait_warp(empty_bar(s), ph ^ 1u, abort_flag, p.err, p.wait_limit_ns)) {
+          ok = false;
+          break;
+        }
+        if (elect_one()) {
           if (leader) mbar_arrive_expect_tx(full_bar(s), 2 * Cfg::kStageBytes);
-          const uint32_t fb = mapa_shared(full_bar(s), 0);
-          tma_load_2d_pair(sA + s * kABytes, &tmA, kb * kBK, w.tm * kTileM + (int)rank * kBM, fb);
+          const uint32_t fb = full_leader + 8u * s;
+          tma_load_2d_pair(sA + s * kABytes, &tmA, kb * kBK, m0, fb);
           const uint32_t b_dst = sB + s * Cfg::kBBytes;
-          const int n0 = w.tn * BN + (int)rank * Cfg::kHalfN;
           if constexpr (B_KMAJOR) {
             tma_load_2d_pair(b_dst, &tmB, kb * kBK, n0, fb);
           } else {
@@ -204,64 +217,63 @@ __global__ void __launch_bounds__(Tc2Cfg<BN, STAGES, B_KMAJOR, EPI, EPI_WARPS, T
             for (int j = 0; j < Cfg::kHalfN / 64; ++j)
               tma_load_2d_pair(b_dst + j * (kBK * 128), &tmB, n0 + 64 * j, kb * kBK, fb);
           }
-          ++g;
+        }
+        __syncwarp();
+        ++g;
+        if (++s == STAGES) {
+          s = 0;
+          ph ^= 1u;
         }
       }
-      if (leader) {
-        const uint32_t first = g > (uint32_t)STAGES ? g - STAGES : 0u;
-        for (uint32_t i = first; i < g; ++i)
-          mbar_wait_drain(full_bar(i % STAGES), (i / STAGES) & 1u, kDrainNs);
-      } else {
-        // the peer's loads complete on the leader's barriers; wait until the
-        // leader's MMAs have released the stages they filled
-        const uint32_t first = g > (uint32_t)STAGES ? g - STAGES : 0u;
-        for (uint32_t i = first; i < g; ++i)
-          mbar_wait_drain(empty_bar(i % STAGES), (i / STAGES) & 1u, kDrainNs);
-      }
     }
+    // Before the CTA may exit: the leader's loads have landed; the peer's
+    // complete on the leader's barriers, so it waits until the leader's MMAs
+    // have released the stages they filled.
+    const uint32_t first = g > (uint32_t)STAGES ? g - STAGES : 0u;
+    for (uint32_t i = first; i < g; ++i)
+      mbar_wait_drain(leader ? full_bar(i % STAGES) : empty_bar(i % STAGES), (i / STAGES) & 1u, kDrainNs);
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer (leader)
-    if (lane == 0 && leader) {
+    if (leader) {
       constexpr uint32_t idesc = idesc_bf16_f32(kTileM, BN, !B_KMAJOR);
-      uint32_t g = 0, acc_cnt = 0;
+      const uint64_t da = smem_desc_sw128(sA, 16, 1024);
+      const uint64_t db = B_KMAJOR ? smem_desc_sw128(sB, 16, 1024) : smem_desc_sw128(sB, kBK * 128, 1024);
+      constexpr uint32_t kBStep = B_KMAJOR ? 32 / 16 : 2048 / 16;
+      uint32_t s = 0, ph = 0, acc_cnt = 0;
       bool ok = true;
       for (int u = cluster; ok && u < num_units; u += num_clusters) {
         const Unit w = decode_unit(p, u);
         for (int kb_s = w.kb0; ok && kb_s < w.kb1; kb_s += p.slab_kb) {
           const int kb_e = min(w.kb1, kb_s + p.slab_kb);
           const uint32_t b = acc_cnt & 1u, aph = (acc_cnt >> 1) & 1u;
-          if (!mbar_wait(acce_bar(b), aph ^ 1u, abort_flag, p.err, p.wait_limit_ns)) {
+          if (!mbar_wait_warp(acce_bar(b), aph ^ 1u, abort_flag, p.err, p.wait_limit_ns)) {
             ok = false;
             break;
           }
           tc_fence_after_sync();
           const uint32_t d_tmem = tmem_base + b * BN;
           for (int kb = kb_s; kb < kb_e; ++kb) {
-            const uint32_t s = g % STAGES, ph = (g / STAGES) & 1u;
-            if (!mbar_wait(full_bar(s), ph, abort_flag, p.err, p.wait_limit_ns)) {
+            if (!mbar_wait_warp(full_bar(s), ph, abort_flag, p.err, p.wait_limit_ns)) {
               ok = false;
               break;
             }
             tc_fence_after_sync();
-            const uint32_t a0 = sA + s * kABytes;
-            const uint32_t b0 = sB + s * Cfg::kBBytes;
-#pragma unroll
-            for (int k = 0; k < kBK / 16; ++k) {
-              const uint64_t ad = smem_desc_sw128(a0 + k * 32, 16, 1024);
-              const uint64_t bd = B_KMAJOR ? smem_desc_sw128(b0 + k * 32, 16, 1024)
-                                           : smem_desc_sw128(b0 + k * 2048, kBK * 128, 1024);
-              tc_mma_bf16_pair(d_tmem, ad, bd, idesc, (kb > kb_s || k > 0) ? 1u : 0u);
+            tc_mma_kstep_pair<kBStep>(d_tmem, da + s * (kABytes / 16), db + s * (Cfg::kBBytes / 16), idesc,
+                                      kb > kb_s ? 1u : 0u, empty_bar(s));
+            if (++s == STAGES) {
+              s = 0;
+              ph ^= 1u;
             }
-            tc_commit_pair_multicast(empty_bar(s));
-            ++g;
           }
           if (!ok) break;
-          tc_commit_pair_multicast(accf_bar(b));
+          if (elect_one()) tc_commit_pair_multicast(accf_bar(b));
+          __syncwarp();
           ++acc_cnt;
         }
       }
-      tc_commit_pair_multicast(drain_bar);
+      if (elect_one()) tc_commit_pair_multicast(drain_bar);
+      __syncwarp();
       mbar_wait_drain(drain_bar, 0, kDrainNs);
     }
     __syncwarp();
