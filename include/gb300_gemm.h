@@ -259,7 +259,10 @@ enum {
   GEMM_ROUTE_SMALL_OPERAND = 3,  /* int8 with one operand of <= 128 rows, converted in the kernel */
   GEMM_ROUTE_TC_SINGLE = 4,      /* tensor-core kernel, one CTA per 128 x BN tile */
   GEMM_ROUTE_TC_PAIR = 5,        /* tensor-core kernel, a CTA pair per 256 x BN tile */
-  GEMM_ROUTE_TINY = 6            /* int8 problem small enough for one CUDA-core launch */
+  GEMM_ROUTE_TINY = 6,           /* int8 problem small enough for one CUDA-core launch */
+  GEMM_ROUTE_FEW_ROWS = 7        /* <= 16 rows (or columns) against a K-contiguous operand, streamed
+                                    into warp matrix instructions (bn: rows of that operand per
+                                    block, splits: blocks of a cluster along K) */
 };
 typedef struct {
   int route;

@@ -78,7 +78,8 @@ namespace {
 // CUDA-core kernel, GB300_GEMM_TMA_STORE=0 direct stores (and scalar atomic
 // adds for the small-operand kernel's split-K), GB300_GEMM_PDL=0
 // plain stream ordering, GB300_GEMM_S8TM=0 the general int8 path for
-// small-operand shapes, GB300_GEMM_TINY_MAX_MACS the largest
+// small-operand shapes; a forced tile plan or small-M limit also turns the
+// few-row kernel off, GB300_GEMM_TINY_MAX_MACS the largest
 // int8 problem (M * N * K) sent to the one-launch CUDA-core kernel (0
 // disables it), GB300_GEMM_DEBUG=1 prints each plan.
 struct Overrides {
@@ -720,6 +721,69 @@ gemm_status_t run_skinny(DeviceState &d, int64_t M, int64_t N, int64_t K, const 
   return GEMM_OK;
 }
 
+// Rows of the small operand up to which gemm_rows_kernel takes a GEMM (0
+// where an override asks for another kernel).  Up to 16 rows it is faster
+// than the kernels that took those shapes before at every size measured
+// (gemm_rows.cu has the figures); its accumulators are built for 16.
+int rows_max(bool int8) {
+  const Overrides o = overrides();
+  if (o.skinny_max_m >= 0 || o.bn > 0 || o.pair >= 0 || o.splits >= 1 || o.tail_splits >= 2) return 0;
+  return int8 && !o.s8tm ? 0 : kRowsMax;
+}
+
+// Which operand gemm_rows_kernel streams, if any: B (stored N x K) against
+// the rows of A, or A against the columns of B (small_n).  A bf16 A with a
+// short K goes to the tensor-core kernels, whose TMA stores take C's narrow
+// rows better (7000 x 16 x 512: 4.3 us against 4.6; 8192 x 8 x 2000: level;
+// 4096 x 16 x 4096: 9.9 against 8.4).
+constexpr int64_t kRowsMinKNarrowBf16 = 1024;
+bool rows_shape(int64_t M, int64_t N, int64_t K, bool b_kmajor, bool int8, bool *small_n) {
+  const int lim = rows_max(int8);
+  *small_n = M > lim;
+  if (*small_n && !int8 && K < kRowsMinKNarrowBf16) return false;
+  return b_kmajor && (M <= lim || N <= lim);
+}
+
+// GEMMs with at most kRowsMax rows of A against a column-major B, or at most
+// kRowsMax columns of a column-major B against A: gemm_rows_kernel streams the
+// other operand, which has to be 16-byte aligned in base and pitch.  Returns
+// false, having launched nothing, for any other.
+bool try_rows(DeviceState &d, int64_t M, int64_t N, int64_t K, const void *A, int64_t lda, const void *B,
+              int64_t ldb, bool b_kmajor, void *C, int64_t ldc, bool int8, int out_bits, int out_shift,
+              cudaStream_t st, gemm_status_t *status) {
+  bool small_n;
+  if (!rows_shape(M, N, K, b_kmajor, int8, &small_n)) return false;
+  const int es = int8 ? 1 : 2;
+  RowsParams p{};
+  p.W = small_n ? A : B;
+  p.ldw = small_n ? lda : ldb;
+  if (!aligned16(p.W) || p.ldw * es % 16 != 0) return false;
+  p.NW = small_n ? M : N;
+  p.X = small_n ? B : A;
+  p.ldx = small_n ? ldb : lda;
+  p.R = (int)(small_n ? N : M);
+  p.scr = small_n ? 1 : ldc;
+  p.scn = small_n ? ldc : 1;
+  p.K = (int)K;
+  p.x_vec = aligned16(p.X) && p.ldx * es % 16 == 0;
+  p.C = C;
+  p.out_bits = out_bits;
+  p.out_shift = out_shift;
+  const int64_t strips = rows_geometry(p.NW, K, int8, d.sms, &p.cluster, &p.kslice);
+  *status = GEMM_ERR_CUDA;
+  const bool prof = g_prof_start && g_prof_stop;
+  if (prof && cudaEventRecord(g_prof_start, st) != cudaSuccess) return true;
+  g_launches.fetch_add(1);
+  const cudaError_t e = launch_rows(p, int8, strips, st);
+  if (e != cudaSuccess) {
+    *status = cuda_failed("few-row kernel launch", e);
+    return true;
+  }
+  if (prof && cudaEventRecord(g_prof_stop, st) != cudaSuccess) return true;
+  *status = GEMM_OK;
+  return true;
+}
+
 }  // namespace
 
 extern "C" {
@@ -738,6 +802,7 @@ gemm_status_t gemm_bf16_f32acc_bf16(int64_t M, int64_t N, int64_t K, const uint1
     return launch_zero_fill(C, M, N, ldc, 2, d->sms, st) == cudaSuccess ? GEMM_OK : GEMM_ERR_CUDA;
   }
   const bool b_kmajor = b_layout == GEMM_B_COL_MAJOR_NxK;
+  if (try_rows(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, false, 0, 0, st, &s)) return s;
   if (M <= skinny_max_m(false))
     return run_skinny(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, false, st);
   Plan pl = make_plan(M, N, K, b_kmajor, kEpiBf16, d->sms, pair_slots());
@@ -976,6 +1041,7 @@ gemm_status_t s8_gemm(int64_t M, int64_t N, int64_t K, const int8_t *A, int64_t 
     return launch_zero_fill(C, M, N, ldc, out_esize, d->sms, st) == cudaSuccess ? GEMM_OK : GEMM_ERR_CUDA;
   }
   const bool b_kmajor = b_layout == GEMM_B_COL_MAJOR_NxK;
+  if (try_rows(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, true, out_bits, shift, st, &s)) return s;
   if (M <= skinny_max_m(true))
     return run_skinny(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, true, st, out_bits, shift);
   if ((double)M * (double)N * (double)K <= (double)tiny_max_macs()) {
@@ -1112,6 +1178,17 @@ gemm_status_t gemm_plan_query(int64_t M, int64_t N, int64_t K, int int8, int b_l
   }
   if (K == 0) {
     out->route = GEMM_ROUTE_ZERO_FILL;
+    return GEMM_OK;
+  }
+  bool small_n;
+  // tight leading dimensions: both operands' pitch is K
+  if (rows_shape(M, N, K, b_kmajor, int8 != 0, &small_n) && K * (int8 ? 1 : 2) % 16 == 0) {
+    int cluster, kslice;
+    const int64_t strips = rows_geometry(small_n ? M : N, K, int8 != 0, sms, &cluster, &kslice);
+    out->route = GEMM_ROUTE_FEW_ROWS;
+    out->bn = 32;
+    out->splits = cluster;
+    out->grid = (int)(strips * cluster);
     return GEMM_OK;
   }
   if (M <= skinny_max_m(int8 != 0)) {

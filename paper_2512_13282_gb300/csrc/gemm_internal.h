@@ -183,6 +183,27 @@ struct TinyParams {
 };
 cudaError_t launch_tiny_s8(const TinyParams &p, bool row_b, cudaStream_t st);
 
+// GEMM with one operand of at most 16 rows (gemm_rows.cu):
+// out(r, n) = sum_k X(r, k) * W(n, k) for r < R, n < NW, stored at element
+// r * scr + n * scn of C.  The rows of W and X are K contiguous; W's start on
+// 16-byte boundaries.
+constexpr int kRowsMax = 16;
+struct RowsParams {
+  const void *W;
+  int64_t ldw;  // row pitch in elements
+  int64_t NW;
+  const void *X;
+  int64_t ldx;
+  int R, K;
+  int x_vec;  // X's rows start on 16-byte boundaries
+  void *C;
+  int64_t scr, scn;
+  int cluster, kslice;  // rows_geometry
+  int out_bits, out_shift;
+};
+int64_t rows_geometry(int64_t NW, int64_t K, bool int8, int sms, int *cluster, int *kslice);
+cudaError_t launch_rows(const RowsParams &p, bool int8, int64_t strips, cudaStream_t st);
+
 // Small-M GEMM on the CUDA cores (gemm_skinny.cu).  M <= 16.
 struct SkinnyParams {
   const void *A;

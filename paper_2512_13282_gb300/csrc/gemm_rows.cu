@@ -1,0 +1,348 @@
+// gemm_rows.cu -- GEMMs with one operand of at most 16 rows against an
+// operand whose rows are K contiguous (a decode batch or one token against
+// weights stored N x K, a tall matrix against a narrow weight): the large
+// operand W goes from HBM into registers that already are operands of warp
+// matrix instructions.
+//
+// With so few rows the time is the time to read W once, plus whatever the
+// kernel spends before its first and after its last byte.  The tcgen05
+// kernels pass every byte through a shared-memory ring (and, for int8,
+// through converter warps and tensor memory) and pay those hand-offs per
+// k-block; here a lane loads 16 bytes of W and multiplies them:
+//
+//   - W is the 16-row A operand of mma.sync m16n8k16, X (the small operand)
+//     the 8-column B operand, so X costs ceil(rows / 8) instructions per
+//     16 x 16 of W.
+//   - The sum over k does not depend on its order, so the four k slots a
+//     lane (g = lane / 4, q = lane % 4) holds of a k16 step are given four
+//     consecutive k of its own 16 bytes, and X is read at the same k: W's
+//     registers are MMA operands as they are loaded, without a shuffle.
+//   - int8: a byte b becomes the fp16 1024 + (b + 128) by placing it under
+//     the exponent of 1024, and one packed subtraction of 1152 leaves b
+//     exactly (five instructions per four values); products are at most
+//     2^14 and an accumulator takes at most 512 of them before it is added
+//     to int32, so every fp32 sum is an integer of at most 2^23, exact.
+//
+// A block of four warps owns 32 rows of W and a K slice; the warps take
+// 128-byte deep batches of the slice in turn and are summed in warp order in
+// shared memory.  K is split over the blocks of a cluster (1-8), whose sums
+// meet in distributed shared memory in rank order: results do not depend on
+// scheduling, and there are no partials in global memory, no counters and no
+// second launch.  Each half of a batch is reloaded as soon as it has been
+// multiplied, so that a lane keeps about 128 bytes in flight.  A block asks
+// for its first batches in L2 before it waits for the previous kernel of the
+// stream (a prefetch reads nothing into the block, so it does not matter
+// whether that kernel still writes W).
+//
+// What bounds it: the HBM stream (5.0-5.6 TB/s of W on 100 MB) and, for the
+// smaller calls, the ~3 us from launch to last store.  Measured on GB300,
+// calls back to back on operands larger than L2, against the kernel that took
+// the shape before (B stored N x K, K = 4096 unless given): int8 16 x 12288
+// 17.7 -> 13.2 us, 16 x 4096 10.4 -> 6.7, 8 x 12288 28.0 -> 11.7, 1 x 12288
+// 15.2 -> 11.4, 16 x 2048 x 2048 25.4 -> 4.1; bf16 1 x 12288 26.4 -> 19.1,
+// 1 x 4096 x 11008 19.5 -> 16.7, 1 x 4096 10.9 -> 7.4, 16 x 12288 21.8 ->
+// 20.0, 16 x 4096 10.9 -> 8.5.
+// Tried: W through a TMA ring with 16 warps (bound by the latency of X and of
+// the consumers, 18-32 us for 16 x 12288), cp.async queues in shared memory
+// (130 KB in flight per SM; 1-3 us slower below 8 rows), and W stored K x N
+// (four k-rows a lane; slower than the CUDA-core kernel at one row and than
+// the tensor-core kernels above).
+#include <cuda_bf16.h>
+#include <cuda_fp16.h>
+
+#include "gemm_internal.h"
+
+namespace gb300 {
+
+namespace {
+
+constexpr int kRowsWarps = 4;
+constexpr int kRowsThreads = kRowsWarps * 32;
+constexpr int kStrip = 32;  // rows of W per block
+// words per row of the shared sums: the accumulators' lanes store to it
+// without bank conflicts
+constexpr int kSumPitch = 36;
+constexpr int kRowsBlocks = 4;  // resident blocks per SM (at most 128 registers a thread; 5 measured no faster)
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// The 32-bit word at the same shared-memory offset in block `rank` of the cluster.
+__device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t addr, uint32_t rank) {
+  uint32_t a, v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(addr), "r"(rank));
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
+template <bool INT8>
+__device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                         uint32_t b0, uint32_t b1) {
+  if constexpr (INT8)
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+  else
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// The 16 bytes at a, of which the first `valid` are read (element by element
+// of `es` bytes) and the rest are zero.  Out of line: the ends of W's and X's
+// rows, and X on odd addresses.
+__device__ __noinline__ uint4 load16_edge(const uint8_t *a, int es, int valid) {
+  uint32_t w[4] = {0u, 0u, 0u, 0u};
+  for (int i = 0; i < 16 && i < valid; i += es) {
+    const uint32_t v =
+        es == 1 ? (uint32_t)__ldg(a + i) : (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(a + i));
+    const uint32_t b = v << (8 * (i & 3));
+    w[0] |= i < 4 ? b : 0u, w[1] |= i >> 2 == 1 ? b : 0u, w[2] |= i >> 2 == 2 ? b : 0u, w[3] |= i >> 2 == 3 ? b : 0u;
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+__device__ __forceinline__ void store_out(const RowsParams &p, bool int8, int64_t at, uint32_t v) {
+  if (!int8) {
+    const __nv_bfloat16 h = __float2bfloat16_rn(__uint_as_float(v));
+    reinterpret_cast<uint16_t *>(p.C)[at] = *reinterpret_cast<const uint16_t *>(&h);
+  } else if (p.out_bits == 32) {
+    reinterpret_cast<int32_t *>(p.C)[at] = (int32_t)v;
+  } else {
+    const int32_t hi = (1 << (p.out_bits - 1)) - 1, lo = -hi - 1;
+    const int32_t q = requantize_s32((int32_t)v, p.out_shift, lo, hi);
+    if (p.out_bits == 16)
+      reinterpret_cast<int16_t *>(p.C)[at] = (int16_t)q;
+    else
+      reinterpret_cast<int8_t *>(p.C)[at] = (int8_t)q;
+  }
+}
+
+// NT: 8-row groups of X.
+template <int NT, bool INT8>
+__global__ void __launch_bounds__(kRowsThreads, kRowsBlocks) gemm_rows_kernel(const RowsParams p) {
+  constexpr int ES = INT8 ? 1 : 2;
+  constexpr int kHalf = 64 / ES;       // k per half batch: 64 bytes of each row, 16 a lane
+  constexpr int kBatch = 2 * kHalf;
+  constexpr int kFlush = 512 / kBatch; // batches after which an accumulator holds 512 products
+  extern __shared__ __align__(16) uint32_t red[];  // [warp][row of X][row of W], then the block's sums
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+  const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+  const uint32_t rank = p.cluster > 1 ? cluster_rank() : 0u;
+  const int64_t n0 = (int64_t)(blockIdx.x / p.cluster) * kStrip;
+  const int kbeg = (int)rank * p.kslice;
+  const int kend = min(p.K, kbeg + p.kslice);  // kbeg < kend (rows_geometry)
+  const int nb = (kend - kbeg + kBatch - 1) / kBatch;
+  const int64_t pitch = p.ldw * ES;
+  const int R = p.R;
+
+  // The lane's bytes of a half batch: 16 q .. of W's rows n0 + 8 i + g and of
+  // X's rows 8 j + g.  Rows past the last repeat another: their sums are not
+  // stored.
+  const uint8_t *wp[4], *xp[NT];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int64_t n = n0 + 8 * i + g;
+    wp[i] = static_cast<const uint8_t *>(p.W) + (n < p.NW ? n : p.NW - 1) * pitch + 16 * q;
+  }
+#pragma unroll
+  for (int j = 0; j < NT; ++j)
+    xp[j] = static_cast<const uint8_t *>(p.X) + (8 * j + g < R ? 8 * j + g : 0) * p.ldx * ES + 16 * q;
+
+  griddep_launch_dependents();
+  {  // the warp's first batch: 128 bytes of row n0 + lane
+    const int64_t n = n0 + lane, k = kbeg + warp * kBatch;
+    if (n < p.NW && k < kend) prefetch_l2(static_cast<const uint8_t *>(p.W) + n * pitch + k * ES);
+  }
+  griddep_wait();
+
+  auto load_half = [&](int k, uint4 (&w)[4], uint4 (&x)[NT]) {
+    const int64_t at = (int64_t)k * ES;
+    const bool whole = k + kHalf <= kend;
+    const int valid = (kend - k) * ES - 16 * q;
+    if (whole) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) w[i] = __ldcs(reinterpret_cast<const uint4 *>(wp[i] + at));
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) w[i] = load16_edge(wp[i] + at, ES, valid);
+    }
+    if (whole && p.x_vec) {
+#pragma unroll
+      for (int j = 0; j < NT; ++j) x[j] = __ldg(reinterpret_cast<const uint4 *>(xp[j] + at));
+    } else {
+#pragma unroll
+      for (int j = 0; j < NT; ++j) x[j] = load16_edge(xp[j] + at, ES, valid);
+    }
+  };
+
+  float acc[2][NT][4];
+  int32_t iacc[INT8 ? 2 : 1][NT][4];  // int8: the exact sums so far
+  auto each = [&](auto &&f) {
+#pragma unroll
+    for (int t = 0; t < 2; ++t)
+#pragma unroll
+      for (int j = 0; j < NT; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) f(t, j, e);
+  };
+  each([&](int t, int j, int e) {
+    acc[t][j][e] = 0.f;
+    if constexpr (INT8) iacc[t][j][e] = 0;
+  });
+
+  auto multiply = [&](const uint4 (&w)[4], const uint4 (&x)[NT]) {
+    uint32_t wr[4][4], xr[NT][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) wr[i][0] = w[i].x, wr[i][1] = w[i].y, wr[i][2] = w[i].z, wr[i][3] = w[i].w;
+#pragma unroll
+    for (int j = 0; j < NT; ++j) xr[j][0] = x[j].x, xr[j][1] = x[j].y, xr[j][2] = x[j].z, xr[j][3] = x[j].w;
+    if constexpr (!INT8) {
+#pragma unroll
+      for (int i = 0; i < 2; ++i)  // four of the lane's 8 k
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+#pragma unroll
+          for (int j = 0; j < NT; ++j)
+            mma16816<INT8>(acc[t][j], wr[2 * t][2 * i], wr[2 * t + 1][2 * i], wr[2 * t][2 * i + 1],
+                           wr[2 * t + 1][2 * i + 1], xr[j][2 * i], xr[j][2 * i + 1]);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {  // four of the lane's 16 k
+        uint32_t b[NT][2];
+#pragma unroll
+        for (int j = 0; j < NT; ++j) s8x4_to_f16x4(xr[j][i], b[j][0], b[j][1]);
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+          uint32_t a[4];
+          s8x4_to_f16x4(wr[2 * t][i], a[0], a[2]);
+          s8x4_to_f16x4(wr[2 * t + 1][i], a[1], a[3]);
+#pragma unroll
+          for (int j = 0; j < NT; ++j) mma16816<INT8>(acc[t][j], a[0], a[1], a[2], a[3], b[j][0], b[j][1]);
+        }
+      }
+    }
+  };
+
+  uint4 w0[4], w1[4], x0[NT], x1[NT];
+  int k = kbeg + warp * kBatch;
+  // halves that start past the slice are neither loaded nor multiplied
+  if (k < kend) load_half(k, w0, x0);
+  if (k + kHalf < kend) load_half(k + kHalf, w1, x1);
+  int held = 0;
+#pragma unroll 1
+  for (int b = warp; b < nb; b += kRowsWarps) {
+    const int kn = k + kRowsWarps * kBatch;
+    multiply(w0, x0);
+    if (kn < kend) load_half(kn, w0, x0);
+    if (k + kHalf < kend) multiply(w1, x1);
+    if (kn + kHalf < kend) load_half(kn + kHalf, w1, x1);
+    k = kn;
+    if (INT8 && ++held == kFlush) {
+      each([&](int t, int j, int e) {
+        iacc[INT8 ? t : 0][j][e] += __float2int_rn(acc[t][j][e]);
+        acc[t][j][e] = 0.f;
+      });
+      held = 0;
+    }
+  }
+
+  // accumulator element e of (tile t, group j): row of X, row of the strip
+  const int words = R * kSumPitch;
+  uint32_t *slot = red + warp * words;
+  each([&](int t, int j, int e) {
+    const int r = 8 * j + 2 * q + (e & 1), c = 16 * t + 8 * (e >> 1) + g;
+    if (r < R)
+      slot[r * kSumPitch + c] = INT8 ? (uint32_t)(iacc[INT8 ? t : 0][j][e] + __float2int_rn(acc[t][j][e]))
+                                     : __float_as_uint(acc[t][j][e]);
+  });
+  __syncthreads();
+
+  // the warps' sums in warp order, then the cluster's in rank order
+  const int total = R * kStrip;
+  const int64_t rows = p.NW - n0 < kStrip ? p.NW - n0 : kStrip;
+  auto add = [](uint32_t a, uint32_t b) {
+    return INT8 ? a + b : __float_as_uint(__uint_as_float(a) + __uint_as_float(b));
+  };
+  auto block_sum = [&](int r, int c) {
+    const uint32_t *s = red + r * kSumPitch + c;
+    uint32_t v = s[0];
+#pragma unroll
+    for (int i = 1; i < kRowsWarps; ++i) v = add(v, s[i * words]);
+    return v;
+  };
+  if (p.cluster == 1) {
+#pragma unroll 2
+    for (int t = threadIdx.x; t < total; t += kRowsThreads) {
+      const int r = t / kStrip, c = t % kStrip;
+      if (c < rows) store_out(p, INT8, r * p.scr + (n0 + c) * p.scn, block_sum(r, c));
+    }
+    return;
+  }
+  uint32_t *part = red + kRowsWarps * words;
+#pragma unroll 2
+  for (int t = threadIdx.x; t < total; t += kRowsThreads) part[t] = block_sum(t / kStrip, t % kStrip);
+  cluster_barrier();
+  const uint32_t part_addr = smem_addr(part);
+#pragma unroll 1
+  for (int t = (int)rank * kRowsThreads + threadIdx.x; t < total; t += p.cluster * kRowsThreads) {
+    const int r = t / kStrip, c = t % kStrip;
+    uint32_t v[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (j < p.cluster) v[j] = ld_cluster_u32(part_addr + 4u * t, j);
+    uint32_t s = v[0];
+#pragma unroll
+    for (int j = 1; j < 8; ++j)
+      if (j < p.cluster) s = add(s, v[j]);
+    if (c < rows) store_out(p, INT8, r * p.scr + (n0 + c) * p.scn, s);
+  }
+  cluster_barrier();  // no block leaves while another may still read its sums
+}
+
+template <int NT, bool INT8>
+cudaError_t launch_nt(const RowsParams &p, int64_t strips, cudaStream_t st) {
+  const size_t smem = (size_t)p.R * 4 * (kRowsWarps * kSumPitch + (p.cluster > 1 ? kStrip : 0));
+  static_assert(8 * NT * 4 * (kRowsWarps * kSumPitch + kStrip) <= 48 * 1024, "no shared-memory opt-in needed");
+  return launch_ex(gemm_rows_kernel<NT, INT8>, dim3((unsigned)(strips * p.cluster)), dim3(kRowsThreads), smem, st,
+                   p.cluster, p);
+}
+
+}  // namespace
+
+// Strips, cluster size and K slice: the cluster (1-8 blocks along K) for
+// which the rounds of resident blocks, each as long as its warps' batches
+// plus the start and end of a block (about six batches), take least.
+int64_t rows_geometry(int64_t NW, int64_t K, bool int8, int sms, int *cluster, int *kslice) {
+  const int batch = int8 ? 128 : 64;
+  const int64_t strips = (NW + kStrip - 1) / kStrip;
+  const int64_t slots = (int64_t)kRowsBlocks * sms;
+  double best = -1;
+  for (int c = 1; c <= 8; ++c) {
+    int64_t ks = (K + c - 1) / c;
+    ks = (ks + batch - 1) / batch * batch;
+    if (c > 1 && ks * (c - 1) >= K) continue;  // an empty slice
+    const double cost = (double)((strips * c + slots - 1) / slots) * ((double)ks / (batch * kRowsWarps) + 6.0);
+    if (best < 0 || cost < best) {
+      best = cost;
+      *cluster = c;
+      *kslice = (int)ks;
+    }
+  }
+  return strips;
+}
+
+cudaError_t launch_rows(const RowsParams &p, bool int8, int64_t strips, cudaStream_t st) {
+  if (int8) return p.R > 8 ? launch_nt<2, true>(p, strips, st) : launch_nt<1, true>(p, strips, st);
+  return p.R > 8 ? launch_nt<2, false>(p, strips, st) : launch_nt<1, false>(p, strips, st);
+}
+
+}  // namespace gb300

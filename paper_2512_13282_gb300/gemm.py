@@ -35,6 +35,7 @@ GEMM_ROUTE_SMALL_OPERAND = 3
 GEMM_ROUTE_TC_SINGLE = 4
 GEMM_ROUTE_TC_PAIR = 5
 GEMM_ROUTE_TINY = 6
+GEMM_ROUTE_FEW_ROWS = 7
 
 
 class gemm_plan_t(ctypes.Structure):

@@ -1,0 +1,102 @@
+"""The few-row kernel (at most 16 rows of A, or columns of B, against a
+K-contiguous operand): every element against the oracle at the edges of its
+strips (32 rows), batches (128 bytes of K), clusters and row groups (8), with
+odd pitches and bases of the small operand and of C, at the int8 extremes, and
+the plan query's route.  int8 is exact; bf16 is held to the library's bound
+|C - ref| <= 2^-8 |ref| + 2^-20 sum |a b|, which one rounding to bf16 and an
+fp32 sum in any order satisfy."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2512_13282_gb300 import gemm as G
+from paper_2512_13282_gb300 import workloads as W
+from tests import gpu_util as U
+
+COL = G.GEMM_B_COL_MAJOR_NxK
+
+
+def _run(dtype, M, N, K, seed, shift=0, **kw):
+    rnd = W.random_bf16 if dtype == "bf16" else W.random_int8
+    A, B = rnd((M, K), seed), rnd((N, K), seed + 1)
+    C = U.run(dtype, A, B, COL, shift=shift, **kw)
+    if dtype == "bf16":
+        ref, mag = oracle.gemm_bf16(A, B, COL)
+        assert oracle.bf16_within_bound(C, ref, mag).all()
+    else:
+        want = oracle.gemm_s8(A, B, COL)
+        if dtype != "int8":
+            want = oracle.requantize(want, shift, 16 if dtype == "int8_int16" else 8)
+        assert np.array_equal(C.astype(np.int64), want)
+
+
+# rows of the small operand x rows of the large one x K
+EDGES = [(1, 1, 16), (1, 33, 128), (7, 31, 144), (8, 32, 2048), (9, 64, 1040), (16, 95, 4112), (16, 129, 496),
+         (3, 700, 16384), (13, 4100, 256)]
+
+
+@pytest.mark.gpu
+@pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a GPU")
+@pytest.mark.parametrize("dtype", ["int8", "bf16", "int8_int8"])
+@pytest.mark.parametrize("R,L,K", EDGES, ids=[f"{r}x{n}x{k}" for r, n, k in EDGES])
+def test_few_rows(dtype, R, L, K):
+    for M, N in ((R, L), (L, R)):
+        st, plan = G.gemm_plan_query(M, N, K, dtype != "bf16", COL)
+        narrow = dtype == "bf16" and M > 16 and K < 1024  # the tensor-core kernels' then
+        assert st == 0 and (plan["route"] == G.GEMM_ROUTE_FEW_ROWS) == (not narrow)
+        _run(dtype, M, N, K, seed=R + L + K, shift=7)
+
+
+@pytest.mark.gpu
+@pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a GPU")
+@pytest.mark.parametrize("dtype", ["int8", "bf16"])
+@pytest.mark.parametrize("K", [1, 15, 130, 1001])
+def test_few_rows_ragged_k_and_odd_small_operand(dtype, K):
+    """K that ends inside a 16-byte piece (the large operand's pitch rounded
+    up to 16 bytes), the small operand and C on odd pitches and bases."""
+    pad = (-K) % 16
+    _run(dtype, 11, 70, K, seed=K, lda=K + 3, ldb=K + pad, ldc=75, a_off=1, c_off=1)
+    _run(dtype, 70, 11, K, seed=K, lda=K + pad, ldb=K + 5, ldc=13, b_off=1, c_off=3)
+
+
+@pytest.mark.gpu
+@pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a GPU")
+def test_few_rows_int8_extremes():
+    """All -128 at the largest K (2147467264), and -128 x 127."""
+    A, B = np.full((16, 131071), -128, np.int8), np.full((40, 131071), -128, np.int8)
+    ld = 131072
+    assert (U.run("int8", A, B, COL, ldb=ld) == 2147467264).all()
+    assert (U.run("int8", B, A, COL, lda=ld) == 2147467264).all()
+    B[:, :] = 127
+    assert (U.run("int8", A, B, COL, ldb=ld) == -16256 * 131071).all()
+
+
+@pytest.mark.gpu
+@pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a GPU")
+def test_few_rows_nan_and_inf_stay_in_their_rows():
+    """A NaN or infinity in a row of either operand reaches that row or
+    column of C and no other (padding rows and columns repeat real ones)."""
+    M, N, K = 5, 45, 300
+    A, B = W.random_bf16((M, K), 3), W.random_bf16((N, K), 4)
+    A[2, 299], B[44, 0] = 0x7FC0, 0x7F80  # NaN; +Inf
+    C = torch.from_numpy(U.run("bf16", A, B, COL, ldb=304).view(np.int16).copy()).view(torch.bfloat16).float().numpy()
+    bad = ~np.isfinite(C)
+    assert np.isnan(C[2]).all() and bad[:, 44].all()
+    bad[2], bad[:, 44] = False, False
+    assert not bad.any()
+
+
+def test_route_limits():
+    """17 rows, a row-major B, an unaligned K pitch or a forced plan take
+    the other kernels."""
+    def route(M, N, K, int8, layout):
+        return G.gemm_plan_query(M, N, K, int8, layout)[1]["route"]
+    from paper_2512_13282_gb300 import build
+    build.build()
+    G.gemm_reload_overrides()
+    few = G.GEMM_ROUTE_FEW_ROWS
+    assert route(16, 4096, 4096, True, COL) == few and route(4096, 16, 4096, False, COL) == few
+    assert route(17, 4096, 4096, True, COL) != few and route(4096, 17, 4096, False, COL) != few
+    assert route(16, 4096, 4096, True, G.GEMM_B_ROW_MAJOR_KxN) != few
+    assert route(16, 4096, 4097, False, COL) != few
