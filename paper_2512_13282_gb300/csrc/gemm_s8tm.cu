@@ -47,8 +47,8 @@
 // every 8 k-blocks of 128 (1024 K elements) and the epilogue converts each
 // slab to int32 (exactly) and adds the slabs in int32 registers.
 //
-// A P stage is free again once every converter warp has read its rows (one
-// arrival per warp), a Q stage once the MMAs that read it have completed
+// A P stage is free again once every converter warp of its group has
+// converted and stored its rows (one arrival per warp), a Q stage once the MMAs that read it have completed
 // (tcgen05.commit), a TMEM P slot likewise.  With P decoupled from the MMA,
 // the P ring keeps its boxes in flight from HBM: measured on GB300, a P box
 // takes about 2 us from issue to arrival under load, so the bytes in flight
@@ -61,10 +61,9 @@ namespace gb300 {
 
 namespace {
 
-constexpr int kConvWarps = 4;
-constexpr int kEpiWarps = 4;
-constexpr int kQWarp = 2 + kEpiWarps + kConvWarps;                // 10: Q producer
-constexpr int kThreadsS8tm = (kQWarp + 1) * 32;                   // 352
+constexpr int kConvWarps = 4;   // converter warps of a group: one per TMEM lane quadrant
+constexpr int kConvGroups = 2;  // groups, which take alternate k-blocks
+constexpr int kEpiCols = 64;    // Q columns an epilogue thread accumulates
 constexpr int kKB = kS8tmKB;                                      // K per k-block
 constexpr uint32_t kPBytes = kBM * kKB;                           // 128 rows x 128 int8
 
@@ -75,6 +74,13 @@ constexpr uint32_t kPBytes = kBM * kKB;                           // 128 rows x 
 template <int QN, int SP, int SQ, int NA>
 struct S8tmCfg {
   static_assert(QN == 64 || QN == 128, "QN is 64 or 128");
+  // A converter group waits for a P stage by parity, so it may be at most one
+  // phase ahead of the stage's use before: the same group's (an even ring), or
+  // one whose MMA the group's free TMEM slot implies.
+  static_assert(SP % kConvGroups == 0 && NA % kConvGroups == 0, "each stage and slot belongs to one group");
+  static constexpr int kEpiWarps = 4 * (QN / kEpiCols);
+  static constexpr int kQWarp = 2 + kEpiWarps + kConvGroups * kConvWarps;  // Q producer
+  static constexpr int kThreads = (kQWarp + 1) * 32;
   static constexpr uint32_t kQHalf = QN * kRowBytes;  // QN x 64 bf16: one half of a Q image
   static constexpr uint32_t kQBytes = 2 * kQHalf;      // the k-block's Q image
   static constexpr uint32_t kPOffset = 0;
@@ -181,7 +187,7 @@ __device__ __forceinline__ void reduce_rows_tma(const CUtensorMap *tm, uint32_t 
 }
 
 template <int QN, int SP, int SQ, int NA, bool PK>
-__global__ void __launch_bounds__(kThreadsS8tm, 1)
+__global__ void __launch_bounds__(S8tmCfg<QN, SP, SQ, NA>::kThreads, 1)
     gemm_s8tm_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CUtensorMap tmC,
                      const S8tmParams p) {
   using Cfg = S8tmCfg<QN, SP, SQ, NA>;
@@ -224,7 +230,7 @@ __global__ void __launch_bounds__(kThreadsS8tm, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(accf_bar(b), 1);
-      mbar_init(acce_bar(b), kEpiWarps * 32);
+      mbar_init(acce_bar(b), Cfg::kEpiWarps * 32);
     }
     mbar_init(drain_bar, 1);
     *abort_flag = 0u;
@@ -237,17 +243,18 @@ __global__ void __launch_bounds__(kThreadsS8tm, 1)
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
-  // The previous kernel of the stream is the Q staging launch (a plain
-  // launch: everything before it on the stream completed before it began).
-  // It writes Q's images and, for split-K into int32 C, zeroes C: the Q
-  // producer and the epilogue wait for it (griddep_wait) before touching
-  // those, while P, written before the staging launch began, is streamed at
-  // once, so that the P ring fills while the staging kernel still runs.
+  // The previous kernel of the stream is the Q staging launch, which lets
+  // this one start only once everything before it has completed.  It writes
+  // Q's images and, for split-K into int32 C, zeroes C: the Q producer and the
+  // epilogue wait for it (griddep_wait) before touching those, while P,
+  // written before the staging launch began its work, is streamed at once, so
+  // that the P ring fills while the staging kernel still runs.
+  griddep_launch_dependents();  // whatever follows waits for this grid to complete
 
   const int num_units = p.tiles_p * p.tiles_q * p.splits;
   constexpr uint64_t kDrainNs = 200ull * 1000 * 1000;
 
-  if (warp == 0 || warp == kQWarp) {
+  if (warp == 0 || warp == Cfg::kQWarp) {
     // -------------------------------------------- producers (P, then Q)
     const bool is_p = warp == 0;
     if (!is_p) griddep_wait();
@@ -289,7 +296,7 @@ __global__ void __launch_bounds__(kThreadsS8tm, 1)
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------- MMA issuer
-    constexpr uint32_t idesc = idesc_bf16_f32(kBM, QN, false);
+    constexpr uint32_t idesc = idesc_f16_f32(kBM, QN);
     // K-major, 128-byte swizzle, 8-row atoms 1024 bytes apart
     const uint64_t dq = smem_desc_sw128(sQ, 16, 1024);
     uint32_t s = 0, ph = 0, a = 0, tph = 0, acc_cnt = 0;
@@ -319,7 +326,7 @@ __global__ void __launch_bounds__(kThreadsS8tm, 1)
             for (int k = 0; k < kKB / 16; ++k)
               // one K step of 16 is 8 packed columns of the P slot, and 32
               // bytes along the rows of Q's half k / 4
-              tc_mma_bf16_tmem_a(d_tmem, a_tmem + k * 8, q0 + (k >> 2) * (Cfg::kQHalf / 16) + (k & 3) * 2, idesc,
+              tc_mma_f16_tmem_a(d_tmem, a_tmem + k * 8, q0 + (k >> 2) * (Cfg::kQHalf / 16) + (k & 3) * 2, idesc,
                                  (kb > kb_s || k > 0) ? 1u : 0u);
             tc_commit(qempty_bar(s));  // the Q stage may be refilled once these MMAs finish
             tc_commit(tempty_bar(a));  // and the P slot reused
@@ -344,47 +351,39 @@ __global__ void __launch_bounds__(kThreadsS8tm, 1)
     __syncwarp();
     mbar_wait_drain(drain_bar, 0, kDrainNs);
     __syncwarp();
-  } else if (warp >= 2 + kEpiWarps) {
+  } else if (warp >= 2 + Cfg::kEpiWarps) {
     // ------------------------------------------------------- converters
-    // Software-pipelined by one k-block: the TMEM store of k-block g is
-    // waited for (and its P slot handed to the MMA warp) only after k-block
-    // g + 1 has been loaded and converted, so the store's latency overlaps
-    // that work.
+    // Two groups of four warps take alternate k-blocks: while one waits for
+    // its TMEM stores and publishes its slot, the other converts.
     const int quad = warp & 3;
     const int r = quad * 32 + lane;               // P row within the tile = TMEM lane
     const uint32_t sw = (uint32_t)r & 7u;         // 128-byte swizzle: chunk j at j ^ (r % 8)
     const uint32_t lane_base = tmem_base + ((uint32_t)(quad * 32) << 16) + Cfg::kPCol0;
+    const uint32_t group = (uint32_t)(warp - 2 - Cfg::kEpiWarps) / kConvWarps;
     uint32_t g = 0;
-    bool ok = true, pending = false;
-    uint32_t pending_slot = 0;
-    auto publish = [&](uint32_t slot) {  // the slot's TMEM store has landed: hand it to the MMA warp
-      tmem_st_wait();
-      tc_fence_before_sync();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(tfull_bar(slot));
-      __syncwarp();
-    };
+    bool ok = true;
     for (int u = blockIdx.x; ok && u < num_units; u += gridDim.x) {
       const S8tmUnit w = decode_s8tm(p, u);
-      for (int kb = w.kb0; kb < w.kb1; ++kb) {
+      for (int kb = w.kb0; kb < w.kb1; ++kb, ++g) {
+        if ((g & (kConvGroups - 1)) != group) continue;
         const uint32_t s = g % SP, ph = (g / SP) & 1u;
         const uint32_t a = g % NA, tph = (g / NA) & 1u;
-        if (!__all_sync(0xffffffffu, mbar_wait(pfull_bar(s), ph, abort_flag, p.err, p.wait_limit_ns)) ||
-            !__all_sync(0xffffffffu, mbar_wait(tempty_bar(a), tph ^ 1u, abort_flag, p.err, p.wait_limit_ns))) {
+        if (!mbar_wait_warp(pfull_bar(s), ph, abort_flag, p.err, p.wait_limit_ns) ||
+            !mbar_wait_warp(tempty_bar(a), tph ^ 1u, abort_flag, p.err, p.wait_limit_ns)) {
           ok = false;
           break;
         }
         tc_fence_after_sync();
-        uint32_t o[64];  // o[c]: bf16 of k = 2c (low half) and 2c + 1
+        uint32_t o[64];  // o[c]: fp16 of k = 2c (low half) and 2c + 1
         if constexpr (PK) {
           const uint32_t row = sP + s * kPBytes + (uint32_t)r * kKB;
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
             const uint4 v = ld_shared_v4(row + (((uint32_t)j ^ sw) << 4));  // k = 16 j .. 16 j + 15
-            s8x4_to_bf16x4(v.x, o[8 * j + 0], o[8 * j + 1]);
-            s8x4_to_bf16x4(v.y, o[8 * j + 2], o[8 * j + 3]);
-            s8x4_to_bf16x4(v.z, o[8 * j + 4], o[8 * j + 5]);
-            s8x4_to_bf16x4(v.w, o[8 * j + 6], o[8 * j + 7]);
+            s8x4_to_f16x4(v.x, o[8 * j + 0], o[8 * j + 1]);
+            s8x4_to_f16x4(v.y, o[8 * j + 2], o[8 * j + 3]);
+            s8x4_to_f16x4(v.z, o[8 * j + 4], o[8 * j + 5]);
+            s8x4_to_f16x4(v.w, o[8 * j + 6], o[8 * j + 7]);
           }
         } else {
           // The box holds 128 k-rows of 128 P rows (byte r of k-row k in
@@ -405,57 +404,63 @@ __global__ void __launch_bounds__(kThreadsS8tm, 1)
               w4[i] = ld_shared_u32(box + k * 128u + ((rc ^ (k & 7u)) << 4) + rw);
             }
             const uint32_t x = __byte_perm(__byte_perm(w4[0], w4[1], sel), __byte_perm(w4[2], w4[3], sel), 0x5410);
-            s8x4_to_bf16x4(x, o[2 * kq], o[2 * kq + 1]);
+            s8x4_to_f16x4(x, o[2 * kq], o[2 * kq + 1]);
           }
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(pempty_bar(s));  // this warp's rows of the P box are read
-        __syncwarp();
-        if (pending) publish(pending_slot);
         tmem_st_32x32b_x64(lane_base + a * 64, o);
-        pending = true;
-        pending_slot = a;
-        ++g;
+        __syncwarp();
+        // The P stage is released only after that store was issued, which
+        // needed every byte this warp reads of it.  An arrival right after the
+        // shared-memory loads were issued let the refill overtake them while
+        // the load queue was backed up (single 16-byte pieces of P wrong).
+        if (lane == 0) mbar_arrive(pempty_bar(s));
+        __syncwarp();
+        tmem_st_wait();
+        tc_fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(tfull_bar(a));  // hand the slot to the MMA warp
+        __syncwarp();
       }
     }
-    if (pending) publish(pending_slot);
   } else {
     // --------------------------------------------------------- epilogue
     griddep_wait();  // C (zeroed by the staging launch) is written below
     const int quad = warp & 3;
     const int r = quad * 32 + lane;
+    const int col0 = ((warp - 2) >> 2) * kEpiCols;  // this warp's Q columns of the tile
     uint32_t acc_cnt = 0;
     bool ok = true;
     for (int u = blockIdx.x; ok && u < num_units; u += gridDim.x) {
       const S8tmUnit w = decode_s8tm(p, u);
-      int32_t acc[QN];
+      int32_t acc[kEpiCols];
 #pragma unroll
-      for (int i = 0; i < QN; ++i) acc[i] = 0;
+      for (int i = 0; i < kEpiCols; ++i) acc[i] = 0;
       for (int kb_s = w.kb0; kb_s < w.kb1; kb_s += p.slab_kb) {
         const uint32_t b = acc_cnt & 1u, aph = (acc_cnt >> 1) & 1u;
-        if (!__all_sync(0xffffffffu, mbar_wait(accf_bar(b), aph, abort_flag, p.err, p.wait_limit_ns))) {
+        if (!mbar_wait_warp(accf_bar(b), aph, abort_flag, p.err, p.wait_limit_ns)) {
           ok = false;
           break;
         }
         tc_fence_after_sync();
-        const uint32_t t0 = tmem_base + b * QN + ((uint32_t)(quad * 32) << 16);
+        const uint32_t t0 = tmem_base + b * QN + ((uint32_t)(quad * 32) << 16) + col0;
 #pragma unroll
-        for (int c = 0; c < QN / 32; ++c) {
-          uint32_t v[32];
-          tmem_ld_32x32b_x32(t0 + c * 32, v);
+        for (int c = 0; c < kEpiCols / 16; ++c) {
+          uint32_t v[16];
+          tmem_ld_32x32b_x16(t0 + c * 16, v);
           tmem_ld_wait();
 #pragma unroll
-          for (int i = 0; i < 32; ++i) acc[c * 32 + i] += __float2int_rn(__uint_as_float(v[i]));
+          for (int i = 0; i < 16; ++i) acc[c * 16 + i] += __float2int_rn(__uint_as_float(v[i]));
         }
         tc_fence_before_sync();
         mbar_arrive(acce_bar(b));
         ++acc_cnt;
       }
       if (!ok) break;
-      const int64_t q0 = (int64_t)w.tq * QN;
+      const int64_t q0 = (int64_t)w.tq * QN + col0;
+      if (q0 >= p.Q_rows) continue;
       if (p.add_into_c && p.c_tma) {  // the whole warp: rows past the matrix are clipped by the TMA
-        reduce_rows_tma<QN>(&tmC, base + Cfg::kEpiOffset + (warp - 2) * 4096, lane, acc, p.swap != 0,
-                            w.tp * kBM + quad * 32, (int32_t)q0, p.P_rows, p.Q_rows);
+        reduce_rows_tma<kEpiCols>(&tmC, base + Cfg::kEpiOffset + (warp - 2) * 4096, lane, acc, p.swap != 0,
+                                  w.tp * kBM + quad * 32, (int32_t)q0, p.P_rows, p.Q_rows);
         continue;
       }
       const int64_t prow = (int64_t)w.tp * kBM + r;
@@ -463,15 +468,14 @@ __global__ void __launch_bounds__(kThreadsS8tm, 1)
       // partials (split-K of int16 / int8 outputs) have row pitch N; C has ldc
       const int64_t ld = (p.splits > 1 && p.out_bits != 32) ? (int64_t)p.N : p.ldc;
       if (p.swap)  // C[q][prow]: per element the warp's lanes store 32 consecutive columns
-        store_row<QN>(p, acc, w.split, q0 * ld + prow, ld, q0);
+        store_row<kEpiCols>(p, acc, w.split, q0 * ld + prow, ld, q0);
       else         // C[prow][q]
-        store_row<QN>(p, acc, w.split, prow * ld + q0, 1, q0);
+        store_row<kEpiCols>(p, acc, w.split, prow * ld + q0, 1, q0);
     }
   }
 
   // the epilogue's TMA reductions have completed before the CTA leaves
-  if (p.c_tma && warp >= 2 && warp < 2 + kEpiWarps && lane == 0) bulk_wait_all();
-  griddep_launch_dependents();  // e.g. the split-K reduction may start setting up
+  if (p.c_tma && warp >= 2 && warp < 2 + Cfg::kEpiWarps && lane == 0) bulk_wait_all();
   __syncwarp();
   tc_fence_before_sync();
   __syncthreads();
@@ -490,7 +494,11 @@ __global__ void __launch_bounds__(256)
     s8tm_stage_q_kernel(const int8_t *__restrict__ src, int64_t sq, int64_t sk, int Q_rows, int K, int qn,
                         int num_kb, uint4 *__restrict__ img, int64_t chunks, int32_t *__restrict__ zero_c,
                         int64_t c_rows, int64_t c_cols, int64_t ldc) {
-  griddep_launch_dependents();  // the GEMM waits for completion before reading
+  // Launched with programmatic dependent launch: scheduled while the previous
+  // kernel drains.  The GEMM may start when every block is past this wait:
+  // it reads P at once and waits for this grid before it reads Q.
+  griddep_wait();
+  griddep_launch_dependents();
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= chunks) {  // the remaining threads zero C (int32, the splits' sums are added into it)
     if (!zero_c) return;
@@ -530,8 +538,8 @@ __global__ void __launch_bounds__(256)
     }
   }
   uint4 o;
-  s8x4_to_bf16x4(w[0], o.x, o.y);
-  s8x4_to_bf16x4(w[1], o.z, o.w);
+  s8x4_to_f16x4(w[0], o.x, o.y);
+  s8x4_to_f16x4(w[1], o.z, o.w);
   const int64_t at = tile * per_tile + h * (qn * 8) + row * 8 + (j ^ (row & 7));
   img[at] = o;
 }
@@ -543,7 +551,7 @@ cudaError_t launch_one(const CUtensorMap &tp, const CUtensorMap &tc, const S8tmP
   auto kern = gemm_s8tm_kernel<QN, SP, SQ, NA, PK>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::kSmemBytes);
   if (e != cudaSuccess) return e;
-  return launch_ex(kern, dim3(grid), dim3(kThreadsS8tm), Cfg::kSmemBytes, st, 1, tp, tc, p);
+  return launch_ex(kern, dim3(grid), dim3(Cfg::kThreads), Cfg::kSmemBytes, st, 1, tp, tc, p);
 }
 
 }  // namespace
@@ -563,21 +571,23 @@ cudaError_t launch_s8tm_stage_q(const int8_t *src, int64_t sq, int64_t sk, int64
   const int64_t quads = zero_c ? c_rows * ((c_cols + 3) / 4) : 0;
   const int64_t extra = quads < 65536 ? quads : 65536;
   if (chunks + extra == 0) return cudaSuccess;
-  s8tm_stage_q_kernel<<<(unsigned)((chunks + extra + 255) / 256), 256, 0, st>>>(
-      src, sq, sk, (int)Q_rows, (int)K, qn, (int)num_kb, static_cast<uint4 *>(img), chunks, zero_c, c_rows, c_cols,
-      ldc);
-  return cudaGetLastError();
+  return launch_ex(s8tm_stage_q_kernel, dim3((unsigned)((chunks + extra + 255) / 256)), dim3(256), 0, st, 1, src, sq,
+                   sk, (int)Q_rows, (int)K, qn, (int)num_kb, static_cast<uint4 *>(img), chunks, zero_c, c_rows, c_cols,
+                   ldc);
 }
 
 cudaError_t launch_s8tm(int qn, bool p_kmajor, const CUtensorMap &tp, const CUtensorMap &tc, const S8tmParams &p,
                         int grid, cudaStream_t st) {
-  // P stages x 16 KB + Q stages x (QN x 256 bytes): 9 x 16 + 2 x 32 KB
-  // (QN 128) or 10 x 16 + 3 x 16 KB (QN 64), and four 4 KB epilogue blocks
+  // P stages x 16 KB + Q stages x (QN x 256 bytes) + a 4 KB block per
+  // epilogue warp: 6 x 16 + 3 x 32 + 32 KB (QN 128) or 8 x 16 + 5 x 16 +
+  // 16 KB (QN 64); TMEM: two accumulators and four (six) 64-column P slots.
+  // Q, read from L2 by every CTA, is up to twice P's bytes: with two Q stages
+  // its latency set the pace (128 x 4096 x 11008 19.3 us, with three 17.2).
   if (qn == 128)
-    return p_kmajor ? launch_one<128, 9, 2, 4, true>(tp, tc, p, grid, st)
-                    : launch_one<128, 9, 2, 4, false>(tp, tc, p, grid, st);
-  return p_kmajor ? launch_one<64, 10, 3, 4, true>(tp, tc, p, grid, st)
-                  : launch_one<64, 10, 3, 4, false>(tp, tc, p, grid, st);
+    return p_kmajor ? launch_one<128, 6, 3, 4, true>(tp, tc, p, grid, st)
+                    : launch_one<128, 6, 3, 4, false>(tp, tc, p, grid, st);
+  return p_kmajor ? launch_one<64, 8, 5, 6, true>(tp, tc, p, grid, st)
+                  : launch_one<64, 8, 5, 6, false>(tp, tc, p, grid, st);
 }
 
 }  // namespace gb300

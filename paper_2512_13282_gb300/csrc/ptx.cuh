@@ -298,9 +298,9 @@ __device__ __forceinline__ void tc_mma_kstep(uint32_t d_tmem, uint64_t a, uint64
 }
 
 // D[tmem] (+)= A[tmem] * B[smem], kind::f16: A is 128 rows (TMEM lanes) of
-// K = 16 bf16 packed two to a 32-bit column (the lower k in the low half),
-// i.e. 8 columns starting at a_tmem.
-__device__ __forceinline__ void tc_mma_bf16_tmem_a(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
+// K = 16 16-bit values packed two to a 32-bit column (the lower k in the low
+// half), i.e. 8 columns starting at a_tmem; the type is the descriptor's.
+__device__ __forceinline__ void tc_mma_f16_tmem_a(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
                                                    uint32_t idesc, uint32_t accumulate) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
@@ -325,6 +325,11 @@ __device__ __forceinline__ void tc_commit(uint32_t bar) {
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(uint32_t m, uint32_t n, bool b_mn_major) {
   return (1u << 4) | (1u << 7) | (1u << 10) | (0u << 15) | ((b_mn_major ? 1u : 0u) << 16) |
          ((n >> 3) << 17) | ((m >> 4) << 24);
+}
+
+// The same with fp16 A/B (format 0), both K-major.
+__host__ __device__ constexpr uint32_t idesc_f16_f32(uint32_t m, uint32_t n) {
+  return (1u << 4) | ((n >> 3) << 17) | ((m >> 4) << 24);
 }
 
 // Shared-memory matrix descriptor, 128-byte swizzle:
