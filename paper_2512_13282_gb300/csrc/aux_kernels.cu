@@ -62,7 +62,6 @@ __device__ __forceinline__ void piece_rc(uint64_t u, uint32_t cpr, int w, int64_
 __global__ void __launch_bounds__(kS8Threads)
     s8_to_bf16_pair_kernel(const S8Job a, const S8Job b, uint32_t cpr_a, uint32_t cpr_b, uint64_t items_a,
                            uint64_t items) {
-  griddep_wait();  // programmatic dependent launch, as every kernel below
   griddep_launch_dependents();
   const uint64_t t = (uint64_t)blockIdx.x * kS8Threads + threadIdx.x;
   if (t >= items) return;
@@ -109,7 +108,6 @@ __global__ void __launch_bounds__(kS8Threads)
 // partial vector (elements % 16) is converted element by element.
 __global__ void __launch_bounds__(kS8Threads)
     s8_to_bf16_dense_kernel(const S8Job a, const S8Job b, int64_t na, int64_t nb) {
-  griddep_wait();
   griddep_launch_dependents();
   const int64_t va = (na + 15) / 16, vtot = va + (nb + 15) / 16;
   const int64_t v = (int64_t)blockIdx.x * kS8Threads + threadIdx.x;
@@ -137,7 +135,6 @@ __global__ void __launch_bounds__(kS8Threads)
 __global__ void __launch_bounds__(kS8Threads)
     pack_u16_kernel(const uint16_t *__restrict__ src, int64_t cols, int64_t ld_src, uint16_t *__restrict__ dst,
                     int64_t ld_dst, uint32_t cpr, uint64_t items) {
-  griddep_wait();
   griddep_launch_dependents();  // the GEMM waits for completion before reading
   const uint64_t t = (uint64_t)blockIdx.x * kS8Threads + threadIdx.x;
   if (t >= items) return;
@@ -260,7 +257,6 @@ __global__ void __launch_bounds__(kThreads)
     splitk_reduce_bf16_kernel(const float *__restrict__ ws, int splits, int64_t M, int64_t N,
                               uint16_t *__restrict__ C, int64_t ldc, uint32_t cpr, const ReduceTiles rt) {
   griddep_wait();  // the partials come from the GEMM launched just before
-  griddep_launch_dependents();
   const uint64_t t = (uint64_t)blockIdx.x * kThreads + threadIdx.x;
   Piece pc;
   if (!reduce_piece(t, cpr, M, N, rt, &pc)) return;
@@ -286,7 +282,6 @@ __global__ void __launch_bounds__(kThreads)
     splitk_reduce_s32_kernel(const int32_t *__restrict__ ws, int splits, int64_t M, int64_t N, void *__restrict__ C,
                              int64_t ldc, int out_bits, int shift, uint32_t cpr, const ReduceTiles rt) {
   griddep_wait();
-  griddep_launch_dependents();
   const uint64_t t = (uint64_t)blockIdx.x * kThreads + threadIdx.x;
   Piece pc;
   if (!reduce_piece(t, cpr, M, N, rt, &pc)) return;
@@ -380,14 +375,15 @@ cudaError_t launch_s8_to_bf16_pair(const S8Job &a, const S8Job &b, int sms, cuda
     const int64_t na = a.rows * a.cols, nb = b.rows * b.cols;
     const int64_t vecs = (na + 15) / 16 + (nb + 15) / 16;
     if (vecs == 0) return cudaSuccess;
-    return launch_ex(s8_to_bf16_dense_kernel, dim3((unsigned)((vecs + kS8Threads - 1) / kS8Threads)), dim3(kS8Threads),
-                     0, st, 1, a, b, na, nb);
+    s8_to_bf16_dense_kernel<<<(unsigned)((vecs + kS8Threads - 1) / kS8Threads), kS8Threads, 0, st>>>(a, b, na, nb);
+    return cudaGetLastError();
   }
   const uint64_t cpr_a = (uint64_t)(a.cols + 15) / 16, cpr_b = (uint64_t)(b.cols + 15) / 16;
   const uint64_t items_a = (uint64_t)a.rows * cpr_a, items = items_a + (uint64_t)b.rows * cpr_b;
   if (items == 0) return cudaSuccess;
-  return launch_ex(s8_to_bf16_pair_kernel, dim3((unsigned)((items + kS8Threads - 1) / kS8Threads)), dim3(kS8Threads), 0,
-                   st, 1, a, b, (uint32_t)(cpr_a ? cpr_a : 1), (uint32_t)(cpr_b ? cpr_b : 1), items_a, items);
+  s8_to_bf16_pair_kernel<<<(unsigned)((items + kS8Threads - 1) / kS8Threads), kS8Threads, 0, st>>>(
+      a, b, (uint32_t)(cpr_a ? cpr_a : 1), (uint32_t)(cpr_b ? cpr_b : 1), items_a, items);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_pack_u16(const uint16_t *src, int64_t rows, int64_t cols, int64_t ld_src,
@@ -395,8 +391,9 @@ cudaError_t launch_pack_u16(const uint16_t *src, int64_t rows, int64_t cols, int
   (void)sms;
   const uint64_t cpr = (uint64_t)(cols + 3) / 4, items = (uint64_t)rows * cpr;
   if (items == 0) return cudaSuccess;
-  return launch_ex(pack_u16_kernel, dim3((unsigned)((items + kS8Threads - 1) / kS8Threads)), dim3(kS8Threads), 0, st, 1,
-                   src, cols, ld_src, dst, ld_dst, (uint32_t)cpr, items);
+  pack_u16_kernel<<<(unsigned)((items + kS8Threads - 1) / kS8Threads), kS8Threads, 0, st>>>(
+      src, cols, ld_src, dst, ld_dst, (uint32_t)cpr, items);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_zero_fill(void *C, int64_t M, int64_t N, int64_t ldc, int esize, int sms,

@@ -662,28 +662,46 @@ gemm_status_t run_tc(DeviceState &d, Plan &pl, const uint16_t *A, int64_t lda, c
   return GEMM_OK;
 }
 
-// Largest int8 problem (M * N * K multiply-adds) computed in one launch on
-// the CUDA cores (gemm_tiny.cu) instead of staging + tensor cores: below it
-// the launches, not the arithmetic, set the time.
-constexpr int64_t kTinyMaxMacs = int64_t(1) << 27;  // 512^3
+// int8 problems computed in one launch on the CUDA cores (gemm_tiny.cu)
+// instead of staging + tensor cores: those where the launches, not the
+// arithmetic, set the time.  A block walks K in slabs of 512, one memory
+// latency each, so the limit is on K as well as on the multiply-adds.
+// Measured on GB300 against the tensor-core routes, back to back: 128^3 3.2 /
+// 5.3 us, 256^3 5.1 / 6.6, 300^3 (odd pitch) 7.7-8.8 / 8.2, 384^3 9.8 / 7.0,
+// 512^3 9.6 / 6.5, 32 x 1024 x 1024 8.7 / 6.3, 128 x 128 x 4096 31 / 9.0.
+constexpr int64_t kTinyMaxMacs = int64_t(1) << 24;  // 256^3
+constexpr int64_t kTinyMaxK = 512;
+// With the small-M limit forced (GB300_GEMM_SKINNY_MAX_M), the tile kernel
+// takes problems by their multiply-adds alone, up to 512^3.
+constexpr int64_t kTinyMaxMacsForced = int64_t(1) << 27;
 
-int64_t tiny_max_macs() {
+bool tiny_shape(int64_t M, int64_t N, int64_t K) {
   const Overrides o = overrides();
   // a forced tile width, family or split asks for the tensor-core kernels
-  if (o.bn > 0 || o.pair >= 0 || o.splits >= 1 || o.tail_splits >= 2) return 0;
-  return o.tiny_max_macs >= 0 ? o.tiny_max_macs : kTinyMaxMacs;
+  if (o.bn > 0 || o.pair >= 0 || o.splits >= 1 || o.tail_splits >= 2) return false;
+  const double macs = (double)M * (double)N * (double)K;
+  if (o.tiny_max_macs >= 0) return macs <= (double)o.tiny_max_macs;
+  if (o.skinny_max_m >= 0) return macs <= (double)kTinyMaxMacsForced;
+  return macs <= (double)kTinyMaxMacs && K <= kTinyMaxK;
 }
 
 // Largest M sent to the CUDA-core small-M kernel: there every B element is
-// used at most a few times and streaming B once is the cost.  Measured on
-// GB300 against the tensor-core path (N = 4096..11008, K = 4096): int8
-// through dp4a, which also skips the staging pass, wins up to M = 8; bf16,
-// accumulating with fp32 FMAs, only up to M = 2.
-// GB300_GEMM_SKINNY_MAX_M overrides (0 disables the kernel).
-int skinny_max_m(bool int8) {
+// used at most a few times and streaming B once is the cost.  bf16,
+// accumulating with fp32 FMAs, wins up to M = 2 (measured on GB300 against
+// the tensor-core path, N = 4096..11008, K = 4096); int8, through dp4a, up to
+// M = 8 where the alternative stages B.  Where the small-operand kernel can
+// read a row-major B as it is (`in_place`), that kernel is faster from M = 2
+// on (K = 4096, back to back: M = 1 x 4096 8.4 / 9.7 us, 2 x 4096 11.0 /
+// 9.7, 4 x 4096 12.9 / 9.8, 8 x 4096 18.1 / 9.9, 4 x 12288 24.1 / 17.0),
+// except M = 2 with a small B (2 x 1024 x 1024 5.9 / 6.2) or a wide one (2 x
+// 12288 16.4 / 17.0).  GB300_GEMM_SKINNY_MAX_M overrides (0 disables the
+// kernel).
+int skinny_max_m(bool int8, int64_t N, int64_t K, bool in_place) {
   const int v = overrides().skinny_max_m;
   if (v >= 0) return v > 16 ? 16 : v;
-  return int8 ? 8 : 2;
+  if (!int8) return 2;
+  if (!in_place) return 8;
+  return N >= 8192 || N * K < (int64_t(1) << 22) ? 2 : 1;
 }
 
 gemm_status_t run_skinny(DeviceState &d, int64_t M, int64_t N, int64_t K, const void *A, int64_t lda,
@@ -803,7 +821,7 @@ gemm_status_t gemm_bf16_f32acc_bf16(int64_t M, int64_t N, int64_t K, const uint1
   }
   const bool b_kmajor = b_layout == GEMM_B_COL_MAJOR_NxK;
   if (try_rows(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, false, 0, 0, st, &s)) return s;
-  if (M <= skinny_max_m(false))
+  if (M <= skinny_max_m(false, N, K, false))
     return run_skinny(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, false, st);
   Plan pl = make_plan(M, N, K, b_kmajor, kEpiBf16, d->sms, pair_slots());
   // TMA needs 16-byte aligned bases and row pitches; re-pitch an operand
@@ -1042,9 +1060,10 @@ gemm_status_t s8_gemm(int64_t M, int64_t N, int64_t K, const int8_t *A, int64_t 
   }
   const bool b_kmajor = b_layout == GEMM_B_COL_MAJOR_NxK;
   if (try_rows(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, true, out_bits, shift, st, &s)) return s;
-  if (M <= skinny_max_m(true))
+  const bool in_place = overrides().s8tm && !b_kmajor && N > kBM && aligned16(B) && ldb % 16 == 0;
+  if (M <= skinny_max_m(true, N, K, in_place))
     return run_skinny(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, true, st, out_bits, shift);
-  if ((double)M * (double)N * (double)K <= (double)tiny_max_macs()) {
+  if (tiny_shape(M, N, K)) {
     const TinyParams tp{A, lda, B, ldb, C, ldc, M, N, K, out_bits, shift};
     const bool prof = g_prof_start && g_prof_stop;
     if (prof && cudaEventRecord(g_prof_start, st) != cudaSuccess) return GEMM_ERR_CUDA;
@@ -1191,11 +1210,12 @@ gemm_status_t gemm_plan_query(int64_t M, int64_t N, int64_t K, int int8, int b_l
     out->grid = (int)(strips * cluster);
     return GEMM_OK;
   }
-  if (M <= skinny_max_m(int8 != 0)) {
+  const bool in_place = overrides().s8tm && !b_kmajor && N > kBM && N % 16 == 0;
+  if (M <= skinny_max_m(int8 != 0, N, K, in_place)) {
     out->route = GEMM_ROUTE_SMALL_M;
     return GEMM_OK;
   }
-  if (int8 && (double)M * (double)N * (double)K <= (double)tiny_max_macs()) {
+  if (int8 && tiny_shape(M, N, K)) {
     out->route = GEMM_ROUTE_TINY;
     out->bn = 32;
     out->splits = 1;

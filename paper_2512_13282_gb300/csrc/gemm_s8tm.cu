@@ -243,13 +243,12 @@ __global__ void __launch_bounds__(S8tmCfg<QN, SP, SQ, NA>::kThreads, 1)
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
-  // The previous kernel of the stream is the Q staging launch, which lets
-  // this one start only once everything before it has completed.  It writes
-  // Q's images and, for split-K into int32 C, zeroes C: the Q producer and the
-  // epilogue wait for it (griddep_wait) before touching those, while P,
-  // written before the staging launch began its work, is streamed at once, so
-  // that the P ring fills while the staging kernel still runs.
-  griddep_launch_dependents();  // whatever follows waits for this grid to complete
+  // The previous kernel of the stream is the Q staging launch (a plain
+  // launch: everything before it on the stream completed before it began).
+  // It writes Q's images and, for split-K into int32 C, zeroes C: the Q
+  // producer and the epilogue wait for it (griddep_wait) before touching
+  // those, while P, written before the staging launch began, is streamed at
+  // once, so that the P ring fills while the staging kernel still runs.
 
   const int num_units = p.tiles_p * p.tiles_q * p.splits;
   constexpr uint64_t kDrainNs = 200ull * 1000 * 1000;
@@ -476,6 +475,7 @@ __global__ void __launch_bounds__(S8tmCfg<QN, SP, SQ, NA>::kThreads, 1)
 
   // the epilogue's TMA reductions have completed before the CTA leaves
   if (p.c_tma && warp >= 2 && warp < 2 + Cfg::kEpiWarps && lane == 0) bulk_wait_all();
+  griddep_launch_dependents();  // e.g. the split-K reduction may start setting up
   __syncwarp();
   tc_fence_before_sync();
   __syncthreads();
@@ -494,11 +494,7 @@ __global__ void __launch_bounds__(256)
     s8tm_stage_q_kernel(const int8_t *__restrict__ src, int64_t sq, int64_t sk, int Q_rows, int K, int qn,
                         int num_kb, uint4 *__restrict__ img, int64_t chunks, int32_t *__restrict__ zero_c,
                         int64_t c_rows, int64_t c_cols, int64_t ldc) {
-  // Launched with programmatic dependent launch: scheduled while the previous
-  // kernel drains.  The GEMM may start when every block is past this wait:
-  // it reads P at once and waits for this grid before it reads Q.
-  griddep_wait();
-  griddep_launch_dependents();
+  griddep_launch_dependents();  // the GEMM waits for completion before reading
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= chunks) {  // the remaining threads zero C (int32, the splits' sums are added into it)
     if (!zero_c) return;
@@ -571,9 +567,10 @@ cudaError_t launch_s8tm_stage_q(const int8_t *src, int64_t sq, int64_t sk, int64
   const int64_t quads = zero_c ? c_rows * ((c_cols + 3) / 4) : 0;
   const int64_t extra = quads < 65536 ? quads : 65536;
   if (chunks + extra == 0) return cudaSuccess;
-  return launch_ex(s8tm_stage_q_kernel, dim3((unsigned)((chunks + extra + 255) / 256)), dim3(256), 0, st, 1, src, sq,
-                   sk, (int)Q_rows, (int)K, qn, (int)num_kb, static_cast<uint4 *>(img), chunks, zero_c, c_rows, c_cols,
-                   ldc);
+  s8tm_stage_q_kernel<<<(unsigned)((chunks + extra + 255) / 256), 256, 0, st>>>(
+      src, sq, sk, (int)Q_rows, (int)K, qn, (int)num_kb, static_cast<uint4 *>(img), chunks, zero_c, c_rows, c_cols,
+      ldc);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_s8tm(int qn, bool p_kmajor, const CUtensorMap &tp, const CUtensorMap &tc, const S8tmParams &p,

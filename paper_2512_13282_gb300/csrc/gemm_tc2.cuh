@@ -188,9 +188,6 @@ __global__ void __launch_bounds__(Tc2Cfg<BN, STAGES, B_KMAJOR, EPI, EPI_WARPS, T
   // kernel parameters, and may overlap the previous kernel of the stream;
   // global memory is touched only after that kernel has completed.
   griddep_wait();
-  // The next kernel of the stream (a reduction, the next call's staging) may
-  // be scheduled beside this one; it waits for this grid to complete.
-  griddep_launch_dependents();
 
   const int num_units = tc_num_units(p);
   constexpr uint64_t kDrainNs = 200ull * 1000 * 1000;
@@ -442,6 +439,7 @@ __global__ void __launch_bounds__(Tc2Cfg<BN, STAGES, B_KMAJOR, EPI, EPI_WARPS, T
   }
 
   if (TMA_OUT && warp >= 2 && lane == 0) bulk_wait_all();  // this warp's TMA stores have landed
+  griddep_launch_dependents();  // e.g. the split-K reduction may start setting up
   __syncwarp();
   tc_fence_before_sync();
   cluster_sync_all();  // no remote arrival or load may target a CTA that has left

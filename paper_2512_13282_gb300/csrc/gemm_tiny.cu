@@ -1,7 +1,7 @@
 // gemm_tiny.cu -- exact int8 GEMM for problems too small to fill the GPU, in
 // one launch on the CUDA cores.
 //
-// Below a few hundred million multiply-adds the time of an int8 GEMM is the
+// Below some ten million multiply-adds the time of an int8 GEMM is the
 // launch and the memory latency, not the arithmetic: the tensor-core path
 // needs two launches (the operands are staged as bf16 first) and a pipeline
 // start per tile, while `__dp4a` (four exact int8 products summed into an
