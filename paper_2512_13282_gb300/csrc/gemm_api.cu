@@ -977,7 +977,7 @@ bool try_s8tm(DeviceState &d, int64_t M, int64_t N, int64_t K, const int8_t *A, 
   *status = GEMM_ERR_CUDA;
   g_launches.fetch_add(1);
   if (launch_s8tm_stage_q(Qs, sq, sk, Q_rows, K, qn, ws, add_into_c ? static_cast<int32_t *>(C) : nullptr, M, N,
-                          ldc, st) != cudaSuccess)
+                          ldc, P_rows * K, st) != cudaSuccess)
     return true;
   CUtensorMap tp;
   if (!(p_kmajor ? encode_s8_rows(&tp, P, (uint64_t)K, (uint64_t)P_rows, (uint64_t)ldp)

@@ -103,10 +103,11 @@ struct S8tmParams {
 size_t s8tm_q_image_bytes(int qn, int64_t Q_rows, int64_t K);
 // Writes Q's images: Q(q, k) = src[q * sq + k * sk] (int8), exact bf16;
 // when zero_c is not null, also sets the c_rows x c_cols int32 matrix at
-// zero_c (row pitch ldc) to zero.
+// zero_c (row pitch ldc) to zero.  p_bytes: the size of P, which decides how
+// the launch overlaps its neighbours.
 cudaError_t launch_s8tm_stage_q(const int8_t *src, int64_t sq, int64_t sk, int64_t Q_rows, int64_t K, int qn,
                                 void *img, int32_t *zero_c, int64_t c_rows, int64_t c_cols, int64_t ldc,
-                                cudaStream_t st);
+                                int64_t p_bytes, cudaStream_t st);
 // qn: 64 or 128 columns of Q per tile.  p_kmajor: P's rows are K
 // contiguous (boxes of 128 k x 128 rows); otherwise P's rows are the
 // contiguous dimension of its storage (boxes of 128 rows x 128 k, read
