@@ -10,6 +10,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <vector>
 
@@ -93,6 +94,11 @@ struct Overrides {
   bool s8tm = true;
   int64_t tiny_max_macs = -1;  // -1: built-in limit
   bool debug = false;
+  bool operator==(const Overrides &o) const {
+    return bn == o.bn && pair == o.pair && splits == o.splits && tail_splits == o.tail_splits &&
+           skinny_max_m == o.skinny_max_m && tma_store == o.tma_store && pdl == o.pdl && s8tm == o.s8tm &&
+           tiny_max_macs == o.tiny_max_macs && debug == o.debug;
+  }
 };
 
 int env_int(const char *name, int dflt) {
@@ -115,18 +121,31 @@ Overrides read_overrides() {
   return o;
 }
 
+// The overrides in force: an immutable snapshot, replaced (never changed) by
+// a reload, so that a call reads it without a lock.  Snapshots stay allocated
+// until the process exits: a concurrent call may still read an old one.
 std::mutex g_ovr_mu;
-Overrides g_ovr;
-bool g_ovr_loaded = false;
+std::vector<std::unique_ptr<const Overrides>> g_ovr_all;
+std::atomic<const Overrides *> g_ovr{nullptr};
 
-// The overrides in force (a copy, so that a concurrent reload cannot tear it).
-Overrides overrides() {
+const Overrides &publish_overrides(bool reload) {
   std::lock_guard<std::mutex> lk(g_ovr_mu);
-  if (!g_ovr_loaded) {
-    g_ovr = read_overrides();
-    g_ovr_loaded = true;
-  }
-  return g_ovr;
+  const Overrides *now = g_ovr.load(std::memory_order_acquire);
+  if (now && !reload) return *now;
+  const Overrides o = read_overrides();
+  for (const auto &p : g_ovr_all)  // a snapshot with these values exists already (tests switch back and forth)
+    if (*p == o) {
+      g_ovr.store(p.get(), std::memory_order_release);
+      return *p;
+    }
+  g_ovr_all.push_back(std::make_unique<const Overrides>(o));
+  g_ovr.store(g_ovr_all.back().get(), std::memory_order_release);
+  return *g_ovr_all.back();
+}
+
+const Overrides &overrides() {
+  const Overrides *p = g_ovr.load(std::memory_order_acquire);
+  return p ? *p : publish_overrides(false);
 }
 
 }  // namespace
@@ -406,8 +425,7 @@ double dram_us(int64_t M, int64_t N, int64_t K, bool int8, bool pair) {
   return (a_bytes + b_bytes * rb + c_bytes) / (plan_table::kHbmGBs * 1e3);
 }
 
-Plan make_plan(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sms, int pairs,
-               bool allow_tail = true) {
+Plan search_plan(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sms, int pairs, bool allow_tail) {
   Plan pl{};
   // compiled widths, widest first: the bf16 single-CTA kernels also come 64
   // and 96 wide (96 for B column-major only), for memory-bound GEMMs with
@@ -415,7 +433,7 @@ Plan make_plan(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sms,
   static const int kWidthsKMajor[] = {256, 224, 192, 128, 96, 64};
   static const int kWidthsMNMajor[] = {256, 192, 128, 64};
   static const int kPairWidthsMNMajor[] = {256, 128};
-  const Overrides ovr = overrides();
+  const Overrides &ovr = overrides();
   const bool int8 = epi == kEpiS32;
   const int64_t num_kb = ceil_div(K, kBK);
   bool best_pair = false;
@@ -543,6 +561,40 @@ Plan make_plan(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sms,
                  (long long)tiles_n, (long long)splits, (long long)best_tail, p.tail_first, pl.grid, best_model, sms,
                  pairs);
   return pl;
+}
+
+// search_plan, remembered per thread for the last shapes it was asked for (a
+// program calls a few shapes over and over; the search costs 1.2 us of a 4 us
+// call).  A plan depends on these sizes, the device's SM counts and the
+// overrides alone; it holds no pointer.
+Plan make_plan(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sms, int pairs, bool allow_tail = true) {
+  struct Entry {
+    int64_t M = -1, N, K;
+    int sms, pairs;
+    int form;  // layout, epilogue and allow_tail
+    const Overrides *ovr;
+    Plan plan;
+  };
+  constexpr uint64_t kEntries = 64;
+  thread_local Entry cache[kEntries];
+  const Overrides *ovr = &overrides();
+  const int form = (b_kmajor ? 1 : 0) | (allow_tail ? 2 : 0) | epi << 2;
+  uint64_t h = (uint64_t)M * 0x9E3779B97F4A7C15ull ^ (uint64_t)N * 0xC2B2AE3D27D4EB4Full ^
+               (uint64_t)K * 0x165667B19E3779F9ull ^ (uint64_t)form;
+  h ^= h >> 29;
+  Entry &e = cache[h % kEntries];
+  if (e.M == M && e.N == N && e.K == K && e.sms == sms && e.pairs == pairs && e.form == form && e.ovr == ovr &&
+      !ovr->debug)
+    return e.plan;
+  e.M = M;
+  e.N = N;
+  e.K = K;
+  e.sms = sms;
+  e.pairs = pairs;
+  e.form = form;
+  e.ovr = ovr;
+  e.plan = search_plan(M, N, K, b_kmajor, epi, sms, pairs, allow_tail);
+  return e.plan;
 }
 
 struct WsLayout {
@@ -676,7 +728,7 @@ constexpr int64_t kTinyMaxK = 512;
 constexpr int64_t kTinyMaxMacsForced = int64_t(1) << 27;
 
 bool tiny_shape(int64_t M, int64_t N, int64_t K) {
-  const Overrides o = overrides();
+  const Overrides &o = overrides();
   // a forced tile width, family or split asks for the tensor-core kernels
   if (o.bn > 0 || o.pair >= 0 || o.splits >= 1 || o.tail_splits >= 2) return false;
   const double macs = (double)M * (double)N * (double)K;
@@ -744,7 +796,7 @@ gemm_status_t run_skinny(DeviceState &d, int64_t M, int64_t N, int64_t K, const 
 // than the kernels that took those shapes before at every size measured
 // (gemm_rows.cu has the figures); its accumulators are built for 16.
 int rows_max(bool int8) {
-  const Overrides o = overrides();
+  const Overrides &o = overrides();
   if (o.skinny_max_m >= 0 || o.bn > 0 || o.pair >= 0 || o.splits >= 1 || o.tail_splits >= 2) return 0;
   return int8 && !o.s8tm ? 0 : kRowsMax;
 }
@@ -945,7 +997,7 @@ bool s8tm_shape(int64_t M, int64_t N, bool b_kmajor, bool *swap, bool *p_kmajor)
 bool try_s8tm(DeviceState &d, int64_t M, int64_t N, int64_t K, const int8_t *A, int64_t lda, const int8_t *B,
               int64_t ldb, bool b_kmajor, void *C, int64_t ldc, int out_bits, int shift, cudaStream_t st,
               gemm_status_t *status) {
-  const Overrides ovr = overrides();
+  const Overrides &ovr = overrides();
   if (!ovr.s8tm) return false;
   bool swap, p_kmajor;  // p_kmajor false: B stored K x N, P's rows are its k-rows
   if (!s8tm_shape(M, N, b_kmajor, &swap, &p_kmajor)) return false;
@@ -1167,10 +1219,7 @@ void gemm_release_resources(void) {
 uint64_t gemm_launch_count(void) { return g_launches.load(); }
 
 void gemm_reload_overrides(void) {
-  const Overrides o = read_overrides();
-  std::lock_guard<std::mutex> lk(g_ovr_mu);
-  g_ovr = o;
-  g_ovr_loaded = true;
+  publish_overrides(true);
 }
 
 gemm_status_t gemm_selftest_wait_timeout(uint64_t limit_ns, gemm_stream_t stream) {

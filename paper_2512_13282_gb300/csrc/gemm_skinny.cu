@@ -451,6 +451,13 @@ __global__ void __launch_bounds__(kSkThreads, colb_blocks(MT)) skinny_colB_kerne
   finish_block<INT8>(p, red, kCols, n0, cols, &ticket);
 }
 
+// Shared memory beyond the 48 KB every kernel may use needs an opt-in.
+template <typename Kern>
+cudaError_t opt_in(Kern kern, size_t smem) {
+  if (smem <= 48 * 1024) return cudaSuccess;
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+
 template <int MT, bool INT8>
 cudaError_t launch_mt(const SkinnyParams &p, dim3 grid, bool row_b, cudaStream_t st) {
   if (row_b) {
@@ -461,7 +468,7 @@ cudaError_t launch_mt(const SkinnyParams &p, dim3 grid, bool row_b, cudaStream_t
     const size_t red_bytes = (size_t)MT * kCols * 4 * (INT8 ? 1 : kSkWarps + 1);
     const size_t smem = a_bytes > red_bytes ? a_bytes : red_bytes;
     auto kern = skinny_rowB_kernel<MT, VB, INT8, sh.rb, sh.bps>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = opt_in(kern, smem);
     if (e != cudaSuccess) return e;
     e = launch_ex(kern, grid, dim3(kSkThreads), smem, st, 1, p);
     if (e != cudaSuccess) return e;
@@ -471,7 +478,7 @@ cudaError_t launch_mt(const SkinnyParams &p, dim3 grid, bool row_b, cudaStream_t
     const size_t red_bytes = (size_t)MT * 32 * 4;
     const size_t smem = a_bytes > red_bytes ? a_bytes : red_bytes;
     auto kern = skinny_colB_kernel<MT, INT8>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = opt_in(kern, smem);
     if (e != cudaSuccess) return e;
     e = launch_ex(kern, grid, dim3(kSkThreads), smem, st, 1, p);
     if (e != cudaSuccess) return e;

@@ -56,6 +56,8 @@ class GemmError(RuntimeError):
 def library():
     """The loaded ``libgb300gemm.so`` (raises if it has not been built)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -99,13 +101,30 @@ def _ptr(x) -> int:
         return 0
     if isinstance(x, int):
         return x
-    return int(x.data_ptr())
+    return x.data_ptr()
+
+
+_current_stream = None  # torch's current stream on the current device, as a handle
+
+
+def _bind_current_stream():
+    """The function behind ``_current_stream``.  ``torch.cuda.current_stream()``
+    builds a Stream object on every call (2.8 us on the Grace cores, more than
+    the rest of this binding); the handle itself is a C call of 0.1 us."""
+    import torch
+    torch.cuda.init()
+    device, raw = getattr(torch._C, "_cuda_getDevice", None), getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if device is None or raw is None:
+        return lambda: int(torch.cuda.current_stream().cuda_stream)
+    return lambda: raw(device())
 
 
 def _stream(s) -> int:
     if s is None:
-        import torch
-        return int(torch.cuda.current_stream().cuda_stream)
+        global _current_stream
+        if _current_stream is None:
+            _current_stream = _bind_current_stream()
+        return _current_stream()
     if isinstance(s, int):
         return s
     return int(s.cuda_stream)
