@@ -245,12 +245,21 @@ __device__ __forceinline__ void sum_piece(const T *__restrict__ ws, int splits, 
 #pragma unroll
   for (int i = 0; i < 4; ++i) v[i] = T(0);
   if (pc.n == 4 && vec) {
-    for (int k = 0; k < splits; ++k) {
-      const uint4 w = __ldcs(reinterpret_cast<const uint4 *>(ws + (int64_t)k * MN + base));
-      T x[4];
-      memcpy(x, &w, sizeof w);
+    // the planes in order, four loads in flight at a time (one after the
+    // other would cost a memory latency per plane)
+    for (int k = 0; k < splits; k += 4) {
+      uint4 w[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) v[i] += x[i];
+      for (int j = 0; j < 4; ++j)
+        if (k + j < splits) w[j] = __ldcs(reinterpret_cast<const uint4 *>(ws + (int64_t)(k + j) * MN + base));
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (k + j >= splits) break;
+        T x[4];
+        memcpy(x, &w[j], sizeof w[j]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] += x[i];
+      }
     }
   } else {
     for (int k = 0; k < splits; ++k)

@@ -166,16 +166,22 @@ __global__ void __launch_bounds__(kRowsThreads, kRowsBlocks) gemm_rows_kernel(co
 
   auto load_half = [&](int k, uint4 (&w)[4], uint4 (&x)[NT]) {
     const int64_t at = (int64_t)k * ES;
-    const bool whole = k + kHalf <= kend;
-    const int valid = (kend - k) * ES - 16 * q;
+    const int valid = (kend - k) * ES - 16 * q;  // bytes of the lane's piece before the slice's end
+    const bool whole = valid >= 16;
     if (whole) {
 #pragma unroll
       for (int i = 0; i < 4; ++i) w[i] = __ldcs(reinterpret_cast<const uint4 *>(wp[i] + at));
+    } else if (valid <= 0) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) w[i] = make_uint4(0u, 0u, 0u, 0u);
     } else {
 #pragma unroll
       for (int i = 0; i < 4; ++i) w[i] = load16_edge(wp[i] + at, ES, valid);
     }
-    if (whole && p.x_vec) {
+    if (valid <= 0) {
+#pragma unroll
+      for (int j = 0; j < NT; ++j) x[j] = make_uint4(0u, 0u, 0u, 0u);
+    } else if (whole && p.x_vec) {
 #pragma unroll
       for (int j = 0; j < NT; ++j) x[j] = __ldg(reinterpret_cast<const uint4 *>(xp[j] + at));
     } else {

@@ -22,18 +22,18 @@ struct StepCost {
 // [0 bf16, 1 int8][0 single CTA, 1 CTA pair][BN 64, 96, 128, 192, 224, 256]; {0, 0}: not compiled
 constexpr StepCost kCost[2][2][6] = {
     {
-        {{0.26885f, 0.0812f}, {0.27958f, 0.0000f}, {0.27863f, 0.1047f}, {0.29486f, 0.5838f}, {0.28341f, 2.6772f}, {0.35269f, 1.0832f}},
-        {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.27831f, 0.7914f}, {0.28422f, 1.2185f}, {0.27975f, 3.0965f}, {0.29593f, 1.6487f}},
+        {{0.14600f, 0.1401f}, {0.16741f, 0.3322f}, {0.21090f, 0.3281f}, {0.28599f, 0.6118f}, {0.25697f, 3.7654f}, {0.34977f, 1.1271f}},
+        {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.16995f, 1.3202f}, {0.23027f, 1.8002f}, {0.23069f, 4.5338f}, {0.29964f, 1.9946f}},
     },
     {
-        {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.27747f, 0.7737f}, {0.32572f, 0.4431f}, {0.32053f, 1.8369f}, {0.34649f, 1.0229f}},
-        {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.27132f, 2.2076f}, {0.28326f, 2.1272f}, {0.28409f, 3.1620f}, {0.28704f, 3.1176f}},
+        {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.18873f, 1.2100f}, {0.30843f, 0.8441f}, {0.28810f, 1.9227f}, {0.35987f, 1.4159f}},
+        {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.16863f, 2.4881f}, {0.21109f, 3.0536f}, {0.23396f, 4.0198f}, {0.27329f, 3.6180f}},
     },
 };
 
 // split-K: [0 bf16, 1 int8]
-constexpr float kSplitFixedUs[2] = {2.6661f, 2.0597f};
-constexpr float kSplitUsPerMB[2] = {0.34096f, 0.19795f};
+constexpr float kSplitFixedUs[2] = {3.0379f, 1.5380f};
+constexpr float kSplitUsPerMB[2] = {0.25321f, 0.20626f};
 
 // Eq. 10: DRAM bandwidth (GB/s) and the L2 capacity the reuse factors use.
 constexpr double kHbmGBs = 6693.8;

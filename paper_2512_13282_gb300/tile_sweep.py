@@ -5,14 +5,16 @@ starting values and each step's efficiency are measured on the device).  For
 each shape of a fixed set -- the tensor-core GEMMs of the benchmark
 workloads and a seeded sample of the roofline sweep sizes -- every plan the
 library can be forced into (kernel family: one CTA per 128-row tile or a CTA
-pair per 256-row tile; tile width BN; split-K factor S; split tail T) is timed with CUDA
-events after a 512 MiB L2 flush: the mean of `reps` launches without the
-fastest and the slowest (the event clock advances in steps of about 1 us on
-GB300, so a median of a few launches of a 10-30 us GEMM is off by up to a
-step; a mean of many is not).  The result is written as JSON; tile_model.py
-fits the planner's cost table to it.
+pair per 256-row tile; tile width BN; split-K factor S; split tail T) is timed
+as a program runs it: calls back to back on one stream, over enough operand
+copies that together they exceed L2 (up to 16), between two CUDA events around
+at least `ms` milliseconds of calls, the median of three such runs after one
+untimed.  Runs that long are under the power limit where a program's would be
+(a burst of 8192^3 GEMMs runs 6 % faster than a stream of them, and favours
+tiles that multiply more padding).  The result is written as JSON;
+tile_model.py fits the planner's cost table to it.
 
-    python -m paper_2512_13282_gb300.tile_sweep OUT.json [--reps 15] [--sample 40]
+    python -m paper_2512_13282_gb300.tile_sweep OUT.json [--ms 4] [--sample 60]
 
 Needs a GPU and the built library.  Results of int8 GEMMs are exact whatever
 the plan, and bf16 results differ only in summation order, so no plan is
@@ -23,7 +25,6 @@ from __future__ import annotations
 import argparse
 import json
 import os
-import statistics
 import sys
 import time
 
@@ -38,10 +39,12 @@ ENV_KEYS = ("GB300_GEMM_BN", "GB300_GEMM_PAIR", "GB300_GEMM_SPLITS", "GB300_GEMM
 TC_ONLY = {"GB300_GEMM_SKINNY_MAX_M": 0, "GB300_GEMM_S8TM": 0, "GB300_GEMM_TINY_MAX_MACS": 0}
 
 
-def sweep_shapes(sample: int = 40, seed: int = 11):
+def sweep_shapes(sample: int = 60, seed: int = 11):
     """(M, N, K, dtype, layout) of the sweep: the workloads' GEMMs with M > 8
     that the tensor-core kernels run (int8-int32 and bf16), then `sample`
-    roofline sizes (both dtypes, B column-major) drawn with `seed`."""
+    roofline sizes (both dtypes, B column- and row-major in turn) drawn with
+    `seed`, and half as many sizes that no tile divides (multiples of 16,
+    uniform in log size from 128 to 8192, one dtype each)."""
     seen, out = set(), []
     for wl in ("square_sweep_512_4096", "square_8192", "transformer_projections", "irregular_skinny",
                "int8_square_256"):
@@ -54,13 +57,19 @@ def sweep_shapes(sample: int = 40, seed: int = 11):
                 out.append(key)
     rng = np.random.default_rng(seed)
     sizes = W.roofline_sweep_sizes()
-    for i in rng.choice(len(sizes), sample, replace=False):
+    for n, i in enumerate(rng.choice(len(sizes), sample, replace=False)):
         M, N, K = sizes[int(i)]
         for dt in ("int8", "bf16"):
-            key = (M, N, K, dt, W.B_COL_MAJOR)
+            key = (M, N, K, dt, W.B_ROW_MAJOR if n % 3 == 2 else W.B_COL_MAJOR)
             if key not in seen:
                 seen.add(key)
                 out.append(key)
+    for n in range(sample // 2):
+        M, N, K = (16 * int(round(np.exp(rng.uniform(np.log(8), np.log(512))))) for _ in range(3))
+        key = (M, N, K, "int8" if n % 2 else "bf16", W.B_ROW_MAJOR if n % 4 >= 2 else W.B_COL_MAJOR)
+        if key not in seen and M * N * K <= 1 << 38:
+            seen.add(key)
+            out.append(key)
     return out
 
 
@@ -72,23 +81,31 @@ def main(argv=None):
 
     ap = argparse.ArgumentParser()
     ap.add_argument("out")
-    ap.add_argument("--reps", type=int, default=15)
-    ap.add_argument("--sample", type=int, default=40)
+    ap.add_argument("--ms", type=float, default=4.0)
+    ap.add_argument("--sample", type=int, default=60)
     args = ap.parse_args(argv)
     Bld.build()
     G.library()
     dev = torch.device("cuda", 0)
     torch.cuda.set_device(dev)
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
-    flush = torch.empty((512 << 20) // 4, dtype=torch.float32, device=dev)
     st = torch.cuda.current_stream()
     shapes = sweep_shapes(args.sample)
-    big = max(max(m * k, k * n) for m, n, k, _, _ in shapes)
-    dA = torch.from_numpy(W.random_int8((big,), 31)).to(dev)
-    dB = torch.from_numpy(W.random_int8((big,), 32)).to(dev)
-    hA16 = torch.from_numpy(W.random_bf16((big,), 33).view(np.int16)).to(dev)
-    hB16 = torch.from_numpy(W.random_bf16((big,), 34).view(np.int16)).to(dev)
-    dC = torch.empty(max(m * n for m, n, _, _, _ in shapes) * 4, dtype=torch.uint8, device=dev)
+
+    def operands(M, N, K, dtype, layout):
+        """Copies of (A, B, C) that together exceed three times L2, at most 16."""
+        b_shape = (K, N) if layout == W.B_ROW_MAJOR else (N, K)
+        esize = 1 if dtype == "int8" else 2
+        copies = []
+        for i in range(max(2, min(16, -(-400_000_000 // (esize * (M * K + N * K)))))):
+            gen = torch.Generator(device="cuda").manual_seed(31 + i)
+            if dtype == "int8":
+                A, B = (torch.randint(-128, 128, s, generator=gen, device=dev, dtype=torch.int8)
+                        for s in ((M, K), b_shape))
+            else:
+                A, B = (torch.randn(s, generator=gen, device=dev).to(torch.bfloat16) for s in ((M, K), b_shape))
+            copies.append((A, B, torch.empty((M, N), device=dev, dtype=torch.int32 if dtype == "int8" else torch.bfloat16)))
+        return copies
 
     def setenv(d):
         for k in ENV_KEYS:
@@ -97,37 +114,41 @@ def main(argv=None):
             os.environ[k] = str(v)
         G.gemm_reload_overrides()
 
-    def time_plan(M, N, K, dtype, layout):
+    def time_plan(M, N, K, dtype, layout, copies):
         ldb = N if layout == W.B_ROW_MAJOR else K
-        if dtype == "int8":
-            fn, A, B, C = G.gemm_s8s8_s32, dA, dB, dC.view(torch.int32)
-        else:
-            fn, A, B, C = G.gemm_bf16_f32acc_bf16, hA16, hB16, dC.view(torch.int16)
-        ts = []
-        for r in range(args.reps + 2):
-            flush.fill_(float(r))
+        fn = G.gemm_s8s8_s32 if dtype == "int8" else G.gemm_bf16_f32acc_bf16
+
+        def calls(n):
+            for i in range(n):
+                A, B, C = copies[i % len(copies)]
+                rc = fn(M, N, K, A, K, B, ldb, layout, C, N, st.cuda_stream)
+                if rc != 0:
+                    raise RuntimeError(f"{dtype} {M}x{N}x{K}: {G.gemm_status_string(rc)}")
+
+        est = max(4e-6, 2.0 * M * N * K / 1.5e15)
+        n = max(4, int(args.ms * 1e-3 / est))
+        times = []
+        for r in range(4):
             a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
             a.record(st)
-            rc = fn(M, N, K, A, K, B, ldb, layout, C, N, st)
+            calls(n)
             b.record(st)
-            if rc != 0:
-                raise RuntimeError(f"{dtype} {M}x{N}x{K}: {G.gemm_status_string(rc)}")
-            if r >= 2:
-                ts.append((a, b))
-        torch.cuda.synchronize()
-        us = sorted(x.elapsed_time(y) * 1e3 for x, y in ts)
-        return statistics.mean(us[1:-1]) if len(us) > 2 else statistics.mean(us)
+            torch.cuda.synchronize()
+            if r:
+                times.append(a.elapsed_time(b) * 1e3 / n)
+        return sorted(times)[1]
 
     rows = []
     t0 = time.time()
     for (M, N, K, dtype, layout) in shapes:
         setenv(TC_ONLY)
-        default_us = time_plan(M, N, K, dtype, layout)
+        copies = operands(M, N, K, dtype, layout)
+        default_us = time_plan(M, N, K, dtype, layout, copies)
         plans = []
         for c in candidate_plans(M, N, K, dtype, layout == W.B_COL_MAJOR, sms=sms, pair_slots=GB300["pair_slots"]):
             setenv(dict(TC_ONLY, GB300_GEMM_PAIR=int(c["pair"]), GB300_GEMM_BN=c["bn"],
                         GB300_GEMM_SPLITS=c["splits"], GB300_GEMM_TAIL_SPLITS=c["tail_splits"]))
-            plans.append(dict(c, us=round(time_plan(M, N, K, dtype, layout), 3)))
+            plans.append(dict(c, us=round(time_plan(M, N, K, dtype, layout, copies), 3)))
         best = min(plans, key=lambda p: p["us"])
         print(f"{dtype:4s} {M}x{N}x{K} {'col' if layout else 'row'}: planner {default_us:8.1f} us, best forced "
               f"{best['us']:8.1f} ({'pair' if best['pair'] else 'single'} BN={best['bn']} S={best['splits']} "
@@ -137,8 +158,8 @@ def main(argv=None):
                      "planner_us": round(default_us, 3), "plans": plans})
     setenv({})
     with open(args.out, "w") as f:
-        json.dump({"device": torch.cuda.get_device_name(dev), "sms": sms, "reps": args.reps,
-                   "flush": "512 MiB write before every launch", "statistic": "mean without min and max",
+        json.dump({"device": torch.cuda.get_device_name(dev), "sms": sms, "ms": args.ms,
+                   "method": "calls back to back over operand copies larger than L2", "statistic": "median of three runs",
                    "seconds": round(time.time() - t0, 1),
                    "shapes": rows}, f, indent=0)
 
