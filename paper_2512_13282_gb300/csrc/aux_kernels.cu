@@ -62,8 +62,9 @@ __device__ __forceinline__ void piece_rc(uint64_t u, uint32_t cpr, int w, int64_
 // flat list of 16-element row pieces -- piece t < items_a is piece t % cpr_a
 // of row t / cpr_a of A (cpr = pieces per row), the rest likewise of B.  A
 // thread reads its 16 bytes with the widest loads the row's address allows
-// (16, 8 or 4 bytes, else bytes), several in flight, and writes 32 bytes
-// with two 16-byte stores (staged rows start 16-byte aligned).
+// (odd rows as five aligned words, shifted; byte by byte they took 1.5 times
+// the GEMM's own time at 1001 x 1503 x 3001) and writes 32 bytes with two
+// 16-byte stores (staged rows start 128-byte aligned).
 __global__ void __launch_bounds__(kS8Threads)
     s8_to_bf16_pair_kernel(const S8Job a, const S8Job b, uint32_t cpr_a, uint32_t cpr_b, uint64_t items_a,
                            uint64_t items) {
@@ -77,24 +78,9 @@ __global__ void __launch_bounds__(kS8Threads)
   const int8_t *src = j.src + r * j.ld_src + c;
   uint16_t *dst = j.dst + r * j.ld_dst + c;
   if (c + 16 <= j.cols) {
-    const uintptr_t al = reinterpret_cast<uintptr_t>(src);
-    int4 raw;
-    if ((al & 15) == 0) {
-      raw = __ldcs(reinterpret_cast<const int4 *>(src));
-    } else if ((al & 7) == 0) {
-      const int2 x = __ldcs(reinterpret_cast<const int2 *>(src)), y = __ldcs(reinterpret_cast<const int2 *>(src) + 1);
-      raw = make_int4(x.x, x.y, y.x, y.y);
-    } else if ((al & 3) == 0) {
-      const int *q = reinterpret_cast<const int *>(src);
-      raw = make_int4(__ldcs(q), __ldcs(q + 1), __ldcs(q + 2), __ldcs(q + 3));
-    } else {
-      uint32_t w[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        w[i] = (uint32_t)(uint8_t)src[4 * i] | ((uint32_t)(uint8_t)src[4 * i + 1] << 8) |
-               ((uint32_t)(uint8_t)src[4 * i + 2] << 16) | ((uint32_t)(uint8_t)src[4 * i + 3] << 24);
-      raw = make_int4((int)w[0], (int)w[1], (int)w[2], (int)w[3]);
-    }
+    const uint8_t *lo8 = reinterpret_cast<const uint8_t *>(j.src), *hi8 = lo8 + (j.rows - 1) * j.ld_src + j.cols;
+    const uint4 v = load16_any<true>(reinterpret_cast<const uint8_t *>(src), lo8, hi8);
+    const int4 raw = make_int4((int)v.x, (int)v.y, (int)v.z, (int)v.w);
     uint4 lo, hi;
     s8x16_to_bf16x16(raw, lo, hi);
     uint4 *d = reinterpret_cast<uint4 *>(dst);
@@ -133,40 +119,22 @@ __global__ void __launch_bounds__(kS8Threads)
   }
 }
 
-// Re-pitch of a bf16 matrix into a buffer whose rows start 16-byte aligned:
-// thread t copies 4-element piece t % cpr of row t / cpr (one 8-byte load
-// where the source row allows it, else two 4-byte or four 2-byte loads; one
-// 8-byte store).
+// Re-pitch of a bf16 matrix into a buffer whose rows start 128-byte aligned:
+// thread t copies 8-element piece t % cpr of row t / cpr with one 16-byte
+// store (the source as for the int8 staging above).
 __global__ void __launch_bounds__(kS8Threads)
-    pack_u16_kernel(const uint16_t *__restrict__ src, int64_t cols, int64_t ld_src, uint16_t *__restrict__ dst,
-                    int64_t ld_dst, uint32_t cpr, uint64_t items) {
+    pack_u16_kernel(const uint16_t *__restrict__ src, int64_t rows, int64_t cols, int64_t ld_src,
+                    uint16_t *__restrict__ dst, int64_t ld_dst, uint32_t cpr, uint64_t items) {
   griddep_wait();
   const uint64_t t = (uint64_t)blockIdx.x * kS8Threads + threadIdx.x;
   if (t >= items) return;
-  uint64_t r, q;
-  if (t <= 0xFFFFFFFFull) {
-    r = (uint32_t)t / cpr;
-    q = (uint32_t)t - (uint32_t)r * cpr;
-  } else {
-    r = t / cpr;
-    q = t - r * cpr;
-  }
-  const int64_t c = (int64_t)q * 4;
-  const uint16_t *s = src + (int64_t)r * ld_src + c;
-  uint16_t *d = dst + (int64_t)r * ld_dst + c;
-  if (c + 4 <= cols) {
-    const uintptr_t al = reinterpret_cast<uintptr_t>(s);
-    uint2 v;
-    if ((al & 7) == 0) {
-      v = __ldcs(reinterpret_cast<const uint2 *>(s));
-    } else if ((al & 3) == 0) {
-      v.x = __ldcs(reinterpret_cast<const unsigned int *>(s));
-      v.y = __ldcs(reinterpret_cast<const unsigned int *>(s) + 1);
-    } else {
-      v.x = (uint32_t)s[0] | ((uint32_t)s[1] << 16);
-      v.y = (uint32_t)s[2] | ((uint32_t)s[3] << 16);
-    }
-    *reinterpret_cast<uint2 *>(d) = v;
+  int64_t r, c;
+  piece_rc(t, cpr, 8, r, c);
+  const uint16_t *s = src + r * ld_src + c;
+  uint16_t *d = dst + r * ld_dst + c;
+  if (c + 8 <= cols) {
+    const uint8_t *lo = reinterpret_cast<const uint8_t *>(src), *hi = lo + ((rows - 1) * ld_src + cols) * 2;
+    *reinterpret_cast<uint4 *>(d) = load16_any<true>(reinterpret_cast<const uint8_t *>(s), lo, hi);
   } else {
     for (int64_t i = 0; c + i < cols; ++i) d[i] = s[i];
   }
@@ -402,10 +370,10 @@ cudaError_t launch_s8_to_bf16_pair(const S8Job &a, const S8Job &b, int sms, cuda
 cudaError_t launch_pack_u16(const uint16_t *src, int64_t rows, int64_t cols, int64_t ld_src,
                             uint16_t *dst, int64_t ld_dst, int sms, cudaStream_t st) {
   (void)sms;
-  const uint64_t cpr = (uint64_t)(cols + 3) / 4, items = (uint64_t)rows * cpr;
+  const uint64_t cpr = (uint64_t)(cols + 7) / 8, items = (uint64_t)rows * cpr;
   if (items == 0) return cudaSuccess;
   return launch_ex(pack_u16_kernel, dim3((unsigned)((items + kS8Threads - 1) / kS8Threads)), dim3(kS8Threads), 0, st, 1,
-                   src, cols, ld_src, dst, ld_dst, (uint32_t)cpr, items);
+                   src, rows, cols, ld_src, dst, ld_dst, (uint32_t)cpr, items);
 }
 
 cudaError_t launch_zero_fill(void *C, int64_t M, int64_t N, int64_t ldc, int esize, int sms,

@@ -597,6 +597,11 @@ Plan make_plan(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sms,
   return e.plan;
 }
 
+// Row pitch (elements) of a staged or re-pitched bf16 copy with rows of n
+// elements: whole 128-byte lines, so that a TMA box row is one line and not
+// the ends of two (int8 2592^3: 41.7 us with rows of 40.5 lines).
+int64_t staged_pitch(int64_t n) { return (n + 63) / 64 * 64; }
+
 struct WsLayout {
   size_t a_off = 0, b_off = 0, part_off = 0, total = 0;
 };
@@ -741,18 +746,21 @@ bool tiny_shape(int64_t M, int64_t N, int64_t K) {
 // used at most a few times and streaming B once is the cost.  bf16,
 // accumulating with fp32 FMAs, wins up to M = 2 (measured on GB300 against
 // the tensor-core path, N = 4096..11008, K = 4096); int8, through dp4a, up to
-// M = 8 where the alternative stages B.  Where the small-operand kernel can
+// M = 8 where the alternative stages a small B (2003 x 3001 stored N x K: M = 8
+// 18.0 / 20.2 us; stored K x N: M = 3 18.6 / 19.6, M = 8 26.9 / 19.8), or up
+// to M = 2 for a larger one (5001 x 5001: M = 2 30.7 / 30.5 and 26.7 / 30.5,
+// M = 3 33.9 / 32.1 and 38.9 / 32.2).  Where the small-operand kernel can
 // read a row-major B as it is (`in_place`), that kernel is faster from M = 2
 // on (K = 4096, back to back: M = 1 x 4096 8.4 / 9.7 us, 2 x 4096 11.0 /
 // 9.7, 4 x 4096 12.9 / 9.8, 8 x 4096 18.1 / 9.9, 4 x 12288 24.1 / 17.0),
 // except M = 2 with a small B (2 x 1024 x 1024 5.9 / 6.2) or a wide one (2 x
 // 12288 16.4 / 17.0).  GB300_GEMM_SKINNY_MAX_M overrides (0 disables the
 // kernel).
-int skinny_max_m(bool int8, int64_t N, int64_t K, bool in_place) {
+int skinny_max_m(bool int8, int64_t N, int64_t K, bool b_kmajor, bool in_place) {
   const int v = overrides().skinny_max_m;
   if (v >= 0) return v > 16 ? 16 : v;
   if (!int8) return 2;
-  if (!in_place) return 8;
+  if (!in_place) return N * K > (int64_t(1) << 23) ? 2 : (b_kmajor ? 8 : 3);
   return N >= 8192 || N * K < (int64_t(1) << 22) ? 2 : 1;
 }
 
@@ -816,8 +824,10 @@ bool rows_shape(int64_t M, int64_t N, int64_t K, bool b_kmajor, bool int8, bool 
 
 // GEMMs with at most kRowsMax rows of A against a column-major B, or at most
 // kRowsMax columns of a column-major B against A: gemm_rows_kernel streams the
-// other operand, which has to be 16-byte aligned in base and pitch.  Returns
-// false, having launched nothing, for any other.
+// other operand, which has to be 16-byte aligned in base and pitch (on odd
+// addresses its lanes would load five words per 16 bytes: 16 x 5000 x 5001
+// bf16 71 us against 30 for re-pitching and the tensor cores).  Returns false,
+// having launched nothing, for any other.
 bool try_rows(DeviceState &d, int64_t M, int64_t N, int64_t K, const void *A, int64_t lda, const void *B,
               int64_t ldb, bool b_kmajor, void *C, int64_t ldc, bool int8, int out_bits, int out_shift,
               cudaStream_t st, gemm_status_t *status) {
@@ -873,7 +883,7 @@ gemm_status_t gemm_bf16_f32acc_bf16(int64_t M, int64_t N, int64_t K, const uint1
   }
   const bool b_kmajor = b_layout == GEMM_B_COL_MAJOR_NxK;
   if (try_rows(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, false, 0, 0, st, &s)) return s;
-  if (M <= skinny_max_m(false, N, K, false))
+  if (M <= skinny_max_m(false, N, K, b_kmajor, false))
     return run_skinny(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, false, st);
   Plan pl = make_plan(M, N, K, b_kmajor, kEpiBf16, d->sms, pair_slots());
   // TMA needs 16-byte aligned bases and row pitches; re-pitch an operand
@@ -881,7 +891,7 @@ gemm_status_t gemm_bf16_f32acc_bf16(int64_t M, int64_t N, int64_t K, const uint1
   const bool pack_a = !(aligned16(A) && (lda * 2) % 16 == 0);
   const bool pack_b = !(aligned16(B) && (ldb * 2) % 16 == 0);
   const int64_t b_rows = b_kmajor ? N : K, b_cols = b_kmajor ? K : N;
-  const int64_t lda_p = (K + 7) / 8 * 8, ldb_p = (b_cols + 7) / 8 * 8;
+  const int64_t lda_p = staged_pitch(K), ldb_p = staged_pitch(b_cols);
   WsLayout L;
   size_t off = 0;
   if (pack_a) { L.a_off = off; off = align_up(off + (size_t)M * lda_p * 2, 256); }
@@ -1113,7 +1123,7 @@ gemm_status_t s8_gemm(int64_t M, int64_t N, int64_t K, const int8_t *A, int64_t 
   const bool b_kmajor = b_layout == GEMM_B_COL_MAJOR_NxK;
   if (try_rows(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, true, out_bits, shift, st, &s)) return s;
   const bool in_place = overrides().s8tm && !b_kmajor && N > kBM && aligned16(B) && ldb % 16 == 0;
-  if (M <= skinny_max_m(true, N, K, in_place))
+  if (M <= skinny_max_m(true, N, K, b_kmajor, in_place))
     return run_skinny(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, true, st, out_bits, shift);
   if (tiny_shape(M, N, K)) {
     const TinyParams tp{A, lda, B, ldb, C, ldc, M, N, K, out_bits, shift};
@@ -1128,9 +1138,9 @@ gemm_status_t s8_gemm(int64_t M, int64_t N, int64_t K, const int8_t *A, int64_t 
   Plan pl = make_plan(M, N, K, b_kmajor, kEpiS32, d->sms, pair_slots());
   pl.p.out_bits = out_bits;
   pl.p.out_shift = shift;
-  // Stage both operands as bf16 (exact for int8) with 16-byte aligned rows.
+  // Stage both operands as bf16 (exact for int8) with 128-byte aligned rows.
   const int64_t b_rows = b_kmajor ? N : K, b_cols = b_kmajor ? K : N;
-  const int64_t lda_p = (K + 7) / 8 * 8, ldb_p = (b_cols + 7) / 8 * 8;
+  const int64_t lda_p = staged_pitch(K), ldb_p = staged_pitch(b_cols);
   WsLayout L;
   size_t off = 0;
   L.a_off = off;
@@ -1260,7 +1270,7 @@ gemm_status_t gemm_plan_query(int64_t M, int64_t N, int64_t K, int int8, int b_l
     return GEMM_OK;
   }
   const bool in_place = overrides().s8tm && !b_kmajor && N > kBM && N % 16 == 0;
-  if (M <= skinny_max_m(int8 != 0, N, K, in_place)) {
+  if (M <= skinny_max_m(int8 != 0, N, K, b_kmajor, in_place)) {
     out->route = GEMM_ROUTE_SMALL_M;
     return GEMM_OK;
   }

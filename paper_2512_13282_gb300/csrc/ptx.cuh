@@ -249,6 +249,39 @@ __device__ __forceinline__ void s8x4_to_f16x4(uint32_t w, uint32_t &lo, uint32_t
   hi = *reinterpret_cast<const uint32_t *>(&y);
 }
 
+// ------------------------------------------------ 16 bytes at any address
+
+// The 16 bytes at a, on any byte boundary, with the widest aligned loads its
+// address allows; on odd addresses five aligned 32-bit words shifted into
+// place, where those lie inside [lo, hi), the matrix the bytes belong to, else
+// byte by byte.
+template <bool STREAM>
+__device__ __forceinline__ uint4 load16_any(const uint8_t *a, const uint8_t *lo, const uint8_t *hi) {
+  const uint32_t m = (uint32_t)reinterpret_cast<uintptr_t>(a) & 15u;
+  if (m == 0)
+    return STREAM ? __ldcs(reinterpret_cast<const uint4 *>(a)) : __ldg(reinterpret_cast<const uint4 *>(a));
+  if ((m & 7u) == 0) {
+    const uint2 x = __ldg(reinterpret_cast<const uint2 *>(a)), y = __ldg(reinterpret_cast<const uint2 *>(a) + 1);
+    return make_uint4(x.x, x.y, y.x, y.y);
+  }
+  const uint32_t sh = 8u * (m & 3u);
+  const uint8_t *al = a - (m & 3u);
+  if (sh == 0 || (al >= lo && al + 20 <= hi)) {
+    const uint32_t *q = reinterpret_cast<const uint32_t *>(al);
+    const uint32_t w0 = __ldg(q), w1 = __ldg(q + 1), w2 = __ldg(q + 2), w3 = __ldg(q + 3);
+    if (sh == 0) return make_uint4(w0, w1, w2, w3);
+    const uint32_t w4 = __ldg(q + 4);
+    return make_uint4(__funnelshift_r(w0, w1, sh), __funnelshift_r(w1, w2, sh), __funnelshift_r(w2, w3, sh),
+                      __funnelshift_r(w3, w4, sh));
+  }
+  uint32_t w[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    w[i] = (uint32_t)a[4 * i] | ((uint32_t)a[4 * i + 1] << 8) | ((uint32_t)a[4 * i + 2] << 16) |
+           ((uint32_t)a[4 * i + 3] << 24);
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
 // ----------------------------------------------------------------- tcgen05
 
 template <uint32_t kCols>
