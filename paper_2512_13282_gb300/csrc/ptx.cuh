@@ -129,6 +129,8 @@ __device__ __forceinline__ bool mbar_wait_drain(uint32_t bar, uint32_t parity, u
 // operations are visible.  A no-op for a grid launched without a
 // programmatic dependency.
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Asks for the 128-byte line of p in L2.
+__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 // Lets the next grid of the stream, if it was launched with programmatic
 // stream serialisation, be scheduled before this one finishes (it still
