@@ -425,7 +425,12 @@ double dram_us(int64_t M, int64_t N, int64_t K, bool int8, bool pair) {
   return (a_bytes + b_bytes * rb + c_bytes) / (plan_table::kHbmGBs * 1e3);
 }
 
-Plan search_plan(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sms, int pairs, bool allow_tail) {
+// The split-K partial planes a plan may ask for: whatever is fastest, no
+// split tail, or none (where the scratch is limited).
+enum class Partials { kAny = 0, kNoTail = 1, kNone = 2 };
+
+Plan search_plan(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sms, int pairs, Partials partials) {
+  const bool allow_tail = partials == Partials::kAny;
   Plan pl{};
   // compiled widths, widest first: the bf16 single-CTA kernels also come 64
   // and 96 wide (96 for B column-major only), for memory-bound GEMMs with
@@ -486,7 +491,7 @@ Plan search_plan(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sm
             bool dup = false;
             for (int j = 0; j < nseen; ++j) dup = dup || seen[j] == s2;
             if (dup) continue;
-            if (s2 > 1 && (kb_per < 4 || tiles * s2 > 2 * slots)) continue;
+            if (s2 > 1 && (partials == Partials::kNone || kb_per < 4 || tiles * s2 > 2 * slots)) continue;
           }
           seen[nseen++] = s2;
           const int64_t rounds = ceil_div(tiles * s2, slots);
@@ -567,18 +572,19 @@ Plan search_plan(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sm
 // program calls a few shapes over and over; the search costs 1.2 us of a 4 us
 // call).  A plan depends on these sizes, the device's SM counts and the
 // overrides alone; it holds no pointer.
-Plan make_plan(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sms, int pairs, bool allow_tail = true) {
+Plan make_plan(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sms, int pairs,
+               Partials partials = Partials::kAny) {
   struct Entry {
     int64_t M = -1, N, K;
     int sms, pairs;
-    int form;  // layout, epilogue and allow_tail
+    int form;  // layout, epilogue and partials
     const Overrides *ovr;
     Plan plan;
   };
   constexpr uint64_t kEntries = 64;
   thread_local Entry cache[kEntries];
   const Overrides *ovr = &overrides();
-  const int form = (b_kmajor ? 1 : 0) | (allow_tail ? 2 : 0) | epi << 2;
+  const int form = (b_kmajor ? 1 : 0) | (int)partials << 1 | epi << 3;
   uint64_t h = (uint64_t)M * 0x9E3779B97F4A7C15ull ^ (uint64_t)N * 0xC2B2AE3D27D4EB4Full ^
                (uint64_t)K * 0x165667B19E3779F9ull ^ (uint64_t)form;
   h ^= h >> 29;
@@ -593,7 +599,7 @@ Plan make_plan(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sms,
   e.pairs = pairs;
   e.form = form;
   e.ovr = ovr;
-  e.plan = search_plan(M, N, K, b_kmajor, epi, sms, pairs, allow_tail);
+  e.plan = search_plan(M, N, K, b_kmajor, epi, sms, pairs, partials);
   return e.plan;
 }
 
@@ -622,6 +628,26 @@ size_t partial_bytes(const Plan &pl) {
   if (pl.p.splits > 1) return (size_t)pl.p.splits * pl.p.M * pl.p.N * 4;
   if (pl.p.tail_splits > 0) return (size_t)pl.p.tail_splits * tail_rows(pl) * pl.v.bn * 4;
   return 0;
+}
+
+// Places a plan's partial planes after the `off` bytes of staged operands and
+// takes the workspace.  A call being captured into a graph cannot grow it:
+// where the workspace has no room for the planes, the plan becomes the fastest
+// one without any.
+gemm_status_t plan_workspace(Plan *pl, WsLayout *L, size_t off, bool b_kmajor, const DeviceState &d, cudaStream_t st) {
+  auto take = [&] {
+    const bool planes = partial_planes(pl->p) > 0;
+    L->part_off = planes ? off : 0;
+    L->total = planes ? align_up(off + partial_bytes(*pl), 256) : off;
+    return L->total ? ensure_workspace(L->total, st) : GEMM_OK;
+  };
+  const gemm_status_t s = take();
+  if (s != GEMM_ERR_UNSUPPORTED || partial_planes(pl->p) == 0 || overrides().splits >= 1) return s;
+  const int out_bits = pl->p.out_bits, out_shift = pl->p.out_shift;
+  *pl = make_plan(pl->p.M, pl->p.N, pl->p.K, b_kmajor, pl->v.epi, d.sms, pair_slots(), Partials::kNone);
+  pl->p.out_bits = out_bits;
+  pl->p.out_shift = out_shift;
+  return take();
 }
 
 // Shared path after staging: encode maps, launch the tcgen05 kernel and the
@@ -728,9 +754,16 @@ gemm_status_t run_tc(DeviceState &d, Plan &pl, const uint16_t *A, int64_t lda, c
 // 512^3 9.6 / 6.5, 32 x 1024 x 1024 8.7 / 6.3, 128 x 128 x 4096 31 / 9.0.
 constexpr int64_t kTinyMaxMacs = int64_t(1) << 24;  // 256^3
 constexpr int64_t kTinyMaxK = 512;
-// With the small-M limit forced (GB300_GEMM_SKINNY_MAX_M), the tile kernel
-// takes problems by their multiply-adds alone, up to 512^3.
+// With the small-M limit forced (GB300_GEMM_SKINNY_MAX_M), or no workspace for
+// another kernel, the tile kernel takes problems by their multiply-adds alone,
+// up to 512^3.
 constexpr int64_t kTinyMaxMacsForced = int64_t(1) << 27;
+
+// Whether no override asks for a particular kernel.
+bool default_routes() {
+  const Overrides &o = overrides();
+  return o.bn <= 0 && o.pair < 0 && o.splits < 1 && o.tail_splits < 2 && o.tiny_max_macs < 0 && o.skinny_max_m < 0;
+}
 
 bool tiny_shape(int64_t M, int64_t N, int64_t K) {
   const Overrides &o = overrides();
@@ -741,6 +774,8 @@ bool tiny_shape(int64_t M, int64_t N, int64_t K) {
   if (o.skinny_max_m >= 0) return macs <= (double)kTinyMaxMacsForced;
   return macs <= (double)kTinyMaxMacs && K <= kTinyMaxK;
 }
+
+constexpr int64_t kSkinnyMaxM = 8;  // the largest limit below
 
 // Largest M sent to the CUDA-core small-M kernel: there every B element is
 // used at most a few times and streaming B once is the cost.  bf16,
@@ -896,12 +931,7 @@ gemm_status_t gemm_bf16_f32acc_bf16(int64_t M, int64_t N, int64_t K, const uint1
   size_t off = 0;
   if (pack_a) { L.a_off = off; off = align_up(off + (size_t)M * lda_p * 2, 256); }
   if (pack_b) { L.b_off = off; off = align_up(off + (size_t)b_rows * ldb_p * 2, 256); }
-  if (partial_planes(pl.p) > 0) {
-    L.part_off = off;
-    off = align_up(off + partial_bytes(pl), 256);
-  }
-  L.total = off;
-  if (L.total && (s = ensure_workspace(L.total, st)) != GEMM_OK) return s;
+  if ((s = plan_workspace(&pl, &L, off, b_kmajor, *d, st)) != GEMM_OK) return s;
   uint8_t *ws = static_cast<uint8_t *>(scratch_ws());
   const uint16_t *Au = A, *Bu = B;
   int64_t lda_u = lda, ldb_u = ldb;
@@ -1125,7 +1155,7 @@ gemm_status_t s8_gemm(int64_t M, int64_t N, int64_t K, const int8_t *A, int64_t 
   const bool in_place = overrides().s8tm && !b_kmajor && N > kBM && aligned16(B) && ldb % 16 == 0;
   if (M <= skinny_max_m(true, N, K, b_kmajor, in_place))
     return run_skinny(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, true, st, out_bits, shift);
-  if (tiny_shape(M, N, K)) {
+  auto run_tiny = [&]() -> gemm_status_t {
     const TinyParams tp{A, lda, B, ldb, C, ldc, M, N, K, out_bits, shift};
     const bool prof = g_prof_start && g_prof_stop;
     if (prof && cudaEventRecord(g_prof_start, st) != cudaSuccess) return GEMM_ERR_CUDA;
@@ -1133,8 +1163,19 @@ gemm_status_t s8_gemm(int64_t M, int64_t N, int64_t K, const int8_t *A, int64_t 
     if (launch_tiny_s8(tp, !b_kmajor, st) != cudaSuccess) return GEMM_ERR_CUDA;
     if (prof && cudaEventRecord(g_prof_stop, st) != cudaSuccess) return GEMM_ERR_CUDA;
     return GEMM_OK;
-  }
-  if (try_s8tm(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, out_bits, shift, st, &s)) return s;
+  };
+  if (tiny_shape(M, N, K)) return run_tiny();
+  // A call being captured into a graph on a stream whose workspace is too
+  // small for its kernel: the CUDA-core kernels, slower there, need little or
+  // none, so small problems can be captured on a stream that has run nothing.
+  auto without_scratch = [&]() -> gemm_status_t {
+    if (!default_routes()) return GEMM_ERR_UNSUPPORTED;
+    if (M <= kSkinnyMaxM)
+      return run_skinny(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, true, st, out_bits, shift);
+    return (double)M * (double)N * (double)K <= (double)kTinyMaxMacsForced ? run_tiny() : GEMM_ERR_UNSUPPORTED;
+  };
+  if (try_s8tm(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, out_bits, shift, st, &s))
+    return s == GEMM_ERR_UNSUPPORTED ? without_scratch() : s;
   Plan pl = make_plan(M, N, K, b_kmajor, kEpiS32, d->sms, pair_slots());
   pl.p.out_bits = out_bits;
   pl.p.out_shift = shift;
@@ -1147,12 +1188,8 @@ gemm_status_t s8_gemm(int64_t M, int64_t N, int64_t K, const int8_t *A, int64_t 
   off = align_up(off + (size_t)M * lda_p * 2, 256);
   L.b_off = off;
   off = align_up(off + (size_t)b_rows * ldb_p * 2, 256);
-  if (partial_planes(pl.p) > 0) {
-    L.part_off = off;
-    off = align_up(off + partial_bytes(pl), 256);
-  }
-  L.total = off;
-  if ((s = ensure_workspace(L.total, st)) != GEMM_OK) return s;
+  if ((s = plan_workspace(&pl, &L, off, b_kmajor, *d, st)) != GEMM_OK)
+    return s == GEMM_ERR_UNSUPPORTED ? without_scratch() : s;
   uint8_t *ws = static_cast<uint8_t *>(scratch_ws());
   uint16_t *Ab = reinterpret_cast<uint16_t *>(ws + L.a_off);
   uint16_t *Bb = reinterpret_cast<uint16_t *>(ws + L.b_off);
@@ -1364,10 +1401,12 @@ gemm_status_t s8_gemm_into_scratch(int64_t M, int64_t N, int64_t K, const int8_t
   auto total_of = [&](const Plan &q) {
     return partial_planes(q.p) > 0 ? align_up(part_off + partial_bytes(q), 256) : part_off;
   };
-  // a split tail's partial planes may not fit the caller's scratch: plan
-  // without one then
+  // partial planes may not fit the caller's scratch: plan without a split
+  // tail then, or without any split
   if (pl.p.tail_splits > 0 && total_of(pl) > capacity)
-    pl = make_plan(M, N, K, b_kmajor, kEpiS32, d->sms, pair_slots(), false);
+    pl = make_plan(M, N, K, b_kmajor, kEpiS32, d->sms, pair_slots(), Partials::kNoTail);
+  if (pl.p.splits > 1 && total_of(pl) > capacity && overrides().splits < 1)
+    pl = make_plan(M, N, K, b_kmajor, kEpiS32, d->sms, pair_slots(), Partials::kNone);
   const size_t total = total_of(pl);
   if (!scratch || total > capacity) return GEMM_ERR_UNSUPPORTED;
   uint8_t *ws = static_cast<uint8_t *>(scratch);

@@ -1,0 +1,93 @@
+"""Edges of the routes: operands that are staged or re-pitched from odd bases
+and pitches (whole 16-byte pieces are read by aligned words there, and the
+first and last elements of a matrix must not be reached past), calls captured
+into a CUDA graph on a stream that has no scratch yet, and the sizes where one
+route ends and the next begins.  int8 is exact; bf16 is held to the library's
+bound |C - ref| <= 2^-8 |ref| + 2^-20 sum |a b|."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2512_13282_gb300 import gemm as G
+from paper_2512_13282_gb300 import workloads as W
+from tests import gpu_util as U
+
+ROW, COL = G.GEMM_B_ROW_MAJOR_KxN, G.GEMM_B_COL_MAJOR_NxK
+needs_gpu = pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a GPU")
+
+
+def _operands(dtype, M, N, K, layout, seed):
+    rnd = W.random_int8 if dtype == "int8" else W.random_bf16
+    return rnd((M, K), seed), rnd((N, K) if layout == COL else (K, N), seed + 1)
+
+
+def _check(dtype, A, B, layout, C):
+    if dtype == "int8":
+        assert np.array_equal(C.astype(np.int64), oracle.gemm_s8(A, B, layout))
+    else:
+        ref, mag = oracle.gemm_bf16(A, B, layout)
+        assert oracle.bf16_within_bound(C, ref, mag).all()
+
+
+@pytest.mark.gpu
+@needs_gpu
+@pytest.mark.parametrize("dtype", ["int8", "bf16"])
+@pytest.mark.parametrize("layout", [ROW, COL])
+@pytest.mark.parametrize("K,pad,off", [(577, 0, 0), (640, 0, 1), (641, 2, 3), (703, 0, 8), (705, 1, 13), (1016, 8, 5)])
+def test_staged_from_odd_bases_and_pitches(dtype, layout, K, pad, off):
+    M, N = 161, 203
+    A, B = _operands(dtype, M, N, K, layout, K)
+    C = U.run(dtype, A, B, layout, lda=K + pad, ldb=B.shape[1] + pad, a_off=off, b_off=off)
+    _check(dtype, A, B, layout, C)
+
+
+@pytest.mark.gpu
+@needs_gpu
+@pytest.mark.parametrize("dtype,M,N,K,layout", [
+    ("int8", 512, 512, 512, COL), ("int8", 40, 300, 4000, ROW), ("int8", 6, 4096, 64, ROW),
+    ("bf16", 256, 512, 3840, COL), ("bf16", 128, 4096, 4096, ROW), ("int8", 16, 4096, 4096, COL)])
+def test_captured_on_a_stream_without_scratch(dtype, M, N, K, layout):
+    G.gemm_reload_overrides()
+    s = torch.cuda.Stream()
+    A, B = _operands(dtype, M, N, K, layout, 9)
+    view = (lambda x: x) if dtype == "int8" else (lambda x: x.view(np.int16))
+    tA, tB = torch.from_numpy(view(A)).cuda(), torch.from_numpy(view(B)).cuda()
+    tC = torch.zeros((M, N), dtype=torch.int32 if dtype == "int8" else torch.int16, device="cuda")
+    fn = G.gemm_s8s8_s32 if dtype == "int8" else G.gemm_bf16_f32acc_bf16
+    torch.cuda.synchronize()
+    G.gemm_release_resources()
+    # another stream's call loads the kernels; the captured stream has no scratch
+    assert fn(M, N, K, tA, K, tB, B.shape[1], layout, tC, N, torch.cuda.default_stream()) == G.GEMM_OK
+    torch.cuda.synchronize()
+    tC.zero_()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        assert fn(M, N, K, tA, K, tB, B.shape[1], layout, tC, N, s) == G.GEMM_OK
+    g.replay()
+    torch.cuda.synchronize()
+    C = tC.cpu().numpy()
+    _check(dtype, A, B, layout, C if dtype == "int8" else C.view(np.uint16))
+
+
+def test_route_limits():
+    from paper_2512_13282_gb300 import build
+    build.build()
+    G.gemm_reload_overrides()
+
+    def route(M, N, K, int8, layout=ROW):
+        st, plan = G.gemm_plan_query(M, N, K, int8, layout)
+        assert st == G.GEMM_OK
+        return plan["route"]
+
+    # the one-launch int8 kernel: 2^24 multiply-adds and K = 512
+    assert route(256, 256, 256, True) == G.GEMM_ROUTE_TINY and route(64, 512, 512, True) == G.GEMM_ROUTE_TINY
+    assert route(256, 272, 256, True) != G.GEMM_ROUTE_TINY and route(64, 64, 513, True) != G.GEMM_ROUTE_TINY
+    # the small-M kernel against the small-operand one, by what each has to move
+    small_m, small_op = G.GEMM_ROUTE_SMALL_M, G.GEMM_ROUTE_SMALL_OPERAND
+    assert [route(m, 4096, 4096, True) for m in (1, 2)] == [small_m, small_op]
+    assert [route(m, 12288, 4096, True) for m in (2, 3)] == [small_m, small_op]
+    assert [route(m, 2003, 3001, True) for m in (3, 4)] == [small_m, G.GEMM_ROUTE_TC_SINGLE]
+    assert [route(m, 2003, 3001, True, COL) for m in (8, 17)] == [small_m, G.GEMM_ROUTE_TC_SINGLE]
+    assert [route(m, 4096, 4096, False) for m in (2, 3)] == [small_m, G.GEMM_ROUTE_TC_SINGLE]
