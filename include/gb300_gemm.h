@@ -34,8 +34,9 @@
  *     once.  gemm_release_resources() frees the scratch.
  *   - CUDA graphs: calls may be captured on a stream that has already run,
  *     outside capture, calls needing at least as much scratch (the same
- *     shapes, say); a captured call that would need more returns
- *     GEMM_ERR_UNSUPPORTED before enqueuing anything.  Scratch that a graph
+ *     shapes, say); a captured call that would need more runs without it
+ *     where a slower kernel can (bf16 on aligned operands, int8 up to
+ *     512^3), else it returns GEMM_ERR_UNSUPPORTED before enqueuing anything.  Scratch that a graph
  *     refers to stays allocated until gemm_release_resources(), after which
  *     graphs captured before must not be launched.
  *   - Environment variables that override the planner, for tests and
@@ -47,8 +48,8 @@
  *     GB300_GEMM_TMA_STORE=0 (results stored, and split-K sums added into
  *     C, element by element instead of by TMA), GB300_GEMM_PDL=0 (plain
  *     stream ordering between the library's kernels), GB300_GEMM_S8TM=0 (int8
- *     GEMMs with one operand of at most 128 rows take the general path
- *     instead of converting the large operand inside the kernel),
+ *     GEMMs with one small operand take the general path instead of
+ *     converting the large operand inside the kernel),
  *     GB300_GEMM_TINY_MAX_MACS (largest M*N*K of an int8 GEMM computed in one
  *     launch on the CUDA cores; 0 disables that kernel, and so does forcing
  *     a tile width, family or split with the variables above) and
@@ -256,7 +257,7 @@ enum {
   GEMM_ROUTE_NONE = 0,           /* M == 0 or N == 0: nothing to do */
   GEMM_ROUTE_ZERO_FILL = 1,      /* K == 0 */
   GEMM_ROUTE_SMALL_M = 2,        /* CUDA-core kernel for very small M */
-  GEMM_ROUTE_SMALL_OPERAND = 3,  /* int8 with one operand of <= 128 rows, converted in the kernel */
+  GEMM_ROUTE_SMALL_OPERAND = 3,  /* int8 with a small operand, the other converted in the kernel */
   GEMM_ROUTE_TC_SINGLE = 4,      /* tensor-core kernel, one CTA per 128 x BN tile */
   GEMM_ROUTE_TC_PAIR = 5,        /* tensor-core kernel, a CTA pair per 256 x BN tile */
   GEMM_ROUTE_TINY = 6,           /* int8 problem small enough for one CUDA-core launch */

@@ -605,7 +605,7 @@ Plan make_plan(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sms,
 
 // Row pitch (elements) of a staged or re-pitched bf16 copy with rows of n
 // elements: whole 128-byte lines, so that a TMA box row is one line and not
-// the ends of two (int8 2592^3: 41.7 us with rows of 40.5 lines).
+// the ends of two (int8 2592^3: 41.7 us with rows of 40.5 lines, 34.3 with 41).
 int64_t staged_pitch(int64_t n) { return (n + 63) / 64 * 64; }
 
 struct WsLayout {
@@ -971,81 +971,109 @@ bool encode_s8_rows(CUtensorMap *map, const void *base, uint64_t inner, uint64_t
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// K splits of the small-operand int8 kernel.  A unit (one P tile, one
-// split) is a chain of k-blocks that each pass the converter, the TMEM store
-// and the MMA in turn, ~0.57 us a k-block on GB300 until every SM streams
-// (then the P stream's rate takes over), and the CTAs (one per SM) run
-// their units one after the other; so the split
-// minimises rounds * (k-blocks per unit + kS8tmUnitKb), the per-unit start
-// and drain counted in k-blocks, plus kS8tmReduceKb when int16 / int8
-// outputs need the reduction launch.  Measured on GB300 (whole GEMM after a
-// 512 MiB flush), this picks the fastest of 1-8 splits for int32 outputs on
-// 128 x 11008 x 4096 (3 splits: 258 units in two rounds of 11 k-blocks,
-// 34.3 -> 30.2 us against one split on 86 SMs), 128 x 12288 x 4096,
-// 128 x 4096 x 11008, 128 x 4096 x 4096, 16 x 4096 x 4096 and
-// 8192 x 64 x 8192, and for int16 outputs on 128 x 11008 / 12288 x 4096
-// (one split: the reduction launch costs more than the shorter chains gain)
-// and 128 x 4096 x 4096 (4 splits).  At least 4 k-blocks (of 128) per split,
-// at most 16 splits (or the forced count); rounded so that no split is
-// empty.
-constexpr int64_t kS8tmUnitKb = 2;
-constexpr int64_t kS8tmReduceKb = 10;
+// What the small-operand int8 kernel does with a GEMM: which operand it
+// streams (P = B for `swap`, else A), whether P is K contiguous (false: B
+// stored K x N, read transposed), the Q rows of a tile, the K splits, and the
+// modelled time of the whole call.
+struct S8tmChoice {
+  bool swap, p_kmajor;
+  int qn;
+  int64_t splits;
+  double model_us;
+};
 
-int64_t s8tm_splits(int64_t tiles, int64_t num_kb, int sms, int forced, bool reduce_launch) {
+// Modelled time, fitted to 1000 forced splits on GB300 (8.5 % RMS; calls back
+// to back, 17 to 1024 rows of Q): the busiest CTA's k-blocks (of 128), C, the
+// staging of Q (per million elements), and the launches.  A k-block is bound
+// by its hand-offs and its P and Q from L2: 0.35 us against 128 rows of Q,
+// 0.28 against 64, 0.45 with P read transposed.  C costs its TMA stores, or for
+// split-K the zeroing and one TMA reduction per split; int16 / int8 outputs
+// are stored element by element (a row per lane, unless swapped) and, split,
+// go through partials and the reduction launch.
+double s8tm_model_us(const S8tmChoice &c, int64_t tiles, int64_t num_kb, int64_t s, double c_mb, bool s32, int sms) {
+  const double kb_us = !c.p_kmajor ? 0.45 : c.qn == 64 ? 0.28 : 0.35;
+  const double t = kb_us * (double)(ceil_div(tiles * s, (int64_t)sms) * ceil_div(num_kb, s));
+  if (s32) return t + (s == 1 ? 0.25 * c_mb : 1.2 + 0.16 * (double)(s + 1) * c_mb);
+  const double store = (c.swap ? 0.25 : 2.5) * c_mb;
+  return t + (s == 1 ? store : 3.5 + (double)s * (store + 0.2 * c_mb));
+}
+
+// Rows of the smaller operand up to which the kernel competes with the general
+// path, and what that path costs beside the planner's model: its staging of
+// both operands per million elements, and its launches.  The split with the
+// least modelled time is 0.4 % (geometric mean) above the best forced one over
+// 168 shapes.  The kernel is taken where its model is 8 % below the general
+// path's (15 % with P read transposed, whose time varies more).  Over 170
+// seeded shapes with 129 to 1024 rows that a margin of 5 % takes, general path
+// / kernel were 1 / 0.86 (geometric mean; 0.47 at best, 1.15 at worst): 256 x
+// 12288 x 4096 53 -> 29.3 us, 256 x 4096 x 4096 23.7 -> 16.1, 512 x 8192 x 4096
+// 45.6 -> 32.7, 8192 x 256 x 4096 36.7 -> 20.0; the other way 1024 x 4096 x 4096
+// 36.5 -> 35.2, 2048^3 22.3 -> 23.7, 480 x 6912 x 4224 transposed 35.6 -> 41.1.
+constexpr int64_t kS8tmMaxRows = 1024;
+constexpr double kS8tmFixedUs = 6.0, kS8tmQUsPerM = 0.45;
+constexpr double kS8tmMargin = 1.08, kS8tmMarginTransposed = 1.15;
+constexpr double kStagedFixedUs = 3.8, kStagedUsPerM = 0.54;
+
+// Whether the small-operand int8 kernel takes a GEMM (P's alignment aside): M
+// or N at most 128 and the other above, always; up to kS8tmMaxRows where it is
+// modelled to be faster and no override asks for another kernel.  `forced` is
+// GB300_GEMM_SPLITS; at least 4 k-blocks per split, at most 16 splits, and no
+// split is empty.
+bool s8tm_choice(int64_t M, int64_t N, int64_t K, bool b_kmajor, int out_bits, int sms, int pairs, S8tmChoice *c) {
+  if (!overrides().s8tm) return false;
+  const int64_t q_rows = M < N ? M : N, p_rows = M < N ? N : M;
+  if (p_rows <= kBM || q_rows > kS8tmMaxRows) return false;
+  c->swap = M < N;
+  c->p_kmajor = !c->swap || b_kmajor;
+  c->qn = q_rows <= 64 ? 64 : 128;
+  const bool always = q_rows <= kBM;
+  if (!always && (!default_routes() || (out_bits != 32 && !c->swap))) return false;
+  const int64_t num_kb = ceil_div(K, kS8tmKB), tiles = ceil_div(p_rows, kBM) * ceil_div(q_rows, c->qn);
+  const int forced = overrides().splits;
   if (forced >= 1) {
     const int64_t f = forced < num_kb ? forced : num_kb;
-    return ceil_div(num_kb, ceil_div(num_kb, f));
+    c->splits = ceil_div(num_kb, ceil_div(num_kb, f));
+    c->model_us = 0;
+    return true;
   }
-  int64_t best = 1, best_cost = -1;
+  const double c_mb = 4e-6 * (double)M * (double)N;
+  double best = -1;
   for (int64_t s = 1; s <= 16 && s <= num_kb; ++s) {
     const int64_t kb_per = ceil_div(num_kb, s);
-    const int64_t s2 = ceil_div(num_kb, kb_per);
-    if (s2 != s || (s2 > 1 && kb_per < 4)) continue;  // a count already seen, or too short a split
-    const int64_t rounds = ceil_div(tiles * s2, (int64_t)sms);
-    const int64_t cost = rounds * (kb_per + kS8tmUnitKb) + (s2 > 1 && reduce_launch ? kS8tmReduceKb : 0);
-    if (best_cost < 0 || cost < best_cost) {
-      best_cost = cost;
-      best = s2;
+    if (ceil_div(num_kb, kb_per) != s || (s > 1 && kb_per < 4)) continue;  // an empty split, or too short a one
+    const double t = s8tm_model_us(*c, tiles, num_kb, s, c_mb, out_bits == 32, sms);
+    if (best < 0 || t < best) {
+      best = t;
+      c->splits = s;
     }
   }
-  return best;
+  c->model_us = best + kS8tmFixedUs + kS8tmQUsPerM * 1e-6 * (double)q_rows * (double)K;
+  if (always) return true;
+  const double staged = make_plan(M, N, K, b_kmajor, kEpiS32, sms, pairs).model_us + kStagedFixedUs +
+                        kStagedUsPerM * 1e-6 * (double)(M + N) * (double)K;
+  return (c->p_kmajor ? kS8tmMargin : kS8tmMarginTransposed) * c->model_us < staged;
 }
 
-// Which operand the small-operand int8 kernel streams, if any: P = B with
-// M <= 128 (swap), P = A with N <= 128 < M; p_kmajor is false for B stored
-// K x N, read transposed.
-bool s8tm_shape(int64_t M, int64_t N, bool b_kmajor, bool *swap, bool *p_kmajor) {
-  if (M <= kBM && N > kBM)
-    *swap = true;
-  else if (N <= kBM && M > kBM)
-    *swap = false;
-  else
-    return false;
-  *p_kmajor = !*swap || b_kmajor;
-  return true;
-}
-
-// Memory-bound int8 shapes, where one operand is far larger than the other:
-// M <= 128 (the weights, P = B, are streamed as int8 and the activations
-// Q = A staged; B stored N x K is read K-major, B stored K x N transposed),
-// or N <= 128 with M > 128 (P = A, Q = B, in either layout).
-// gemm_s8tm_kernel converts P inside the kernel, so P moves once as int8
-// instead of three times as staged bf16.  Returns false, having launched
-// nothing, when the shape or P's alignment (16-byte base and pitch, for
-// TMA) rules the path out; GB300_GEMM_S8TM=0 turns it off and
+// int8 GEMMs with one operand larger than the other (s8tm_choice): with M < N
+// the weights, P = B, are streamed as int8 and the activations Q = A staged (B
+// stored N x K is read K-major, B stored K x N transposed), with N < M P = A
+// and Q = B in either layout.  gemm_s8tm_kernel converts P inside the kernel,
+// so P moves as int8 instead of three times as staged bf16.  Returns false,
+// having launched nothing, when the shape or P's alignment (16-byte base and
+// pitch, for TMA) rules the path out; GB300_GEMM_S8TM=0 turns it off and
 // GB300_GEMM_SPLITS forces the split-K factor.
 bool try_s8tm(DeviceState &d, int64_t M, int64_t N, int64_t K, const int8_t *A, int64_t lda, const int8_t *B,
               int64_t ldb, bool b_kmajor, void *C, int64_t ldc, int out_bits, int shift, cudaStream_t st,
               gemm_status_t *status) {
   const Overrides &ovr = overrides();
-  if (!ovr.s8tm) return false;
-  bool swap, p_kmajor;  // p_kmajor false: B stored K x N, P's rows are its k-rows
-  if (!s8tm_shape(M, N, b_kmajor, &swap, &p_kmajor)) return false;
+  S8tmChoice c;
+  if (!s8tm_choice(M, N, K, b_kmajor, out_bits, d.sms, pair_slots(), &c)) return false;
+  const bool swap = c.swap, p_kmajor = c.p_kmajor;
   const int8_t *P = swap ? B : A;
   const int64_t ldp = swap ? ldb : lda;
   if (!aligned16(P) || ldp % 16 != 0) return false;
   const int64_t P_rows = swap ? N : M, Q_rows = swap ? M : N;
-  const int qn = Q_rows <= 64 ? 64 : 128;
+  const int qn = c.qn;
   // Q(q, k): A[q][k] when swapped; else B, stored N x K or K x N.
   const int8_t *Qs = swap ? A : B;
   const int64_t sq = (swap || b_kmajor) ? (swap ? lda : ldb) : 1;
@@ -1053,7 +1081,7 @@ bool try_s8tm(DeviceState &d, int64_t M, int64_t N, int64_t K, const int8_t *A, 
   const int64_t num_kb = ceil_div(K, kS8tmKB);
   const int64_t tiles_p = ceil_div(P_rows, kBM), tiles_q = ceil_div(Q_rows, qn);
   const int64_t tiles = tiles_p * tiles_q;
-  int64_t splits = s8tm_splits(tiles, num_kb, d.sms, ovr.splits, out_bits != 32);
+  const int64_t splits = c.splits;
   const int64_t kb_per = ceil_div(num_kb, splits);
   gemm_status_t s;
   // split-K: int32 outputs are added into C (zeroed by the staging launch),
@@ -1097,13 +1125,14 @@ bool try_s8tm(DeviceState &d, int64_t M, int64_t N, int64_t K, const int8_t *A, 
   p.out_bits = out_bits;
   p.out_shift = shift;
   p.q_img = ws;
-  // Split-K into int32 C by TMA reductions where C's base, pitch and row
-  // ends allow TMA (rows ending on a 16-byte boundary: a clipped TMA
-  // reduction would touch the rest of the row's last 16-byte piece), else
-  // by element-wise atomic adds.
+  // int32 C by TMA stores, or for split-K TMA reductions, where C's base,
+  // pitch and row ends allow TMA (rows ending on a 16-byte boundary: a clipped
+  // TMA store touches the rest of the row's last 16-byte piece), else element
+  // by element: 8192 x 128 x 512 unsplit 17.9 -> 7.7 us (a row per lane), 128 x
+  // 8192 x 2048 14.3 -> 13.5.
   CUtensorMap tc = tp;
   p.c_tma = 0;
-  if (add_into_c && overrides().tma_store && aligned16(C) && (ldc * 4) % 16 == 0 && (N * 4) % 16 == 0) {
+  if (out_bits == 32 && overrides().tma_store && aligned16(C) && (ldc * 4) % 16 == 0 && (N * 4) % 16 == 0) {
     if (!encode_out(&tc, CU_TENSOR_MAP_DATA_TYPE_INT32, 4, C, (uint64_t)N, (uint64_t)M, (uint64_t)ldc, 1))
       return true;
     p.c_tma = 1;
@@ -1318,14 +1347,12 @@ gemm_status_t gemm_plan_query(int64_t M, int64_t N, int64_t K, int int8, int b_l
     out->grid = (int)(ceil_div(M, 32) * ceil_div(N, 32));
     return GEMM_OK;
   }
-  bool swap, p_kmajor;
+  S8tmChoice c;
   // tight leading dimensions: P's pitch is K (K-major) or N (B stored K x N)
-  if (int8 && overrides().s8tm && s8tm_shape(M, N, b_kmajor, &swap, &p_kmajor) &&
-      (p_kmajor ? K : N) % 16 == 0) {
-    const int64_t Q_rows = swap ? M : N, P_rows = swap ? N : M;
-    const int qn = Q_rows <= 64 ? 64 : 128;
-    const int64_t tiles = ceil_div(P_rows, kBM) * ceil_div(Q_rows, qn);
-    const int64_t splits = s8tm_splits(tiles, ceil_div(K, kS8tmKB), sms, overrides().splits, false);
+  if (int8 && s8tm_choice(M, N, K, b_kmajor, 32, sms, pair_slots_, &c) && (c.p_kmajor ? K : N) % 16 == 0) {
+    const int64_t Q_rows = c.swap ? M : N, P_rows = c.swap ? N : M;
+    const int qn = c.qn;
+    const int64_t tiles = ceil_div(P_rows, kBM) * ceil_div(Q_rows, qn), splits = c.splits;
     out->route = GEMM_ROUTE_SMALL_OPERAND;
     out->bn = qn;
     out->splits = (int)splits;

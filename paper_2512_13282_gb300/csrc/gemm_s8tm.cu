@@ -1,14 +1,13 @@
-// gemm_s8tm.cu -- exact int8 GEMM for memory-bound shapes: one operand is
-// converted to bf16 inside the kernel, straight into tensor memory.
+// gemm_s8tm.cu -- exact int8 GEMM for shapes with a small operand: the large
+// one is converted inside the kernel, straight into tensor memory.
 //
-// When one operand is much larger than the other (a few rows of
-// activations against a weight matrix, or a weight matrix a few columns
-// wide), the time is the time to stream the large operand from HBM once.
-// The general int8 path first stages both operands as bf16 (one launch that
-// reads 1 byte and writes 2 per element), then the GEMM reads those 2 bytes
-// again: 5 bytes of traffic per element of the large operand instead of 1.
-// This kernel stages only the small operand and streams the large one as
-// int8:
+// When one operand is much larger than the other (a batch of activations
+// against a weight matrix, or a weight matrix a few columns wide), streaming
+// and converting the large operand is most of the time.  The general int8
+// path first stages both operands as bf16 (one launch that reads 1 byte and
+// writes 2 per element), then the GEMM reads those 2 bytes again: 5 bytes of
+// traffic per element of the large operand instead of 1.  This kernel stages
+// only the small operand and streams the large one as int8:
 //
 //   P  the large operand, int8: B when M is small (P row = column n of C),
 //      or A when N is small (P row = row m).  It is the MMA's 128-row A
@@ -17,29 +16,35 @@
 //      128 k-rows of 128 P rows, and the converters read it transposed).
 //   Q  the small operand, staged beforehand (s8tm_stage_q_kernel) as the
 //      exact shared-memory image the MMA reads for each (Q tile, k-block):
-//      bf16, K-major, 128-byte swizzled, QN rows x 128 K = QN x 256 bytes,
+//      fp16, K-major, 128-byte swizzled, QN rows x 128 K = QN x 256 bytes,
 //      contiguous; zero outside the matrix.  It is the MMA's QN-column B
 //      operand.
 //
-// Roles (11 warps):
+// Roles (15 warps with QN = 64, 19 with QN = 128):
 //   warp 0             P producer: per k-block of 128 a 128 x 128 int8 TMA
 //                      box of P (128-byte rows, 128-byte swizzle) into a
 //                      deep ring of its own.  Every row of a TMA box is a
 //                      request of its own; 128-byte rows move twice the
 //                      bytes per request of 64-byte ones (measured on
 //                      GB300: twice the bytes per second per SM).
-//   warp 10            Q producer: Q's image with one bulk copy into a
-//                      shallow ring (Q is read from L2).
-//   warps 6..9         converters: lane r of the warp with TMEM lane
-//                      quadrant q converts P row 32 q + r (128 int8, read
-//                      with eight conflict-free 16-byte loads) to 64 packed
-//                      bf16 pairs and writes them to one of NA P slots in
-//                      TMEM (tcgen05.st, lane = row, the lower k of a pair
-//                      in the low half).
+//   last warp          Q producer: Q's image with one bulk copy into a
+//                      ring of its own (Q is read from L2).
+//   8 converter warps  two groups of four that take alternate k-blocks:
+//                      lane r of the warp with TMEM lane quadrant q converts
+//                      P row 32 q + r (128 int8, read with eight
+//                      conflict-free 16-byte loads) to 64 packed fp16 pairs
+//                      and writes them to one of NA P slots in TMEM
+//                      (tcgen05.st, lane = row, the lower k of a pair in the
+//                      low half).  One group waits for its stores while the
+//                      other converts; a single group left the MMAs idle for
+//                      a store's latency per k-block (128 x 4096 x 4096 back
+//                      to back 16.7 -> 12.9 us with the fp16 conversion,
+//                      which takes half the instructions of the bf16 one).
 //   warp 1             MMA issuer: tcgen05.mma kind::f16 with A in TMEM and
 //                      B in shared memory, into one of two TMEM accumulators
 //                      of QN fp32 columns.
-//   warps 2..5         epilogue: lane r of quadrant q owns P row 32 q + r.
+//   4 or 8 warps       epilogue, 64 accumulator columns each: lane r of
+//                      quadrant q owns P row 32 q + r.
 //
 // Exactness is the general int8 path's: every product is at most 2^14 in
 // magnitude, so a partial sum of at most 1024 of them is an integer below
@@ -48,11 +53,13 @@
 // slab to int32 (exactly) and adds the slabs in int32 registers.
 //
 // A P stage is free again once every converter warp of its group has
-// converted and stored its rows (one arrival per warp), a Q stage once the MMAs that read it have completed
-// (tcgen05.commit), a TMEM P slot likewise.  With P decoupled from the MMA,
-// the P ring keeps its boxes in flight from HBM: measured on GB300, a P box
-// takes about 2 us from issue to arrival under load, so the bytes in flight
-// per SM, not the converters or the MMAs, set the stream rate.
+// converted and stored its rows (one arrival per warp), a Q stage once the
+// MMAs that read it have completed (tcgen05.commit), a TMEM P slot likewise.
+// With P decoupled from the MMA, the P ring keeps its boxes in flight from
+// HBM: measured on GB300, a P box takes about 2 us from issue to arrival
+// under load.  What bounds a long unit is the k-block itself, 0.42 us for
+// 128 x 128 x 128 (512 x 12288 x 4096: 16 KB of P and 32 KB of Q from L2 and
+// 0.33 us of MMA); short ones wait for their first box and their last slab.
 #include <cuda_bf16.h>
 
 #include "gemm_internal.h"
@@ -85,8 +92,8 @@ struct S8tmCfg {
   static constexpr uint32_t kQBytes = 2 * kQHalf;      // the k-block's Q image
   static constexpr uint32_t kPOffset = 0;
   static constexpr uint32_t kQOffset = SP * kPBytes;  // 1024-byte aligned
-  // one 32 x 32 int32 block per epilogue warp, staging the TMA reductions
-  // of split-K into C (128-byte swizzle; 1024-byte aligned)
+  // one 32 x 32 int32 block per epilogue warp, staging the TMA stores of C
+  // (128-byte swizzle; 1024-byte aligned)
   static constexpr uint32_t kEpiOffset = kQOffset + SQ * kQBytes;
   static constexpr uint32_t kBarOffset = kEpiOffset + kEpiWarps * 4096;
   static constexpr uint32_t kNumBars = 2 * SP + 2 * SQ + 2 * NA + 5;
@@ -106,8 +113,8 @@ __device__ __forceinline__ S8tmUnit decode_s8tm(const S8tmParams &p, int u) {
   S8tmUnit w;
   w.split = u / tiles;
   const int t = u - w.split * tiles;
-  w.tq = t / p.tiles_p;
-  w.tp = t - w.tq * p.tiles_p;
+  w.tp = t / p.tiles_q;  // the Q tiles of a P tile run side by side: P comes from HBM once
+  w.tq = t - w.tp * p.tiles_q;
   w.kb0 = w.split * p.kb_per_split;
   w.kb1 = min(p.num_kb, w.kb0 + p.kb_per_split);
   return w;
@@ -149,14 +156,14 @@ __device__ __forceinline__ void store_row(const S8tmParams &p, const int32_t (&a
   }
 }
 
-// Split-K of int32 C with TMA reductions: the warp's QN sums of its 32 P
-// rows, 32 Q columns at a time, staged as a 32 x 32 block (128-byte rows,
-// 16-byte chunk j of row r at chunk j ^ (r % 8)) and added into C by one TMA
-// reduction (element-wise atomic; the TMA clips a block that crosses C's
-// edges, and a block that starts outside C is not issued).  C[q][prow]
-// (swap): block row = q, column = lane; else C[prow][q]: row = lane.
+// int32 C by TMA: the warp's QN sums of its 32 P rows, 32 Q columns at a time,
+// staged as a 32 x 32 block (128-byte rows, 16-byte chunk j of row r at chunk
+// j ^ (r % 8)) and stored, or for split-K added into C by one TMA reduction
+// (element-wise atomic); the TMA clips a block that crosses C's edges, and a
+// block that starts outside C is not issued.  C[q][prow] (swap): block row =
+// q, column = lane; else C[prow][q]: row = lane.
 template <int QN>
-__device__ __forceinline__ void reduce_rows_tma(const CUtensorMap *tm, uint32_t buf, int lane, const int32_t (&acc)[QN],
+__device__ __forceinline__ void out_rows_tma(bool add, const CUtensorMap *tm, uint32_t buf, int lane, const int32_t (&acc)[QN],
                                                 bool swap, int32_t prow0, int32_t q0, int32_t P_rows, int32_t Q_rows) {
 #pragma unroll
   for (int c = 0; c < QN / 32; ++c) {
@@ -177,10 +184,11 @@ __device__ __forceinline__ void reduce_rows_tma(const CUtensorMap *tm, uint32_t 
     fence_proxy_async_smem();
     __syncwarp();
     if (lane == 0 && prow0 < P_rows && q0 + c * 32 < Q_rows) {
-      if (swap)
-        tma_reduce_add_2d(tm, buf, prow0, q0 + c * 32);
+      const int32_t x = swap ? prow0 : q0 + c * 32, y = swap ? q0 + c * 32 : prow0;
+      if (add)
+        tma_reduce_add_2d(tm, buf, x, y);
       else
-        tma_reduce_add_2d(tm, buf, q0 + c * 32, prow0);
+        tma_store_2d(tm, buf, x, y);
       bulk_commit();
     }
   }
@@ -457,8 +465,8 @@ __global__ void __launch_bounds__(S8tmCfg<QN, SP, SQ, NA>::kThreads, 1)
       if (!ok) break;
       const int64_t q0 = (int64_t)w.tq * QN + col0;
       if (q0 >= p.Q_rows) continue;
-      if (p.add_into_c && p.c_tma) {  // the whole warp: rows past the matrix are clipped by the TMA
-        reduce_rows_tma<kEpiCols>(&tmC, base + Cfg::kEpiOffset + (warp - 2) * 4096, lane, acc, p.swap != 0,
+      if (p.c_tma) {  // the whole warp: rows past the matrix are clipped by the TMA
+        out_rows_tma<kEpiCols>(p.add_into_c != 0, &tmC, base + Cfg::kEpiOffset + (warp - 2) * 4096, lane, acc, p.swap != 0,
                                   w.tp * kBM + quad * 32, (int32_t)q0, p.P_rows, p.Q_rows);
         continue;
       }
@@ -473,7 +481,7 @@ __global__ void __launch_bounds__(S8tmCfg<QN, SP, SQ, NA>::kThreads, 1)
     }
   }
 
-  // the epilogue's TMA reductions have completed before the CTA leaves
+  // the epilogue's TMA stores have completed before the CTA leaves
   if (p.c_tma && warp >= 2 && warp < 2 + Cfg::kEpiWarps && lane == 0) bulk_wait_all();
   griddep_launch_dependents();  // e.g. the split-K reduction may start setting up
   __syncwarp();

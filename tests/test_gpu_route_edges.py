@@ -71,6 +71,33 @@ def test_captured_on_a_stream_without_scratch(dtype, M, N, K, layout):
     _check(dtype, A, B, layout, C if dtype == "int8" else C.view(np.uint16))
 
 
+# 129 rows and more of the small operand: several Q tiles, one or more K
+# splits, ragged edges of both operands; C stored by TMA or, with an odd pitch
+# or base, element by element
+@pytest.mark.gpu
+@needs_gpu
+@pytest.mark.parametrize("dtype,M,N,K,layout,kw", [
+    ("int8", 129, 4096, 2048, COL, {}), ("int8", 129, 4096, 2048, ROW, {}), ("int8", 257, 2064, 4100, COL, {"ldb": 4112}),
+    ("int8", 200, 3000, 4099, ROW, {"ldb": 3008, "ldc": 3001}), ("int8", 385, 12288, 1040, COL, {}),
+    ("int8", 385, 8193, 2048, COL, {"ldc": 8193, "c_off": 1}), ("int8", 4096, 129, 2048, ROW, {}),
+    ("int8", 3001, 200, 4096, COL, {}), ("int8", 2049, 300, 4096, ROW, {"ldc": 301}), ("int8", 8192, 520, 2064, COL, {}),
+    ("int8_int16", 200, 4096, 4096, COL, {"shift": 9}), ("int8_int8", 192, 4096, 4096, ROW, {"shift": 14})])
+def test_small_operand_kernel_with_several_tiles(dtype, M, N, K, layout, kw):
+    rng = np.random.default_rng(M + N + K)
+    A = rng.integers(-128, 128, (M, K), dtype=np.int8)
+    B = rng.integers(-128, 128, (N, K) if layout == COL else (K, N), dtype=np.int8)
+    A[-1], B[-1] = -128, -128
+    # the query takes tight pitches: ask for the K or N that the call's pitch makes of it
+    pk, pn = (kw.get("ldb", K), N) if layout == COL else (K, kw.get("ldb", N))
+    st, plan = G.gemm_plan_query(M, pn, pk, True, layout)
+    assert st == G.GEMM_OK and plan["route"] == G.GEMM_ROUTE_SMALL_OPERAND and plan["bn"] == 128
+    C = U.run(dtype, A, B, layout, **kw)
+    want = oracle.gemm_s8(A, B, layout)
+    if dtype != "int8":
+        want = oracle.requantize(want, kw["shift"], 16 if dtype == "int8_int16" else 8)
+    assert np.array_equal(C.astype(np.int64), want)
+
+
 def test_route_limits():
     from paper_2512_13282_gb300 import build
     build.build()
@@ -90,4 +117,7 @@ def test_route_limits():
     assert [route(m, 12288, 4096, True) for m in (2, 3)] == [small_m, small_op]
     assert [route(m, 2003, 3001, True) for m in (3, 4)] == [small_m, G.GEMM_ROUTE_TC_SINGLE]
     assert [route(m, 2003, 3001, True, COL) for m in (8, 17)] == [small_m, G.GEMM_ROUTE_TC_SINGLE]
+    # several Q tiles of the small-operand kernel against the general path
+    assert route(512, 4096, 4096, True, COL) == small_op and route(4096, 256, 4096, True) == small_op
+    assert route(1024, 4096, 4096, True, COL) == G.GEMM_ROUTE_TC_PAIR and route(256, 1024, 1024, True) != small_op
     assert [route(m, 4096, 4096, False) for m in (2, 3)] == [small_m, G.GEMM_ROUTE_TC_SINGLE]
