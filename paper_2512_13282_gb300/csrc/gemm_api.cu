@@ -982,27 +982,27 @@ struct S8tmChoice {
   double model_us;
 };
 
-// Modelled time, fitted to 1000 forced splits on GB300 (8.5 % RMS; calls back
+// Modelled time, fitted to 1700 forced splits on GB300 (10 % RMS; calls back
 // to back, 17 to 1024 rows of Q): the busiest CTA's k-blocks (of 128), C, the
 // staging of Q (per million elements), and the launches.  A k-block is bound
 // by its hand-offs and its P and Q from L2: 0.35 us against 128 rows of Q,
-// 0.28 against 64, 0.45 with P read transposed.  C costs its TMA stores, or for
+// 0.33 against 64, 0.45 with P read transposed.  C costs its TMA stores, or for
 // split-K the zeroing and one TMA reduction per split; int16 / int8 outputs
-// are stored element by element (a row per lane, unless swapped) and, split,
-// go through partials and the reduction launch.
+// are stored by the lanes and, split, go through partials and the reduction
+// launch.
 double s8tm_model_us(const S8tmChoice &c, int64_t tiles, int64_t num_kb, int64_t s, double c_mb, bool s32, int sms) {
-  const double kb_us = !c.p_kmajor ? 0.45 : c.qn == 64 ? 0.28 : 0.35;
+  const double kb_us = !c.p_kmajor ? 0.45 : c.qn == 64 ? 0.33 : 0.35;
   const double t = kb_us * (double)(ceil_div(tiles * s, (int64_t)sms) * ceil_div(num_kb, s));
-  if (s32) return t + (s == 1 ? 0.25 * c_mb : 1.2 + 0.16 * (double)(s + 1) * c_mb);
-  const double store = (c.swap ? 0.25 : 2.5) * c_mb;
-  return t + (s == 1 ? store : 3.5 + (double)s * (store + 0.2 * c_mb));
+  if (s32) return t + (s == 1 ? 0.25 * c_mb : 0.9 + 0.16 * (double)(s + 1) * c_mb);
+  const double store = (c.swap ? 0.2 : 0.6) * c_mb;
+  return t + (s == 1 ? store : 1.0 + (double)s * (store + 0.3 * c_mb));
 }
 
 // Rows of the smaller operand up to which the kernel competes with the general
 // path, and what that path costs beside the planner's model: its staging of
 // both operands per million elements, and its launches.  The split with the
-// least modelled time is 0.4 % (geometric mean) above the best forced one over
-// 168 shapes.  The kernel is taken where its model is 8 % below the general
+// least modelled time is 0.4 % (geometric mean; 14 % at worst) above the best
+// forced one over 300 shapes.  The kernel is taken where its model is 8 % below the general
 // path's (15 % with P read transposed, whose time varies more).  Over 170
 // seeded shapes with 129 to 1024 rows that a margin of 5 % takes, general path
 // / kernel were 1 / 0.86 (geometric mean; 0.47 at best, 1.15 at worst): 256 x
@@ -1027,7 +1027,7 @@ bool s8tm_choice(int64_t M, int64_t N, int64_t K, bool b_kmajor, int out_bits, i
   c->p_kmajor = !c->swap || b_kmajor;
   c->qn = q_rows <= 64 ? 64 : 128;
   const bool always = q_rows <= kBM;
-  if (!always && (!default_routes() || (out_bits != 32 && !c->swap))) return false;
+  if (!always && !default_routes()) return false;
   const int64_t num_kb = ceil_div(K, kS8tmKB), tiles = ceil_div(p_rows, kBM) * ceil_div(q_rows, c->qn);
   const int forced = overrides().splits;
   if (forced >= 1) {

@@ -123,8 +123,9 @@ __device__ __forceinline__ S8tmUnit decode_s8tm(const S8tmParams &p, int u) {
 // Stores the QN int32 sums of one P row: element i goes to offset
 // off0 + i * step of the destination (C, or the split's partials), for the
 // elements whose Q index q0 + i is inside the matrix; int32, or requantised
-// to int16 / int8.  Every branch is taken per thread, outside the unrolled
-// loops, so that acc stays in registers.
+// to int16 / int8.  Where the elements are contiguous (C[prow][q]) a lane
+// stores 16 bytes at a time: int16 8848 x 32 x 1648 unsplit 18.3 (general path)
+// -> 13.0 us, int8 9616 x 64 x 3200 27.7 -> 15.0.  acc stays in registers.
 template <int QN>
 __device__ __forceinline__ void store_row(const S8tmParams &p, const int32_t (&acc)[QN], int split, int64_t off0,
                                           int64_t step, int64_t q0) {
@@ -137,22 +138,61 @@ __device__ __forceinline__ void store_row(const S8tmParams &p, const int32_t (&a
 #pragma unroll
     for (int i = 0; i < QN; ++i)
       if (i < nq) atomicAdd(dst + i * step, acc[i]);
-  } else if (p.splits > 1 || p.out_bits == 32) {
+    return;
+  }
+  // Where the lane's elements are contiguous (C[prow][q]), 16 bytes at a time
+  // with the widest stores their address allows.
+  if (p.splits > 1 || p.out_bits == 32) {
     int32_t *dst = reinterpret_cast<int32_t *>(p.splits > 1 ? p.ws : p.C) +
                    (p.splits > 1 ? (int64_t)split * p.M * p.N : 0) + off0;
 #pragma unroll
-    for (int i = 0; i < QN; ++i)
-      if (i < nq) dst[i * step] = acc[i];
-  } else if (p.out_bits == 16) {
-    int16_t *dst = reinterpret_cast<int16_t *>(p.C) + off0;
+    for (int c = 0; c < QN; c += 4) {
+      if (step == 1 && c + 4 <= nq) {
+        const uint32_t w[4] = {(uint32_t)acc[c], (uint32_t)acc[c + 1], (uint32_t)acc[c + 2], (uint32_t)acc[c + 3]};
+        store_chunk_aligned<4>(dst + c, w);
+      } else {
 #pragma unroll
-    for (int i = 0; i < QN; ++i)
-      if (i < nq) dst[i * step] = static_cast<int16_t>(requantize_s32(acc[i], p.out_shift, -32768, 32767));
-  } else {
-    int8_t *dst = reinterpret_cast<int8_t *>(p.C) + off0;
+        for (int i = c; i < c + 4; ++i)
+          if (i < nq) dst[i * step] = acc[i];
+      }
+    }
+    return;
+  }
+  const int32_t hi = (1 << (p.out_bits - 1)) - 1, lo = -hi - 1;
+  const int esize = p.out_bits / 8;
+  uint8_t *dst = reinterpret_cast<uint8_t *>(p.C) + off0 * esize;
+  const bool words = step == 1 && (reinterpret_cast<uintptr_t>(dst) & 3) == 0;
 #pragma unroll
-    for (int i = 0; i < QN; ++i)
-      if (i < nq) dst[i * step] = static_cast<int8_t>(requantize_s32(acc[i], p.out_shift, -128, 127));
+  for (int c = 0; c < QN; c += 16) {
+    uint32_t q[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) q[i] = (uint32_t)requantize_s32(acc[c + i], p.out_shift, lo, hi);
+    if (words && c + 16 <= nq) {
+      uint32_t h[4];
+      if (esize == 2) {
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) h[i] = __byte_perm(q[8 * half + 2 * i], q[8 * half + 2 * i + 1], 0x5410);
+          store_chunk_aligned<4>(dst + (c + 8 * half) * 2, h);
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          h[i] = __byte_perm(__byte_perm(q[4 * i], q[4 * i + 1], 0x0040),
+                             __byte_perm(q[4 * i + 2], q[4 * i + 3], 0x0040), 0x5410);
+        store_chunk_aligned<4>(dst + c, h);
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < 16; ++i)
+        if (c + i < nq) {
+          if (esize == 2)
+            reinterpret_cast<int16_t *>(dst)[(c + i) * step] = (int16_t)q[i];
+          else
+            reinterpret_cast<int8_t *>(dst)[(c + i) * step] = (int8_t)q[i];
+        }
+    }
   }
 }
 
@@ -167,7 +207,7 @@ __device__ __forceinline__ void out_rows_tma(bool add, const CUtensorMap *tm, ui
                                                 bool swap, int32_t prow0, int32_t q0, int32_t P_rows, int32_t Q_rows) {
 #pragma unroll
   for (int c = 0; c < QN / 32; ++c) {
-    if (lane == 0) bulk_wait_read_all();  // the previous reduction has read the block
+    if (lane == 0) bulk_wait_read_all();  // the previous store has read the block
     __syncwarp();
     if (swap) {
 #pragma unroll

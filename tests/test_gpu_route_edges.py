@@ -81,7 +81,10 @@ def test_captured_on_a_stream_without_scratch(dtype, M, N, K, layout):
     ("int8", 200, 3000, 4099, ROW, {"ldb": 3008, "ldc": 3001}), ("int8", 385, 12288, 1040, COL, {}),
     ("int8", 385, 8193, 2048, COL, {"ldc": 8193, "c_off": 1}), ("int8", 4096, 129, 2048, ROW, {}),
     ("int8", 3001, 200, 4096, COL, {}), ("int8", 2049, 300, 4096, ROW, {"ldc": 301}), ("int8", 8192, 520, 2064, COL, {}),
-    ("int8_int16", 200, 4096, 4096, COL, {"shift": 9}), ("int8_int8", 192, 4096, 4096, ROW, {"shift": 14})])
+    ("int8_int16", 200, 4096, 4096, COL, {"shift": 9}), ("int8_int8", 192, 4096, 4096, ROW, {"shift": 14}),
+    ("int8_int8", 4096, 200, 4096, COL, {"shift": 14}), ("int8_int16", 3001, 77, 4096, ROW, {"shift": 9}),
+    ("int8_int8", 2000, 132, 4096, COL, {"shift": 13, "ldc": 133, "c_off": 1}),
+    ("int8_int16", 8192, 520, 2064, ROW, {"shift": 8})])
 def test_small_operand_kernel_with_several_tiles(dtype, M, N, K, layout, kw):
     rng = np.random.default_rng(M + N + K)
     A = rng.integers(-128, 128, (M, K), dtype=np.int8)
