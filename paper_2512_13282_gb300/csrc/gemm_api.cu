@@ -680,11 +680,16 @@ gemm_status_t run_tc(DeviceState &d, Plan &pl, const uint16_t *A, int64_t lda, c
   const bool tma_ok = overrides().tma_store &&
                       (p.splits > 1 ? p.N % 4 == 0 && pl.v.tma_out == 1
                                     : p.c_vec != 0 && ((int64_t)p.N * esize) % 16 == 0);
+  // Rows on 8-byte boundaries are then stored by their lanes, others row by row
+  // through the staging blocks (rows_out; back to back with 8-byte rows 16.7 us
+  // for bf16 2048^3 where an odd pitch took 38.7).
+  const int64_t odd_bytes = p.splits > 1 ? (int64_t)p.N * 4 : (int64_t)(reinterpret_cast<uintptr_t>(C) | (uint64_t)(ldc * esize));
+  const bool rows = !tma_ok && overrides().tma_store && odd_bytes % 8 != 0;
   // An output that will be stored directly wants the variant with the extra
   // pipeline stage where one exists (int8 at 192 / 224).
-  if (!tma_ok && s32 && (pl.v.bn == 192 || pl.v.bn == 224)) pl.v.tma_out = 0;
+  if (!tma_ok && s32 && (pl.v.bn == 192 || pl.v.bn == 224)) pl.v.tma_out = rows ? 1 : 0;
   CUtensorMap tout = tb, tws = tb;
-  p.out_tma = kOutDirect;
+  p.out_tma = rows && (pl.v.tma_out == 1 || (pl.v.tma_out == 2 && p.splits == 1)) ? kOutRows : kOutDirect;
   p.ws_tma = 0;
   // a split tail's compact partials go through TMA in the variants with
   // 4 KB staging blocks (their rows, BN words, always end on 16 bytes)

@@ -22,9 +22,10 @@
 //                      Stores that each lane makes to its own row touch 32
 //                      lines per instruction and compete with the operand
 //                      traffic; lanes store their rows directly only where
-//                      C's address or pitch rules TMA out, and in the int8
-//                      variants that trade the staging blocks for a pipeline
-//                      stage (long reductions).  Two accumulators let the
+//                      C's address or pitch rules TMA out but its rows lie on
+//                      8-byte boundaries, and in the int8 variants that trade
+//                      the staging blocks for a pipeline stage (long
+//                      reductions).  Odder rows leave row by row (rows_out).  Two accumulators let the
 //                      epilogue of one tile overlap the main loop of the
 //                      next (the paper keeps a single C buffer for lack of
 //                      L1 space, Sec. 5.3.2; TMEM has room for two).
@@ -70,7 +71,7 @@ struct TcParams {
   uint64_t wait_limit_ns;
   int out_bits;      // int8 path: 32 (exact int32 C), 16 or 8 (requantised C)
   int out_shift;     // int8 path with out_bits < 32: right shift, 0..31
-  int out_tma;       // kOutDirect, kOutTmaC (tmOut maps C) or kOutTmaWs (tmOut maps the partials)
+  int out_tma;       // kOutDirect, kOutTmaC (tmOut maps C), kOutTmaWs (tmOut maps the partials) or kOutRows (rows_out)
   // Split tail (tail_splits >= 2, splits == 1): the tiles of the last,
   // partly filled round -- raster positions tail_first .. -- are each split
   // into tail_splits units of tail_kb_per k-blocks that write partials for
@@ -84,7 +85,11 @@ struct TcParams {
 };
 
 // How the epilogue writes its results.
-enum OutMode : int { kOutDirect = 0, kOutTmaC = 1, kOutTmaWs = 2 };
+enum OutMode : int { kOutDirect = 0, kOutTmaC = 1, kOutTmaWs = 2, kOutRows = 3 };
+// Added to a variant's TMA_OUT: the same kernel for C (or partials) by rows_out.
+// A variant of its own, since the code costs the others registers and 0.6 us
+// a call (int8 8192 x 512 x 512 11.2 -> 11.7 us).
+constexpr int kTmaOutRows = 4;
 
 __host__ __device__ constexpr uint32_t pow2_at_least(uint32_t x) {
   uint32_t p = 32;
@@ -128,13 +133,13 @@ struct TcCfg {
   // TMA_OUT 1: per epilogue warp, one 32 x 32 block of 32-bit words (int32
   // results or split-K partials of either path; bf16 results use half of
   // it); TMA_OUT 2 (bf16 C only): a 1 KB block of 32 rows x 16 bf16
-  static constexpr uint32_t kEpiWarpBytes = TMA_OUT == 1 ? 4096 : TMA_OUT == 2 ? 1024 : 0;
+  static constexpr uint32_t kEpiWarpBytes = (TMA_OUT & 3) == 1 ? 4096 : (TMA_OUT & 3) == 2 ? 1024 : 0;
   static constexpr uint32_t kEpiOffset = STAGES * kStageBytes;  // 1024-byte aligned
   static constexpr uint32_t kBarOffset = kEpiOffset + EPI_WARPS * kEpiWarpBytes;
   static constexpr uint32_t kNumBars = 2 * STAGES + 4 + 1;
   static constexpr uint32_t kSmemBytes = kBarOffset + kNumBars * 8 + 16 + 1024;
   static_assert(kSmemBytes <= 232448, "shared memory per CTA is 227 KB");
-  static_assert(kSmemBytes == tc_smem_bytes(STAGES, BN, EPI_WARPS, TMA_OUT), "layout and model agree");
+  static_assert(kSmemBytes == tc_smem_bytes(STAGES, BN, EPI_WARPS, TMA_OUT & 3), "layout and model agree");
   static_assert(kTmemCols <= 512, "TMEM has 512 columns");
 };
 
@@ -434,15 +439,116 @@ __device__ __forceinline__ void tma_out_narrow(const CUtensorMap *tm, uint32_t b
   }
 }
 
+// Output whose rows do not allow wide stores (odd pitch or base): a warp passes
+// its 32 rows x COLS elements of ES bytes (W words of `h` per lane = row)
+// through its shared-memory block and stores them row by row, 32 / COLS rows
+// per instruction and an element per lane, so that a store touches the lines
+// of one row or two instead of 32.  Word j of row r lies at j ^ (r / (32 / W)),
+// without bank conflicts either way.  dst is element (0, 0) of the block;
+// `rows` x `cols` of it are inside the output.  Back to back on GB300, odd
+// ldc, a lane storing its row / this: bf16 4096 x 4096 x 1024 107 / 52 us,
+// 2048^3 38.7 / 23.7 (26 and 14.8 by TMA), int8 2048^3 int32 36.3 / 26.
+template <int ES, int COLS>
+__device__ __forceinline__ void rows_out(uint32_t buf, int lane, const uint32_t (&h)[ES * COLS / 4], uint8_t *dst,
+                                         int64_t pitch, int rows, int cols) {
+  constexpr int W = ES * COLS / 4;
+  if (lane == 0) bulk_wait_read_all();
+  __syncwarp();  // the block's previous contents have been read
+#pragma unroll
+  for (int j = 0; j < W; ++j) st_shared_u32(buf + (lane * W + (j ^ ((lane / (32 / W)) & (W - 1)))) * 4, h[j]);
+  __syncwarp();
+  const int c = lane % COLS, r0 = lane / COLS, j = c * ES / 4, sh = 8 * (c * ES & 3);
+  uint8_t *d = dst + (int64_t)r0 * pitch + c * ES;
+#pragma unroll 8
+  for (int i = 0; i < COLS; ++i) {
+    const int r = i * (32 / COLS) + r0;
+    if (r < rows && c < cols) {
+      const uint32_t v = ld_shared_u32(buf + (r * W + (j ^ ((r / (32 / W)) & (W - 1)))) * 4) >> sh;
+      uint8_t *e = d + (int64_t)i * (32 / COLS) * pitch;
+      if (ES == 4)
+        *reinterpret_cast<uint32_t *>(e) = v;
+      else if (ES == 2)
+        *reinterpret_cast<uint16_t *>(e) = static_cast<uint16_t>(v);
+      else
+        *e = static_cast<uint8_t>(v);
+    }
+  }
+}
+
+// rows_out of COLS int32 results of each lane's row, requantised where C is
+// narrow; block origin (y, x) of C.
+template <int COLS>
+__device__ __forceinline__ void rows_out_s8(const TcParams &p, uint32_t buf, int lane, const uint32_t (&v)[COLS], int x,
+                                            int y) {
+  const int rows = min(32, p.M - y), cols = min(COLS, p.N - x);
+  const int64_t at = (int64_t)y * p.ldc + x;
+  uint8_t *C = static_cast<uint8_t *>(p.C);
+  if (p.out_bits == 32) {
+    rows_out<4, COLS>(buf, lane, v, C + 4 * at, 4 * p.ldc, rows, cols);
+    return;
+  }
+  const RneShift rq(p.out_shift);
+  if (p.out_bits == 16) {
+    uint32_t h[COLS / 2];
+#pragma unroll
+    for (int i = 0; i < COLS / 2; ++i) h[i] = pack_sat_s16x2(rq((int32_t)v[2 * i]), rq((int32_t)v[2 * i + 1]));
+    rows_out<2, COLS>(buf, lane, h, C + 2 * at, 2 * p.ldc, rows, cols);
+  } else {
+    uint32_t h[COLS / 4];
+#pragma unroll
+    for (int i = 0; i < COLS / 4; ++i)
+      h[i] = pack_sat_s8x4(rq((int32_t)v[4 * i]), rq((int32_t)v[4 * i + 1]), rq((int32_t)v[4 * i + 2]),
+                           rq((int32_t)v[4 * i + 3]));
+    rows_out<1, COLS>(buf, lane, h, C + at, p.ldc, rows, cols);
+  }
+}
+
+// ... of 32 32-bit partials of each lane's row; wrow0 is the block's first
+// row of the partials (pitch pn words), x its first column there.
+__device__ __forceinline__ void rows_out_partials(uint32_t buf, int lane, const uint32_t (&v)[32], uint32_t *wrow0, int x,
+                                                  int pn, int rows) {
+  rows_out<4, 32>(buf, lane, v, reinterpret_cast<uint8_t *>(wrow0 + x), 4 * (int64_t)pn, min(32, rows), min(32, pn - x));
+}
+
+// ... of 32 fp32 sums of each lane's row rounded to bf16, through a block of at
+// least 2 KB, or in two halves through 1 KB.
+template <bool HALVES>
+__device__ __forceinline__ void rows_out_bf16(const TcParams &p, uint32_t buf, int lane, const uint32_t (&r)[32], int x,
+                                              int y) {
+  uint8_t *dst = static_cast<uint8_t *>(p.C) + 2 * ((int64_t)y * p.ldc + x);
+  const int rows = min(32, p.M - y), cols = p.N - x;
+  if constexpr (HALVES) {
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      uint32_t h[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        h[i] = pack_bf16x2(__uint_as_float(r[16 * half + 2 * i]), __uint_as_float(r[16 * half + 2 * i + 1]));
+      rows_out<2, 16>(buf, lane, h, dst + 32 * half, 2 * p.ldc, rows, min(16, cols - 16 * half));
+    }
+  } else {
+    uint32_t h[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) h[i] = pack_bf16x2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]));
+    rows_out<2, 32>(buf, lane, h, dst, 2 * p.ldc, rows, min(32, cols));
+  }
+}
+
 // One 32-column chunk of a lane's int32 sums (row `row`, columns x ..): to
 // C (int32, or requantised) or to the split's partials (wrow), through the
 // warp's TMA staging block when out_tma says so (the warp's rows y0 ..),
 // else directly.
+template <bool ROWS>
 __device__ __forceinline__ void store_s32_chunk(const TcParams &p, const CUtensorMap *tm, uint32_t ebuf, int lane,
                                                 int out_tma, const uint32_t (&v)[32], int x, int y0, int split,
                                                 bool row_ok, int64_t row, uint32_t *wrow, bool ws_vec, int px,
                                                 int py, int pn) {
-  if (out_tma != kOutDirect) {
+  if (ROWS && out_tma == kOutRows) {
+    if (wrow)
+      rows_out_partials(ebuf, lane, v, wrow - (int64_t)lane * pn, x - px, pn, p.M - y0);
+    else
+      rows_out_s8<32>(p, ebuf, lane, v, x, y0);
+  } else if (out_tma != kOutDirect) {
     if (out_tma == kOutTmaWs)
       tma_out_words32<true>(tm, ebuf, lane, v, x - px, y0 - py, split, y0 < p.M && x < p.N);
     else if (p.out_bits == 32)
@@ -471,9 +577,10 @@ __global__ void __launch_bounds__(TcCfg<BN, STAGES, B_KMAJOR, EPI, EPI_WARPS, TM
                    const __grid_constant__ CUtensorMap tmOut, const __grid_constant__ CUtensorMap tmWs,
                    const TcParams p) {
   using Cfg = TcCfg<BN, STAGES, B_KMAJOR, EPI, EPI_WARPS, TMA_OUT>;
-  const int out_tma = TMA_OUT != 0 ? p.out_tma : (int)kOutDirect;
+  constexpr bool kRows = (TMA_OUT & kTmaOutRows) != 0;
+  const int out_tma = kRows ? (int)kOutRows : TMA_OUT != 0 ? p.out_tma : (int)kOutDirect;
   // the split tail's partials: through tmWs by the 4 KB staging blocks, or directly
-  const int tail_out = (TMA_OUT == 1 && p.ws_tma) ? (int)kOutTmaWs : (int)kOutDirect;
+  const int tail_out = ((TMA_OUT & 3) == 1 && p.ws_tma) ? (int)kOutTmaWs : (int)kOutDirect;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_addr(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;  // swizzle atoms need 1024-byte alignment
@@ -655,7 +762,7 @@ __global__ void __launch_bounds__(TcCfg<BN, STAGES, B_KMAJOR, EPI, EPI_WARPS, TM
             tmem_ld_wait();
 #pragma unroll
             for (int i = 0; i < 32; ++i) v[i] = static_cast<uint32_t>(__float2int_rn(__uint_as_float(v[i])));
-            store_s32_chunk(p, om, ebuf, lane, uo, v, col0 + c * 32, y0, w.split, row_ok, row, wrow, ws_vec, px, py, pn);
+            store_s32_chunk<kRows>(p, om, ebuf, lane, uo, v, col0 + c * 32, y0, w.split, row_ok, row, wrow, ws_vec, px, py, pn);
           }
           if constexpr (CPT % 32 != 0) {  // a 16-column tail: each lane stores its row
             constexpr int kTail = (CPT / 32) * 32;
@@ -664,7 +771,9 @@ __global__ void __launch_bounds__(TcCfg<BN, STAGES, B_KMAJOR, EPI, EPI_WARPS, TM
             tmem_ld_wait();
 #pragma unroll
             for (int i = 0; i < 16; ++i) v[i] = static_cast<uint32_t>(__float2int_rn(__uint_as_float(v[i])));
-            if (row_ok) {
+            if (kRows && uo == kOutRows && !split) {
+              rows_out_s8<16>(p, ebuf, lane, v, col0 + kTail, y0);
+            } else if (row_ok) {
               if (split)
                 store_words<16>(wrow, col0 + kTail - px, pn, ws_vec, v);
               else
@@ -721,6 +830,10 @@ __global__ void __launch_bounds__(TcCfg<BN, STAGES, B_KMAJOR, EPI, EPI_WARPS, TM
             const int x = col0 + c * 32;
             if (uo == kOutTmaWs)
               tma_out_words32<true>(om, ebuf, lane, v, x - px, y0 - py, w.split, y0 < p.M && x < p.N);
+            else if (kRows && split)
+              rows_out_partials(ebuf, lane, v, wrow - (int64_t)lane * pn, x - px, pn, p.M - y0);
+            else if (kRows)
+              rows_out_s8<32>(p, ebuf, lane, v, x, y0);
             else if (p.out_bits == 32)
               tma_out_words32<false>(om, ebuf, lane, v, x, y0, 0, y0 < p.M && x < p.N);
             else
@@ -728,10 +841,12 @@ __global__ void __launch_bounds__(TcCfg<BN, STAGES, B_KMAJOR, EPI, EPI_WARPS, TM
           }
           if constexpr (CPT % 32 != 0) {  // a 16-column tail: each lane stores its row
             constexpr int kTail = (CPT / 32) * 32;
-            if (row_ok) {
-              uint32_t v[16];
+            uint32_t v[16];
 #pragma unroll
-              for (int i = 0; i < 16; ++i) v[i] = static_cast<uint32_t>(acc[kTail + i]);
+            for (int i = 0; i < 16; ++i) v[i] = static_cast<uint32_t>(acc[kTail + i]);
+            if (kRows && uo == kOutRows && !split) {
+              rows_out_s8<16>(p, ebuf, lane, v, col0 + kTail, y0);
+            } else if (row_ok) {
               if (split)
                 store_words<16>(wrow, col0 + kTail - px, pn, ws_vec, v);
               else
@@ -777,12 +892,16 @@ __global__ void __launch_bounds__(TcCfg<BN, STAGES, B_KMAJOR, EPI, EPI_WARPS, TM
           tmem_ld<32>(t0 + c * 32, r);
           tmem_ld_wait();
           const int x = col0 + c * 32;
-          if (TMA_OUT == 1 && uo == kOutTmaWs) {
+          if ((TMA_OUT & 3) == 1 && uo == kOutTmaWs) {
             tma_out_words32<true>(om, ebuf, lane, r, x - px, y0 - py, w.split, y0 < p.M && x < p.N);
           } else if (TMA_OUT == 1 && uo == kOutTmaC) {
             tma_out_bf16x32(om, ebuf, lane, r, x, y0, y0 < p.M && x < p.N);
           } else if (TMA_OUT == 2 && uo == kOutTmaC) {
             tma_out_bf16x16x2(om, ebuf, lane, r, x, y0, p.M, p.N);
+          } else if (kRows && (TMA_OUT & 3) == 1 && uo == kOutRows && split) {
+            rows_out_partials(ebuf, lane, r, wrow - (int64_t)lane * pn, x - px, pn, p.M - y0);
+          } else if (kRows && uo == kOutRows && !split) {
+            rows_out_bf16<(TMA_OUT & 3) == 2>(p, ebuf, lane, r, x, y0);
           } else if (row_ok) {
             if (split)
               store_words<32>(wrow, x - px, pn, ws_vec, r);

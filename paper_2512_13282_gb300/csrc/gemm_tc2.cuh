@@ -115,13 +115,13 @@ struct Tc2Cfg {
   static constexpr int kEpiThreads = EPI_WARPS * 32;
   static constexpr int kColsPerThread = BN / (EPI_WARPS / 4);
   static_assert(kColsPerThread % 16 == 0, "epilogue chunks are 32 columns, plus one of 16");
-  static constexpr uint32_t kEpiWarpBytes = TMA_OUT == 1 ? 4096 : TMA_OUT == 2 ? 1024 : 0;  // one 32 x 32 block of 32-bit words
+  static constexpr uint32_t kEpiWarpBytes = (TMA_OUT & 3) == 1 ? 4096 : (TMA_OUT & 3) == 2 ? 1024 : 0;  // one 32 x 32 block of 32-bit words
   static constexpr uint32_t kEpiOffset = STAGES * kStageBytes;
   static constexpr uint32_t kBarOffset = kEpiOffset + EPI_WARPS * kEpiWarpBytes;
   static constexpr uint32_t kNumBars = 2 * STAGES + 4 + 1;
   static constexpr uint32_t kSmemBytes = kBarOffset + kNumBars * 8 + 16 + 1024;
   static_assert(kSmemBytes <= 232448, "shared memory per CTA is 227 KB");
-  static_assert(kSmemBytes == tc_smem_bytes(STAGES, kHalfN, EPI_WARPS, TMA_OUT), "layout and model agree");
+  static_assert(kSmemBytes == tc_smem_bytes(STAGES, kHalfN, EPI_WARPS, TMA_OUT & 3), "layout and model agree");
   static_assert(kTmemCols <= 512, "TMEM has 512 columns");
 };
 
@@ -133,9 +133,10 @@ __global__ void __launch_bounds__(Tc2Cfg<BN, STAGES, B_KMAJOR, EPI, EPI_WARPS, T
                     const __grid_constant__ CUtensorMap tmOut, const __grid_constant__ CUtensorMap tmWs,
                     const TcParams p) {
   using Cfg = Tc2Cfg<BN, STAGES, B_KMAJOR, EPI, EPI_WARPS, TMA_OUT>;
-  const int out_tma = TMA_OUT != 0 ? p.out_tma : (int)kOutDirect;
+  constexpr bool kRows = (TMA_OUT & kTmaOutRows) != 0;
+  const int out_tma = kRows ? (int)kOutRows : TMA_OUT != 0 ? p.out_tma : (int)kOutDirect;
   // the split tail's partials: through tmWs by the 4 KB staging blocks, or directly
-  const int tail_out = (TMA_OUT == 1 && p.ws_tma) ? (int)kOutTmaWs : (int)kOutDirect;
+  const int tail_out = ((TMA_OUT & 3) == 1 && p.ws_tma) ? (int)kOutTmaWs : (int)kOutDirect;
   constexpr int kTileM = 2 * kBM;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_addr(smem_raw);
@@ -350,6 +351,10 @@ __global__ void __launch_bounds__(Tc2Cfg<BN, STAGES, B_KMAJOR, EPI, EPI_WARPS, T
             const int x = col0 + c * 32;
             if (uo == kOutTmaWs)
               tma_out_words32<true>(om, ebuf, lane, v, x - px, y0 - py, w.split, y0 < p.M && x < p.N);
+            else if (kRows && split)
+              rows_out_partials(ebuf, lane, v, wrow - (int64_t)lane * pn, x - px, pn, p.M - y0);
+            else if (kRows)
+              rows_out_s8<32>(p, ebuf, lane, v, x, y0);
             else if (p.out_bits == 32)
               tma_out_words32<false>(om, ebuf, lane, v, x, y0, 0, y0 < p.M && x < p.N);
             else
@@ -357,10 +362,12 @@ __global__ void __launch_bounds__(Tc2Cfg<BN, STAGES, B_KMAJOR, EPI, EPI_WARPS, T
           }
           if constexpr (CPT % 32 != 0) {  // a 16-column tail: each lane stores its row
             constexpr int kTail = (CPT / 32) * 32;
-            if (row_ok) {
-              uint32_t v[16];
+            uint32_t v[16];
 #pragma unroll
-              for (int i = 0; i < 16; ++i) v[i] = static_cast<uint32_t>(acc[kTail + i]);
+            for (int i = 0; i < 16; ++i) v[i] = static_cast<uint32_t>(acc[kTail + i]);
+            if (kRows && uo == kOutRows && !split) {
+              rows_out_s8<16>(p, ebuf, lane, v, col0 + kTail, y0);
+            } else if (row_ok) {
               if (split)
                 store_words<16>(wrow, col0 + kTail - px, pn, ws_vec, v);
               else
@@ -406,12 +413,16 @@ __global__ void __launch_bounds__(Tc2Cfg<BN, STAGES, B_KMAJOR, EPI, EPI_WARPS, T
           tmem_ld<32>(t0 + c * 32, r);
           tmem_ld_wait();
           const int x = col0 + c * 32;
-          if (TMA_OUT == 1 && uo == kOutTmaWs) {
+          if ((TMA_OUT & 3) == 1 && uo == kOutTmaWs) {
             tma_out_words32<true>(om, ebuf, lane, r, x - px, y0 - py, w.split, y0 < p.M && x < p.N);
           } else if (TMA_OUT == 1 && uo == kOutTmaC) {
             tma_out_bf16x32(om, ebuf, lane, r, x, y0, y0 < p.M && x < p.N);
           } else if (TMA_OUT == 2 && uo == kOutTmaC) {
             tma_out_bf16x16x2(om, ebuf, lane, r, x, y0, p.M, p.N);
+          } else if (kRows && (TMA_OUT & 3) == 1 && uo == kOutRows && split) {
+            rows_out_partials(ebuf, lane, r, wrow - (int64_t)lane * pn, x - px, pn, p.M - y0);
+          } else if (kRows && uo == kOutRows && !split) {
+            rows_out_bf16<(TMA_OUT & 3) == 2>(p, ebuf, lane, r, x, y0);
           } else if (row_ok) {
             if (split)
               store_words<32>(wrow, x - px, pn, ws_vec, r);

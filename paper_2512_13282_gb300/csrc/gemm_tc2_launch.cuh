@@ -7,7 +7,7 @@
 namespace gb300 {
 
 template <int BN, int STAGES, bool KM, int EPI, int EW, int TMA>
-cudaError_t launch_pair(const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap &o, const CUtensorMap &w, const TcParams &p,
+cudaError_t launch_pair_variant(const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap &o, const CUtensorMap &w, const TcParams &p,
                         int grid,
                         cudaStream_t st) {
   using Cfg = Tc2Cfg<BN, STAGES, KM, EPI, EW, TMA>;
@@ -23,6 +23,15 @@ cudaError_t launch_pair(const CUtensorMap &a, const CUtensorMap &b, const CUtens
   }
   // grid is even: a whole number of pairs
   return launch_ex(kern, dim3((unsigned)grid), dim3(Cfg::kThreads), Cfg::kSmemBytes, st, 2, a, b, o, w, p);
+}
+
+template <int BN, int STAGES, bool KM, int EPI, int EW, int TMA>
+cudaError_t launch_pair(const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap &o, const CUtensorMap &w,
+                       const TcParams &p, int grid, cudaStream_t st) {
+  if constexpr (TMA != 0)
+    if (p.out_tma == kOutRows)
+      return launch_pair_variant<BN, STAGES, KM, EPI, EW, TMA | kTmaOutRows>(a, b, o, w, p, grid, st);
+  return launch_pair_variant<BN, STAGES, KM, EPI, EW, TMA>(a, b, o, w, p, grid, st);
 }
 
 }  // namespace gb300

@@ -5,7 +5,7 @@ namespace gb300 {
 
 namespace {
 template <int BN, int STAGES, bool KM, int EPI, int EW, int TMA>
-cudaError_t launch_one(const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap &o, const CUtensorMap &w, const TcParams &p,
+cudaError_t launch_one_variant(const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap &o, const CUtensorMap &w, const TcParams &p,
                        int grid,
                        cudaStream_t st) {
   using Cfg = TcCfg<BN, STAGES, KM, EPI, EW, TMA>;
@@ -21,6 +21,15 @@ cudaError_t launch_one(const CUtensorMap &a, const CUtensorMap &b, const CUtenso
     if (dev >= 0 && dev < 64) opted_in[dev] = true;
   }
   return launch_ex(kern, dim3((unsigned)grid), dim3(Cfg::kThreads), Cfg::kSmemBytes, st, 1, a, b, o, w, p);
+}
+
+template <int BN, int STAGES, bool KM, int EPI, int EW, int TMA>
+cudaError_t launch_one(const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap &o, const CUtensorMap &w,
+                       const TcParams &p, int grid, cudaStream_t st) {
+  if constexpr (TMA != 0)
+    if (p.out_tma == kOutRows)
+      return launch_one_variant<BN, STAGES, KM, EPI, EW, TMA | kTmaOutRows>(a, b, o, w, p, grid, st);
+  return launch_one_variant<BN, STAGES, KM, EPI, EW, TMA>(a, b, o, w, p, grid, st);
 }
 }  // namespace
 

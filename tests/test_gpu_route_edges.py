@@ -71,6 +71,46 @@ def test_captured_on_a_stream_without_scratch(dtype, M, N, K, layout):
     _check(dtype, A, B, layout, C if dtype == "int8" else C.view(np.uint16))
 
 
+# C rows that allow no wide store leave row by row through the staging blocks:
+# every tile width and family, partials with an odd pitch, a split tail
+@pytest.mark.gpu
+@needs_gpu
+@pytest.mark.parametrize("dtype", ["bf16", "int8", "int8_int16", "int8_int8"])
+@pytest.mark.parametrize("bn,pair", [(64, 0), (96, 0), (128, 0), (128, 1), (192, 0), (192, 1), (224, 0), (224, 1), (256, 0),
+                                     (256, 1)])
+def test_odd_output_rows(monkeypatch, dtype, bn, pair):
+    if dtype != "bf16" and bn < 128:
+        pytest.skip("not compiled for int8")
+    monkeypatch.setenv("GB300_GEMM_S8TM", "0")
+    monkeypatch.setenv("GB300_GEMM_BN", str(bn))
+    monkeypatch.setenv("GB300_GEMM_PAIR", str(pair))
+    for M, N, K, ldc, off, extra in ((300, 259, 512, 261, 1, None), (513, 259, 1600, 259, 3, None),
+                                     (200, 131, 2064, 133, 0, ("GB300_GEMM_SPLITS", "3")),
+                                     (1300, 4099, 512, 4099, 0, ("GB300_GEMM_TAIL_SPLITS", "2"))):
+        with monkeypatch.context() as m:
+            if extra:
+                m.setenv(*extra)
+            kind = "bf16" if dtype == "bf16" else "int8"
+            A, B = _operands(kind, M, N, K, COL, bn + M)
+            C = U.run(dtype, A, B, COL, ldc=ldc, c_off=off, shift=9)
+            if dtype in ("bf16", "int8"):
+                _check(kind, A, B, COL, C)
+            else:
+                want = oracle.requantize(oracle.gemm_s8(A, B, COL), 9, 16 if dtype == "int8_int16" else 8)
+                assert np.array_equal(C.astype(np.int64), want)
+
+
+# the CUDA-core kernel with an unaligned column-major B, whose lanes read their
+# pieces by aligned words inside the matrix
+@pytest.mark.gpu
+@needs_gpu
+@pytest.mark.parametrize("dtype", ["int8", "bf16"])
+@pytest.mark.parametrize("M,N,K,off", [(1, 33, 1001, 0), (2, 70, 515, 1), (2, 4, 17, 3), (1, 301, 4099, 5)])
+def test_small_m_unaligned_column_major(dtype, M, N, K, off):
+    A, B = _operands(dtype, M, N, K, COL, M + K)
+    _check(dtype, A, B, COL, U.run(dtype, A, B, COL, b_off=off))
+
+
 # 129 rows and more of the small operand: several Q tiles, one or more K
 # splits, ragged edges of both operands; C stored by TMA or, with an odd pitch
 # or base, element by element
