@@ -17,6 +17,7 @@
 #include "gb300_gemm.h"
 #include "gemm_internal.h"
 #include "plan_table.h"
+#include "range_table.h"
 
 using namespace gb300;
 
@@ -401,12 +402,18 @@ struct Plan {
 // ceil(units / slots) of kb_per steps each; a split tail (the tiles of a
 // last, partly filled round split in tail_splits) gives the full rounds of
 // whole tiles plus one round of a tail unit's steps.
-double modelled_us(bool int8, bool pair, int bn, int64_t steps, int64_t rounds, double partial_mb) {
+struct Costs {
+  const plan_table::StepCost (*step)[2][6];
+  const float *split_fixed_us, *split_us_per_mb;
+};
+constexpr Costs kPlanCosts{plan_table::kCost, plan_table::kSplitFixedUs, plan_table::kSplitUsPerMB};
+constexpr Costs kRangeCosts{range_table::kCost, range_table::kSplitFixedUs, range_table::kSplitUsPerMB};  // bf16 only
+
+double modelled_us(const Costs &ct, bool int8, bool pair, int bn, int64_t steps, int64_t rounds, double partial_mb) {
   const int wi = bn == 64 ? 0 : bn == 96 ? 1 : bn == 128 ? 2 : bn == 192 ? 3 : bn == 224 ? 4 : 5;
-  const plan_table::StepCost c = plan_table::kCost[int8 ? 1 : 0][pair ? 1 : 0][wi];
+  const plan_table::StepCost c = ct.step[int8 ? 1 : 0][pair ? 1 : 0][wi];
   double t = (double)steps * c.kstep_us + (double)rounds * c.unit_us;
-  if (partial_mb > 0)
-    t += plan_table::kSplitFixedUs[int8 ? 1 : 0] + plan_table::kSplitUsPerMB[int8 ? 1 : 0] * partial_mb;
+  if (partial_mb > 0) t += ct.split_fixed_us[int8 ? 1 : 0] + ct.split_us_per_mb[int8 ? 1 : 0] * partial_mb;
   return t;
 }
 
@@ -429,9 +436,23 @@ double dram_us(int64_t M, int64_t N, int64_t K, bool int8, bool pair) {
 // split tail, or none (where the scratch is limited).
 enum class Partials { kAny = 0, kNoTail = 1, kNone = 2 };
 
-Plan search_plan(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sms, int pairs, Partials partials) {
-  const bool allow_tail = partials == Partials::kAny;
-  Plan pl{};
+struct Choice {
+  bool found = false, pair = false;
+  int bn = 128;
+  int64_t splits = 1, tail_splits = 0, kb_tail = 0;
+  double model_us = 0.0;
+};
+
+// Extra time of a K range summed in registers (bf16, one split) beyond the
+// first, per tile: its accumulator is read while the next one fills, so only
+// the hand-over shows.
+constexpr double kSlabUs = 0.2;
+
+// The fastest plan by `costs`.  ranges > 0 (bf16): only plans that sum K in
+// that many ranges, as splits or, on the tiles compiled for it, in registers.
+Choice best_choice(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sms, int pairs, Partials partials,
+                   const Costs &costs, int64_t ranges) {
+  const bool allow_tail = partials == Partials::kAny && ranges <= 1;
   // compiled widths, widest first: the bf16 single-CTA kernels also come 64
   // and 96 wide (96 for B column-major only), for memory-bound GEMMs with
   // few rows
@@ -441,21 +462,14 @@ Plan search_plan(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sm
   const Overrides &ovr = overrides();
   const bool int8 = epi == kEpiS32;
   const int64_t num_kb = ceil_div(K, kBK);
-  bool best_pair = false;
-  int best_bn = 128;
-  int64_t best_splits = 1, best_tail = 0, best_kb_tail = 0;
-  double best_cost = -1.0, best_model = 0.0;
+  Choice best;
+  double best_cost = -1.0;
   const double mem_rank = plan_table::kMemWeight;
   auto consider = [&](bool pair, int bn, int64_t splits, int64_t tail_splits, int64_t kb_tail, double model) {
     const double cost = model + mem_rank * dram_us(M, N, K, int8, pair);
     if (best_cost < 0 || cost < best_cost - 1e-9) {
       best_cost = cost;
-      best_model = model;
-      best_pair = pair;
-      best_bn = bn;
-      best_splits = splits;
-      best_tail = tail_splits;
-      best_kb_tail = kb_tail;
+      best = Choice{true, pair, bn, splits, tail_splits, kb_tail, model};
     }
   };
   // A forced tail split (GB300_GEMM_TAIL_SPLITS >= 2) searches the split-tail
@@ -494,9 +508,12 @@ Plan search_plan(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sm
             if (s2 > 1 && (partials == Partials::kNone || kb_per < 4 || tiles * s2 > 2 * slots)) continue;
           }
           seen[nseen++] = s2;
+          const bool in_regs = ranges > 1 && s2 == 1 && bn <= kMaxSlabBN;
+          if (ranges > 0 && s2 != ranges && !in_regs) continue;
           const int64_t rounds = ceil_div(tiles * s2, slots);
           consider(pair, bn, s2, 0, 0,
-                   modelled_us(int8, pair, bn, rounds * kb_per, rounds, s2 > 1 ? 4.0 * s2 * M * N / 1e6 : 0.0));
+                   modelled_us(costs, int8, pair, bn, rounds * kb_per, rounds, s2 > 1 ? 4.0 * s2 * M * N / 1e6 : 0.0) +
+                       (in_regs ? kSlabUs * (double)(rounds * (ranges - 1)) : 0.0));
         }
         // Split tail: whole tiles for the full rounds, the last round's
         // tiles (at most half a round of them) split in S so that they fill
@@ -508,19 +525,38 @@ Plan search_plan(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sm
           const int64_t kb_tail = ceil_div(num_kb, st2);
           if (ceil_div(num_kb, kb_tail) != st2 || kb_tail < 4) continue;
           const double part_mb = 4.0 * st2 * tail * (pair ? 2 * kBM : kBM) * bn / 1e6;
-          consider(pair, bn, 1, st2, kb_tail, modelled_us(int8, pair, bn, full * num_kb + kb_tail, full + 1, part_mb));
+          consider(pair, bn, 1, st2, kb_tail,
+                   modelled_us(costs, int8, pair, bn, full * num_kb + kb_tail, full + 1, part_mb));
         }
       }
     }
   }
-  const bool pair = best_pair;
-  const int bn = best_bn;
+  return best;
+}
+
+Plan search_plan(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sms, int pairs, Partials partials) {
+  const Overrides &ovr = overrides();
+  const int64_t num_kb = ceil_div(K, kBK);
+  // bf16: the K ranges come from a table of their own (range_table.h), so that
+  // the costs a plan is ranked by never change what a sum rounds to.
+  int64_t ranges = 0;
+  if (epi == kEpiBf16 && ovr.splits < 1)
+    ranges = best_choice(M, N, K, b_kmajor, epi, sms, pairs, Partials::kAny, kRangeCosts, 0).splits;
+  Choice best = best_choice(M, N, K, b_kmajor, epi, sms, pairs, partials, kPlanCosts, ranges);
+  if (!best.found && ranges > 1) {  // a forced tile without a variant that sums ranges in registers, and no partials
+    ranges = 0;
+    best = best_choice(M, N, K, b_kmajor, epi, sms, pairs, partials, kPlanCosts, 0);
+  }
+  Plan pl{};
+  const bool pair = best.pair;
+  const int bn = best.bn;
   const int64_t slots = pair ? pairs : sms;
   const int64_t tiles_m = ceil_div(M, pair ? 2 * kBM : kBM);
   const int64_t tiles_n = ceil_div(N, bn);
   const int64_t tiles = tiles_m * tiles_n;
-  const int64_t kb_per = ceil_div(num_kb, best_splits);
+  const int64_t kb_per = ceil_div(num_kb, best.splits);
   const int64_t splits = ceil_div(num_kb, kb_per);
+  const int64_t best_tail = best.tail_splits;
   const int64_t full_rounds = best_tail > 0 ? tiles / slots : 0;
   // Output path: the bf16 224-wide kernels keep a pipeline stage and stage
   // their TMA stores through 1 KB blocks; for int8 at 192/224, TMA stores
@@ -534,7 +570,7 @@ Plan search_plan(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sm
   else
     tma_out = ((bn != 224 && bn != 192) || kb_per <= 128) ? 1 : 0;
   pl.v = TcVariant{bn, b_kmajor, epi, pair, tma_out};
-  pl.model_us = best_model;
+  pl.model_us = best.model_us;
   TcParams &p = pl.p;
   p.M = (int)M;
   p.N = (int)N;
@@ -544,13 +580,13 @@ Plan search_plan(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sm
   p.num_kb = (int)num_kb;
   p.splits = (int)splits;
   p.kb_per_split = (int)kb_per;
-  p.slab_kb = epi == kEpiS32 ? 1024 / kBK : (int)num_kb;
+  p.slab_kb = epi == kEpiS32 ? 1024 / kBK : (int)(splits == 1 && ranges > 1 ? ceil_div(num_kb, ranges) : num_kb);
   p.group_m = 8;
   p.out_bits = 32;
   p.out_shift = 0;
   p.tail_first = (int)(full_rounds * slots);
   p.tail_splits = (int)best_tail;
-  p.tail_kb_per = (int)best_kb_tail;
+  p.tail_kb_per = (int)best.kb_tail;
   p.ws_tma = 0;
   const int64_t units = best_tail > 0 ? full_rounds * slots + (tiles - full_rounds * slots) * best_tail
                                       : tiles * splits;
@@ -563,7 +599,7 @@ Plan search_plan(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sm
                  (long long)M, (long long)N, (long long)K, epi == kEpiS32 ? "int8" : "bf16",
                  b_kmajor ? "col" : "row", pair ? "pair" : "single", bn,
                  tma_out == 2 ? " tma-store-1k" : tma_out ? " tma-store" : "", (long long)tiles_m,
-                 (long long)tiles_n, (long long)splits, (long long)best_tail, p.tail_first, pl.grid, best_model, sms,
+                 (long long)tiles_n, (long long)splits, (long long)best_tail, p.tail_first, pl.grid, best.model_us, sms,
                  pairs);
   return pl;
 }

@@ -90,6 +90,14 @@ enum OutMode : int { kOutDirect = 0, kOutTmaC = 1, kOutTmaWs = 2, kOutRows = 3 }
 // A variant of its own, since the code costs the others registers and 0.6 us
 // a call (int8 8192 x 512 x 512 11.2 -> 11.7 us).
 constexpr int kTmaOutRows = 4;
+// Added to a bf16 variant's TMA_OUT: the unit's K ranges of slab_kb k-blocks
+// are summed in registers, one fp32 sum per accumulator column, in order -- the
+// additions of the split-K reduction, without its partials and launch (bf16
+// 128 x 11008 x 4096 in two ranges 25.5 -> 19.0 us; one range 18.7).  A variant
+// of its own for the registers (BN of them); compiled up to 128 columns: the
+// measured shapes lose no more with wider ones left out.
+constexpr int kTmaOutSlabs = 8;
+constexpr int kMaxSlabBN = 128;
 
 __host__ __device__ constexpr uint32_t pow2_at_least(uint32_t x) {
   uint32_t p = 32;
@@ -571,6 +579,31 @@ __device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&r)[W]) {
     tmem_ld_32x32b_x16(taddr, r);
 }
 
+// 32 fp32 sums of each lane's row as bf16 C, by the path uo.
+template <int TMA_OUT>
+__device__ __forceinline__ void store_bf16_chunk(const TcParams &p, const CUtensorMap *tm, uint32_t ebuf, int lane, int uo,
+                                                 const uint32_t (&r)[32], int x, int y0, int64_t row) {
+  if ((TMA_OUT & 3) == 1 && uo == kOutTmaC)
+    tma_out_bf16x32(tm, ebuf, lane, r, x, y0, y0 < p.M && x < p.N);
+  else if ((TMA_OUT & kTmaOutRows) != 0)
+    rows_out_bf16<(TMA_OUT & 3) == 2>(p, ebuf, lane, r, x, y0);
+  else if (row < p.M)
+    store_bf16<32>(reinterpret_cast<uint16_t *>(p.C) + row * p.ldc, x, p.N, p.c_vec != 0, r);
+}
+
+// acc += the CPT accumulator columns at t0.
+template <int CPT>
+__device__ __forceinline__ void add_columns(uint32_t t0, float (&acc)[CPT]) {
+#pragma unroll
+  for (int c = 0; c < CPT / 32; ++c) {
+    uint32_t r[32];
+    tmem_ld<32>(t0 + c * 32, r);
+    tmem_ld_wait();
+#pragma unroll
+    for (int i = 0; i < 32; ++i) acc[c * 32 + i] += __uint_as_float(r[i]);
+  }
+}
+
 template <int BN, int STAGES, bool B_KMAJOR, int EPI, int EPI_WARPS, int TMA_OUT>
 __global__ void __launch_bounds__(TcCfg<BN, STAGES, B_KMAJOR, EPI, EPI_WARPS, TMA_OUT>::kThreads, 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -874,6 +907,31 @@ __global__ void __launch_bounds__(TcCfg<BN, STAGES, B_KMAJOR, EPI, EPI_WARPS, TM
             else
               store_s8_result<16>(p, row, col0 + kTail, v);
           }
+        }
+      } else if constexpr ((TMA_OUT & kTmaOutSlabs) != 0) {
+        static_assert(CPT % 32 == 0, "whole 32-column chunks");
+        float acc[CPT];
+#pragma unroll
+        for (int i = 0; i < CPT; ++i) acc[i] = 0.f;
+        for (int kb_s = w.kb0; kb_s < w.kb1; kb_s += p.slab_kb) {
+          const uint32_t b = acc_cnt & 1u, aph = (acc_cnt >> 1) & 1u;
+          if (!__all_sync(0xffffffffu, mbar_wait(accf_bar(b), aph, abort_flag, p.err, p.wait_limit_ns))) {
+            ok = false;
+            break;
+          }
+          tc_fence_after_sync();
+          add_columns<CPT>(tmem_base + b * BN + ((uint32_t)(quad * 32) << 16) + colpart * CPT, acc);
+          tc_fence_before_sync();
+          mbar_arrive(acce_bar(b));
+          ++acc_cnt;
+        }
+        if (!ok) break;
+#pragma unroll
+        for (int c = 0; c < CPT / 32; ++c) {
+          uint32_t r[32];
+#pragma unroll
+          for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(acc[c * 32 + i]);
+          store_bf16_chunk<TMA_OUT>(p, om, ebuf, lane, uo, r, col0 + c * 32, y0, row);
         }
       } else {
         const uint32_t b = acc_cnt & 1u, aph = (acc_cnt >> 1) & 1u;

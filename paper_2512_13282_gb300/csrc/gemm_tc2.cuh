@@ -396,6 +396,31 @@ __global__ void __launch_bounds__(Tc2Cfg<BN, STAGES, B_KMAJOR, EPI, EPI_WARPS, T
               store_s8_result<16>(p, row, col0 + kTail, v);
           }
         }
+      } else if constexpr ((TMA_OUT & kTmaOutSlabs) != 0) {
+        static_assert(CPT % 32 == 0, "whole 32-column chunks");
+        float acc[CPT];
+#pragma unroll
+        for (int i = 0; i < CPT; ++i) acc[i] = 0.f;
+        for (int kb_s = w.kb0; kb_s < w.kb1; kb_s += p.slab_kb) {
+          const uint32_t b = acc_cnt & 1u, aph = (acc_cnt >> 1) & 1u;
+          if (!__all_sync(0xffffffffu, mbar_wait(accf_bar(b), aph, abort_flag, p.err, p.wait_limit_ns))) {
+            ok = false;
+            break;
+          }
+          tc_fence_after_sync();
+          add_columns<CPT>(tmem_base + b * BN + ((uint32_t)(quad * 32) << 16) + colpart * CPT, acc);
+          tc_fence_before_sync();
+          mbar_arrive_cluster(mapa_shared(acce_bar(b), 0));
+          ++acc_cnt;
+        }
+        if (!ok) break;
+#pragma unroll
+        for (int c = 0; c < CPT / 32; ++c) {
+          uint32_t r[32];
+#pragma unroll
+          for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(acc[c * 32 + i]);
+          store_bf16_chunk<TMA_OUT>(p, om, ebuf, lane, uo, r, col0 + c * 32, y0, row);
+        }
       } else {
         const uint32_t b = acc_cnt & 1u, aph = (acc_cnt >> 1) & 1u;
         if (!__all_sync(0xffffffffu, mbar_wait(accf_bar(b), aph, abort_flag, p.err, p.wait_limit_ns))) {

@@ -28,6 +28,11 @@ cudaError_t launch_pair_variant(const CUtensorMap &a, const CUtensorMap &b, cons
 template <int BN, int STAGES, bool KM, int EPI, int EW, int TMA>
 cudaError_t launch_pair(const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap &o, const CUtensorMap &w,
                        const TcParams &p, int grid, cudaStream_t st) {
+  if constexpr (EPI == kEpiBf16 && BN <= kMaxSlabBN)
+    if (p.slab_kb < p.kb_per_split)
+      return p.out_tma == kOutRows
+                 ? launch_pair_variant<BN, STAGES, KM, EPI, EW, TMA | kTmaOutSlabs | kTmaOutRows>(a, b, o, w, p, grid, st)
+                 : launch_pair_variant<BN, STAGES, KM, EPI, EW, TMA | kTmaOutSlabs>(a, b, o, w, p, grid, st);
   if constexpr (TMA != 0)
     if (p.out_tma == kOutRows)
       return launch_pair_variant<BN, STAGES, KM, EPI, EW, TMA | kTmaOutRows>(a, b, o, w, p, grid, st);

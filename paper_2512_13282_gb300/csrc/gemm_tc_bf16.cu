@@ -26,6 +26,11 @@ cudaError_t launch_one_variant(const CUtensorMap &a, const CUtensorMap &b, const
 template <int BN, int STAGES, bool KM, int EPI, int EW, int TMA>
 cudaError_t launch_one(const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap &o, const CUtensorMap &w,
                        const TcParams &p, int grid, cudaStream_t st) {
+  if constexpr (BN <= kMaxSlabBN)
+    if (p.slab_kb < p.kb_per_split)
+      return p.out_tma == kOutRows
+                 ? launch_one_variant<BN, STAGES, KM, EPI, EW, TMA | kTmaOutSlabs | kTmaOutRows>(a, b, o, w, p, grid, st)
+                 : launch_one_variant<BN, STAGES, KM, EPI, EW, TMA | kTmaOutSlabs>(a, b, o, w, p, grid, st);
   if constexpr (TMA != 0)
     if (p.out_tma == kOutRows)
       return launch_one_variant<BN, STAGES, KM, EPI, EW, TMA | kTmaOutRows>(a, b, o, w, p, grid, st);

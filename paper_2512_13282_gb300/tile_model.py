@@ -59,6 +59,7 @@ decide, and the walk stops at the first slowdown.
 """
 from __future__ import annotations
 
+import functools
 import json
 import math
 import os
@@ -68,6 +69,7 @@ import numpy as np
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 HEADER = os.path.join(HERE, "csrc", "plan_table.h")
+RANGE_HEADER = os.path.join(HERE, "csrc", "range_table.h")
 MEASUREMENTS = os.path.join(HERE, "plan_measurements.json")
 
 # GB300 resources (one GPU): SMs, co-resident SM pairs for one CTA per SM,
@@ -85,6 +87,10 @@ WIDTHS = (64, 96, 128, 192, 224, 256)
 # only): tiles for memory-bound GEMMs with few rows, which fill the SMs
 # without a K split; they do not meet Eq. 4 and are chosen only by time
 NARROW = (64, 96)
+# tiles whose bf16 kernels can sum K ranges in registers, and what a range
+# beyond the first costs there (kMaxSlabBN and kSlabUs in csrc)
+MAX_SLAB_BN = 128
+SLAB_US = 0.2
 
 
 class Variant:
@@ -294,6 +300,8 @@ def plan_cost_us(M, N, K, dtype, plan, table):
     if mb > 0:
         sp = table["split"][dtype]
         t_split = sp["fixed_us"] + sp["us_per_mb"] * mb
+    if plan.get("slabs", 1) > 1:  # K ranges summed in registers
+        t_split = SLAB_US * rounds * (plan["slabs"] - 1)
     return t_comp + t_split
 
 
@@ -309,11 +317,32 @@ def rank_us(M, N, K, dtype, plan, table):
     return plan_cost_us(M, N, K, dtype, plan, table) + table.get("mem_weight", 0.0) * mem_time_us(M, N, K, dtype, plan)
 
 
+def sum_ranges(M, N, K, b_kmajor, sms=None, pair_slots=None):
+    """The K ranges a bf16 GEMM is summed in (csrc/range_table.h): the split
+    of the plan of least rank_us by the costs fixed there, whatever costs the
+    kernel is then chosen by."""
+    return _least(M, N, K, "bf16", candidate_plans(M, N, K, "bf16", b_kmajor, sms, pair_slots), _range_table())["splits"]
+
+
 def choose_plan(M, N, K, dtype, b_kmajor, table, sms=None, pair_slots=None):
     """The planner: the candidate of least rank_us (the first one, in
-    candidate order, on a tie)."""
+    candidate order, on a tie).  bf16: of those that sum K in sum_ranges
+    ranges, as splits or, unsplit on tiles of at most MAX_SLAB_BN columns, in
+    registers (the plan's "slabs")."""
+    cands = candidate_plans(M, N, K, dtype, b_kmajor, sms, pair_slots)
+    if dtype == "bf16":
+        r = sum_ranges(M, N, K, b_kmajor, sms, pair_slots)
+        if r > 1:
+            cands = [p if p["splits"] == r else dict(p, slabs=r) for p in cands
+                     if p["splits"] == r or (p["splits"] == 1 and not p["tail_splits"] and p["bn"] <= MAX_SLAB_BN)]
+        else:
+            cands = [p for p in cands if p["splits"] == 1]
+    return _least(M, N, K, dtype, cands, table)
+
+
+def _least(M, N, K, dtype, cands, table):
     best, best_c = None, math.inf
-    for p in candidate_plans(M, N, K, dtype, b_kmajor, sms, pair_slots):
+    for p in cands:
         c = rank_us(M, N, K, dtype, p, table)
         if c < best_c - 1e-9:
             best, best_c = p, c
@@ -506,6 +535,24 @@ def header_text(table, source="plan_measurements.json"):
         "",
     ]
     return "\n".join(lines)
+
+
+@functools.lru_cache(maxsize=1)
+def _range_table():
+    """csrc/range_table.h's costs (bf16 only)."""
+    import re
+    with open(RANGE_HEADER) as f:
+        text = f.read()
+    nums = iter([float(x) for x in re.findall(r"([0-9.]+)f", text.split("kCost")[1].split("};")[0])])
+    groups = {}
+    for fam in ("single", "pair"):
+        for bn in WIDTHS:
+            k, u = next(nums), next(nums)
+            if k > 0:
+                groups[f"bf16/{fam}/{bn}"] = {"kstep_us": k, "unit_us": u}
+    one = lambda name: float(re.findall(name + r"\[1\] = \{([0-9.]+)f\}", text)[0])
+    return {"groups": groups, "split": {"bf16": {"fixed_us": one("kSplitFixedUs"), "us_per_mb": one("kSplitUsPerMB")}},
+            "mem_weight": load_table()["mem_weight"]}
 
 
 def table_from_header(text):
