@@ -894,6 +894,7 @@ constexpr int64_t kRowsMinKNarrowBf16 = 1024;
 bool rows_shape(int64_t M, int64_t N, int64_t K, bool b_kmajor, bool int8, bool *small_n) {
   const int lim = rows_max(int8);
   *small_n = M > lim;
+  if (K > kRowsMaxK) return false;
   if (*small_n && !int8 && K < kRowsMinKNarrowBf16) return false;
   return b_kmajor && (M <= lim || N <= lim);
 }

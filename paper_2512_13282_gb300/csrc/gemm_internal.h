@@ -189,6 +189,10 @@ cudaError_t launch_tiny_s8(const TinyParams &p, bool row_b, cudaStream_t st);
 // r * scr + n * scn of C.  The rows of W and X are K contiguous; W's start on
 // 16-byte boundaries.
 constexpr int kRowsMax = 16;
+// The kernel's k indexes are int, and run up to a cluster's rounded slices and
+// a round of batches past K: eight slices of at most 128 more than their share
+// and 4 x 128.
+constexpr int64_t kRowsMaxK = int64_t(1) << 30;
 struct RowsParams {
   const void *W;
   int64_t ldw;  // row pitch in elements

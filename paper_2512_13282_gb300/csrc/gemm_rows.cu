@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(kRowsThreads, kRowsBlocks) gemm_rows_kernel(co
   const uint32_t rank = p.cluster > 1 ? cluster_rank() : 0u;
   const int64_t n0 = (int64_t)(blockIdx.x / p.cluster) * kStrip;
   const int kbeg = (int)rank * p.kslice;
-  const int kend = min(p.K, kbeg + p.kslice);  // kbeg < kend (rows_geometry)
+  const int kend = min(p.K, kbeg + p.kslice);  // kbeg < kend (rows_geometry), no overflow (kRowsMaxK)
   const int nb = (kend - kbeg + kBatch - 1) / kBatch;
   const int64_t pitch = p.ldw * ES;
   const int R = p.R;

@@ -100,3 +100,19 @@ def test_route_limits():
     assert route(17, 4096, 4096, True, COL) != few and route(4096, 17, 4096, False, COL) != few
     assert route(16, 4096, 4096, True, G.GEMM_B_ROW_MAJOR_KxN) != few
     assert route(16, 4096, 4097, False, COL) != few
+
+
+def test_few_row_indexes_fit_an_int():
+    """K up to INT32_MAX is accepted: the calls that the few-row kernel takes
+    have every k index it forms (the cluster's slices and a round of batches
+    past them) below 2^31, longer ones go elsewhere."""
+    from paper_2512_13282_gb300 import build
+    build.build()
+    G.gemm_reload_overrides()
+    for K in (1 << 20, 1 << 28, 1 << 30, (1 << 30) + 8, (1 << 31) - 512, (1 << 31) - 8):
+        for M, N in ((2, 32), (16, 1000), (64, 8), (1, 1 << 20)):
+            st, plan = G.gemm_plan_query(M, N, K, False, COL)
+            assert st == G.GEMM_OK
+            if plan["route"] == G.GEMM_ROUTE_FEW_ROWS:
+                slice_ = -(-(-(-K // plan["splits"])) // 64) * 64
+                assert plan["splits"] * slice_ + 4 * 64 + 32 < 1 << 31, (M, N, K)
