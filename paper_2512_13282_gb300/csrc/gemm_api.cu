@@ -903,8 +903,15 @@ bool rows_shape(int64_t M, int64_t N, int64_t K, bool b_kmajor, bool int8, bool 
 // kRowsMax columns of a column-major B against A: gemm_rows_kernel streams the
 // other operand, which has to be 16-byte aligned in base and pitch (on odd
 // addresses its lanes would load five words per 16 bytes: 16 x 5000 x 5001
-// bf16 71 us against 30 for re-pitching and the tensor cores).  Returns false,
-// having launched nothing, for any other.
+// bf16 71 us against 30 for re-pitching and the tensor cores).  The small
+// operand may lie anywhere; against more than 8 unaligned rows of it, whose
+// words then load the lanes as much as the stream does, large streams go to the
+// tensor-core kernels, which re-pitch or stage them (kRowsMaxOddX elements:
+// bf16 16 x 4096 x 4096 12.6 / 13.0 us, 16 x 12288 x 2048 18.7 / 18.5, 16 x
+// 8192 x 4096 20.7 / 16.8, 16 x 12288 x 4096 33.1 / 21.8; int8 10.3 / 10.8,
+// 13.2 / 12.7, 15.0 / 14.3, 21.9 / 16.9).  Returns false, having launched
+// nothing, for any other.
+constexpr int64_t kRowsMaxOddX = int64_t(1) << 25;
 bool try_rows(DeviceState &d, int64_t M, int64_t N, int64_t K, const void *A, int64_t lda, const void *B,
               int64_t ldb, bool b_kmajor, void *C, int64_t ldc, bool int8, int out_bits, int out_shift,
               cudaStream_t st, gemm_status_t *status) {
@@ -923,6 +930,7 @@ bool try_rows(DeviceState &d, int64_t M, int64_t N, int64_t K, const void *A, in
   p.scn = small_n ? ldc : 1;
   p.K = (int)K;
   p.x_vec = aligned16(p.X) && p.ldx * es % 16 == 0;
+  if (!p.x_vec && p.R > 8 && p.NW * K >= kRowsMaxOddX) return false;
   p.C = C;
   p.out_bits = out_bits;
   p.out_shift = out_shift;

@@ -50,6 +50,8 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
 #include "gemm_internal.h"
 
 namespace gb300 {
@@ -97,7 +99,7 @@ __device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1
 
 // The 16 bytes at a, of which the first `valid` are read (element by element
 // of `es` bytes) and the rest are zero.  Out of line: the ends of W's and X's
-// rows, and X on odd addresses.
+// rows.
 __device__ __noinline__ uint4 load16_edge(const uint8_t *a, int es, int valid) {
   uint32_t w[4] = {0u, 0u, 0u, 0u};
   for (int i = 0; i < 16 && i < valid; i += es) {
@@ -125,8 +127,24 @@ __device__ __forceinline__ void store_out(const RowsParams &p, bool int8, int64_
   }
 }
 
-// NT: 8-row groups of X.
-template <int NT, bool INT8>
+// The 16 bytes at a, on any boundary of X = [lo, hi), as four or five aligned
+// words, shifted (X on odd addresses): element by element they took longer
+// than the stream (odd X pitch, element by element / this: bf16 4 x 12288 x 4096
+// 51.3 / 23.0 us, 16 x 4096 x 4096 29.8 / 12.5, int8 4 x
+// 4096 x 4096 14.5 / 8.1, 16 x 4096 x 4096 26.5 / 10.3).
+__device__ __forceinline__ uint4 load16_words(const uint8_t *a, const uint8_t *lo, const uint8_t *hi, int es) {
+  const uint32_t off = (uint32_t)reinterpret_cast<uintptr_t>(a) & 3u, sh = 8u * off;
+  const uint8_t *al = a - off;
+  if (al < lo || al + (off ? 20 : 16) > hi) return load16_edge(a, es, 16);
+  const uint32_t *q = reinterpret_cast<const uint32_t *>(al);
+  const uint32_t w0 = __ldg(q), w1 = __ldg(q + 1), w2 = __ldg(q + 2), w3 = __ldg(q + 3), w4 = off ? __ldg(q + 4) : 0u;
+  return make_uint4(__funnelshift_r(w0, w1, sh), __funnelshift_r(w1, w2, sh), __funnelshift_r(w2, w3, sh),
+                    __funnelshift_r(w3, w4, sh));
+}
+
+// NT: 8-row groups of X.  XVEC: X's rows start on 16-byte boundaries (a kernel
+// of its own for those that do not, whose loads need more registers).
+template <int NT, bool INT8, bool XVEC>
 __global__ void __launch_bounds__(kRowsThreads, kRowsBlocks) gemm_rows_kernel(const RowsParams p) {
   constexpr int ES = INT8 ? 1 : 2;
   constexpr int kHalf = 64 / ES;       // k per half batch: 64 bytes of each row, 16 a lane
@@ -155,6 +173,7 @@ __global__ void __launch_bounds__(kRowsThreads, kRowsBlocks) gemm_rows_kernel(co
 #pragma unroll
   for (int j = 0; j < NT; ++j)
     xp[j] = static_cast<const uint8_t *>(p.X) + (8 * j + g < R ? 8 * j + g : 0) * p.ldx * ES + 16 * q;
+  const uint8_t *x_lo = static_cast<const uint8_t *>(p.X), *x_hi = x_lo + ((R - 1) * p.ldx + p.K) * ES;
 
   griddep_launch_dependents();
   {  // the warp's first batch: 128 bytes of row n0 + lane
@@ -180,9 +199,12 @@ __global__ void __launch_bounds__(kRowsThreads, kRowsBlocks) gemm_rows_kernel(co
     if (valid <= 0) {
 #pragma unroll
       for (int j = 0; j < NT; ++j) x[j] = make_uint4(0u, 0u, 0u, 0u);
-    } else if (whole && p.x_vec) {
+    } else if (whole && XVEC) {
 #pragma unroll
       for (int j = 0; j < NT; ++j) x[j] = __ldg(reinterpret_cast<const uint4 *>(xp[j] + at));
+    } else if (whole) {
+#pragma unroll
+      for (int j = 0; j < NT; ++j) x[j] = load16_words(xp[j] + at, x_lo, x_hi, ES);
     } else {
 #pragma unroll
       for (int j = 0; j < NT; ++j) x[j] = load16_edge(xp[j] + at, ES, valid);
@@ -313,11 +335,11 @@ __global__ void __launch_bounds__(kRowsThreads, kRowsBlocks) gemm_rows_kernel(co
   cluster_barrier();  // no block leaves while another may still read its sums
 }
 
-template <int NT, bool INT8>
+template <int NT, bool INT8, bool XVEC>
 cudaError_t launch_nt(const RowsParams &p, int64_t strips, cudaStream_t st) {
   const size_t smem = (size_t)p.R * 4 * (kRowsWarps * kSumPitch + (p.cluster > 1 ? kStrip : 0));
   static_assert(8 * NT * 4 * (kRowsWarps * kSumPitch + kStrip) <= 48 * 1024, "no shared-memory opt-in needed");
-  return launch_ex(gemm_rows_kernel<NT, INT8>, dim3((unsigned)(strips * p.cluster)), dim3(kRowsThreads), smem, st,
+  return launch_ex(gemm_rows_kernel<NT, INT8, XVEC>, dim3((unsigned)(strips * p.cluster)), dim3(kRowsThreads), smem, st,
                    p.cluster, p);
 }
 
@@ -346,8 +368,15 @@ int64_t rows_geometry(int64_t NW, int64_t K, bool int8, int sms, int *cluster, i
 }
 
 cudaError_t launch_rows(const RowsParams &p, bool int8, int64_t strips, cudaStream_t st) {
-  if (int8) return p.R > 8 ? launch_nt<2, true>(p, strips, st) : launch_nt<1, true>(p, strips, st);
-  return p.R > 8 ? launch_nt<2, false>(p, strips, st) : launch_nt<1, false>(p, strips, st);
+  auto by_x = [&](auto nt, auto is_int8) {
+    constexpr int NT = decltype(nt)::value;
+    constexpr bool INT8 = decltype(is_int8)::value;
+    return p.x_vec ? launch_nt<NT, INT8, true>(p, strips, st) : launch_nt<NT, INT8, false>(p, strips, st);
+  };
+  using std::integral_constant;
+  if (int8)
+    return p.R > 8 ? by_x(integral_constant<int, 2>{}, std::true_type{}) : by_x(integral_constant<int, 1>{}, std::true_type{});
+  return p.R > 8 ? by_x(integral_constant<int, 2>{}, std::false_type{}) : by_x(integral_constant<int, 1>{}, std::false_type{});
 }
 
 }  // namespace gb300

@@ -62,6 +62,19 @@ def test_few_rows_ragged_k_and_odd_small_operand(dtype, K):
 
 @pytest.mark.gpu
 @pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a GPU")
+@pytest.mark.parametrize("dtype,R,K,pad,off", [("int8", 16, 2048, 1, 0), ("int8", 9, 640, 2, 3), ("int8", 3, 1040, 4, 1),
+                                               ("int8", 8, 512, 8, 0), ("int8", 1, 2064, 0, 2), ("bf16", 16, 1032, 1, 0),
+                                               ("bf16", 8, 2048, 2, 3), ("bf16", 2, 1024, 4, 1), ("bf16", 1, 1544, 0, 1)])
+def test_few_rows_small_operand_by_words(dtype, R, K, pad, off):
+    """A small operand on every alignment that is not 16 bytes, over several
+    batches: read by aligned words, at its first and last bytes element by
+    element."""
+    _run(dtype, R, 130, K, seed=K + R, lda=K + pad, a_off=off)
+    _run(dtype, 1100, R, K, seed=K - R, ldb=K + pad, b_off=off)
+
+
+@pytest.mark.gpu
+@pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a GPU")
 def test_few_rows_int8_extremes():
     """All -128 at the largest K (2147467264), and -128 x 127."""
     A, B = np.full((16, 131071), -128, np.int8), np.full((40, 131071), -128, np.int8)
