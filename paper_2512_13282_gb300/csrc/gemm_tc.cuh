@@ -23,9 +23,10 @@
 //                      lines per instruction and compete with the operand
 //                      traffic; lanes store their rows directly only where
 //                      C's address or pitch rules TMA out but its rows lie on
-//                      8-byte boundaries, and in the int8 variants that trade
-//                      the staging blocks for a pipeline stage (long
-//                      reductions).  Odder rows leave row by row (rows_out).  Two accumulators let the
+//                      8-byte boundaries (4-byte for 16- and 8-bit outputs) or
+//                      are short, and in the int8 variants that trade the
+//                      staging blocks for a pipeline stage (long reductions).
+//                      Odder rows leave row by row (rows_out).  Two accumulators let the
 //                      epilogue of one tile overlap the main loop of the
 //                      next (the paper keeps a single C buffer for lack of
 //                      L1 space, Sec. 5.3.2; TMEM has room for two).

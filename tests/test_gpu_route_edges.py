@@ -164,3 +164,30 @@ def test_route_limits():
     assert route(512, 4096, 4096, True, COL) == small_op and route(4096, 256, 4096, True) == small_op
     assert route(1024, 4096, 4096, True, COL) == G.GEMM_ROUTE_TC_PAIR and route(256, 1024, 1024, True) != small_op
     assert [route(m, 4096, 4096, False) for m in (2, 3)] == [small_m, G.GEMM_ROUTE_TC_SINGLE]
+
+
+# how C is stored where TMA cannot: by the lanes where they can store whole
+# words (two for 32-bit outputs) or C is a few columns or one block of rows
+# tall, else row by row
+@pytest.mark.gpu
+@needs_gpu
+@pytest.mark.parametrize("dtype,M,N,ldc,off,how", [
+    ("bf16", 200, 130, 130, 0, "lanes"), ("bf16", 200, 130, 131, 0, "rows"), ("bf16", 200, 130, 130, 1, "rows"),
+    ("int8_int16", 200, 130, 130, 0, "lanes"), ("int8_int16", 200, 130, 131, 0, "rows"),
+    ("int8_int8", 200, 132, 132, 0, "lanes"), ("int8_int8", 200, 130, 130, 0, "rows"), ("int8_int8", 200, 132, 132, 2, "rows"),
+    ("int8", 200, 130, 130, 0, "lanes"), ("int8", 200, 129, 129, 0, "rows"), ("int8", 200, 127, 127, 0, "lanes"),
+    ("bf16", 65, 23, 23, 0, "lanes"), ("bf16", 65, 25, 25, 0, "rows"), ("bf16", 32, 131, 131, 0, "lanes"),
+    ("bf16", 33, 131, 131, 0, "rows"), ("int8_int8", 65, 23, 23, 0, "lanes"), ("int8_int8", 32, 131, 131, 0, "lanes")])
+def test_how_odd_output_rows_are_stored(monkeypatch, capfd, dtype, M, N, ldc, off, how):
+    for var, v in (("S8TM", 0), ("TINY_MAX_MACS", 0), ("SPLITS", 1), ("DEBUG", 1)):
+        monkeypatch.setenv("GB300_GEMM_" + var, str(v))
+    kind = "bf16" if dtype == "bf16" else "int8"
+    A, B = _operands(kind, M, N, 640, COL, M + N)
+    capfd.readouterr()
+    C = U.run(dtype, A, B, COL, ldc=ldc, c_off=off, shift=9)
+    assert f"output by {how}" in capfd.readouterr().err
+    if dtype in ("bf16", "int8"):
+        _check(kind, A, B, COL, C)
+    else:
+        want = oracle.requantize(oracle.gemm_s8(A, B, COL), 9, 16 if dtype == "int8_int16" else 8)
+        assert np.array_equal(C.astype(np.int64), want)
