@@ -64,7 +64,10 @@ __device__ __forceinline__ void piece_rc(uint64_t u, uint32_t cpr, int w, int64_
 // thread reads its 16 bytes with the widest loads the row's address allows
 // (odd rows as five aligned words, shifted; byte by byte they took 1.5 times
 // the GEMM's own time at 1001 x 1503 x 3001) and writes 32 bytes with two
-// 16-byte stores (staged rows start 128-byte aligned).
+// 16-byte stores (staged rows start 16-byte aligned).  A row's last, partial
+// piece does the same where its 16 bytes lie inside the matrix and its 32 inside
+// the staged row: what follows the row is read, converted and never used (element
+// by element, each load waited for, they set the time of short rows).
 __global__ void __launch_bounds__(kS8Threads)
     s8_to_bf16_pair_kernel(const S8Job a, const S8Job b, uint32_t cpr_a, uint32_t cpr_b, uint64_t items_a,
                            uint64_t items) {
@@ -77,8 +80,8 @@ __global__ void __launch_bounds__(kS8Threads)
   piece_rc(in_a ? t : t - items_a, in_a ? cpr_a : cpr_b, 16, r, c);
   const int8_t *src = j.src + r * j.ld_src + c;
   uint16_t *dst = j.dst + r * j.ld_dst + c;
-  if (c + 16 <= j.cols) {
-    const uint8_t *lo8 = reinterpret_cast<const uint8_t *>(j.src), *hi8 = lo8 + (j.rows - 1) * j.ld_src + j.cols;
+  const uint8_t *lo8 = reinterpret_cast<const uint8_t *>(j.src), *hi8 = lo8 + (j.rows - 1) * j.ld_src + j.cols;
+  if (c + 16 <= j.cols || (c + 16 <= j.ld_dst && reinterpret_cast<const uint8_t *>(src) + 16 <= hi8)) {
     const uint4 v = load16_any<true>(reinterpret_cast<const uint8_t *>(src), lo8, hi8);
     const int4 raw = make_int4((int)v.x, (int)v.y, (int)v.z, (int)v.w);
     uint4 lo, hi;
@@ -119,9 +122,9 @@ __global__ void __launch_bounds__(kS8Threads)
   }
 }
 
-// Re-pitch of a bf16 matrix into a buffer whose rows start 128-byte aligned:
+// Re-pitch of a bf16 matrix into a buffer whose rows start 16-byte aligned:
 // thread t copies 8-element piece t % cpr of row t / cpr with one 16-byte
-// store (the source as for the int8 staging above).
+// store (the source and a row's last piece as for the int8 staging above).
 __global__ void __launch_bounds__(kS8Threads)
     pack_u16_kernel(const uint16_t *__restrict__ src, int64_t rows, int64_t cols, int64_t ld_src,
                     uint16_t *__restrict__ dst, int64_t ld_dst, uint32_t cpr, uint64_t items) {
@@ -132,8 +135,8 @@ __global__ void __launch_bounds__(kS8Threads)
   piece_rc(t, cpr, 8, r, c);
   const uint16_t *s = src + r * ld_src + c;
   uint16_t *d = dst + r * ld_dst + c;
-  if (c + 8 <= cols) {
-    const uint8_t *lo = reinterpret_cast<const uint8_t *>(src), *hi = lo + ((rows - 1) * ld_src + cols) * 2;
+  const uint8_t *lo = reinterpret_cast<const uint8_t *>(src), *hi = lo + ((rows - 1) * ld_src + cols) * 2;
+  if (c + 8 <= cols || reinterpret_cast<const uint8_t *>(s) + 16 <= hi) {
     *reinterpret_cast<uint4 *>(d) = load16_any<true>(reinterpret_cast<const uint8_t *>(s), lo, hi);
   } else {
     for (int64_t i = 0; c + i < cols; ++i) d[i] = s[i];

@@ -642,7 +642,15 @@ Plan make_plan(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sms,
 // Row pitch (elements) of a staged or re-pitched bf16 copy with rows of n
 // elements: whole 128-byte lines, so that a TMA box row is one line and not
 // the ends of two (int8 2592^3: 41.7 us with rows of 40.5 lines, 34.3 with 41).
-int64_t staged_pitch(int64_t n) { return (n + 63) / 64 * 64; }
+// Rows of a few lines keep their length, rounded to the 16 elements a thread of
+// the staging kernels writes (a multiple of 8 stays: such matrices are staged as
+// one flat array): whole lines would multiply the copy, up to 8 times for 16
+// elements (int8 19776 x 256 x 40 21.8 -> 14.8 us, 1034048 x 64 x 14 236 -> 175,
+// 4096 x 1000 x 300 14.7 -> 13.1; level from 520 elements on).
+int64_t staged_pitch(int64_t n) {
+  if (n >= 512) return (n + 63) / 64 * 64;
+  return n % 8 == 0 ? n : (n + 15) / 16 * 16;
+}
 
 struct WsLayout {
   size_t a_off = 0, b_off = 0, part_off = 0, total = 0;
@@ -1269,7 +1277,7 @@ gemm_status_t s8_gemm(int64_t M, int64_t N, int64_t K, const int8_t *A, int64_t 
   Plan pl = make_plan(M, N, K, b_kmajor, kEpiS32, d->sms, pair_slots());
   pl.p.out_bits = out_bits;
   pl.p.out_shift = shift;
-  // Stage both operands as bf16 (exact for int8) with 128-byte aligned rows.
+  // Stage both operands as bf16 (exact for int8) with rows a TMA can read.
   const int64_t b_rows = b_kmajor ? N : K, b_cols = b_kmajor ? K : N;
   const int64_t lda_p = staged_pitch(K), ldb_p = staged_pitch(b_cols);
   WsLayout L;

@@ -191,3 +191,41 @@ def test_how_odd_output_rows_are_stored(monkeypatch, capfd, dtype, M, N, ldc, of
     else:
         want = oracle.requantize(oracle.gemm_s8(A, B, COL), 9, 16 if dtype == "int8_int16" else 8)
         assert np.array_equal(C.astype(np.int64), want)
+
+
+# the copies of operands with short rows: not much longer than the operand, and
+# right at the ends of the rows and of the matrix, whose last pieces are read
+# past the row where the matrix goes on
+@pytest.mark.gpu
+@needs_gpu
+def test_short_rows_are_copied_at_their_length():
+    M, N, K = 2_000_000, 24, 5
+    A, B = W.random_bf16((M, K), 1), W.random_bf16((N, K), 2)
+    tA, tB = (torch.from_numpy(x.view(np.int16)).cuda() for x in (A, B))
+    tC = torch.zeros((M, N), dtype=torch.int16, device="cuda")
+    G.gemm_release_resources()
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    assert G.gemm_bf16_f32acc_bf16(M, N, K, tA, K, tB, K, COL, tC, N) == G.GEMM_OK
+    torch.cuda.synchronize()
+    used = free - torch.cuda.mem_get_info()[0]
+    assert used < 5 * M * K * 2, used  # rows of 16 elements and a quarter to spare, not of 64
+    C = tC.cpu().numpy().view(np.uint16)
+    for rows in (slice(0, 300), slice(M - 300, M)):
+        ref, mag = oracle.gemm_bf16(A[rows], B, COL)
+        assert oracle.bf16_within_bound(C[rows], ref, mag).all()
+
+
+@pytest.mark.gpu
+@needs_gpu
+@pytest.mark.parametrize("dtype", ["int8", "bf16"])
+@pytest.mark.parametrize("K,pad,off", [(1, 0, 0), (7, 0, 1), (9, 1, 0), (21, 0, 3), (40, 0, 0), (47, 2, 1), (255, 0, 5),
+                                       (300, 0, 0), (501, 3, 0), (513, 0, 7)])
+def test_short_rows_staged(monkeypatch, dtype, K, pad, off):
+    for var in ("S8TM", "TINY_MAX_MACS"):
+        monkeypatch.setenv("GB300_GEMM_" + var, "0")
+    M, N = 333, 77
+    for layout in (ROW, COL):
+        A, B = _operands(dtype, M, N, K, layout, K)
+        C = U.run(dtype, A, B, layout, lda=K + pad, ldb=B.shape[1] + pad, a_off=off, b_off=off)
+        _check(dtype, A, B, layout, C)
