@@ -643,13 +643,13 @@ Plan make_plan(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sms,
 // elements: whole 128-byte lines, so that a TMA box row is one line and not
 // the ends of two (int8 2592^3: 41.7 us with rows of 40.5 lines, 34.3 with 41).
 // Rows of a few lines keep their length, rounded to the 16 elements a thread of
-// the staging kernels writes (a multiple of 8 stays: such matrices are staged as
-// one flat array): whole lines would multiply the copy, up to 8 times for 16
-// elements (int8 19776 x 256 x 40 21.8 -> 14.8 us, 1034048 x 64 x 14 236 -> 175,
+// the staging kernels writes (8 for 8 or fewer, and a multiple of 8 stays: such
+// matrices are staged as one flat array): whole lines would multiply the copy,
+// up to 8 times (int8 19776 x 256 x 40 21.8 -> 14.8 us, 1034048 x 64 x 14 236 -> 175,
 // 4096 x 1000 x 300 14.7 -> 13.1; level from 520 elements on).
 int64_t staged_pitch(int64_t n) {
   if (n >= 512) return (n + 63) / 64 * 64;
-  return n % 8 == 0 ? n : (n + 15) / 16 * 16;
+  return n % 8 == 0 ? n : n < 8 ? 8 : (n + 15) / 16 * 16;
 }
 
 struct WsLayout {
