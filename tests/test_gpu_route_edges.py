@@ -229,3 +229,17 @@ def test_short_rows_staged(monkeypatch, dtype, K, pad, off):
         A, B = _operands(dtype, M, N, K, layout, K)
         C = U.run(dtype, A, B, layout, lda=K + pad, ldb=B.shape[1] + pad, a_off=off, b_off=off)
         _check(dtype, A, B, layout, C)
+
+
+# the CUDA-core kernel reads aligned and unaligned column-major rows by code of
+# its own each: the same sums, in the same order
+@pytest.mark.gpu
+@needs_gpu
+@pytest.mark.parametrize("dtype", ["int8", "bf16"])
+@pytest.mark.parametrize("M,N,K", [(1, 70, 2064), (2, 33, 4096), (5, 129, 1040), (8, 31, 527), (16, 64, 784)])
+def test_small_m_aligned_and_unaligned_columns_agree(monkeypatch, dtype, M, N, K):
+    monkeypatch.setenv("GB300_GEMM_SKINNY_MAX_M", "16")
+    A, B = _operands(dtype, M, N, K, COL, M + N)
+    C = U.run(dtype, A, B, COL, ldb=(K + 15) // 16 * 16)
+    _check(dtype, A, B, COL, C)
+    assert np.array_equal(C, U.run(dtype, A, B, COL, ldb=(K + 15) // 16 * 16 + 1, b_off=1))
