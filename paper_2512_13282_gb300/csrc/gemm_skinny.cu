@@ -466,10 +466,12 @@ __global__ void __launch_bounds__(kSkThreads, colb_blocks(MT)) skinny_colB_kerne
   finish_block<INT8>(p, red, kCols, n0, cols, &ticket);
 }
 
-// Shared memory beyond the 48 KB every kernel may use needs an opt-in.
+// Shared memory beyond the 48 KB that every kernel may use, its static words
+// among them, needs an opt-in.
+constexpr size_t kStaticSmem = 16;  // the ticket, rounded up
 template <typename Kern>
 cudaError_t opt_in(Kern kern, size_t smem) {
-  if (smem <= 48 * 1024) return cudaSuccess;
+  if (smem + kStaticSmem <= 48 * 1024) return cudaSuccess;
   return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 

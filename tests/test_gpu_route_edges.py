@@ -243,3 +243,16 @@ def test_small_m_aligned_and_unaligned_columns_agree(monkeypatch, dtype, M, N, K
     C = U.run(dtype, A, B, COL, ldb=(K + 15) // 16 * 16)
     _check(dtype, A, B, COL, C)
     assert np.array_equal(C, U.run(dtype, A, B, COL, ldb=(K + 15) // 16 * 16 + 1, b_off=1))
+
+
+# slices of A that fill the 48 KB of shared memory a kernel may use unasked
+# (16 rows x 1536 bf16) or all but a little more
+@pytest.mark.gpu
+@needs_gpu
+@pytest.mark.parametrize("K", [1504, 1536, 1568, 3072])
+def test_small_m_kernel_at_the_shared_memory_limit(monkeypatch, K):
+    monkeypatch.setenv("GB300_GEMM_SKINNY_MAX_M", "16")
+    # as many columns as give one slice of K per wave of blocks
+    N = 32 * 608
+    A, B = _operands("bf16", 12, N, K, COL, K)
+    _check("bf16", A, B, COL, U.run("bf16", A, B, COL))
