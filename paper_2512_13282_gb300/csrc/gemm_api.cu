@@ -895,9 +895,8 @@ gemm_status_t run_skinny(DeviceState &d, int64_t M, int64_t N, int64_t K, const 
 }
 
 // Rows of the small operand up to which gemm_rows_kernel takes a GEMM (0
-// where an override asks for another kernel).  Up to 16 rows it is faster
-// than the kernels that took those shapes before at every size measured
-// (gemm_rows.cu has the figures); its accumulators are built for 16.
+// where an override asks for another kernel): its accumulators are built for
+// 16.  Up to there rows_faster decides (gemm_rows.cu has the figures).
 int rows_max(bool int8) {
   const Overrides &o = overrides();
   if (o.skinny_max_m >= 0 || o.bn > 0 || o.pair >= 0 || o.splits >= 1 || o.tail_splits >= 2) return 0;
@@ -910,12 +909,12 @@ int rows_max(bool int8) {
 // rows better (7000 x 16 x 512: 4.3 us against 4.6; 8192 x 8 x 2000: level;
 // 4096 x 16 x 4096: 9.9 against 8.4).
 constexpr int64_t kRowsMinKNarrowBf16 = 1024;
-bool rows_shape(int64_t M, int64_t N, int64_t K, bool b_kmajor, bool int8, bool *small_n) {
+bool rows_shape(int64_t M, int64_t N, int64_t K, bool b_kmajor, bool int8, int sms, bool *small_n) {
   const int lim = rows_max(int8);
   *small_n = M > lim;
-  if (K > kRowsMaxK) return false;
+  if (!b_kmajor || (M > lim && N > lim) || K > kRowsMaxK) return false;
   if (*small_n && !int8 && K < kRowsMinKNarrowBf16) return false;
-  return b_kmajor && (M <= lim || N <= lim);
+  return *small_n ? rows_faster(M, K, (int)N, int8, false, sms) : rows_faster(N, K, (int)M, int8, true, sms);
 }
 
 // GEMMs with at most kRowsMax rows of A against a column-major B, or at most
@@ -935,7 +934,7 @@ bool try_rows(DeviceState &d, int64_t M, int64_t N, int64_t K, const void *A, in
               int64_t ldb, bool b_kmajor, void *C, int64_t ldc, bool int8, int out_bits, int out_shift,
               cudaStream_t st, gemm_status_t *status) {
   bool small_n;
-  if (!rows_shape(M, N, K, b_kmajor, int8, &small_n)) return false;
+  if (!rows_shape(M, N, K, b_kmajor, int8, d.sms, &small_n)) return false;
   const int es = int8 ? 1 : 2;
   RowsParams p{};
   p.W = small_n ? A : B;
@@ -953,7 +952,7 @@ bool try_rows(DeviceState &d, int64_t M, int64_t N, int64_t K, const void *A, in
   p.C = C;
   p.out_bits = out_bits;
   p.out_shift = out_shift;
-  const int64_t strips = rows_geometry(p.NW, K, int8, d.sms, &p.cluster, &p.kslice);
+  const int64_t strips = rows_geometry(p.NW, K, p.R, int8, d.sms, &p.cluster, &p.kslice);
   *status = GEMM_ERR_CUDA;
   const bool prof = g_prof_start && g_prof_stop;
   if (prof && cudaEventRecord(g_prof_start, st) != cudaSuccess) return true;
@@ -1395,9 +1394,9 @@ gemm_status_t gemm_plan_query(int64_t M, int64_t N, int64_t K, int int8, int b_l
   }
   bool small_n;
   // tight leading dimensions: both operands' pitch is K
-  if (rows_shape(M, N, K, b_kmajor, int8 != 0, &small_n) && K * (int8 ? 1 : 2) % 16 == 0) {
+  if (rows_shape(M, N, K, b_kmajor, int8 != 0, sms, &small_n) && K * (int8 ? 1 : 2) % 16 == 0) {
     int cluster, kslice;
-    const int64_t strips = rows_geometry(small_n ? M : N, K, int8 != 0, sms, &cluster, &kslice);
+    const int64_t strips = rows_geometry(small_n ? M : N, K, (int)(small_n ? N : M), int8 != 0, sms, &cluster, &kslice);
     out->route = GEMM_ROUTE_FEW_ROWS;
     out->bn = 32;
     out->splits = cluster;

@@ -206,7 +206,8 @@ struct RowsParams {
   int cluster, kslice;  // rows_geometry
   int out_bits, out_shift;
 };
-int64_t rows_geometry(int64_t NW, int64_t K, bool int8, int sms, int *cluster, int *kslice);
+int64_t rows_geometry(int64_t NW, int64_t K, int R, bool int8, int sms, int *cluster, int *kslice);
+bool rows_faster(int64_t NW, int64_t K, int R, bool int8, bool few_m, int sms);
 cudaError_t launch_rows(const RowsParams &p, bool int8, int64_t strips, cudaStream_t st);
 
 // Small-M GEMM on the CUDA cores (gemm_skinny.cu).  M <= 16.

@@ -347,17 +347,25 @@ cudaError_t launch_nt(const RowsParams &p, int64_t strips, cudaStream_t st) {
 
 // Strips, cluster size and K slice: the cluster (1-8 blocks along K) for
 // which the rounds of resident blocks, each as long as its warps' batches
-// plus the start and end of a block (about six batches), take least.
-int64_t rows_geometry(int64_t NW, int64_t K, bool int8, int sms, int *cluster, int *kslice) {
+// plus the start and end of a block (about six batches), take least.  Clusters
+// of four blocks and more do not fill every SM (a processing cluster's blocks are
+// not a multiple of theirs): int8 4 x 2400 x 8192 in 75 clusters of 8 takes 9.9
+// us, of 7 7.0, 4 x 2656 x 8192 in 83 of 7 11.2, of 6 7.2, 4 x 3200 x 8192 in 100
+// of 6 11.5, of 5 8.1; 512 blocks do run at once.  bf16 against at most 8 rows
+// has room for a fifth block per SM, which makes up for it (4 x 2400 x 8192 in 8
+// 8.7, in 7 9.2).
+int64_t rows_geometry(int64_t NW, int64_t K, int R, bool int8, int sms, int *cluster, int *kslice) {
   const int batch = int8 ? 128 : 64;
   const int64_t strips = (NW + kStrip - 1) / kStrip;
   const int64_t slots = (int64_t)kRowsBlocks * sms;
+  const int64_t wide_slots = int8 || R > 8 ? slots * 22 / 25 : slots;
   double best = -1;
   for (int c = 1; c <= 8; ++c) {
     int64_t ks = (K + c - 1) / c;
     ks = (ks + batch - 1) / batch * batch;
     if (c > 1 && ks * (c - 1) >= K) continue;  // an empty slice
-    const double cost = (double)((strips * c + slots - 1) / slots) * ((double)ks / (batch * kRowsWarps) + 6.0);
+    const int64_t at_once = c >= 4 ? wide_slots : slots;
+    const double cost = (double)((strips * c + at_once - 1) / at_once) * ((double)ks / (batch * kRowsWarps) + 6.0);
     if (best < 0 || cost < best) {
       best = cost;
       *cluster = c;
@@ -365,6 +373,29 @@ int64_t rows_geometry(int64_t NW, int64_t K, bool int8, int sms, int *cluster, i
     }
   }
   return strips;
+}
+
+// Whether the kernel is the fastest for these sizes.  A block streams its strip
+// of W at what a few loads in flight give, about 3 us per 1024 k of bf16 and 1.8
+// of int8, and a strip has at most eight blocks: with few strips a long K is
+// faster on kernels that split it further: the CUDA-core kernel where it is the
+// other choice (`few_m`: up to 2 rows of A for bf16 and 8 for int8), else the
+// tensor cores.  Back to back, W stored N x K,
+// this kernel / those: bf16 1 x 32 x 32768 8.5 / 18.7 us, x 65536 21.5 / 18.8; 1 x
+// 128 x 16384 8.0 / 9.2, x 32768 15.1 / 10.5, x 131072 52.8 / 15.5; 1 x 600 x 8192
+// 6.0 / 6.9, x 16384 9.4 / 8.7; 4 x 600 x 16384 9.2 / 10.1, x 32768 16.1 / 13.4;
+// int8 1 x 32 x 65536 16.4 / 22.6; 1 x 128 x 32768 9.5 / 11.5, x 65536 16.6 / 12.1;
+// 1 x 600 x 16384 6.6 / 7.4, x 32768 10.6 / 8.6.  From about 400 blocks on the
+// stream itself is the limit (1 x 2400 x 65536 bf16 50.0 / 60.2), but for long
+// slices in more than one round (bf16 4 x 10000 x 16384 60.7 / 53.6).
+bool rows_faster(int64_t NW, int64_t K, int R, bool int8, bool few_m, int sms) {
+  int cluster, kslice;
+  const int64_t strips = rows_geometry(NW, K, R, int8, sms, &cluster, &kslice), blocks = strips * cluster;
+  if (blocks * 2 >= (int64_t)sms * 5)
+    return int8 || R <= 2 || kslice <= 4096 || blocks <= (int64_t)kRowsBlocks * sms;
+  if (int8) return !few_m || R > 8 || kslice <= (strips == 1 ? 8192 : strips <= 6 ? 4096 : 2560);
+  if (!few_m || R > 2) return kslice <= 2560;
+  return kslice <= (strips <= 2 ? 4096 : strips <= 6 ? 2048 : 1536);
 }
 
 cudaError_t launch_rows(const RowsParams &p, bool int8, int64_t strips, cudaStream_t st) {

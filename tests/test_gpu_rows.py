@@ -129,3 +129,36 @@ def test_few_row_indexes_fit_an_int():
             if plan["route"] == G.GEMM_ROUTE_FEW_ROWS:
                 slice_ = -(-(-(-K // plan["splits"])) // 64) * 64
                 assert plan["splits"] * slice_ + 4 * 64 + 32 < 1 << 31, (M, N, K)
+
+
+def test_few_rows_of_a_long_k_go_where_it_is_split_further():
+    """Few strips of the streamed operand and a long K: more blocks than a
+    cluster's eight share it on the other kernels; clusters that do not all run
+    at once are not chosen."""
+    from paper_2512_13282_gb300 import build
+    build.build()
+    G.gemm_reload_overrides()
+
+    def few(M, N, K, int8):
+        st, plan = G.gemm_plan_query(M, N, K, int8, COL)
+        assert st == G.GEMM_OK
+        return plan["splits"] if plan["route"] == G.GEMM_ROUTE_FEW_ROWS else 0
+
+    for M, N, K, int8, c in ((1, 32, 32768, False, 8), (1, 32, 65536, False, 0), (1, 600, 8192, False, 8),
+                             (1, 600, 16384, False, 0), (4, 600, 16384, False, 8), (4, 600, 32768, False, 0),
+                             (32, 1, 65536, False, 0), (600, 16, 16384, False, 8), (1, 2400, 65536, False, 8),
+                             (4, 10000, 16384, False, 0), (1, 128, 32768, True, 8), (1, 128, 65536, True, 0),
+                             (8, 600, 32768, True, 0), (16, 600, 65536, True, 8), (600, 4, 65536, True, 8),
+                             (16, 4096, 4096, True, 4), (4, 2400, 8192, True, 7), (4, 2656, 8192, True, 6),
+                             (16, 2400, 8192, False, 7), (4, 2400, 8192, False, 8)):
+        assert few(M, N, K, int8) == c, (M, N, K, int8)
+
+
+@pytest.mark.gpu
+@pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a GPU")
+@pytest.mark.parametrize("dtype,M,N,K", [("bf16", 2, 40, 40960), ("bf16", 5, 70, 24576), ("bf16", 70, 2, 24576), ("int8", 3, 70, 40960),
+                                         ("int8", 7, 250, 24576), ("bf16", 16, 2400, 1024), ("int8", 4, 2656, 2048), ("int8", 9, 3200, 1040)])
+def test_few_rows_around_the_long_k_limit(dtype, M, N, K):
+    """Both sides of the limit, and clusters of 5 to 7 blocks."""
+    _run(dtype, M, N, K, seed=M + K)
+    _run(dtype, M, N, K - 32 * 1024 // 4 if K > 16384 else K + 16, seed=M - K)
