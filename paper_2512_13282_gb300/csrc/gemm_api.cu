@@ -840,23 +840,35 @@ constexpr int64_t kSkinnyMaxM = 8;  // the largest limit below
 // Largest M sent to the CUDA-core small-M kernel: there every B element is
 // used at most a few times and streaming B once is the cost.  bf16,
 // accumulating with fp32 FMAs, wins up to M = 2 (measured on GB300 against
-// the tensor-core path, N = 4096..11008, K = 4096); int8, through dp4a, up to
-// M = 8 where the alternative stages a small B (2003 x 3001 stored N x K: M = 8
-// 18.0 / 20.2 us; stored K x N: M = 3 18.6 / 19.6, M = 8 26.9 / 19.8), or up
-// to M = 2 for a larger one (5001 x 5001: M = 2 30.7 / 30.5 and 26.7 / 30.5,
-// M = 3 33.9 / 32.1 and 38.9 / 32.2).  Where the small-operand kernel can
-// read a row-major B as it is (`in_place`), that kernel is faster from M = 2
-// on (K = 4096, back to back: M = 1 x 4096 8.4 / 9.7 us, 2 x 4096 11.0 /
-// 9.7, 4 x 4096 12.9 / 9.8, 8 x 4096 18.1 / 9.9, 4 x 12288 24.1 / 17.0),
-// except M = 2 with a small B (2 x 1024 x 1024 5.9 / 6.2) or a wide one (2 x
-// 12288 16.4 / 17.0).  GB300_GEMM_SKINNY_MAX_M overrides (0 disables the
-// kernel).
-int skinny_max_m(bool int8, int64_t N, int64_t K, bool b_kmajor, bool in_place) {
+// the tensor-core path, N = 4096..11008, K = 4096).  int8, through dp4a, has two
+// alternatives (back to back, this kernel / that):
+//   - B would be staged.  Stored N x K: up to M = 8 (2003 x 3001 M = 8 13.3 /
+//     22.3 us, 12289 x 4097 M = 3 30.6 / 54.3, M = 8 47.0 / 58.7, 20001 x 20001 M
+//     = 3 163 / 347).  Stored K x N: up to M = 3 for a small B (2003 x 3001 16.2 /
+//     21.9) and 2 for a larger one (5001 x 5001 M = 2 25.4 / 36.1, M = 3 40.7 /
+//     35.2), but further for a few columns and a K to split (M = 4: 5 x 700 6.9 /
+//     8.1, 33 x 1500 9.4 / 11.2; M = 8: 17 x 3001 10.5 / 12.9).
+//   - the small-operand kernel reads a row-major B as it is (`in_place`): with
+//     int32 outputs that is faster from M = 2 on (M = 1 x 4096 x 4096 8.4 / 9.7
+//     us, 2 x 4096 11.0 / 9.7, 8 x 4096 18.1 / 9.9), except M = 2 with a small B
+//     (2 x 1024 x 1024 5.9 / 6.2) or a wide one (2 x 12288 x 4096 16.4 / 17.0).
+//     Narrow outputs cost it a reduction launch: from M = 3 on (2 x 4096 x 4096
+//     11.9 / 12.9, 2 x 8192 x 8192 20.0 / 29.2, 3 x 4096 x 4096 13.3 / 12.9), a
+//     short K from 4 or 7 on (3 x 4096 x 1024 8.8 / 9.4, 6 x 1024 x 1024 8.4 / 9.0),
+//     a large B from 4 (3 x 8192 x 8192 26.3 / 29.1, 3 x 16384 x 8192 44.9 / 37.0).
+// GB300_GEMM_SKINNY_MAX_M overrides (0 disables the kernel).
+int skinny_max_m(bool int8, int64_t N, int64_t K, bool b_kmajor, bool in_place, int out_bits) {
   const int v = overrides().skinny_max_m;
   if (v >= 0) return v > 16 ? 16 : v;
   if (!int8) return 2;
-  if (!in_place) return N * K > (int64_t(1) << 23) ? 2 : (b_kmajor ? 8 : 3);
-  return N >= 8192 || N * K < (int64_t(1) << 22) ? 2 : 1;
+  if (!in_place) {
+    if (b_kmajor || (N <= 48 && K >= 2048)) return 8;
+    if (N <= 8 || (N <= 48 && K >= 1024)) return 4;
+    return N * K > (int64_t(1) << 23) ? 2 : 3;
+  }
+  if (out_bits == 32) return N >= 8192 || N * K < (int64_t(1) << 22) ? 2 : 1;
+  if (K <= 1024) return N <= 2048 ? 6 : 3;
+  return K >= 8192 && N <= 8192 ? 3 : 2;
 }
 
 gemm_status_t run_skinny(DeviceState &d, int64_t M, int64_t N, int64_t K, const void *A, int64_t lda,
@@ -986,7 +998,7 @@ gemm_status_t gemm_bf16_f32acc_bf16(int64_t M, int64_t N, int64_t K, const uint1
   }
   const bool b_kmajor = b_layout == GEMM_B_COL_MAJOR_NxK;
   if (try_rows(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, false, 0, 0, st, &s)) return s;
-  if (M <= skinny_max_m(false, N, K, b_kmajor, false))
+  if (M <= skinny_max_m(false, N, K, b_kmajor, false, 16))
     return run_skinny(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, false, st);
   Plan pl = make_plan(M, N, K, b_kmajor, kEpiBf16, d->sms, pair_slots());
   // TMA needs 16-byte aligned bases and row pitches; re-pitch an operand
@@ -1250,7 +1262,7 @@ gemm_status_t s8_gemm(int64_t M, int64_t N, int64_t K, const int8_t *A, int64_t 
   const bool b_kmajor = b_layout == GEMM_B_COL_MAJOR_NxK;
   if (try_rows(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, true, out_bits, shift, st, &s)) return s;
   const bool in_place = overrides().s8tm && !b_kmajor && N > kBM && aligned16(B) && ldb % 16 == 0;
-  if (M <= skinny_max_m(true, N, K, b_kmajor, in_place))
+  if (M <= skinny_max_m(true, N, K, b_kmajor, in_place, out_bits))
     return run_skinny(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, true, st, out_bits, shift);
   auto run_tiny = [&]() -> gemm_status_t {
     const TinyParams tp{A, lda, B, ldb, C, ldc, M, N, K, out_bits, shift};
@@ -1404,7 +1416,7 @@ gemm_status_t gemm_plan_query(int64_t M, int64_t N, int64_t K, int int8, int b_l
     return GEMM_OK;
   }
   const bool in_place = overrides().s8tm && !b_kmajor && N > kBM && N % 16 == 0;
-  if (M <= skinny_max_m(int8 != 0, N, K, b_kmajor, in_place)) {
+  if (M <= skinny_max_m(int8 != 0, N, K, b_kmajor, in_place, 32)) {
     out->route = GEMM_ROUTE_SMALL_M;
     return GEMM_OK;
   }

@@ -256,3 +256,35 @@ def test_small_m_kernel_at_the_shared_memory_limit(monkeypatch, K):
     N = 32 * 608
     A, B = _operands("bf16", 12, N, K, COL, K)
     _check("bf16", A, B, COL, U.run("bf16", A, B, COL))
+
+
+def test_small_m_limits():
+    """The CUDA-core kernel keeps a B that the others would have to stage."""
+    from paper_2512_13282_gb300 import build
+    build.build()
+    G.gemm_reload_overrides()
+
+    def small(M, N, K, layout):
+        st, plan = G.gemm_plan_query(M, N, K, True, layout)
+        assert st == G.GEMM_OK
+        return plan["route"] == G.GEMM_ROUTE_SMALL_M
+
+    assert all(small(m, n, k, COL) for m in (3, 8) for n, k in ((12289, 4097), (9001, 16385), (20001, 20001)))
+    assert [small(m, 5001, 5001, ROW) for m in (2, 3)] == [True, False]
+    assert [small(m, 5, 700, ROW) for m in (4, 5)] == [True, False] and small(4, 33, 1500, ROW)
+    assert small(8, 17, 3001, ROW) and not small(8, 65, 3001, ROW)
+
+
+@pytest.mark.gpu
+@needs_gpu
+@pytest.mark.parametrize("dtype", ["int8", "int8_int16", "int8_int8"])
+@pytest.mark.parametrize("M,N,K,layout", [(8, 301, 4097, COL), (3, 4099, 2049, COL), (4, 5, 700, ROW), (8, 17, 3001, ROW), (4, 33, 1500, ROW),
+                                          (2, 4096, 2048, ROW), (3, 2064, 1024, ROW), (4, 2064, 1024, ROW), (6, 1024, 1024, ROW),
+                                          (7, 1024, 1024, ROW), (3, 1040, 8192, ROW)])
+def test_small_m_limits_results(dtype, M, N, K, layout):
+    A, B = _operands("int8", M, N, K, layout, M + N)
+    C = U.run(dtype, A, B, layout, shift=10)
+    want = oracle.gemm_s8(A, B, layout)
+    if dtype != "int8":
+        want = oracle.requantize(want, 10, 16 if dtype == "int8_int16" else 8)
+    assert np.array_equal(C.astype(np.int64), want)
