@@ -812,8 +812,16 @@ gemm_status_t run_tc(DeviceState &d, Plan &pl, const uint16_t *A, int64_t lda, c
 // Measured on GB300 against the tensor-core routes, back to back: 128^3 3.2 /
 // 5.3 us, 256^3 5.1 / 6.6, 300^3 (odd pitch) 7.7-8.8 / 8.2, 384^3 9.8 / 7.0,
 // 512^3 9.6 / 6.5, 32 x 1024 x 1024 8.7 / 6.3, 128 x 128 x 4096 31 / 9.0.
+// Two kinds of larger problem stay with it: those of one short round of tiles
+// (128 x 512 x 512 5.3 / 8.6, 64 x 1024 x 512 5.3 / 7.5), and those with an
+// operand or C off the 16-byte grid, which the others stage and store more slowly
+// (640 x 89 x 416 8.3 / 11.2, 500 x 500 x 200 int8 outputs 6.6 / 10.9, 511 x 511 x
+// 129 7.7 / 11.0, x 400 11.1 / 12.5, x 511 14.5 / 12.5; 1023 x 511 x 90 8.1 / 11.1,
+// 4001 x 131 x 127 12.3 / 11.1).
 constexpr int64_t kTinyMaxMacs = int64_t(1) << 24;  // 256^3
 constexpr int64_t kTinyMaxK = 512;
+constexpr int64_t kTinyShortTiles = 64;                                             // 32 x 32 tiles
+constexpr int64_t kTinyMaxMacsOdd = int64_t(3) << 25, kTinyMaxTilesOdd = 512;
 // With the small-M limit forced (GB300_GEMM_SKINNY_MAX_M), or no workspace for
 // another kernel, the tile kernel takes problems by their multiply-adds alone,
 // up to 512^3.
@@ -825,14 +833,18 @@ bool default_routes() {
   return o.bn <= 0 && o.pair < 0 && o.splits < 1 && o.tail_splits < 2 && o.tiny_max_macs < 0 && o.skinny_max_m < 0;
 }
 
-bool tiny_shape(int64_t M, int64_t N, int64_t K) {
+// `odd`: an operand or C does not start each row on a 16-byte boundary.
+bool tiny_shape(int64_t M, int64_t N, int64_t K, bool odd) {
   const Overrides &o = overrides();
   // a forced tile width, family or split asks for the tensor-core kernels
   if (o.bn > 0 || o.pair >= 0 || o.splits >= 1 || o.tail_splits >= 2) return false;
   const double macs = (double)M * (double)N * (double)K;
   if (o.tiny_max_macs >= 0) return macs <= (double)o.tiny_max_macs;
   if (o.skinny_max_m >= 0) return macs <= (double)kTinyMaxMacsForced;
-  return macs <= (double)kTinyMaxMacs && K <= kTinyMaxK;
+  if (K > kTinyMaxK) return false;
+  const double tiles = (double)ceil_div(M, (int64_t)32) * (double)ceil_div(N, (int64_t)32);
+  return macs <= (double)kTinyMaxMacs || tiles <= (double)kTinyShortTiles ||
+         (odd && macs <= (double)kTinyMaxMacsOdd && tiles <= (double)kTinyMaxTilesOdd);
 }
 
 constexpr int64_t kSkinnyMaxM = 8;  // the largest limit below
@@ -1273,7 +1285,9 @@ gemm_status_t s8_gemm(int64_t M, int64_t N, int64_t K, const int8_t *A, int64_t 
     if (prof && cudaEventRecord(g_prof_stop, st) != cudaSuccess) return GEMM_ERR_CUDA;
     return GEMM_OK;
   };
-  if (tiny_shape(M, N, K)) return run_tiny();
+  const int64_t es_c = out_bits / 8;
+  const bool odd = !aligned16(A) || !aligned16(B) || !aligned16(C) || (lda | ldb | (ldc * es_c)) % 16 != 0;
+  if (tiny_shape(M, N, K, odd)) return run_tiny();
   // A call being captured into a graph on a stream whose workspace is too
   // small for its kernel: the CUDA-core kernels, slower there, need little or
   // none, so small problems can be captured on a stream that has run nothing.
@@ -1420,7 +1434,8 @@ gemm_status_t gemm_plan_query(int64_t M, int64_t N, int64_t K, int int8, int b_l
     out->route = GEMM_ROUTE_SMALL_M;
     return GEMM_OK;
   }
-  if (int8 && tiny_shape(M, N, K)) {
+  const bool odd = (K | (b_kmajor ? K : N) | (N * 4)) % 16 != 0;  // tight leading dimensions, int32 C
+  if (int8 && tiny_shape(M, N, K, odd)) {
     out->route = GEMM_ROUTE_TINY;
     out->bn = 32;
     out->splits = 1;

@@ -288,3 +288,34 @@ def test_small_m_limits_results(dtype, M, N, K, layout):
     if dtype != "int8":
         want = oracle.requantize(want, 10, 16 if dtype == "int8_int16" else 8)
     assert np.array_equal(C.astype(np.int64), want)
+
+
+def test_tiny_limits():
+    """The one-launch kernel beyond 2^24 multiply-adds: a short round of tiles, or
+    rows off the 16-byte grid."""
+    from paper_2512_13282_gb300 import build
+    build.build()
+    G.gemm_reload_overrides()
+
+    def tiny(M, N, K, layout=ROW):
+        st, plan = G.gemm_plan_query(M, N, K, True, layout)
+        assert st == G.GEMM_OK
+        return plan["route"] == G.GEMM_ROUTE_TINY
+
+    assert tiny(128, 512, 512) and tiny(64, 1024, 512) and not tiny(64, 1040, 512) and not tiny(128, 512, 528)
+    assert tiny(640, 89, 416) and tiny(511, 511, 129, COL) and tiny(511, 511, 385) and not tiny(511, 511, 386)
+    assert tiny(1023, 511, 90) and not tiny(1025, 511, 90) and not tiny(1024, 512, 96) and not tiny(4001, 131, 127)
+
+
+@pytest.mark.gpu
+@needs_gpu
+@pytest.mark.parametrize("dtype", ["int8", "int8_int16", "int8_int8"])
+@pytest.mark.parametrize("M,N,K,layout,pad,off", [(128, 512, 512, ROW, 0, 0), (640, 89, 416, COL, 0, 0), (511, 511, 385, ROW, 0, 1),
+                                                  (1023, 511, 90, COL, 1, 3), (512, 512, 128, ROW, 4, 0), (512, 512, 384, ROW, 0, 0)])
+def test_tiny_limits_results(dtype, M, N, K, layout, pad, off):
+    A, B = _operands("int8", M, N, K, layout, M + N)
+    C = U.run(dtype, A, B, layout, lda=K + pad, ldb=B.shape[1] + pad, ldc=N + pad, a_off=off, c_off=off, shift=8)
+    want = oracle.gemm_s8(A, B, layout)
+    if dtype != "int8":
+        want = oracle.requantize(want, 8, 16 if dtype == "int8_int16" else 8)
+    assert np.array_equal(C.astype(np.int64), want)
