@@ -35,10 +35,12 @@
  *   - CUDA graphs: calls may be captured on a stream that has already run,
  *     outside capture, calls needing at least as much scratch (the same
  *     shapes, say); a captured call that would need more runs without it
- *     where a slower kernel can (bf16 on aligned operands, int8 up to
- *     512^3), else it returns GEMM_ERR_UNSUPPORTED before enqueuing anything.  Scratch that a graph
- *     refers to stays allocated until gemm_release_resources(), after which
- *     graphs captured before must not be launched.
+ *     where a slower kernel can (bf16 on operands with 16-byte aligned bases
+ *     and pitches, int8 up to 2^27 multiply-adds), unless an override below
+ *     asks for a particular kernel; else it returns GEMM_ERR_UNSUPPORTED
+ *     before enqueuing anything.  Scratch that a graph refers to stays
+ *     allocated until gemm_release_resources(), after which graphs captured
+ *     before must not be launched.
  *   - Environment variables that override the planner, for tests and
  *     benchmarks (int8 results are identical either way; bf16 results may
  *     differ in summation order, within the same accuracy): GB300_GEMM_BN,

@@ -1010,8 +1010,12 @@ gemm_status_t gemm_bf16_f32acc_bf16(int64_t M, int64_t N, int64_t K, const uint1
   }
   const bool b_kmajor = b_layout == GEMM_B_COL_MAJOR_NxK;
   if (try_rows(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, false, 0, 0, st, &s)) return s;
-  if (M <= skinny_max_m(false, N, K, b_kmajor, false, 16))
-    return run_skinny(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, false, st);
+  if (M <= skinny_max_m(false, N, K, b_kmajor, false, 16)) {
+    s = run_skinny(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, false, st);
+    // no scratch for its partials inside a capture: the tensor-core kernels need
+    // none for aligned operands
+    if (s != GEMM_ERR_UNSUPPORTED || !default_routes()) return s;
+  }
   Plan pl = make_plan(M, N, K, b_kmajor, kEpiBf16, d->sms, pair_slots());
   // TMA needs 16-byte aligned bases and row pitches; re-pitch an operand
   // that is not, into the workspace.
@@ -1273,9 +1277,6 @@ gemm_status_t s8_gemm(int64_t M, int64_t N, int64_t K, const int8_t *A, int64_t 
   }
   const bool b_kmajor = b_layout == GEMM_B_COL_MAJOR_NxK;
   if (try_rows(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, true, out_bits, shift, st, &s)) return s;
-  const bool in_place = overrides().s8tm && !b_kmajor && N > kBM && aligned16(B) && ldb % 16 == 0;
-  if (M <= skinny_max_m(true, N, K, b_kmajor, in_place, out_bits))
-    return run_skinny(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, true, st, out_bits, shift);
   auto run_tiny = [&]() -> gemm_status_t {
     const TinyParams tp{A, lda, B, ldb, C, ldc, M, N, K, out_bits, shift};
     const bool prof = g_prof_start && g_prof_stop;
@@ -1285,20 +1286,28 @@ gemm_status_t s8_gemm(int64_t M, int64_t N, int64_t K, const int8_t *A, int64_t 
     if (prof && cudaEventRecord(g_prof_stop, st) != cudaSuccess) return GEMM_ERR_CUDA;
     return GEMM_OK;
   };
+  // A call being captured into a graph on a stream whose scratch is too small
+  // for its kernel (UNSUPPORTED, with nothing enqueued): the CUDA-core kernels,
+  // slower there, need less or none, so small problems can be captured on a
+  // stream that has run nothing.
+  auto without_scratch = [&](bool try_small_m) -> gemm_status_t {
+    if (!default_routes()) return GEMM_ERR_UNSUPPORTED;
+    if (try_small_m && M <= kSkinnyMaxM) {
+      const gemm_status_t r = run_skinny(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, true, st, out_bits, shift);
+      if (r != GEMM_ERR_UNSUPPORTED) return r;
+    }
+    return (double)M * (double)N * (double)K <= (double)kTinyMaxMacsForced ? run_tiny() : GEMM_ERR_UNSUPPORTED;
+  };
+  const bool in_place = overrides().s8tm && !b_kmajor && N > kBM && aligned16(B) && ldb % 16 == 0;
+  if (M <= skinny_max_m(true, N, K, b_kmajor, in_place, out_bits)) {
+    s = run_skinny(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, true, st, out_bits, shift);
+    return s == GEMM_ERR_UNSUPPORTED ? without_scratch(false) : s;
+  }
   const int64_t es_c = out_bits / 8;
   const bool odd = !aligned16(A) || !aligned16(B) || !aligned16(C) || (lda | ldb | (ldc * es_c)) % 16 != 0;
   if (tiny_shape(M, N, K, odd)) return run_tiny();
-  // A call being captured into a graph on a stream whose workspace is too
-  // small for its kernel: the CUDA-core kernels, slower there, need little or
-  // none, so small problems can be captured on a stream that has run nothing.
-  auto without_scratch = [&]() -> gemm_status_t {
-    if (!default_routes()) return GEMM_ERR_UNSUPPORTED;
-    if (M <= kSkinnyMaxM)
-      return run_skinny(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, true, st, out_bits, shift);
-    return (double)M * (double)N * (double)K <= (double)kTinyMaxMacsForced ? run_tiny() : GEMM_ERR_UNSUPPORTED;
-  };
   if (try_s8tm(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, out_bits, shift, st, &s))
-    return s == GEMM_ERR_UNSUPPORTED ? without_scratch() : s;
+    return s == GEMM_ERR_UNSUPPORTED ? without_scratch(true) : s;
   Plan pl = make_plan(M, N, K, b_kmajor, kEpiS32, d->sms, pair_slots());
   pl.p.out_bits = out_bits;
   pl.p.out_shift = shift;
@@ -1312,7 +1321,7 @@ gemm_status_t s8_gemm(int64_t M, int64_t N, int64_t K, const int8_t *A, int64_t 
   L.b_off = off;
   off = align_up(off + (size_t)b_rows * ldb_p * 2, 256);
   if ((s = plan_workspace(&pl, &L, off, b_kmajor, *d, st)) != GEMM_OK)
-    return s == GEMM_ERR_UNSUPPORTED ? without_scratch() : s;
+    return s == GEMM_ERR_UNSUPPORTED ? without_scratch(true) : s;
   uint8_t *ws = static_cast<uint8_t *>(scratch_ws());
   uint16_t *Ab = reinterpret_cast<uint16_t *>(ws + L.a_off);
   uint16_t *Bb = reinterpret_cast<uint16_t *>(ws + L.b_off);

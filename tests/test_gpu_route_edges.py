@@ -319,3 +319,13 @@ def test_tiny_limits_results(dtype, M, N, K, layout, pad, off):
     if dtype != "int8":
         want = oracle.requantize(want, 8, 16 if dtype == "int8_int16" else 8)
     assert np.array_equal(C.astype(np.int64), want)
+
+
+# ... whose kernel for few rows would keep K-slice partials and counters
+@pytest.mark.gpu
+@needs_gpu
+@pytest.mark.parametrize("dtype,M,N,K,layout", [
+    ("int8", 6, 4096, 1024, ROW), ("int8", 1, 4096, 4096, ROW), ("int8", 3, 4099, 4099, COL), ("int8", 8, 17, 3001, ROW),
+    ("bf16", 2, 4096, 4096, ROW), ("bf16", 1, 1024, 8192, ROW), ("bf16", 1, 64, 65536, COL), ("bf16", 5, 600, 32768, COL)])
+def test_captured_few_rows_on_a_stream_without_scratch(dtype, M, N, K, layout):
+    test_captured_on_a_stream_without_scratch(dtype, M, N, K, layout)
