@@ -538,11 +538,25 @@ Plan search_plan(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sm
   const Overrides &ovr = overrides();
   const int64_t num_kb = ceil_div(K, kBK);
   // bf16: the K ranges come from a table of their own (range_table.h), so that
-  // the costs a plan is ranked by never change what a sum rounds to.
+  // the costs a plan is ranked by never change what a sum rounds to.  Which tiles
+  // a split tail covers depends on the tile, so that a plan with one stands as it
+  // is, and no other gets one.
   int64_t ranges = 0;
-  if (epi == kEpiBf16 && ovr.splits < 1)
-    ranges = best_choice(M, N, K, b_kmajor, epi, sms, pairs, Partials::kAny, kRangeCosts, 0).splits;
-  Choice best = best_choice(M, N, K, b_kmajor, epi, sms, pairs, partials, kPlanCosts, ranges);
+  Choice best;
+  if (epi == kEpiBf16 && ovr.splits < 1) {
+    best = best_choice(M, N, K, b_kmajor, epi, sms, pairs, Partials::kAny, kRangeCosts, 0);
+    ranges = best.splits;
+    if (partials == Partials::kAny) partials = Partials::kNoTail;
+    else best.tail_splits = 0;
+  }
+  if (best.tail_splits > 0) {
+    const int64_t slots = best.pair ? pairs : sms, rows = best.pair ? 2 * kBM : kBM;
+    const int64_t tiles = ceil_div(M, rows) * ceil_div(N, (int64_t)best.bn), full = tiles / slots;
+    best.model_us = modelled_us(kPlanCosts, false, best.pair, best.bn, full * num_kb + best.kb_tail, full + 1,
+                                4e-6 * (double)(best.tail_splits * (tiles - full * slots) * rows * best.bn));
+  } else {
+    best = best_choice(M, N, K, b_kmajor, epi, sms, pairs, partials, kPlanCosts, ranges);
+  }
   if (!best.found && ranges > 1) {  // a forced tile without a variant that sums ranges in registers, and no partials
     ranges = 0;
     best = best_choice(M, N, K, b_kmajor, epi, sms, pairs, partials, kPlanCosts, 0);

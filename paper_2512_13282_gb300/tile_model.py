@@ -317,24 +317,33 @@ def rank_us(M, N, K, dtype, plan, table):
     return plan_cost_us(M, N, K, dtype, plan, table) + table.get("mem_weight", 0.0) * mem_time_us(M, N, K, dtype, plan)
 
 
+def range_plan(M, N, K, b_kmajor, sms=None, pair_slots=None):
+    """The plan whose K ranges (splits, or split tail) a bf16 GEMM is summed
+    in: the one of least rank_us by the costs fixed in csrc/range_table.h,
+    whatever costs the kernel is then chosen by."""
+    return _least(M, N, K, "bf16", candidate_plans(M, N, K, "bf16", b_kmajor, sms, pair_slots), _range_table())
+
+
 def sum_ranges(M, N, K, b_kmajor, sms=None, pair_slots=None):
-    """The K ranges a bf16 GEMM is summed in (csrc/range_table.h): the split
-    of the plan of least rank_us by the costs fixed there, whatever costs the
-    kernel is then chosen by."""
-    return _least(M, N, K, "bf16", candidate_plans(M, N, K, "bf16", b_kmajor, sms, pair_slots), _range_table())["splits"]
+    """The K ranges of a bf16 GEMM's sums (of those outside a split tail)."""
+    return range_plan(M, N, K, b_kmajor, sms, pair_slots)["splits"]
 
 
 def choose_plan(M, N, K, dtype, b_kmajor, table, sms=None, pair_slots=None):
     """The planner: the candidate of least rank_us (the first one, in
-    candidate order, on a tie).  bf16: of those that sum K in sum_ranges
-    ranges, as splits or, unsplit on tiles of at most MAX_SLAB_BN columns, in
-    registers (the plan's "slabs")."""
+    candidate order, on a tie).  bf16: range_plan itself where it has a split
+    tail; else of those that sum K in its ranges, as splits or, unsplit on
+    tiles of at most MAX_SLAB_BN columns, in registers (the plan's "slabs")."""
     cands = candidate_plans(M, N, K, dtype, b_kmajor, sms, pair_slots)
     if dtype == "bf16":
-        r = sum_ranges(M, N, K, b_kmajor, sms, pair_slots)
+        rp = range_plan(M, N, K, b_kmajor, sms, pair_slots)
+        if rp["tail_splits"]:
+            return rp
+        cands = [p for p in cands if not p["tail_splits"]]
+        r = rp["splits"]
         if r > 1:
             cands = [p if p["splits"] == r else dict(p, slabs=r) for p in cands
-                     if p["splits"] == r or (p["splits"] == 1 and not p["tail_splits"] and p["bn"] <= MAX_SLAB_BN)]
+                     if p["splits"] == r or (p["splits"] == 1 and p["bn"] <= MAX_SLAB_BN)]
         else:
             cands = [p for p in cands if p["splits"] == 1]
     return _least(M, N, K, dtype, cands, table)

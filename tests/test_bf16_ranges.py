@@ -65,3 +65,26 @@ def test_ranges_in_registers_equal_split_k(M, N, K, layout, bn, kw, monkeypatch)
     rows = np.arange(M) != M // 2
     ref, mag = oracle.gemm_bf16(A[rows], B, layout)
     assert oracle.bf16_within_bound(C[rows], ref, mag).all()
+
+
+def test_split_tails_are_a_property_of_the_sizes():
+    """A split tail, with the tiles it covers, belongs to the ranges too: it
+    stands as the fixed costs choose it, and no other plan gets one."""
+    from paper_2512_13282_gb300 import build
+    build.build()
+    G.gemm_reload_overrides()
+    for M, N, K, layout, bn, pair, tails in ((1072, 4848, 6800, COL, 256, True, 4), (8192, 1072, 4304, COL, 256, True, 5),
+                                             (992, 7632, 8000, ROW, None, None, 0)):
+        st, plan = G.gemm_plan_query(M, N, K, False, layout)
+        assert st == G.GEMM_OK and plan["tail_splits"] == tails
+        if tails:
+            assert plan["bn"] == bn and (plan["route"] == G.GEMM_ROUTE_TC_PAIR) == pair
+    rng = random.Random(4)
+    for _ in range(400):
+        M, N, K = (int(2 ** rng.uniform(9, 13)) for _ in range(3))
+        layout = rng.randint(0, 1)
+        st, plan = G.gemm_plan_query(M, N, K, False, layout)
+        want = T.range_plan(M, N, K, layout == COL)
+        assert st == G.GEMM_OK and plan["tail_splits"] == want["tail_splits"]
+        if want["tail_splits"]:
+            assert (plan["bn"], plan["route"] == G.GEMM_ROUTE_TC_PAIR) == (want["bn"], want["pair"])
