@@ -385,41 +385,34 @@ __global__ void __launch_bounds__(kSkThreads, colb_blocks(MT)) skinny_colB_kerne
       facc[m][j] = 0.f;
       iacc[m][j] = 0;
     }
-  // The 16-byte chunk at k = kk of the warp's four columns.  Aligned rows have
-  // code of their own: the ways that load16_any may take, between the loads of
-  // the four columns, keep them from being in flight together (bf16 1 x 32 x
-  // 32768 27 us with one code for all rows, 18 with two).
-  auto load_chunk = [&](int kk, uint32_t (&w)[kColsPerWarp][4], auto aligned) {
-    constexpr int ES = INT8 ? 1 : 2, kPer = 4 / ES;
+  for (int ch = lane; ch < chunks; ch += 32) {
+    const int kk = ch * kElems;
+    uint32_t w[kColsPerWarp][4];
 #pragma unroll
     for (int j = 0; j < kColsPerWarp; ++j) {
       w[j][0] = w[j][1] = w[j][2] = w[j][3] = 0;
       const int64_t n = n0 + warp * kColsPerWarp + j;
       if (n >= p.N) continue;
-      const uint8_t *row = b_lo + (n * p.ldb + k0 + kk) * ES;
-      if (kk + kElems <= kb) {
-        uint4 v;
-        if constexpr (decltype(aligned)::value)
-          v = __ldcs(reinterpret_cast<const uint4 *>(row));
-        else
-          v = load16_any<true>(row, b_lo, b_hi);
-        w[j][0] = v.x; w[j][1] = v.y; w[j][2] = v.z; w[j][3] = v.w;
+      if (INT8) {
+        const int8_t *row = reinterpret_cast<const int8_t *>(p.B) + n * p.ldb + k0 + kk;
+        if (kk + kElems <= kb) {
+          const uint4 v = load16_any<true>(reinterpret_cast<const uint8_t *>(row), b_lo, b_hi);
+          w[j][0] = v.x; w[j][1] = v.y; w[j][2] = v.z; w[j][3] = v.w;
+        } else {
+          for (int i = 0; i < kElems; ++i)
+            if (kk + i < kb) w[j][i >> 2] |= (uint32_t)(uint8_t)row[i] << (8 * (i & 3));
+        }
       } else {
-        for (int i = 0; i < kElems; ++i)
-          if (kk + i < kb) {
-            const uint32_t e = INT8 ? (uint32_t)row[i] : (uint32_t)reinterpret_cast<const uint16_t *>(row)[i];
-            w[j][i / kPer] |= e << (8 * ES * (i % kPer));
-          }
+        const uint16_t *row = reinterpret_cast<const uint16_t *>(p.B) + n * p.ldb + k0 + kk;
+        if (kk + kElems <= kb) {
+          const uint4 v = load16_any<true>(reinterpret_cast<const uint8_t *>(row), b_lo, b_hi);
+          w[j][0] = v.x; w[j][1] = v.y; w[j][2] = v.z; w[j][3] = v.w;
+        } else {
+          for (int i = 0; i < kElems; ++i)
+            if (kk + i < kb) w[j][i >> 1] |= (uint32_t)row[i] << (16 * (i & 1));
+        }
       }
     }
-  };
-  const bool vec = p.b_align >= 16;
-  for (int ch = lane; ch < chunks; ch += 32) {
-    uint32_t w[kColsPerWarp][4];
-    if (vec)
-      load_chunk(ch * kElems, w, std::true_type{});
-    else
-      load_chunk(ch * kElems, w, std::false_type{});
 #pragma unroll
     for (int m = 0; m < MT; ++m) {
       const uint4 av = *reinterpret_cast<const uint4 *>(&a_s[(m * chunks + ch) * 4]);
