@@ -965,9 +965,11 @@ bool rows_shape(int64_t M, int64_t N, int64_t K, bool b_kmajor, bool int8, int s
 // tensor-core kernels, which re-pitch or stage them (kRowsMaxOddX elements:
 // bf16 16 x 4096 x 4096 12.6 / 13.0 us, 16 x 12288 x 2048 18.7 / 18.5, 16 x
 // 8192 x 4096 20.7 / 16.8, 16 x 12288 x 4096 33.1 / 21.8; int8 10.3 / 10.8,
-// 13.2 / 12.7, 15.0 / 14.3, 21.9 / 16.9).  Returns false, having launched
-// nothing, for any other.
+// 13.2 / 12.7, 15.0 / 14.3, 21.9 / 16.9), and so do long slices of K (int8 13 x
+// 256 x 59712 35.0 / 22.1).  Returns false, having launched nothing, for any
+// other.
 constexpr int64_t kRowsMaxOddX = int64_t(1) << 25;
+constexpr int kRowsMaxSliceOddX = 4096;
 bool try_rows(DeviceState &d, int64_t M, int64_t N, int64_t K, const void *A, int64_t lda, const void *B,
               int64_t ldb, bool b_kmajor, void *C, int64_t ldc, bool int8, int out_bits, int out_shift,
               cudaStream_t st, gemm_status_t *status) {
@@ -991,6 +993,7 @@ bool try_rows(DeviceState &d, int64_t M, int64_t N, int64_t K, const void *A, in
   p.out_bits = out_bits;
   p.out_shift = out_shift;
   const int64_t strips = rows_geometry(p.NW, K, p.R, int8, d.sms, &p.cluster, &p.kslice);
+  if (!p.x_vec && p.R > 8 && p.kslice > kRowsMaxSliceOddX) return false;
   *status = GEMM_ERR_CUDA;
   const bool prof = g_prof_start && g_prof_stop;
   if (prof && cudaEventRecord(g_prof_start, st) != cudaSuccess) return true;

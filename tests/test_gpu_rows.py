@@ -162,3 +162,13 @@ def test_few_rows_around_the_long_k_limit(dtype, M, N, K):
     """Both sides of the limit, and clusters of 5 to 7 blocks."""
     _run(dtype, M, N, K, seed=M + K)
     _run(dtype, M, N, K - 32 * 1024 // 4 if K > 16384 else K + 16, seed=M - K)
+
+
+@pytest.mark.gpu
+@pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a GPU")
+@pytest.mark.parametrize("K", [32768, 40960])
+def test_many_unaligned_rows_of_a_long_k(K):
+    """More than 8 rows off the 16-byte grid: long slices go to other kernels."""
+    before = G.gemm_launch_count()
+    _run("int8", 13, 70, K, seed=K, lda=K + 8)
+    assert (G.gemm_launch_count() - before == 1) == (K == 32768)
