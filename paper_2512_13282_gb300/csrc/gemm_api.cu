@@ -872,8 +872,10 @@ constexpr int64_t kSkinnyMaxM = 8;  // the largest limit below
 //     22.3 us, 12289 x 4097 M = 3 30.6 / 54.3, M = 8 47.0 / 58.7, 20001 x 20001 M
 //     = 3 163 / 347).  Stored K x N: up to M = 3 for a small B (2003 x 3001 16.2 /
 //     21.9) and 2 for a larger one (5001 x 5001 M = 2 25.4 / 36.1, M = 3 40.7 /
-//     35.2), but further for a few columns and a K to split (M = 4: 5 x 700 6.9 /
-//     8.1, 33 x 1500 9.4 / 11.2; M = 8: 17 x 3001 10.5 / 12.9).
+//     35.2), but to 8 where a lane's loads are whole (`lanes`: B's rows on 8-byte
+//     boundaries; 8 x 8192 x 4288 24.3 / 36.5), and further for a few columns and
+//     a K to split (M = 4: 5 x 700 6.9 / 8.1, 33 x 1500 9.4 / 11.2; M = 8: 17 x
+//     3001 10.5 / 12.9).
 //   - the small-operand kernel reads a row-major B as it is (`in_place`): with
 //     int32 outputs that is faster from M = 2 on (M = 1 x 4096 x 4096 8.4 / 9.7
 //     us, 2 x 4096 11.0 / 9.7, 8 x 4096 18.1 / 9.9), except M = 2 with a small B
@@ -883,14 +885,14 @@ constexpr int64_t kSkinnyMaxM = 8;  // the largest limit below
 //     short K from 4 or 7 on (3 x 4096 x 1024 8.8 / 9.4, 6 x 1024 x 1024 8.4 / 9.0),
 //     a large B from 4 (3 x 8192 x 8192 26.3 / 29.1, 3 x 16384 x 8192 44.9 / 37.0).
 // GB300_GEMM_SKINNY_MAX_M overrides (0 disables the kernel).
-int skinny_max_m(bool int8, int64_t N, int64_t K, bool b_kmajor, bool in_place, int out_bits) {
+int skinny_max_m(bool int8, int64_t N, int64_t K, bool b_kmajor, bool in_place, bool lanes, int out_bits) {
   const int v = overrides().skinny_max_m;
   if (v >= 0) return v > 16 ? 16 : v;
   if (!int8) return 2;
   if (!in_place) {
     if (b_kmajor || (N <= 48 && K >= 2048)) return 8;
     if (N <= 8 || (N <= 48 && K >= 1024)) return 4;
-    return N * K > (int64_t(1) << 23) ? 2 : 3;
+    return N * K <= (int64_t(1) << 23) ? 3 : lanes ? 8 : 2;
   }
   if (out_bits == 32) return N >= 8192 || N * K < (int64_t(1) << 22) ? 2 : 1;
   if (K <= 1024) return N <= 2048 ? 6 : 3;
@@ -1027,7 +1029,7 @@ gemm_status_t gemm_bf16_f32acc_bf16(int64_t M, int64_t N, int64_t K, const uint1
   }
   const bool b_kmajor = b_layout == GEMM_B_COL_MAJOR_NxK;
   if (try_rows(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, false, 0, 0, st, &s)) return s;
-  if (M <= skinny_max_m(false, N, K, b_kmajor, false, 16)) {
+  if (M <= skinny_max_m(false, N, K, b_kmajor, false, false, 16)) {
     s = run_skinny(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, false, st);
     // no scratch for its partials inside a capture: the tensor-core kernels need
     // none for aligned operands
@@ -1316,7 +1318,7 @@ gemm_status_t s8_gemm(int64_t M, int64_t N, int64_t K, const int8_t *A, int64_t 
     return (double)M * (double)N * (double)K <= (double)kTinyMaxMacsForced ? run_tiny() : GEMM_ERR_UNSUPPORTED;
   };
   const bool in_place = overrides().s8tm && !b_kmajor && N > kBM && aligned16(B) && ldb % 16 == 0;
-  if (M <= skinny_max_m(true, N, K, b_kmajor, in_place, out_bits)) {
+  if (M <= skinny_max_m(true, N, K, b_kmajor, in_place, ((uintptr_t)B | (uint64_t)ldb) % 8 == 0, out_bits)) {
     s = run_skinny(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, true, st, out_bits, shift);
     return s == GEMM_ERR_UNSUPPORTED ? without_scratch(false) : s;
   }
@@ -1456,7 +1458,7 @@ gemm_status_t gemm_plan_query(int64_t M, int64_t N, int64_t K, int int8, int b_l
     return GEMM_OK;
   }
   const bool in_place = overrides().s8tm && !b_kmajor && N > kBM && N % 16 == 0;
-  if (M <= skinny_max_m(int8 != 0, N, K, b_kmajor, in_place, 32)) {
+  if (M <= skinny_max_m(int8 != 0, N, K, b_kmajor, in_place, N % 8 == 0, 32)) {
     out->route = GEMM_ROUTE_SMALL_M;
     return GEMM_OK;
   }

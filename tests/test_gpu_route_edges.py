@@ -273,6 +273,7 @@ def test_small_m_limits():
     assert [small(m, 5001, 5001, ROW) for m in (2, 3)] == [True, False]
     assert [small(m, 5, 700, ROW) for m in (4, 5)] == [True, False] and small(4, 33, 1500, ROW)
     assert small(8, 17, 3001, ROW) and not small(8, 65, 3001, ROW)
+    assert small(8, 8200, 4288, ROW) and not small(8, 8204, 4288, ROW) and not small(8, 2008, 1500, ROW)
 
 
 @pytest.mark.gpu
