@@ -831,11 +831,13 @@ gemm_status_t run_tc(DeviceState &d, Plan &pl, const uint16_t *A, int64_t lda, c
 // operand or C off the 16-byte grid, which the others stage and store more slowly
 // (640 x 89 x 416 8.3 / 11.2, 500 x 500 x 200 int8 outputs 6.6 / 10.9, 511 x 511 x
 // 129 7.7 / 11.0, x 400 11.1 / 12.5, x 511 14.5 / 12.5; 1023 x 511 x 90 8.1 / 11.1,
-// 4001 x 131 x 127 12.3 / 11.1).
+// 4001 x 131 x 127 12.3 / 11.1; a little more tiles of a short K: 512 x 1257 x 80
+// 8.3 / 11.7, 1023 x 1023 x 31 12.0 / 11.1).
 constexpr int64_t kTinyMaxMacs = int64_t(1) << 24;  // 256^3
 constexpr int64_t kTinyMaxK = 512;
 constexpr int64_t kTinyShortTiles = 64;                                             // 32 x 32 tiles
 constexpr int64_t kTinyMaxMacsOdd = int64_t(3) << 25, kTinyMaxTilesOdd = 512;
+constexpr int64_t kTinyShortK = 96, kTinyMaxTilesOddShortK = 704;
 // With the small-M limit forced (GB300_GEMM_SKINNY_MAX_M), or no workspace for
 // another kernel, the tile kernel takes problems by their multiply-adds alone,
 // up to 512^3.
@@ -858,7 +860,8 @@ bool tiny_shape(int64_t M, int64_t N, int64_t K, bool odd) {
   if (K > kTinyMaxK) return false;
   const double tiles = (double)ceil_div(M, (int64_t)32) * (double)ceil_div(N, (int64_t)32);
   return macs <= (double)kTinyMaxMacs || tiles <= (double)kTinyShortTiles ||
-         (odd && macs <= (double)kTinyMaxMacsOdd && tiles <= (double)kTinyMaxTilesOdd);
+         (odd && macs <= (double)kTinyMaxMacsOdd &&
+          tiles <= (double)(K <= kTinyShortK ? kTinyMaxTilesOddShortK : kTinyMaxTilesOdd));
 }
 
 constexpr int64_t kSkinnyMaxM = 8;  // the largest limit below

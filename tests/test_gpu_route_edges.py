@@ -305,7 +305,8 @@ def test_tiny_limits():
 
     assert tiny(128, 512, 512) and tiny(64, 1024, 512) and not tiny(64, 1040, 512) and not tiny(128, 512, 528)
     assert tiny(640, 89, 416) and tiny(511, 511, 129, COL) and tiny(511, 511, 385) and not tiny(511, 511, 386)
-    assert tiny(1023, 511, 90) and not tiny(1025, 511, 90) and not tiny(1024, 512, 96) and not tiny(4001, 131, 127)
+    assert tiny(1023, 511, 97) and not tiny(1025, 511, 97) and not tiny(1024, 512, 97 + 15) and not tiny(4001, 131, 127)
+    assert tiny(512, 1257, 80) and tiny(1025, 511, 96) and not tiny(1023, 1023, 31)
 
 
 @pytest.mark.gpu
