@@ -1125,8 +1125,10 @@ double s8tm_model_us(const S8tmChoice &c, int64_t tiles, int64_t num_kb, int64_t
 // seeded shapes with 129 to 1024 rows that a margin of 5 % takes, general path
 // / kernel were 1 / 0.86 (geometric mean; 0.47 at best, 1.15 at worst): 256 x
 // 12288 x 4096 53 -> 29.3 us, 256 x 4096 x 4096 23.7 -> 16.1, 512 x 8192 x 4096
-// 45.6 -> 32.7, 8192 x 256 x 4096 36.7 -> 20.0; the other way 1024 x 4096 x 4096
-// 36.5 -> 35.2, 2048^3 22.3 -> 23.7, 480 x 6912 x 4224 transposed 35.6 -> 41.1.
+// 45.6 -> 32.7, 8192 x 256 x 4096 36.7 -> 20.0.  The worst of them, 480 x 6912 x
+// 4224 transposed 35.6 -> 41.1, and those that gain little (1024 x 4096 x 4096
+// 36.5 -> 35.2) are outside the margins kept, and 2048^3 (22.3 -> 23.7) outside
+// the rows.
 constexpr int64_t kS8tmMaxRows = 1024;
 constexpr double kS8tmFixedUs = 6.0, kS8tmQUsPerM = 0.45;
 constexpr double kS8tmMargin = 1.08, kS8tmMarginTransposed = 1.15;
@@ -1200,6 +1202,9 @@ bool try_s8tm(DeviceState &d, int64_t M, int64_t N, int64_t K, const int8_t *A, 
   const int64_t tiles_p = ceil_div(P_rows, kBM), tiles_q = ceil_div(Q_rows, qn);
   const int64_t tiles = tiles_p * tiles_q;
   const int64_t splits = c.splits;
+  if (ovr.debug)
+    std::fprintf(stderr, "[gb300_gemm] M=%lld N=%lld K=%lld small operand: %lld x %lld tiles of 128 x %d, %lld splits\n",
+                 (long long)M, (long long)N, (long long)K, (long long)tiles_p, (long long)tiles_q, qn, (long long)splits);
   const int64_t kb_per = ceil_div(num_kb, splits);
   gemm_status_t s;
   // split-K: int32 outputs are added into C (zeroed by the staging launch),

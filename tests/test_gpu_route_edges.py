@@ -331,3 +331,21 @@ def test_tiny_limits_results(dtype, M, N, K, layout, pad, off):
     ("bf16", 2, 4096, 4096, ROW), ("bf16", 1, 1024, 8192, ROW), ("bf16", 1, 64, 65536, COL), ("bf16", 5, 600, 32768, COL)])
 def test_captured_few_rows_on_a_stream_without_scratch(dtype, M, N, K, layout):
     test_captured_on_a_stream_without_scratch(dtype, M, N, K, layout)
+
+
+# narrow outputs through several tiles of the small-operand kernel (its choice
+# depends on the output width; GB300_GEMM_DEBUG tells which kernel a call takes)
+@pytest.mark.gpu
+@needs_gpu
+@pytest.mark.parametrize("dtype,M,N,K,layout,tiles,splits,kw", [
+    ("int8_int16", 300, 12288, 4096, COL, (96, 3), 1, {"shift": 9}), ("int8_int8", 12288, 280, 4096, ROW, (96, 3), 1, {"shift": 14}),
+    ("int8_int8", 300, 12280, 4096, COL, (96, 3), 1, {"shift": 14, "ldc": 12281, "c_off": 1}),
+    ("int8_int16", 200, 4096, 4096, COL, (32, 2), 2, {"shift": 9, "ldc": 4099})])
+def test_narrow_outputs_of_several_small_operand_tiles(monkeypatch, capfd, dtype, M, N, K, layout, tiles, splits, kw):
+    monkeypatch.setenv("GB300_GEMM_DEBUG", "1")
+    A, B = _operands("int8", M, N, K, layout, M)
+    capfd.readouterr()
+    C = U.run(dtype, A, B, layout, **kw)
+    assert f"small operand: {tiles[0]} x {tiles[1]} tiles of 128 x 128, {splits} splits" in capfd.readouterr().err
+    want = oracle.requantize(oracle.gemm_s8(A, B, layout), kw["shift"], 16 if dtype == "int8_int16" else 8)
+    assert np.array_equal(C.astype(np.int64), want)
