@@ -385,13 +385,13 @@ int64_t rows_geometry(int64_t NW, int64_t K, int R, bool int8, int sms, int *clu
 // 128 x 16384 8.0 / 9.2, x 32768 15.1 / 10.5, x 131072 52.8 / 15.5; 1 x 600 x 8192
 // 6.0 / 6.9, x 16384 9.4 / 8.7; 4 x 600 x 16384 9.2 / 10.1, x 32768 16.1 / 13.4;
 // int8 1 x 32 x 65536 16.4 / 22.6; 1 x 128 x 32768 9.5 / 11.5, x 65536 16.6 / 12.1;
-// 1 x 600 x 16384 6.6 / 7.4, x 32768 10.6 / 8.6.  From about 400 blocks on the
+// 1 x 600 x 16384 6.6 / 7.4, x 32768 10.6 / 8.6.  From about 48 strips on the
 // stream itself is the limit (1 x 2400 x 65536 bf16 50.0 / 60.2), but for long
 // slices in more than one round (bf16 4 x 10000 x 16384 60.7 / 53.6).
 bool rows_faster(int64_t NW, int64_t K, int R, bool int8, bool few_m, int sms) {
   int cluster, kslice;
   const int64_t strips = rows_geometry(NW, K, R, int8, sms, &cluster, &kslice), blocks = strips * cluster;
-  if (blocks * 2 >= (int64_t)sms * 5)
+  if (strips * 16 >= (int64_t)sms * 5)  // 2.5 blocks per SM, were each strip given eight
     return int8 || R <= 2 || kslice <= 4096 || blocks <= (int64_t)kRowsBlocks * sms;
   if (int8) return !few_m || R > 8 || kslice <= (strips == 1 ? 8192 : strips <= 6 ? 4096 : 2560);
   if (!few_m || R > 2) return kslice <= 2560;

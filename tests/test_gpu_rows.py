@@ -150,7 +150,8 @@ def test_few_rows_of_a_long_k_go_where_it_is_split_further():
                              (4, 10000, 16384, False, 0), (1, 128, 32768, True, 8), (1, 128, 65536, True, 0),
                              (8, 600, 32768, True, 0), (16, 600, 65536, True, 8), (600, 4, 65536, True, 8),
                              (16, 4096, 4096, True, 4), (4, 2400, 8192, True, 7), (4, 2656, 8192, True, 6),
-                             (16, 2400, 8192, False, 7), (4, 2400, 8192, False, 8)):
+                             (16, 2400, 8192, False, 7), (4, 2400, 8192, False, 8),
+                             (4, 11008, 4096, False, 1), (1, 11008, 4096, True, 1), (1, 12288, 4096, False, 1)):
         assert few(M, N, K, int8) == c, (M, N, K, int8)
 
 
