@@ -402,17 +402,32 @@ struct Plan {
 // ceil(units / slots) of kb_per steps each; a split tail (the tiles of a
 // last, partly filled round split in tail_splits) gives the full rounds of
 // whole tiles plus one round of a tail unit's steps.
+//
+// With an A of fewer than 128 KB (a few rows) a K step takes at least
+// kSmallAStepUs for each CTA at work, whatever the tile: loads through a tensor
+// map of that size are slow where every CTA makes them (bf16 M x 11008 x 4096 on
+// 115 tiles of 96 columns 30.2 us for M = 4 to 14, 18.1 for M = 16 = 128 KB; M x
+// 12368 x 2576 on 97 tiles of 128 21.5 for M = 13 and 16, 14.6 for M = 32).  Fewer
+// and longer steps win there (three splits of 256 columns 21.9 and 18.7 us).
+constexpr double kSmallAStepUs = 0.0039;
+constexpr int64_t kSmallABytes = int64_t(128) << 10, kSmallAMaxM = 64;  // 100 x 11008 x 512 shows none of it
+bool small_a_map(int64_t M, int64_t K) { return M <= kSmallAMaxM && M * K * 2 < kSmallABytes; }
+
 struct Costs {
   const plan_table::StepCost (*step)[2][6];
   const float *split_fixed_us, *split_us_per_mb;
+  double small_a_step_us;
 };
-constexpr Costs kPlanCosts{plan_table::kCost, plan_table::kSplitFixedUs, plan_table::kSplitUsPerMB};
-constexpr Costs kRangeCosts{range_table::kCost, range_table::kSplitFixedUs, range_table::kSplitUsPerMB};  // bf16 only
+constexpr Costs kPlanCosts{plan_table::kCost, plan_table::kSplitFixedUs, plan_table::kSplitUsPerMB, kSmallAStepUs};
+constexpr Costs kRangeCosts{range_table::kCost, range_table::kSplitFixedUs, range_table::kSplitUsPerMB, 0.0};  // bf16 only
 
-double modelled_us(const Costs &ct, bool int8, bool pair, int bn, int64_t steps, int64_t rounds, double partial_mb) {
+// small_a_ctas: CTAs at work at a time where A is small, else 0.
+double modelled_us(const Costs &ct, bool int8, bool pair, int bn, int64_t steps, int64_t rounds, double partial_mb,
+                   int64_t small_a_ctas) {
   const int wi = bn == 64 ? 0 : bn == 96 ? 1 : bn == 128 ? 2 : bn == 192 ? 3 : bn == 224 ? 4 : 5;
   const plan_table::StepCost c = ct.step[int8 ? 1 : 0][pair ? 1 : 0][wi];
-  double t = (double)steps * c.kstep_us + (double)rounds * c.unit_us;
+  const double floor_us = ct.small_a_step_us * (double)small_a_ctas;
+  double t = (double)steps * (floor_us > c.kstep_us ? floor_us : c.kstep_us) + (double)rounds * c.unit_us;
   if (partial_mb > 0) t += ct.split_fixed_us[int8 ? 1 : 0] + ct.split_us_per_mb[int8 ? 1 : 0] * partial_mb;
   return t;
 }
@@ -460,7 +475,7 @@ Choice best_choice(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int 
   static const int kWidthsMNMajor[] = {256, 192, 128, 64};
   static const int kPairWidthsMNMajor[] = {256, 128};
   const Overrides &ovr = overrides();
-  const bool int8 = epi == kEpiS32;
+  const bool int8 = epi == kEpiS32, small_a = small_a_map(M, K);
   const int64_t num_kb = ceil_div(K, kBK);
   Choice best;
   double best_cost = -1.0;
@@ -486,6 +501,7 @@ Choice best_choice(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int 
       const int nw = b_kmajor ? (narrow ? 6 : 4) : (pair ? 2 : (narrow ? 4 : 3));
       const int64_t slots = pair ? pairs : sms;
       const int64_t tiles_m = ceil_div(M, pair ? 2 * kBM : kBM);
+      auto ctas = [&](int64_t units) { return (units < slots ? units : slots) * (pair ? 2 : 1); };
       for (int i = 0; i < nw; ++i) {
         const int bn = widths[i];
         if (N <= 128 && bn > 128) continue;
@@ -512,7 +528,8 @@ Choice best_choice(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int 
           if (ranges > 0 && s2 != ranges && !in_regs) continue;
           const int64_t rounds = ceil_div(tiles * s2, slots);
           consider(pair, bn, s2, 0, 0,
-                   modelled_us(costs, int8, pair, bn, rounds * kb_per, rounds, s2 > 1 ? 4.0 * s2 * M * N / 1e6 : 0.0) +
+                   modelled_us(costs, int8, pair, bn, rounds * kb_per, rounds, s2 > 1 ? 4.0 * s2 * M * N / 1e6 : 0.0,
+                               small_a ? ctas(tiles * s2) : 0) +
                        (in_regs ? kSlabUs * (double)(rounds * (ranges - 1)) : 0.0));
         }
         // Split tail: whole tiles for the full rounds, the last round's
@@ -526,7 +543,8 @@ Choice best_choice(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int 
           if (ceil_div(num_kb, kb_tail) != st2 || kb_tail < 4) continue;
           const double part_mb = 4.0 * st2 * tail * (pair ? 2 * kBM : kBM) * bn / 1e6;
           consider(pair, bn, 1, st2, kb_tail,
-                   modelled_us(costs, int8, pair, bn, full * num_kb + kb_tail, full + 1, part_mb));
+                   modelled_us(costs, int8, pair, bn, full * num_kb + kb_tail, full + 1, part_mb,
+                               small_a ? ctas(slots) : 0));
         }
       }
     }
@@ -553,7 +571,8 @@ Plan search_plan(int64_t M, int64_t N, int64_t K, bool b_kmajor, int epi, int sm
     const int64_t slots = best.pair ? pairs : sms, rows = best.pair ? 2 * kBM : kBM;
     const int64_t tiles = ceil_div(M, rows) * ceil_div(N, (int64_t)best.bn), full = tiles / slots;
     best.model_us = modelled_us(kPlanCosts, false, best.pair, best.bn, full * num_kb + best.kb_tail, full + 1,
-                                4e-6 * (double)(best.tail_splits * (tiles - full * slots) * rows * best.bn));
+                                4e-6 * (double)(best.tail_splits * (tiles - full * slots) * rows * best.bn),
+                                small_a_map(M, K) ? slots * (best.pair ? 2 : 1) : 0);
   } else {
     best = best_choice(M, N, K, b_kmajor, epi, sms, pairs, partials, kPlanCosts, ranges);
   }

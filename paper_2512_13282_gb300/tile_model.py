@@ -91,6 +91,9 @@ NARROW = (64, 96)
 # beyond the first costs there (kMaxSlabBN and kSlabUs in csrc)
 MAX_SLAB_BN = 128
 SLAB_US = 0.2
+# least time of a K step per CTA at work where A has at most SMALL_A_MAX_M rows and is smaller than SMALL_A_BYTES
+# (kSmallAStepUs in csrc)
+SMALL_A_STEP_US, SMALL_A_BYTES, SMALL_A_MAX_M = 0.0039, 128 << 10, 64
 
 
 class Variant:
@@ -295,7 +298,12 @@ def plan_cost_us(M, N, K, dtype, plan, table):
     if g is None:
         return math.inf
     steps, rounds, mb = plan_terms(M, N, plan)
-    t_comp = steps * g["kstep_us"] + rounds * g["unit_us"]
+    kstep = g["kstep_us"]
+    if M <= SMALL_A_MAX_M and M * K * 2 < SMALL_A_BYTES and not table.get("ranges"):
+        slots = GB300["pair_slots"] if plan["pair"] else GB300["sms"]
+        units = slots if plan.get("tail_splits", 0) else min(plan["tiles"] * plan["splits"], slots)
+        kstep = max(kstep, SMALL_A_STEP_US * units * (2 if plan["pair"] else 1))
+    t_comp = steps * kstep + rounds * g["unit_us"]
     t_split = 0.0
     if mb > 0:
         sp = table["split"][dtype]
@@ -561,7 +569,7 @@ def _range_table():
                 groups[f"bf16/{fam}/{bn}"] = {"kstep_us": k, "unit_us": u}
     one = lambda name: float(re.findall(name + r"\[1\] = \{([0-9.]+)f\}", text)[0])
     return {"groups": groups, "split": {"bf16": {"fixed_us": one("kSplitFixedUs"), "us_per_mb": one("kSplitUsPerMB")}},
-            "mem_weight": load_table()["mem_weight"]}
+            "mem_weight": load_table()["mem_weight"], "ranges": True}
 
 
 def table_from_header(text):

@@ -88,3 +88,16 @@ def test_split_tails_are_a_property_of_the_sizes():
         assert st == G.GEMM_OK and plan["tail_splits"] == want["tail_splits"]
         if want["tail_splits"]:
             assert (plan["bn"], plan["route"] == G.GEMM_ROUTE_TC_PAIR) == (want["bn"], want["pair"])
+
+
+def test_small_a_takes_long_steps():
+    """Few rows with an A below 128 KB: fewer CTAs and longer K steps than for
+    the same tiles with a larger A; the ranges stay."""
+    from paper_2512_13282_gb300 import build
+    build.build()
+    G.gemm_reload_overrides()
+    for M, N, K in ((14, 12368, 2576), (6, 8960, 1705), (6, 11008, 2048)):
+        st, few = G.gemm_plan_query(M, N, K, False, ROW)
+        assert st == G.GEMM_OK and few["splits"] == T.sum_ranges(M, N, K, False) == 3
+    st, many = G.gemm_plan_query(32, 12368, 2576, False, ROW)
+    assert st == G.GEMM_OK and many["splits"] == 1 and T.sum_ranges(32, 12368, 2576, False) == 3
