@@ -173,3 +173,44 @@ def test_many_unaligned_rows_of_a_long_k(K):
     before = G.gemm_launch_count()
     _run("int8", 13, 70, K, seed=K, lda=K + 8)
     assert (G.gemm_launch_count() - before == 1) == (K == 32768)
+
+
+@pytest.mark.gpu
+@pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a GPU")
+@pytest.mark.parametrize("dtype", ["int8", "bf16"])
+@pytest.mark.parametrize("R", [3, 16])
+@pytest.mark.parametrize("K,pad", [(271, 1), (500, 12), (1003, 5), (1009, 15), (2047, 1), (1030, 26)])
+def test_few_rows_last_pieces(dtype, R, K, pad):
+    """A K off the 16-byte grid: the last piece of a row is cut from what follows
+    it, NaN and extremes there included, and the last row's ends at the matrix."""
+    L = 70
+    rng = np.random.default_rng(K)
+    ld = K + pad
+
+    def filled(rows):
+        if dtype == "bf16":
+            buf = np.full((rows, ld), 0x7FC0, np.uint16)  # NaN behind each row
+            buf[:, :K] = W.random_bf16((rows, K), int(rng.integers(1 << 30)))
+        else:
+            buf = np.full((rows, ld), -128, np.int8)
+            buf[:, :K] = W.random_int8((rows, K), int(rng.integers(1 << 30)))
+        return buf
+
+    A, B = filled(R), filled(L)
+    for X, Y in ((A, B), (B, A)):
+        M, N = X.shape[0], Y.shape[0]
+        view = (lambda a: a.view(np.int16)) if dtype == "bf16" else (lambda a: a)
+        tx, ty = torch.from_numpy(view(X)).cuda(), torch.from_numpy(view(Y)).cuda()
+        c = torch.zeros((M, N), dtype=torch.int16 if dtype == "bf16" else torch.int32, device="cuda")
+        fn = G.gemm_bf16_f32acc_bf16 if dtype == "bf16" else G.gemm_s8s8_s32
+        G.gemm_reload_overrides()
+        # the pitch of the small operand need not be a multiple of 16 bytes, the large one's is
+        assert fn(M, N, K, tx, ld, ty, ld, COL, c, N) == G.GEMM_OK
+        torch.cuda.synchronize()
+        C = c.cpu().numpy()
+        x, y = np.ascontiguousarray(X[:, :K]), np.ascontiguousarray(Y[:, :K])
+        if dtype == "bf16":
+            ref, mag = oracle.gemm_bf16(x, y, COL)
+            assert oracle.bf16_within_bound(C.view(np.uint16), ref, mag).all()
+        else:
+            assert np.array_equal(C.astype(np.int64), oracle.gemm_s8(x, y, COL))
