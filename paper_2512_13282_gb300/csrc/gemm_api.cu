@@ -762,14 +762,14 @@ gemm_status_t run_tc(DeviceState &d, Plan &pl, const uint16_t *A, int64_t lda, c
   // through the staging blocks (rows_out).  By a lane / by rows, back to back:
   // int32 on 4-byte rows 4096 x 4096 x 1024 82.4 / 44.2 us; bf16 on 4-byte rows
   // 42.2 / 52.8 and on odd ones 110.6 / 52.3; int8 37.9 / 49.0 and 143.4 / 48.8.
-  // By a lane, too, where a block has few columns or there is one block of rows
-  // (bf16 60000 x 15 x 64 11.4 / 16.6, 60000 x 29 x 64 21.9 / 17.3, 32 x 515 x
-  // 128 6.0 / 7.5; int32 300000 x 97 x 16 115.7 / 121.5, 60000 x 129 x 64 37.1 /
+  // By a lane, too, where a block has few columns or there are few blocks of rows
+  // (bf16 60000 x 15 x 64 11.4 / 16.6, 60000 x 29 x 64 21.9 / 17.3; 33 x 2051 x 2048
+  // 11.8 / 15.2, 64 x 2051 x 2048 14.2 / 15.9, 96 x 2051 x 2048 14.4 / 13.8; int32 300000 x 97 x 16 115.7 / 121.5, 60000 x 129 x 64 37.1 /
   // 31.4).
   const bool words = p.splits > 1 || esize == 4;
   const int64_t odd_bytes = p.splits > 1 ? (int64_t)p.N * 4 : (int64_t)(reinterpret_cast<uintptr_t>(C) | (uint64_t)(ldc * esize));
   const bool rows = !tma_ok && overrides().tma_store && odd_bytes % (words ? 8 : 4) != 0 &&
-                    p.N >= (words ? 128 : 24) && p.M > 32;
+                    p.N >= (words ? 128 : 24) && p.M > 64;
   // An output that will be stored directly wants the variant with the extra
   // pipeline stage where one exists (int8 at 192 / 224).
   if (!tma_ok && s32 && (pl.v.bn == 192 || pl.v.bn == 224)) pl.v.tma_out = rows ? 1 : 0;
