@@ -846,7 +846,9 @@ gemm_status_t run_tc(DeviceState &d, Plan &pl, const uint16_t *A, int64_t lda, c
 // 5.3 us, 256^3 5.1 / 6.6, 300^3 (odd pitch) 7.7-8.8 / 8.2, 384^3 9.8 / 7.0,
 // 512^3 9.6 / 6.5, 32 x 1024 x 1024 8.7 / 6.3, 128 x 128 x 4096 31 / 9.0.
 // Two kinds of larger problem stay with it: those of one short round of tiles
-// (128 x 512 x 512 5.3 / 8.6, 64 x 1024 x 512 5.3 / 7.5), and those with an
+// (128 x 512 x 512 5.3 / 8.6, 64 x 1024 x 512 5.3 / 7.5), of more tiles for a short
+// K (512 x 512 x 128 5.6 / 6.6, 2400 x 80 x 112 5.7 / 8.0) or narrow outputs (768 x
+// 96 x 512 5.1 / 8.4, 384^3 6.4 / 6.9), and those with an
 // operand or C off the 16-byte grid, which the others stage and store more slowly
 // (640 x 89 x 416 8.3 / 11.2, 500 x 500 x 200 int8 outputs 6.6 / 10.9, 511 x 511 x
 // 129 7.7 / 11.0, x 400 11.1 / 12.5, x 511 14.5 / 12.5; 1023 x 511 x 90 8.1 / 11.1,
@@ -854,7 +856,8 @@ gemm_status_t run_tc(DeviceState &d, Plan &pl, const uint16_t *A, int64_t lda, c
 // 8.3 / 11.7, 1023 x 1023 x 31 12.0 / 11.1).
 constexpr int64_t kTinyMaxMacs = int64_t(1) << 24;  // 256^3
 constexpr int64_t kTinyMaxK = 512;
-constexpr int64_t kTinyShortTiles = 64;                                             // 32 x 32 tiles
+constexpr int64_t kTinyShortTiles = 64, kTinyShortTilesNarrow = 144;  // 32 x 32 tiles
+constexpr int64_t kTinyShortTilesShortK = 256, kTinyShorterK = 192;
 constexpr int64_t kTinyMaxMacsOdd = int64_t(3) << 25, kTinyMaxTilesOdd = 512;
 constexpr int64_t kTinyShortK = 96, kTinyMaxTilesOddShortK = 704;
 // With the small-M limit forced (GB300_GEMM_SKINNY_MAX_M), or no workspace for
@@ -869,7 +872,7 @@ bool default_routes() {
 }
 
 // `odd`: an operand or C does not start each row on a 16-byte boundary.
-bool tiny_shape(int64_t M, int64_t N, int64_t K, bool odd) {
+bool tiny_shape(int64_t M, int64_t N, int64_t K, bool odd, int out_bits) {
   const Overrides &o = overrides();
   // a forced tile width, family or split asks for the tensor-core kernels
   if (o.bn > 0 || o.pair >= 0 || o.splits >= 1 || o.tail_splits >= 2) return false;
@@ -878,7 +881,8 @@ bool tiny_shape(int64_t M, int64_t N, int64_t K, bool odd) {
   if (o.skinny_max_m >= 0) return macs <= (double)kTinyMaxMacsForced;
   if (K > kTinyMaxK) return false;
   const double tiles = (double)ceil_div(M, (int64_t)32) * (double)ceil_div(N, (int64_t)32);
-  return macs <= (double)kTinyMaxMacs || tiles <= (double)kTinyShortTiles ||
+  const int64_t short_tiles = K <= kTinyShorterK ? kTinyShortTilesShortK : out_bits < 32 ? kTinyShortTilesNarrow : kTinyShortTiles;
+  return macs <= (double)kTinyMaxMacs || tiles <= (double)short_tiles ||
          (odd && macs <= (double)kTinyMaxMacsOdd &&
           tiles <= (double)(K <= kTinyShortK ? kTinyMaxTilesOddShortK : kTinyMaxTilesOdd));
 }
@@ -1351,7 +1355,7 @@ gemm_status_t s8_gemm(int64_t M, int64_t N, int64_t K, const int8_t *A, int64_t 
   }
   const int64_t es_c = out_bits / 8;
   const bool odd = !aligned16(A) || !aligned16(B) || !aligned16(C) || (lda | ldb | (ldc * es_c)) % 16 != 0;
-  if (tiny_shape(M, N, K, odd)) return run_tiny();
+  if (tiny_shape(M, N, K, odd, out_bits)) return run_tiny();
   if (try_s8tm(*d, M, N, K, A, lda, B, ldb, b_kmajor, C, ldc, out_bits, shift, st, &s))
     return s == GEMM_ERR_UNSUPPORTED ? without_scratch(true) : s;
   Plan pl = make_plan(M, N, K, b_kmajor, kEpiS32, d->sms, pair_slots());
@@ -1490,7 +1494,7 @@ gemm_status_t gemm_plan_query(int64_t M, int64_t N, int64_t K, int int8, int b_l
     return GEMM_OK;
   }
   const bool odd = (K | (b_kmajor ? K : N) | (N * 4)) % 16 != 0;  // tight leading dimensions, int32 C
-  if (int8 && tiny_shape(M, N, K, odd)) {
+  if (int8 && tiny_shape(M, N, K, odd, 32)) {
     out->route = GEMM_ROUTE_TINY;
     out->bn = 32;
     out->splits = 1;

@@ -307,13 +307,15 @@ def test_tiny_limits():
     assert tiny(640, 89, 416) and tiny(511, 511, 129, COL) and tiny(511, 511, 385) and not tiny(511, 511, 386)
     assert tiny(1023, 511, 97) and not tiny(1025, 511, 97) and not tiny(1024, 512, 97 + 15) and not tiny(4001, 131, 127)
     assert tiny(512, 1257, 80) and tiny(1025, 511, 96) and not tiny(1023, 1023, 31)
+    assert tiny(512, 512, 192) and not tiny(512, 512, 208) and not tiny(512, 528, 192)
 
 
 @pytest.mark.gpu
 @needs_gpu
 @pytest.mark.parametrize("dtype", ["int8", "int8_int16", "int8_int8"])
 @pytest.mark.parametrize("M,N,K,layout,pad,off", [(128, 512, 512, ROW, 0, 0), (640, 89, 416, COL, 0, 0), (511, 511, 385, ROW, 0, 1),
-                                                  (1023, 511, 90, COL, 1, 3), (512, 512, 128, ROW, 4, 0), (512, 512, 384, ROW, 0, 0)])
+                                                  (1023, 511, 90, COL, 1, 3), (512, 512, 128, ROW, 4, 0), (512, 512, 384, ROW, 0, 0),
+                                                  (512, 512, 192, COL, 0, 0), (384, 384, 512, ROW, 0, 0), (384, 400, 512, COL, 0, 0)])
 def test_tiny_limits_results(dtype, M, N, K, layout, pad, off):
     A, B = _operands("int8", M, N, K, layout, M + N)
     C = U.run(dtype, A, B, layout, lda=K + pad, ldb=B.shape[1] + pad, ldc=N + pad, a_off=off, c_off=off, shift=8)
