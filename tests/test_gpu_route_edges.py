@@ -351,3 +351,13 @@ def test_narrow_outputs_of_several_small_operand_tiles(monkeypatch, capfd, dtype
     assert f"small operand: {tiles[0]} x {tiles[1]} tiles of 128 x 128, {splits} splits" in capfd.readouterr().err
     want = oracle.requantize(oracle.gemm_s8(A, B, layout), kw["shift"], 16 if dtype == "int8_int16" else 8)
     assert np.array_equal(C.astype(np.int64), want)
+
+
+@pytest.mark.gpu
+@needs_gpu
+@pytest.mark.parametrize("M,N,K,layout,kw", [(7978, 321, 640, ROW, {}), (2048, 300, 4096, COL, {"ldc": 301}), (321, 4097, 2048, COL, {}),
+                                             (4096, 201, 4096, ROW, {"c_off": 1}), (3000, 131, 2048, ROW, {})])
+def test_small_operand_int32_rows_off_the_grid(M, N, K, layout, kw):
+    """C that TMA cannot write: whichever kernel its stores leave the faster one."""
+    A, B = _operands("int8", M, N, K, layout, M + N)
+    _check("int8", A, B, layout, U.run("int8", A, B, layout, **kw))
