@@ -240,9 +240,10 @@ gemm_status_t gemm_selftest_wait_timeout(uint64_t limit_ns, gemm_stream_t stream
  * and K splits it takes the least modelled time, from per-variant costs
  * fitted to measurements on GB300.
  *   int8: nonzero for the int8 entry points, with int32 outputs (int16 and
- *   int8 outputs cost some kernels a reduction launch or narrow stores, so
- *   that gemm_s8s8_s16 / _s8 may take another route or split, with the same
- *   results; GB300_GEMM_DEBUG=1 prints a call's own), 0 for bf16.  b_layout
+ *   int8 outputs cost some kernels a reduction launch or narrow stores, and
+ *   an int32 C whose rows do not start and end on 16 bytes costs them stores
+ *   by the lanes, so that such calls may take another route or split, with
+ *   the same results; GB300_GEMM_DEBUG=1 prints a call's own), 0 for bf16.  b_layout
  *   as in the GEMM calls.  sms: SMs of the device (152 on GB300); pair_slots:
  *   co-resident CTA pairs (76).  Operands are taken as tight (lda = K, ldb
  *   and ldc = N or K) and 16-byte aligned; the planner overrides in force

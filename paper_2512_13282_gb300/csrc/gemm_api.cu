@@ -1508,7 +1508,7 @@ gemm_status_t gemm_plan_query(int64_t M, int64_t N, int64_t K, int int8, int b_l
   }
   S8tmChoice c;
   // tight leading dimensions: P's pitch is K (K-major) or N (B stored K x N)
-  if (int8 && s8tm_choice(M, N, K, b_kmajor, 32, N % 4 == 0, sms, pair_slots_, &c) && (c.p_kmajor ? K : N) % 16 == 0) {
+  if (int8 && s8tm_choice(M, N, K, b_kmajor, 32, true, sms, pair_slots_, &c) && (c.p_kmajor ? K : N) % 16 == 0) {
     const int64_t Q_rows = c.swap ? M : N, P_rows = c.swap ? N : M;
     const int qn = c.qn;
     const int64_t tiles = ceil_div(P_rows, kBM) * ceil_div(Q_rows, qn), splits = c.splits;
