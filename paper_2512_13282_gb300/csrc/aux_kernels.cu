@@ -53,11 +53,26 @@ __device__ __forceinline__ void piece_rc(uint64_t u, uint32_t cpr, int w, int64_
   c = (int64_t)q * w;
 }
 
-// The staging and re-pitch kernels are programmatic launches that wait for
-// the previous kernel at their start and let the next one start when they
-// end: a plain launch in the chain of a stream's kernels costs up to 2 us
-// more on GB300 (int8 1024^3 back to back 10.3 -> 9.8 us).
-//
+// The staging and re-pitch kernels are programmatic launches that wait for the
+// previous kernel at their start: a plain launch in the chain of a stream's
+// kernels costs up to 2 us more on GB300 (int8 1024^3 back to back 10.3 -> 9.8
+// us).  Replayed from a graph it is the other way round (1376 x 3276 x 112 10.9
+// us programmatic, 8.6 plain; 2048^3 23.1 and 22.0), so that captured launches are
+// plain.  Either way everything before them has completed when they let the next
+// kernel start, which sets itself up while they run and shares the GPU with them
+// alone.
+__device__ __forceinline__ void staging_begins() {
+  griddep_wait();
+  griddep_launch_dependents();
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_staging(void (*kern)(KArgs...), int64_t threads, cudaStream_t st, Args... args) {
+  const dim3 grid((unsigned)((threads + kS8Threads - 1) / kS8Threads));
+  if (!capturing(st)) return launch_ex(kern, grid, dim3(kS8Threads), 0, st, 1, args...);
+  kern<<<grid, kS8Threads, 0, st>>>(args...);
+  return cudaGetLastError();
+}
+
 // General path (any alignment, any leading dimension): both matrices as one
 // flat list of 16-element row pieces -- piece t < items_a is piece t % cpr_a
 // of row t / cpr_a of A (cpr = pieces per row), the rest likewise of B.  A
@@ -71,7 +86,7 @@ __device__ __forceinline__ void piece_rc(uint64_t u, uint32_t cpr, int w, int64_
 __global__ void __launch_bounds__(kS8Threads)
     s8_to_bf16_pair_kernel(const S8Job a, const S8Job b, uint32_t cpr_a, uint32_t cpr_b, uint64_t items_a,
                            uint64_t items) {
-  griddep_wait();
+  staging_begins();
   const uint64_t t = (uint64_t)blockIdx.x * kS8Threads + threadIdx.x;
   if (t >= items) return;
   const bool in_a = t < items_a;
@@ -102,7 +117,7 @@ __global__ void __launch_bounds__(kS8Threads)
 // partial vector (elements % 16) is converted element by element.
 __global__ void __launch_bounds__(kS8Threads)
     s8_to_bf16_dense_kernel(const S8Job a, const S8Job b, int64_t na, int64_t nb) {
-  griddep_wait();
+  staging_begins();
   const int64_t va = (na + 15) / 16, vtot = va + (nb + 15) / 16;
   const int64_t v = (int64_t)blockIdx.x * kS8Threads + threadIdx.x;
   if (v >= vtot) return;
@@ -128,7 +143,7 @@ __global__ void __launch_bounds__(kS8Threads)
 __global__ void __launch_bounds__(kS8Threads)
     pack_u16_kernel(const uint16_t *__restrict__ src, int64_t rows, int64_t cols, int64_t ld_src,
                     uint16_t *__restrict__ dst, int64_t ld_dst, uint32_t cpr, uint64_t items) {
-  griddep_wait();
+  staging_begins();
   const uint64_t t = (uint64_t)blockIdx.x * kS8Threads + threadIdx.x;
   if (t >= items) return;
   int64_t r, c;
@@ -360,14 +375,13 @@ cudaError_t launch_s8_to_bf16_pair(const S8Job &a, const S8Job &b, int sms, cuda
     const int64_t na = a.rows * a.cols, nb = b.rows * b.cols;
     const int64_t vecs = (na + 15) / 16 + (nb + 15) / 16;
     if (vecs == 0) return cudaSuccess;
-    return launch_ex(s8_to_bf16_dense_kernel, dim3((unsigned)((vecs + kS8Threads - 1) / kS8Threads)), dim3(kS8Threads),
-                     0, st, 1, a, b, na, nb);
+    return launch_staging(s8_to_bf16_dense_kernel, vecs, st, a, b, na, nb);
   }
   const uint64_t cpr_a = (uint64_t)(a.cols + 15) / 16, cpr_b = (uint64_t)(b.cols + 15) / 16;
   const uint64_t items_a = (uint64_t)a.rows * cpr_a, items = items_a + (uint64_t)b.rows * cpr_b;
   if (items == 0) return cudaSuccess;
-  return launch_ex(s8_to_bf16_pair_kernel, dim3((unsigned)((items + kS8Threads - 1) / kS8Threads)), dim3(kS8Threads), 0,
-                   st, 1, a, b, (uint32_t)(cpr_a ? cpr_a : 1), (uint32_t)(cpr_b ? cpr_b : 1), items_a, items);
+  return launch_staging(s8_to_bf16_pair_kernel, (int64_t)items, st, a, b, (uint32_t)(cpr_a ? cpr_a : 1),
+                        (uint32_t)(cpr_b ? cpr_b : 1), items_a, items);
 }
 
 cudaError_t launch_pack_u16(const uint16_t *src, int64_t rows, int64_t cols, int64_t ld_src,
@@ -375,8 +389,7 @@ cudaError_t launch_pack_u16(const uint16_t *src, int64_t rows, int64_t cols, int
   (void)sms;
   const uint64_t cpr = (uint64_t)(cols + 7) / 8, items = (uint64_t)rows * cpr;
   if (items == 0) return cudaSuccess;
-  return launch_ex(pack_u16_kernel, dim3((unsigned)((items + kS8Threads - 1) / kS8Threads)), dim3(kS8Threads), 0, st, 1,
-                   src, rows, cols, ld_src, dst, ld_dst, (uint32_t)cpr, items);
+  return launch_staging(pack_u16_kernel, (int64_t)items, st, src, rows, cols, ld_src, dst, ld_dst, (uint32_t)cpr, items);
 }
 
 cudaError_t launch_zero_fill(void *C, int64_t M, int64_t N, int64_t ldc, int esize, int sms,

@@ -153,6 +153,11 @@ const Overrides &overrides() {
 
 bool gb300::pdl_enabled() { return overrides().pdl; }
 
+bool gb300::capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone;
+}
+
 namespace {
 
 uint64_t wait_limit_ns() {
@@ -237,12 +242,6 @@ class ScratchLease {
   Scratch *s_ = nullptr;
   Scratch temp_;
 };
-
-// Whether `st` is being captured into a CUDA graph.
-bool capturing(cudaStream_t st) {
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  return cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone;
-}
 
 // Scratch of a stream's own slot needed by a call being captured into a
 // CUDA graph: it must exist already (the stream has run a call at least as

@@ -47,6 +47,9 @@ cudaError_t launch_ex(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem
   return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
 
+// Whether `st` is being captured into a CUDA graph.
+bool capturing(cudaStream_t st);
+
 // One compiled variant of the tcgen05 kernel.
 struct TcVariant {
   int bn;        // tile width (see the instantiation files for the compiled set)

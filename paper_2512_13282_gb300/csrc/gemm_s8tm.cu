@@ -623,7 +623,8 @@ cudaError_t launch_s8tm_stage_q(const int8_t *src, int64_t sq, int64_t sk, int64
   // it ends.  Measured on GB300, calls back to back (plain / programmatic):
   // 64 x 2048 x 2048 8.2 / 7.1 us, 32 x 4096 x 4096 12.3 / 10.9, 128 x 4096 x
   // 4096 14.3 / 12.9, 128 x 12288 x 4096 20.6 / 22.0, 8192 x 64 x 8192 20.8 /
-  // 21.3.
+  // 21.3.  Replayed from a graph the plain one is faster at every size (128 x 4096
+  // x 4096 12.8 / 14.1, 64 x 2048 x 2048 7.0 / 7.2).
   constexpr int64_t kStageOverlapBytes = int64_t(32) << 20;
   const int64_t num_kb = (K + kKB - 1) / kKB;
   const int64_t chunks = (int64_t)s8tm_q_image_bytes(qn, Q_rows, K) / 16;
@@ -633,7 +634,7 @@ cudaError_t launch_s8tm_stage_q(const int8_t *src, int64_t sq, int64_t sk, int64
   const int64_t extra = quads < 65536 ? quads : 65536;
   if (chunks + extra == 0) return cudaSuccess;
   const dim3 grid((unsigned)((chunks + extra + 255) / 256));
-  if (p_bytes >= kStageOverlapBytes || !pdl_enabled()) {
+  if (p_bytes >= kStageOverlapBytes || !pdl_enabled() || capturing(st)) {
     s8tm_stage_q_kernel<<<grid, 256, 0, st>>>(src, sq, sk, (int)Q_rows, (int)K, qn, (int)num_kb,
                                               static_cast<uint4 *>(img), chunks, zero_c, c_rows, c_cols, ldc, 1);
     return cudaGetLastError();

@@ -120,3 +120,49 @@ def test_capture_refuses_growth():
     g.replay()
     torch.cuda.synchronize()
     small.check()
+
+
+@pytest.mark.gpu
+@pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a GPU")
+def test_chain_of_dependent_calls_in_a_stream_and_a_graph():
+    """Each call's int8 output is the next one's A, through kernels that start
+    early, stage an operand or split K: in a stream and, with other launches for
+    the staging kernels, replayed from a graph."""
+    G.gemm_reload_overrides()
+    rng = np.random.default_rng(3)
+    M = 40
+    dims = [(640, 513), (513, 300), (300, 4096), (4096, 272), (272, 2064), (2064, 129), (129, 1000), (1000, 640)]  # K, N
+    Bs = [rng.integers(-30, 30, (N, K) if i % 2 else (K, N), dtype=np.int8) for i, (K, N) in enumerate(dims)]
+    A = rng.integers(-128, 128, (M, 640), dtype=np.int8)
+    shift = 10
+    want, x = [], A
+    for i, B in enumerate(Bs):
+        x = oracle.requantize(oracle.gemm_s8(x, B, i % 2), shift, 8).astype(np.int8)
+        want.append(x)
+    tB = [torch.from_numpy(b).cuda() for b in Bs]
+    tA = torch.from_numpy(A).cuda()
+    outs = [torch.zeros((M, N), dtype=torch.int8, device="cuda") for _, N in dims]
+
+    def chain(s):
+        a = tA
+        for i, (K, N) in enumerate(dims):
+            assert G.gemm_s8s8_s8(M, N, K, a, K, tB[i], tB[i].shape[1], i % 2, outs[i], N, shift, s) == G.GEMM_OK
+            a = outs[i]
+
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for _ in range(3):
+        chain(s)
+    s.synchronize()
+    for got, w in zip(outs, want):
+        assert np.array_equal(got.cpu().numpy(), w)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        chain(s)
+    for _ in range(3):
+        for o in outs:
+            o.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        for got, w in zip(outs, want):
+            assert np.array_equal(got.cpu().numpy(), w)
