@@ -24,8 +24,8 @@
 //     to int32, so every fp32 sum is an integer of at most 2^23, exact.
 //
 // A block of four warps owns 32 rows of W and a K slice; the warps take
-// 128-byte deep batches of the slice in turn and are summed in warp order in
-// shared memory.  K is split over the blocks of a cluster (1-8), whose sums
+// 128-byte deep batches of the slice in turn and are summed in warp order (one or
+// two bf16 rows pairwise) in shared memory.  K is split over the blocks of a cluster (1-8), whose sums
 // meet in distributed shared memory in rank order: results do not depend on
 // scheduling, and there are no partials in global memory, no counters and no
 // second launch.  Each half of a batch is reloaded as soon as it has been
@@ -159,12 +159,24 @@ __device__ __forceinline__ uint4 first_bytes(uint4 v, int valid) {
 
 // NT: 8-row groups of X.  XVEC: X's rows start on 16-byte boundaries (a kernel
 // of its own for those that do not, whose loads need more registers).
-template <int NT, bool INT8, bool XVEC>
+//
+// FINE: one or two rows of X in bf16.  An MMA leaves its fp32 sum truncated, and
+// one chain of MMAs over a warp's share of K was further off than the fp32 FMAs of
+// the CUDA-core kernel that took those rows before: 0.035 % of the results were
+// not the nearest bf16 against 0.009 % (K = 1024 to 12288; for 4 to 16 rows, where
+// the other choice is the tensor cores, 0.033 against 0.062).  Here a chain ends
+// with its batch (four MMAs), four batches are added in fp32 and their sums again:
+// 0.0102 % of 13.2 M results, 0.0099 on the CUDA cores, in the same time (1 x 12288
+// x 4096 19.1 us).  (Compensated sums, or chains spread over MMA columns that
+// multiply zeros, would make NaN of infinities.)
+template <int NT, bool INT8, bool XVEC, bool FINE>
 __global__ void __launch_bounds__(kRowsThreads, rows_blocks<NT, INT8>()) gemm_rows_kernel(const RowsParams p) {
   constexpr int ES = INT8 ? 1 : 2;
   constexpr int kHalf = 64 / ES;       // k per half batch: 64 bytes of each row, 16 a lane
   constexpr int kBatch = 2 * kHalf;
-  constexpr int kFlush = 512 / kBatch; // batches after which an accumulator holds 512 products
+  // batches after which an accumulator holds 512 products; FINE: that are added up
+  constexpr int kFlush = INT8 ? 512 / kBatch : 4;
+  static_assert(!FINE || (NT == 1 && !INT8), "one or two bf16 rows");
   extern __shared__ __align__(16) uint32_t red[];  // [warp][row of X][row of W], then the block's sums
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
   const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
@@ -243,6 +255,7 @@ __global__ void __launch_bounds__(kRowsThreads, rows_blocks<NT, INT8>()) gemm_ro
 
   float acc[2][NT][4];
   int32_t iacc[INT8 ? 2 : 1][NT][4];  // int8: the exact sums so far
+  float near[FINE ? 2 : 1][NT][4], far[FINE ? 2 : 1][NT][4];  // FINE: the sums of up to kFlush batches, and of those
   auto each = [&](auto &&f) {
 #pragma unroll
     for (int t = 0; t < 2; ++t)
@@ -254,6 +267,7 @@ __global__ void __launch_bounds__(kRowsThreads, rows_blocks<NT, INT8>()) gemm_ro
   each([&](int t, int j, int e) {
     acc[t][j][e] = 0.f;
     if constexpr (INT8) iacc[t][j][e] = 0;
+    if constexpr (FINE) near[t][j][e] = far[t][j][e] = 0.f;
   });
 
   auto multiply = [&](const uint4 (&w)[4], const uint4 (&x)[NT]) {
@@ -303,6 +317,18 @@ __global__ void __launch_bounds__(kRowsThreads, rows_blocks<NT, INT8>()) gemm_ro
     if (k + kHalf < kend) multiply(w1, x1);
     if (kn + kHalf < kend) load_half(kn + kHalf, w1, x1);
     k = kn;
+    if constexpr (FINE) {
+      const bool flush = ++held == kFlush;
+      each([&](int t, int j, int e) {
+        near[FINE ? t : 0][j][e] += acc[t][j][e];
+        acc[t][j][e] = 0.f;
+        if (flush) {
+          far[FINE ? t : 0][j][e] += near[FINE ? t : 0][j][e];
+          near[FINE ? t : 0][j][e] = 0.f;
+        }
+      });
+      if (flush) held = 0;
+    }
     if (INT8 && ++held == kFlush) {
       each([&](int t, int j, int e) {
         iacc[INT8 ? t : 0][j][e] += __float2int_rn(acc[t][j][e]);
@@ -312,6 +338,8 @@ __global__ void __launch_bounds__(kRowsThreads, rows_blocks<NT, INT8>()) gemm_ro
     }
   }
 
+  if constexpr (FINE)
+    each([&](int t, int j, int e) { acc[t][j][e] = near[FINE ? t : 0][j][e] + far[FINE ? t : 0][j][e]; });
   // accumulator element e of (tile t, group j): row of X, row of the strip
   const int words = R * kSumPitch;
   uint32_t *slot = red + warp * words;
@@ -331,6 +359,7 @@ __global__ void __launch_bounds__(kRowsThreads, rows_blocks<NT, INT8>()) gemm_ro
   };
   auto block_sum = [&](int r, int c) {
     const uint32_t *s = red + r * kSumPitch + c;
+    if (FINE) return add(add(s[0], s[words]), add(s[2 * words], s[3 * words]));
     uint32_t v = s[0];
 #pragma unroll
     for (int i = 1; i < kRowsWarps; ++i) v = add(v, s[i * words]);
@@ -365,12 +394,12 @@ __global__ void __launch_bounds__(kRowsThreads, rows_blocks<NT, INT8>()) gemm_ro
   cluster_barrier();  // no block leaves while another may still read its sums
 }
 
-template <int NT, bool INT8, bool XVEC>
+template <int NT, bool INT8, bool XVEC, bool FINE = false>
 cudaError_t launch_nt(const RowsParams &p, int64_t strips, cudaStream_t st) {
   const size_t smem = (size_t)p.R * 4 * (kRowsWarps * kSumPitch + (p.cluster > 1 ? kStrip : 0));
   static_assert(8 * NT * 4 * (kRowsWarps * kSumPitch + kStrip) <= 48 * 1024, "no shared-memory opt-in needed");
-  return launch_ex(gemm_rows_kernel<NT, INT8, XVEC>, dim3((unsigned)(strips * p.cluster)), dim3(kRowsThreads), smem, st,
-                   p.cluster, p);
+  return launch_ex(gemm_rows_kernel<NT, INT8, XVEC, FINE>, dim3((unsigned)(strips * p.cluster)), dim3(kRowsThreads), smem,
+                   st, p.cluster, p);
 }
 
 }  // namespace
@@ -435,6 +464,8 @@ cudaError_t launch_rows(const RowsParams &p, bool int8, int64_t strips, cudaStre
     return p.x_vec ? launch_nt<NT, INT8, true>(p, strips, st) : launch_nt<NT, INT8, false>(p, strips, st);
   };
   using std::integral_constant;
+  if (!int8 && p.R <= 2)
+    return p.x_vec ? launch_nt<1, false, true, true>(p, strips, st) : launch_nt<1, false, false, true>(p, strips, st);
   if (int8)
     return p.R > 8 ? by_x(integral_constant<int, 2>{}, std::true_type{}) : by_x(integral_constant<int, 1>{}, std::true_type{});
   return p.R > 8 ? by_x(integral_constant<int, 2>{}, std::false_type{}) : by_x(integral_constant<int, 1>{}, std::false_type{});
