@@ -148,13 +148,25 @@ __device__ __forceinline__ uint4 load16_words(const uint8_t *a, const uint8_t *l
                     __funnelshift_r(w3, w4, sh));
 }
 
-// The first `valid` (1-15) bytes of v, the rest zero.
-__device__ __forceinline__ uint4 first_bytes(uint4 v, int valid) {
+// The same of a row in [lo, hi): a row's last, partial piece is read whole and cut
+// where the matrix goes on behind it, element by element only at its end (element
+// by element everywhere it took as long as the rest of a small call: int8 16 x 64 x
+// 271 8.7 us, 3.1 for K = 256).  Out of line for int8 against 16 rows, whose loop
+// it cost 6 % inlined (16 x 11008 x 4096 14.6 us, 13.5 out of line); inlined
+// elsewhere, where the call costs small calls 0.5 us.
+__device__ __forceinline__ uint4 load16_part(const uint8_t *a, const uint8_t *lo, const uint8_t *hi, int es, int valid) {
+  if (a + 16 > hi) return load16_edge(a, es, valid);
+  const uint4 v = (reinterpret_cast<uintptr_t>(a) & 15u) == 0 ? __ldg(reinterpret_cast<const uint4 *>(a))
+                                                               : load16_words(a, lo, hi, es);
   auto keep = [&](uint32_t w, int at) {
     const int n = valid - at;
     return n >= 4 ? w : n <= 0 ? 0u : w & (0xffffffffu >> (32 - 8 * n));
   };
   return make_uint4(keep(v.x, 0), keep(v.y, 4), keep(v.z, 8), keep(v.w, 12));
+}
+
+__device__ __noinline__ uint4 load16_part_call(const uint8_t *a, const uint8_t *lo, const uint8_t *hi, int es, int valid) {
+  return load16_part(a, lo, hi, es, valid);
 }
 
 // NT: 8-row groups of X.  XVEC: X's rows start on 16-byte boundaries (a kernel
@@ -209,12 +221,9 @@ __global__ void __launch_bounds__(kRowsThreads, rows_blocks<NT, INT8>()) gemm_ro
   }
   griddep_wait();
 
-  const uint8_t *w_hi = static_cast<const uint8_t *>(p.W) + (p.NW - 1) * pitch + (int64_t)p.K * ES;
-
-  // A row's last, partial piece is read whole and cut where the matrix goes on
-  // behind it, element by element only at its end: element by element everywhere
-  // it took as long as the rest of a small call (int8 16 x 64 x 271 8.7 us, 3.1
-  // for K = 256).
+  auto load_part = [&](const uint8_t *a, const uint8_t *lo, const uint8_t *hi, int valid) {
+    return INT8 && NT == 2 ? load16_part_call(a, lo, hi, ES, valid) : load16_part(a, lo, hi, ES, valid);
+  };
   auto load_half = [&](int k, uint4 (&w)[4], uint4 (&x)[NT]) {
     const int64_t at = (int64_t)k * ES;
     const int valid = (kend - k) * ES - 16 * q;  // bytes of the lane's piece before the slice's end
@@ -228,8 +237,8 @@ __global__ void __launch_bounds__(kRowsThreads, rows_blocks<NT, INT8>()) gemm_ro
     } else {
 #pragma unroll
       for (int i = 0; i < 4; ++i)
-        w[i] = wp[i] + at + 16 <= w_hi ? first_bytes(__ldcs(reinterpret_cast<const uint4 *>(wp[i] + at)), valid)
-                                       : load16_edge(wp[i] + at, ES, valid);
+        w[i] = load_part(wp[i] + at, static_cast<const uint8_t *>(p.W),
+                         static_cast<const uint8_t *>(p.W) + (p.NW - 1) * pitch + (int64_t)p.K * ES, valid);
     }
     if (valid <= 0) {
 #pragma unroll
@@ -242,14 +251,7 @@ __global__ void __launch_bounds__(kRowsThreads, rows_blocks<NT, INT8>()) gemm_ro
       for (int j = 0; j < NT; ++j) x[j] = load16_words(xp[j] + at, x_lo, x_hi, ES);
     } else {
 #pragma unroll
-      for (int j = 0; j < NT; ++j) {
-        if (xp[j] + at + 16 > x_hi)
-          x[j] = load16_edge(xp[j] + at, ES, valid);
-        else if (XVEC)
-          x[j] = first_bytes(__ldg(reinterpret_cast<const uint4 *>(xp[j] + at)), valid);
-        else
-          x[j] = first_bytes(load16_words(xp[j] + at, x_lo, x_hi, ES), valid);
-      }
+      for (int j = 0; j < NT; ++j) x[j] = load_part(xp[j] + at, x_lo, x_hi, valid);
     }
   };
 
