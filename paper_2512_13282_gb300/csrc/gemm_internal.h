@@ -75,10 +75,10 @@ cudaError_t launch_tc2_bf16(const TcVariant &v, const CUtensorMap &a, const CUte
 cudaError_t launch_tc2_s32(const TcVariant &v, const CUtensorMap &a, const CUtensorMap &b,
                            const CUtensorMap &o, const CUtensorMap &w, const TcParams &p, int grid, cudaStream_t st);
 
-// int8 GEMM for memory-bound shapes with the large operand converted to bf16
+// int8 GEMM with a small operand, the large one converted to fp16
 // inside the kernel (gemm_s8tm.cu).  P (int8, K contiguous, P_rows x K) is
 // the operand streamed from HBM; Q (Q_rows x K) the small one, staged by
-// launch_s8tm_stage_q as bf16 shared-memory images.  The sum over k of
+// launch_s8tm_stage_q as fp16 shared-memory images.  The sum over k of
 // P[p][k] * Q[q][k] is C[q][p] when swap (P = B stored N x K, Q = A) and
 // C[p][q] otherwise (P = A, Q = B).
 constexpr int kS8tmKB = 128;  // K per k-block of gemm_s8tm_kernel
@@ -90,7 +90,7 @@ struct S8tmParams {
   int splits, kb_per_split;
   int slab_kb;       // k-blocks per exact fp32 slab (1024 / kS8tmKB)
   int add_into_c;    // splits add their exact sums into C (int32, zeroed by the Q staging launch)
-  int c_tma;         // ... with TMA reductions through tmC (else element by element)
+  int c_tma;         // int32 C is stored, or the splits' sums added, by TMA through tmC (else by the lanes)
   int swap;
   void *C;
   int64_t ldc;
@@ -104,7 +104,7 @@ struct S8tmParams {
 };
 // Bytes of Q's images for QN = qn columns per tile.
 size_t s8tm_q_image_bytes(int qn, int64_t Q_rows, int64_t K);
-// Writes Q's images: Q(q, k) = src[q * sq + k * sk] (int8), exact bf16;
+// Writes Q's images: Q(q, k) = src[q * sq + k * sk] (int8), exact fp16;
 // when zero_c is not null, also sets the c_rows x c_cols int32 matrix at
 // zero_c (row pitch ldc) to zero.  p_bytes: the size of P, which decides how
 // the launch overlaps its neighbours.

@@ -57,9 +57,9 @@
 // MMAs that read it have completed (tcgen05.commit), a TMEM P slot likewise.
 // With P decoupled from the MMA, the P ring keeps its boxes in flight from
 // HBM: measured on GB300, a P box takes about 2 us from issue to arrival
-// under load.  What bounds a long unit is the k-block itself, 0.42 us for
-// 128 x 128 x 128 (512 x 12288 x 4096: 16 KB of P and 32 KB of Q from L2 and
-// 0.33 us of MMA); short ones wait for their first box and their last slab.
+// under load.  What bounds a long unit is the k-block itself, 0.35 us for
+// 128 x 128 x 128 (16 KB of P and 32 KB of Q from L2, and 0.27 us of MMA at its
+// peak rate); short ones wait for their first box and their last slab.
 #include <cuda_bf16.h>
 
 #include "gemm_internal.h"
@@ -88,7 +88,7 @@ struct S8tmCfg {
   static constexpr int kEpiWarps = 4 * (QN / kEpiCols);
   static constexpr int kQWarp = 2 + kEpiWarps + kConvGroups * kConvWarps;  // Q producer
   static constexpr int kThreads = (kQWarp + 1) * 32;
-  static constexpr uint32_t kQHalf = QN * kRowBytes;  // QN x 64 bf16: one half of a Q image
+  static constexpr uint32_t kQHalf = QN * kRowBytes;  // QN x 64 fp16: one half of a Q image
   static constexpr uint32_t kQBytes = 2 * kQHalf;      // the k-block's Q image
   static constexpr uint32_t kPOffset = 0;
   static constexpr uint32_t kQOffset = SP * kPBytes;  // 1024-byte aligned
@@ -534,7 +534,7 @@ __global__ void __launch_bounds__(S8tmCfg<QN, SP, SQ, NA>::kThreads, 1)
   }
 }
 
-// Q's image for one (Q tile, k-block): QN rows x 128 K of bf16 as two
+// Q's image for one (Q tile, k-block): QN rows x 128 K of fp16 as two
 // 64-K halves of QN 128-byte rows, 16-byte chunk j of row r stored at chunk
 // j ^ (r % 8) (the 128-byte swizzle).  One thread writes one 16-byte chunk
 // (8 consecutive k of one row), reading Q(q, k) at src + q * sq + k * sk.

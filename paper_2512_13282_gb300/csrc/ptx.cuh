@@ -240,7 +240,8 @@ __device__ __forceinline__ void s8x4_to_bf16x4(uint32_t w, uint32_t &lo, uint32_
 // Four int8 (byte i is element i) -> four fp16, exactly: byte b, flipped to
 // b + 128, placed under the exponent of 1024 is the fp16 1024 + (b + 128),
 // and one packed subtraction of 1152 leaves b (fp16 holds every integer up
-// to 2048).  Five instructions; the bf16 conversion above takes eleven.
+// to 2048): the biased-exponent ("magic number") conversion of integers to
+// floating point.  Five instructions; the bf16 conversion above takes eleven.
 __device__ __forceinline__ void s8x4_to_f16x4(uint32_t w, uint32_t &lo, uint32_t &hi) {
   const uint32_t u = w ^ 0x80808080u;
   const uint32_t a = __byte_perm(u, 0x64u, 0x4140), b = __byte_perm(u, 0x64u, 0x4342);
