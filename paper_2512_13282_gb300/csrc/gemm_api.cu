@@ -855,8 +855,10 @@ gemm_status_t run_tc(DeviceState &d, Plan &pl, const uint16_t *A, int64_t lda, c
 // 8.3 / 11.7, 1023 x 1023 x 31 12.0 / 11.1).
 constexpr int64_t kTinyMaxMacs = int64_t(1) << 24;  // 256^3
 constexpr int64_t kTinyMaxK = 512;
-constexpr int64_t kTinyShortTiles = 64, kTinyShortTilesNarrow = 144;  // 32 x 32 tiles
-constexpr int64_t kTinyShortTilesShortK = 256, kTinyShorterK = 192;
+struct TinyTiles {
+  int64_t max_k, tiles, tiles_narrow;  // 32 x 32 tiles with int32 and with narrow outputs
+};
+constexpr TinyTiles kTinyTiles[] = {{96, 608, 608}, {128, 304, 304}, {192, 256, 256}, {256, 64, 208}, {kTinyMaxK, 64, 144}};
 constexpr int64_t kTinyMaxMacsOdd = int64_t(3) << 25, kTinyMaxTilesOdd = 512;
 constexpr int64_t kTinyShortK = 96, kTinyMaxTilesOddShortK = 704;
 // With the small-M limit forced (GB300_GEMM_SKINNY_MAX_M), or no workspace for
@@ -880,8 +882,9 @@ bool tiny_shape(int64_t M, int64_t N, int64_t K, bool odd, int out_bits) {
   if (o.skinny_max_m >= 0) return macs <= (double)kTinyMaxMacsForced;
   if (K > kTinyMaxK) return false;
   const double tiles = (double)ceil_div(M, (int64_t)32) * (double)ceil_div(N, (int64_t)32);
-  const int64_t short_tiles = K <= kTinyShorterK ? kTinyShortTilesShortK : out_bits < 32 ? kTinyShortTilesNarrow : kTinyShortTiles;
-  return macs <= (double)kTinyMaxMacs || tiles <= (double)short_tiles ||
+  const TinyTiles *row = kTinyTiles;
+  while (K > row->max_k) ++row;  // the last row's is kTinyMaxK
+  return macs <= (double)kTinyMaxMacs || tiles <= (double)(out_bits < 32 ? row->tiles_narrow : row->tiles) ||
          (odd && macs <= (double)kTinyMaxMacsOdd &&
           tiles <= (double)(K <= kTinyShortK ? kTinyMaxTilesOddShortK : kTinyMaxTilesOdd));
 }

@@ -308,6 +308,8 @@ def test_tiny_limits():
     assert tiny(1023, 511, 97) and not tiny(1025, 511, 97) and not tiny(1024, 512, 97 + 15) and not tiny(4001, 131, 127)
     assert tiny(512, 1257, 80) and tiny(1025, 511, 96) and not tiny(1023, 1023, 31)
     assert tiny(512, 512, 192) and not tiny(512, 512, 208) and not tiny(512, 528, 192)
+    assert tiny(608, 1024, 96) and tiny(4800, 128, 64, COL) and not tiny(609, 1024, 64) and not tiny(608, 1024, 112)
+    assert tiny(512, 608, 128) and not tiny(512, 624, 128) and not tiny(512, 608, 144)
 
 
 @pytest.mark.gpu
@@ -315,7 +317,9 @@ def test_tiny_limits():
 @pytest.mark.parametrize("dtype", ["int8", "int8_int16", "int8_int8"])
 @pytest.mark.parametrize("M,N,K,layout,pad,off", [(128, 512, 512, ROW, 0, 0), (640, 89, 416, COL, 0, 0), (511, 511, 385, ROW, 0, 1),
                                                   (1023, 511, 90, COL, 1, 3), (512, 512, 128, ROW, 4, 0), (512, 512, 384, ROW, 0, 0),
-                                                  (512, 512, 192, COL, 0, 0), (384, 384, 512, ROW, 0, 0), (384, 400, 512, COL, 0, 0)])
+                                                  (512, 512, 192, COL, 0, 0), (384, 384, 512, ROW, 0, 0), (384, 400, 512, COL, 0, 0),
+                                                  (608, 1024, 96, COL, 0, 0), (4800, 128, 64, ROW, 0, 0), (512, 608, 128, ROW, 0, 0),
+                                                  (416, 512, 256, COL, 0, 0), (416, 528, 256, ROW, 0, 0)])
 def test_tiny_limits_results(dtype, M, N, K, layout, pad, off):
     A, B = _operands("int8", M, N, K, layout, M + N)
     C = U.run(dtype, A, B, layout, lda=K + pad, ldb=B.shape[1] + pad, ldc=N + pad, a_off=off, c_off=off, shift=8)
